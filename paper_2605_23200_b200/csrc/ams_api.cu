@@ -264,6 +264,7 @@ int ams_compress(ams_state *st, void *k_pages, void *v_pages, int64_t num_pages,
     p.quotas = (int *)(st->ws + y.quotas); p.keep_idx = (int *)(st->ws + y.keep_idx);
     p.raw_cuts = (int *)(st->ws + y.raw_cuts);
     p.mass_dbg = dbg ? dbg->mass : nullptr;
+    p.seg_out = dbg && (dbg->n_segments || dbg->seg_bounds || dbg->quotas || dbg->keep_idx);
     p.part = (float *)(st->ws + y.part); p.fin = (float *)(st->ws + y.fin);
     p.slice_len = y.slice_len; p.n_slices = y.n_slices;
     p.rows_pad = scorer_id == AMS_SCORER_TOVA ? rows_padded(p.rows) : kHeadDim;
@@ -312,11 +313,8 @@ int ams_compress(ams_state *st, void *k_pages, void *v_pages, int64_t num_pages,
         cudaError_t e = cudaSuccess;
         if (dbg->scores && e == cudaSuccess) e = cudaMemcpyAsync(dbg->scores, p.scores, U * p.T_cap * 4, cudaMemcpyDeviceToDevice, s);
         if (dbg->usage && e == cudaSuccess) e = cudaMemcpyAsync(dbg->usage, p.usage, U * p.T_cap * 4, cudaMemcpyDeviceToDevice, s);
-        if (dbg->n_segments && e == cudaSuccess) e = cudaMemcpyAsync(dbg->n_segments, p.n_seg, U * 4, cudaMemcpyDeviceToDevice, s);
-        if (dbg->seg_bounds && e == cudaSuccess) e = cudaMemcpyAsync(dbg->seg_bounds, p.seg_bounds, U * (size_t)(p.seg_cap + 1) * 4, cudaMemcpyDeviceToDevice, s);
-        if (dbg->quotas && e == cudaSuccess) e = cudaMemcpyAsync(dbg->quotas, p.quotas, U * (size_t)p.seg_cap * 4, cudaMemcpyDeviceToDevice, s);
-        if (dbg->keep_idx && e == cudaSuccess) e = cudaMemcpyAsync(dbg->keep_idx, p.keep_idx, U * (size_t)p.Tk * 4, cudaMemcpyDeviceToDevice, s);
         if (e != cudaSuccess) rc = AMS_ERR_CUDA;
+        if (rc == AMS_OK && p.seg_out) rc = launch_inspect(p, *dbg, ctx);
         if (rc == AMS_OK && dbg->prev_kept && dbg->retained_iou) rc = launch_retained_iou(p, dbg->prev_kept, dbg->retained_iou, ctx);
     }
     if (rc == AMS_OK) rc = launch_gather(p, ctx);

@@ -47,6 +47,7 @@ struct DevParams {
     int *keep_idx;                    // [Tk]
     int *raw_cuts;                    // [S + 1]  cut after the token that reaches mass quantile k (T: none)
     float *mass_dbg;                  // [T_cap] or null
+    int seg_out;                      // segments and quotas are wanted by the caller: write n_seg, seg_bounds, quotas
     // scorer scratch
     float *part;                      // per (unit, slice) partials
     float *fin;                       // per unit finals
@@ -262,7 +263,9 @@ int launch_score_keydiff(const DevParams &p, LaunchCtx &ctx);
 bool expected_supported(const DevParams &p);
 int launch_score_expected(const DevParams &p, LaunchCtx &ctx);
 bool segsel_supported(const DevParams &p);   // shared-memory need of the selection kernels fits (always, within the configuration limits)
-int launch_segsel(const DevParams &p, LaunchCtx &ctx); // Algorithm 1 steps 1-5: three kernels
+int launch_segsel(const DevParams &p, LaunchCtx &ctx); // Algorithm 1 steps 1-5: k_mass_scan, then launch_select
+size_t select_smem_bytes(const DevParams &p);
+int launch_select(const DevParams &p, LaunchCtx &ctx);
 int launch_gather(const DevParams &p, LaunchCtx &ctx);
 int launch_smooth_usage(const DevParams &p, const float *src, float *dst, int k, LaunchCtx &ctx);
 // First kernel of an event: validates lengths and page ids, writes the effective lengths (lens_in: the caller's).
@@ -297,6 +300,7 @@ inline bool grant_dynamic_smem(K kernel, size_t smem, SmemGrant &g)
     }
     return true;
 }
+int launch_inspect(const DevParams &p, const ams_debug_views &v, LaunchCtx &ctx); // segments, quotas, kept positions -> views
 int launch_retained_iou(const DevParams &p, const int *prev_kept, float *out, LaunchCtx &ctx); // before the lengths are rewritten
 
 } // namespace ams

@@ -55,6 +55,25 @@ __global__ void __launch_bounds__(128) k_retained_iou(DevParams p, const int *pr
     out[uid] = either > 0 ? __fdiv_rn((float)both, (float)either) : 0.0f;
 }
 
+// Inspection views of the selection, one block per unit: segments, quotas and kept positions go to the caller's arrays in
+// one launch.  Units that were skipped are left untouched.
+__global__ void __launch_bounds__(256) k_inspect(DevParams p, ams_debug_views v)
+{
+    wait_for_previous_kernel(); // the selection
+    const int uid = blockIdx.x, tid = threadIdx.x;
+    const int T = p.seq_lens[(uid / p.H) % p.B];
+    if (T <= p.Tk || T > p.T_cap) return;
+    const int n = p.n_seg[uid];
+    const size_t sc = (size_t)p.seg_cap, u = (size_t)uid;
+    if (v.n_segments && tid == 0) v.n_segments[uid] = n;
+    if (v.seg_bounds)
+        for (int i = tid; i <= n; i += 256) v.seg_bounds[u * (sc + 1) + i] = p.seg_bounds[u * (sc + 1) + i];
+    if (v.quotas)
+        for (int i = tid; i < n; i += 256) v.quotas[u * sc + i] = p.quotas[u * sc + i];
+    if (v.keep_idx)
+        for (int i = tid; i < p.Tk; i += 256) v.keep_idx[u * p.Tk + i] = p.keep_idx[u * p.Tk + i];
+}
+
 // First kernel of an event, one block per sequence: the effective length the other kernels work with.
 // A sequence within the budget has nothing to evict (effective length 0: every kernel skips it).  A
 // sequence over the configured capacity, shorter than the observation window, or whose block-table
@@ -120,6 +139,13 @@ int launch_expire_wait(int *status, uint32_t polls, cudaStream_t s)
 {
     k_expire_wait<<<1, 1, 0, s>>>(status, polls);
     return cudaGetLastError() == cudaSuccess ? AMS_OK : AMS_ERR_CUDA;
+}
+
+int launch_inspect(const DevParams &p, const ams_debug_views &v, LaunchCtx &ctx)
+{
+    if (launch_after(k_inspect, dim3((unsigned)(p.L * p.B * p.H)), dim3(256), 0, ctx.s, p, v) != cudaSuccess) return AMS_ERR_CUDA;
+    ctx.mark(kKernQuota);
+    return AMS_OK;
 }
 
 int launch_retained_iou(const DevParams &p, const int *prev_kept, float *out, LaunchCtx &ctx)
