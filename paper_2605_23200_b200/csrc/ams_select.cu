@@ -4,18 +4,18 @@
 // block per unit, one kept bit per token in shared memory.
 //
 // Selection order is (score key descending, position ascending), a strict total order, so a segment and its quota have
-// exactly one answer however it is found.  The block searches all segments at once, in three walks over the unit's
-// scores (the first from L2, the others mostly from L1):
-//   1. smallest and largest key of every segment;
-//   2. a histogram per segment, its bins spread evenly over that range of keys;
-//   3. a warp per segment has found the bin of the q-th key: keys above it are kept, the few inside it go to a list
-//      in which every entry counts the entries of its segment before it.
-// A segment whose bin holds too many keys gets another histogram over that bin first (ties by the hundred end with a
-// bin of one key).  The work per token does not depend on how long the segments are, every warp has the same share of
-// it, and the number of block-wide steps is fixed; fixing key bits segment by segment, as this kernel once did, is a
-// chain of 16 to 20 dependent warp-wide counts per segment.
-// The backfill takes its bound from the best rejected key of every chunk, which walk 3 leaves behind, instead of
-// walking the sequence twice more.
+// exactly one answer however it is found.  Finding the q-th largest key is what costs.  It is bound by latency and issue
+// slots, not by memory (4 bytes per token, from L2):
+//   * a segment of at most 256 tokens lives in the registers of one warp.  A histogram of 128 bins over the segment's own
+//     range of keys leads to the bin of the q-th key, a second one over that bin usually ends the search: two short
+//     steps instead of 16 to 20 dependent warp-wide counts, one per key bit.
+//   * longer segments are searched together by the whole block, in three walks over their 256-token pieces: range of
+//     keys, histogram per segment, then keys above the threshold's bin are kept and the few inside it go to a list in which
+//     every entry counts the entries of its segment before it.  (A bin that is still crowded gets another histogram
+//     first; ties by the hundred end with a bin of one key.)  Every warp has the same share of the walks whatever the
+//     lengths of the segments.
+// The backfill takes its bound from the best rejected key of every piece, which the searches leave behind, and looks only
+// at pieces that reach it, instead of walking the sequence twice.
 #include "ams_common.cuh"
 #include "ams_select.cuh"
 
@@ -26,18 +26,22 @@ using namespace sel;
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kBatch = 256;         // segments searched together
-constexpr int kMaxBins = 1024;      // histogram bins per segment
-constexpr int kMaxChunks = 256;     // entries of the table of best rejected keys
-constexpr int kGroup = 8;           // 32-token windows whose scores a warp fetches together
+constexpr int kPiece = 256;         // tokens a warp holds in registers, eight per lane
+constexpr int kPer = kPiece / 32;
+constexpr int kWarpBins = 128;      // bins of a warp's own histogram
+constexpr int kBatch = 256;         // long segments searched together
+constexpr int kMaxBins = 1024;      // histogram bins per long segment
+constexpr int kBest = 1024;         // entries of the table of best rejected keys
 
-// Working arrays of the search, one entry per segment of the batch.
+// Working arrays of the search of long segments, one entry per segment of the batch.
 struct SegTab {
-    unsigned lo[kBatch], hi[kBatch]; // range of keys of the histogram (hi inclusive)
+    unsigned lo[kBatch], w[kBatch];  // the histogram covers the keys [lo, lo + w]
     unsigned L[kBatch], U[kBatch];   // keys >= U win, keys < L lose
     int above[kBatch];               // keys above the range of the histogram
     int r[kBatch], m[kBatch];        // r of the m keys in [L, U) win
     int base[kBatch], cnt[kBatch];   // part of the list
+    unsigned short seg[kBatch];
+    int piece0[kBatch + 1];          // first piece
     unsigned char shift[kBatch];     // bin = (key - lo) >> shift
     unsigned char state[kBatch];
 };
@@ -45,39 +49,38 @@ enum { kDone = 0, kSearch = 1, kTies = 2 };
 
 template <int NT> struct Tune {
     static constexpr int kBins = NT <= 256 ? 8192 : 16384; // histogram bins of a batch
-    static constexpr int kList = NT <= 256 ? 1024 : 2048;  // candidates
+    static constexpr int kList = NT <= 256 ? 1024 : 2048;  // candidates, of the long segments and then of the backfill
 };
 
-struct SelSmem { size_t mask, ms, bounds, quota, tab, hist, list, total; };
+struct SelSmem { size_t mask, ms, bounds, quota, best, list, hist, lhist, tab, total; };
 template <int NT>
-__host__ __device__ inline SelSmem sel_smem(int T_cap, int sc, int S)
+__host__ __device__ inline SelSmem sel_smem(int T_cap, int sc, int S, bool longs)
 {
     SelSmem m;
     size_t o = 0;
-    m.mask = o;   o += (size_t)((T_cap + 31) / 32 + 1) * 4;
+    m.mask = o;   o += (size_t)((T_cap + 31) / 32 + 2) * 4;
     o = (o + 15) & ~(size_t)15;
     m.ms = o;     o += (size_t)sc * 8;
     m.bounds = o; o += (size_t)(sc + 1) * 4;
     m.quota = o;  o += (size_t)sc * 4;
     o = (o + 15) & ~(size_t)15;
-    m.tab = o;    o += sizeof(SegTab);
-    o = (o + 15) & ~(size_t)15;
-    m.hist = o;   // also: scratch of the quota computation, which comes before
-    const size_t h = (size_t)Tune<NT>::kBins * 4, q = (size_t)(S + 1) * 12 + (size_t)sc * 4;
-    o += (h > q ? h : q);
-    o = (o + 15) & ~(size_t)15;
-    m.list = o;   o += (size_t)Tune<NT>::kList * 8;
+    m.best = o;   o += (size_t)kBest * 4;
+    m.hist = o;   o += (size_t)(NT / 32) * kWarpBins * 4;
+    // the quota computation, which comes first, uses the list (and what follows) as scratch
+    const size_t q = (size_t)(S + 1) * 8 + (size_t)sc * 4, l = (size_t)Tune<NT>::kList * 8 + (longs ? (size_t)Tune<NT>::kBins * 4 + sizeof(SegTab) : 0);
+    m.list = o;
+    m.lhist = o + (size_t)Tune<NT>::kList * 8;
+    m.tab = m.lhist + (size_t)Tune<NT>::kBins * 4;
+    o += q > l ? q : l;
     m.total = (o + 15) & ~(size_t)15;
     return m;
 }
 
 struct SelShared {
     int wc[2][32];   // per-warp counts of even / odd rounds of a block-wide count
-    unsigned cmax[kMaxChunks];
-    int n_list, n_clist, total;
+    int n_list, n_long, total;
     unsigned bound;
     int n_merged, n_seg, level, rem;
-    unsigned short clist[kMaxChunks];
 };
 
 __device__ __forceinline__ int warp_sum(int v) { return (int)__reduce_add_sync(kFull, v); }
@@ -143,57 +146,68 @@ __device__ int block_distribute(int sign, int D, const int *cap, int *quota, con
     }
     __syncthreads();
     const int level = sh.level, rem = sh.rem, left = sh.total;
-    for (int i = tid; i < n_seg; i += NT) {
-        int g = min(cap[i], level);
-        if (rem > 0 && cap[i] > level) {
-            int rank = 0;
+    for (int i = tid >> 5; i < n_seg; i += NT / 32) { // a warp per segment: its rank in visiting order among those with room
+        const int ci = cap[i];
+        int g = min(ci, level);
+        if (rem > 0 && ci > level) {
             const u64 Mi = M[i];
-            for (int j = 0; j < n_seg; ++j) {
-                if (cap[j] <= level) continue;
+            int rank = 0;
+            for (int j = lane; j < n_seg; j += 32) {
                 const u64 Mj = M[j];
-                rank += sign > 0 ? (Mj > Mi || (Mj == Mi && j < i)) : (Mj < Mi || (Mj == Mi && j > i));
+                const bool before = sign > 0 ? (Mj > Mi || (Mj == Mi && j < i)) : (Mj < Mi || (Mj == Mi && j > i));
+                rank += cap[j] > level && before;
             }
-            g += rank < rem;
+            g += warp_sum(rank) < rem;
         }
-        quota[i] += sign * g;
+        if (lane == 0) quota[i] += sign * g;
     }
     __syncthreads();
     return left;
 }
 
+// floor(x / y) for a quotient below 2^20 and x < 2^62: the fp64 quotient is off by less than one, the remainder corrects it.
+__device__ __forceinline__ u64 quotient(u64 x, u64 y)
+{
+    u64 q = (u64)((double)x / (double)y);
+    const long long rem = (long long)(x - q * y);
+    if (rem < 0) --q;
+    else if (rem >= (long long)y) ++q;
+    return q;
+}
+
 // Merge of short and split of long segments, quotas with their adjustment (Section 3.3 of the paper; Algorithm 1 steps
 // 3-4): bounds[0..n], quota[0..n).  Returns n, or -1 if the tables cannot hold the segments.  Bq: the budget less the
-// must-keep positions.  `tmp`: 3 (S + 1) + seg_cap ints.
+// must-keep positions.  `tmp`: 2 (S + 1) + seg_cap ints.
 template <int NT>
 __device__ int segments_and_quotas(const DevParams &p, int uid, int T, int Bq, u64 *Ms, int *bounds, int *quota, int *tmp,
                                    SelShared &sh, int &round)
 {
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    int *raw = tmp, *merged = raw + p.S + 1, *poff = merged + p.S + 1, *cap = poff + p.S + 1;
+    int *merged = tmp, *poff = merged + p.S + 1, *cap = poff + p.S + 1;
     const u64 *C = p.cbuf + (size_t)uid * p.T_cap;
     const u64 SH = C[T - 1];
     if (warp == 0) {
-        // raw cuts of the mass quantiles, found by the scan kernel (a cut at or beyond T means "none")
-        for (int k = lane + 1; k < p.S; k += 32)
-            raw[k] = p.fixed_seg ? (int)(((long long)k * T) / p.S) // component ablation: boundary k at floor(k T / S)
-                                 : p.raw_cuts[(size_t)uid * (p.S + 1) + k];
-        __syncwarp();
-        int nm = 0;
-        if (lane == 0) { // merge short raw segments forward, fold a short tail left
-            int last = 0, start = 0;
-            merged[nm++] = 0;
-            for (int k = 1; k < p.S; ++k) {
-                const int e = raw[k];
-                if (e <= last || e >= T) continue;
-                last = e;
-                if (e - start >= p.l_min) { merged[nm++] = e; start = e; }
+        // raw cuts of the mass quantiles, ascending, found by the scan kernel (a cut at or beyond T means "none"); short raw
+        // segments merge forward: the next boundary is the first cut at least l_min past the last one
+        int nm = 0, start = 0;
+        if (lane == 0) merged[0] = 0;
+        for (int k0 = 1; k0 < p.S; k0 += 32) {
+            const int k = k0 + lane;
+            int e = T;
+            if (k < p.S) e = p.fixed_seg ? (int)(((long long)k * T) / p.S) // component ablation: boundary k at floor(k T / S)
+                                         : p.raw_cuts[(size_t)uid * (p.S + 1) + k];
+            for (;;) {
+                const unsigned can = __ballot_sync(kFull, e < T && e - start >= p.l_min);
+                if (!can) break;
+                start = __shfl_sync(kFull, e, __ffs(can) - 1);
+                ++nm;
+                if (lane == 0) merged[nm] = start;
             }
-            if (nm > 1 && T - start < p.l_min) --nm;
-            merged[nm] = T; // nm segments
         }
+        if (nm == 0 || T - start >= p.l_min) ++nm; // (otherwise the short tail folds left)
+        if (lane == 0) merged[nm] = T;
         __syncwarp();
-        nm = __shfl_sync(kFull, nm, 0);
         int off = 0; // pieces of the segments before
         for (int i0 = 0; i0 < nm; i0 += 32) {
             const int i = i0 + lane;
@@ -230,7 +244,7 @@ __device__ int segments_and_quotas(const DevParams &p, int uid, int T, int Bq, u
     for (int i = tid; i < n_seg; i += NT) {
         const int L = bounds[i + 1] - bounds[i];
         long long qi = max(0, min(p.q_min, L));
-        if (Trem >= 0) qi += (long long)((2ull * (u64)Trem * Ms[i] + SHq) / (2ull * SHq));
+        if (Trem >= 0) qi += (long long)quotient(2ull * (u64)Trem * Ms[i] + SHq, 2ull * SHq);
         if (qi > L) qi = L;
         quota[i] = (int)qi;
         sq += (int)qi;
@@ -252,74 +266,187 @@ __device__ int segments_and_quotas(const DevParams &p, int uid, int T, int Bq, u
     return n_seg;
 }
 
-// ------------------------------------------------------------------------------------------ walks
+// ------------------------------------------------------------------------------------------ searches
 
-// Walks the tokens [bounds[0], bounds[n]) of the batch's segments in windows of 32 (one token per lane, aligned to words of
-// the kept mask); a warp takes one run of consecutive windows, kGroup of them fetched ahead.  f(t, s, in, key, crossing):
-// s is the lane's segment; `crossing` (warp-uniform) says that the lanes may differ in it or in `in`; enter(s) is called
-// when the warp moves to segment s as a whole, done(w) after the last window of a run or of a chunk of 2^chunk_log windows.
-template <int NT, typename Enter, typename F, typename Done>
-__device__ __forceinline__ void walk(const float *g, const int *bounds, int n, int chunk_log, Enter enter, F f, Done done)
+struct Cut { unsigned key; int ties; }; // the keys above `key` win, and `ties` of those equal to it (-1: all of them)
+
+// Bin of a warp's histogram of kWarpBins bins that holds the q-th key from the top (1 <= q <= number of keys counted): bin,
+// keys in it, keys above it.
+__device__ __forceinline__ void find_bin(const unsigned *hist, int q, int &bin, int &m, int &above)
 {
-    constexpr int NW = NT / 32;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int A = bounds[0], E = bounds[n];
-    const int w0 = A >> 5, n_win = ((E + 31) >> 5) - w0;
-    const int per = ((n_win + NW - 1) / NW + kGroup - 1) / kGroup * kGroup;
-    const int wb = w0 + warp * per, we = min(w0 + n_win, wb + per);
-    if (wb >= we) return;
-    int s = 0;
-    { // the segment of the run's first token
-        int hi = n;
-        const int t = max(A, wb * 32);
-        while (hi - s > 1) {
-            const int mid = (s + hi) >> 1;
-            if (bounds[mid] <= t) s = mid; else hi = mid;
-        }
+    const int lane = threadIdx.x & 31;
+    const uint4 v = reinterpret_cast<const uint4 *>(hist)[31 - lane]; // lane 0 has the top four bins
+    const int c0 = (int)v.w, c1 = c0 + (int)v.z, c2 = c1 + (int)v.y, c3 = c2 + (int)v.x;
+    const int inc = warp_incl_scan(c3), exc = inc - c3, rest = q - exc;
+    const int src = __ffs(__ballot_sync(kFull, inc >= q)) - 1; // the first lane that covers q
+    const int i = (rest > c0) + (rest > c1) + (rest > c2);
+    const int below = i == 0 ? 0 : (i == 1 ? c0 : (i == 2 ? c1 : c2)), upto = i == 0 ? c0 : (i == 1 ? c1 : (i == 2 ? c2 : c3));
+    bin = __shfl_sync(kFull, (31 - lane) * 4 + 3 - i, src);
+    m = __shfl_sync(kFull, upto - below, src);
+    above = __shfl_sync(kFull, exc + below, src);
+}
+
+// The q-th largest (0 < q < n) of n keys in a warp's registers, kPL per lane, key number j * 32 + lane in register j, unused
+// registers 0.  hist: kWarpBins words of the warp's own.
+template <int kPL>
+__device__ __forceinline__ Cut warp_cut(const unsigned (&k)[kPL], int n, int q, unsigned *hist)
+{
+    const int lane = threadIdx.x & 31, room = n - lane;
+    unsigned mx = 0u, mn = kFull;
+#pragma unroll
+    for (int j = 0; j < kPL; ++j) {
+        mx = max(mx, k[j]);
+        mn = min(mn, j * 32 < room ? k[j] : kFull);
     }
-    int next = bounds[s + 1];
-    enter(s);
-    for (int g0 = wb; g0 < we; g0 += kGroup) {
-        float x[kGroup];
+    mx = __reduce_max_sync(kFull, mx);
+    mn = __reduce_min_sync(kFull, mn);
+    if (mn == mx) return {mn, q};
+    if (mn == 0u) { // NaN scores (and unused registers) stay out of the histogram
+        int c = 0;
+        mn = kFull;
 #pragma unroll
-        for (int j = 0; j < kGroup; ++j) {
-            const int t = (g0 + j) * 32 + lane;
-            x[j] = (g0 + j < we && t >= A && t < E) ? g[t] : 0.0f;
-        }
+        for (int j = 0; j < kPL; ++j) { c += k[j] > 0u; mn = min(mn, k[j] - 1u); }
+        c = warp_sum(c);
+        if (c < q) return {0u, q - c};
+        mn = __reduce_min_sync(kFull, mn) + 1u;
+    }
+    unsigned lo = mn, w = mx - mn;
+    for (;;) {
+        const int shift = max(0, 25 - __clz(w)); // w >> shift < kWarpBins
+        reinterpret_cast<uint4 *>(hist)[lane] = make_uint4(0, 0, 0, 0);
+        __syncwarp();
 #pragma unroll
-        for (int j = 0; j < kGroup; ++j) {
-            const int w = g0 + j;
-            if (w >= we) break;
-            const int ts = w * 32, t = ts + lane;
-            const unsigned key = score_key(x[j]);
-            if (ts >= next) {
-                while (ts >= next) next = bounds[++s + 1];
-                enter(s);
-            }
-            if (ts >= A && ts + 32 <= next) {
-                f(t, s, true, key, false);
-            } else {
-                const bool in = t >= A && t < E;
-                int sl = s;
-                if (in) while (t >= bounds[sl + 1]) ++sl;
-                f(t, sl, in, key, true);
-            }
-            if ((((w + 1) >> chunk_log) << chunk_log) == w + 1 || w + 1 == we) done(w);
+        for (int j = 0; j < kPL; ++j) {
+            const unsigned d = k[j] - lo;
+            if (d <= w) atomicAdd(&hist[d >> shift], 1u);
         }
+        __syncwarp();
+        int bin, m, above;
+        find_bin(hist, q, bin, m, above);
+        q -= above;
+        lo += (unsigned)bin << shift;
+        if (q == m) return {lo, -1};
+        w = min((1u << shift) - 1u, w - ((unsigned)bin << shift));
+        if (w == 0u) return {lo, q};
+        __syncwarp();
     }
 }
 
-// A warp finds the bin of segment s that holds its q-th key and what is left to decide in it.
-__device__ __forceinline__ void find_bin(SegTab &tb, const unsigned *hist, int nb, int s, int q)
+// Kept bits of a piece of at most kPiece tokens from position a: lane j's word holds tokens a + 32 j .., shifted onto
+// the words of the mask.
+__device__ __forceinline__ void mask_or(unsigned *mask, int a, unsigned word)
 {
     const int lane = threadIdx.x & 31;
-    const uint4 *h4 = reinterpret_cast<const uint4 *>(hist + s * nb);
-    int above = tb.above[s];
+    const unsigned prev = __shfl_up_sync(kFull, word, 1);
+    const unsigned w = __funnelshift_l(lane ? prev : 0u, word, a & 31);
+    if (lane <= kPer && w) atomicOr(&mask[(a >> 5) + lane], w);
+}
+
+// Best rejected key of a piece (slot): one entry per eight lanes while there are few pieces, one per piece otherwise.
+__device__ __forceinline__ void note_best(unsigned *best, int slot, bool fine, unsigned key)
+{
+    const int lane = threadIdx.x & 31;
+    if (fine) {
+#pragma unroll
+        for (int d = 1; d < 8; d <<= 1) key = max(key, __shfl_xor_sync(kFull, key, d));
+        if ((lane & 7) == 0) best[slot * 4 + (lane >> 3)] = key;
+    } else {
+        key = __reduce_max_sync(kFull, key);
+        if (lane == 0) atomicMax(&best[slot & (kBest - 1)], key);
+    }
+}
+
+__device__ __forceinline__ void load_piece(const float *g, int a, int len, float (&x)[kPer])
+{
+    const float *src = g + a + (threadIdx.x & 31);
+    const int room = len - (int)(threadIdx.x & 31);
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) x[j] = j * 32 < room ? src[j * 32] : __uint_as_float(0x7fffffffu); // NaN: key 0
+}
+
+// One segment of at most kPiece tokens.
+__device__ __forceinline__ void warp_segment(const float (&x)[kPer], unsigned *mask, unsigned *best, unsigned *hist, int slot, bool fine,
+                                             int a, int L, int q, int ns, int t_last)
+{
+    const int lane = threadIdx.x & 31, room = L - lane;
+    unsigned k[kPer];
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) k[j] = score_key(x[j]);
+    Cut cut = {kFull, 0};                    // none of it
+    if (q >= L) cut = {0u, -1};              // all of it
+    else if (q > 0) cut = warp_cut<kPer>(k, L, q, hist);
+    const bool plain = a >= ns && a + L <= t_last; // no must-keep position in it
+    auto may_fill = [&](int j) { return plain || (a + j * 32 + lane >= ns && a + j * 32 + lane < t_last); };
+    unsigned word = 0, rej = 0;
+    if (cut.ties < 0 && cut.key > 0u) {      // the usual end: the keys from cut.key on
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const bool kept = k[j] >= cut.key;
+            const unsigned bal = __ballot_sync(kFull, kept);
+            if (lane == j) word = bal;
+            if (!kept && may_fill(j)) rej = max(rej, k[j]);
+        }
+    } else {                                 // the first ties in position order
+        int seen = 0;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const bool in = j * 32 < room, tie = in && k[j] == cut.key;
+            const unsigned tb = __ballot_sync(kFull, tie);
+            const bool kept = in && (k[j] > cut.key || (tie && (cut.ties < 0 || seen + __popc(tb & ((1u << lane) - 1u)) < cut.ties)));
+            seen += __popc(tb);
+            const unsigned bal = __ballot_sync(kFull, kept);
+            if (lane == j) word = bal;
+            if (!kept && may_fill(j)) rej = max(rej, k[j]);
+        }
+    }
+    mask_or(mask, a, word);
+    note_best(best, slot, fine, rej);
+}
+
+// Walks the pieces of the batch's long segments, a run of consecutive pieces per warp, the next piece's scores on their way
+// while f(i, piece, a, len, x) works on this one's; i is the segment's entry in the table, enter(i) announces it.
+template <int NT, typename Enter, typename F>
+__device__ __forceinline__ void walk_long(const float *g, const int *bounds, const SegTab &tb, int n, Enter enter, F f)
+{
+    constexpr int NW = NT / 32;
+    const int warp = threadIdx.x >> 5, n_piece = tb.piece0[n];
+    const int p0 = (int)((long long)n_piece * warp / NW), p1 = (int)((long long)n_piece * (warp + 1) / NW);
+    if (p0 >= p1) return;
+    int i = 0;
+    for (int hi = n; hi - i > 1;) {
+        const int mid = (i + hi) >> 1;
+        if (tb.piece0[mid] <= p0) i = mid; else hi = mid;
+    }
+    int next = tb.piece0[i + 1], e = bounds[tb.seg[i] + 1], a = bounds[tb.seg[i]] + (p0 - tb.piece0[i]) * kPiece;
+    float x[kPer];
+    load_piece(g, a, e - a, x);
+    enter(i);
+    for (int pc = p0; pc < p1; ++pc) {
+        float y[kPer];
+        const int ca = a, cl = min(kPiece, e - a), ci = i;
+        if (pc + 1 < p1) {
+            a += kPiece;
+            if (pc + 1 == next) { ++i; next = tb.piece0[i + 1]; a = bounds[tb.seg[i]]; e = bounds[tb.seg[i] + 1]; }
+            load_piece(g, a, e - a, y);
+        }
+        f(ci, pc, ca, cl, x);
+        if (i != ci) enter(i);
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) x[j] = y[j];
+    }
+}
+
+// A warp finds the bin of long segment i that holds its q-th key and what is left to decide in it.
+__device__ __forceinline__ void find_long_bin(SegTab &tb, const unsigned *hist, int nb, int i, int q)
+{
+    const int lane = threadIdx.x & 31;
+    const uint4 *h4 = reinterpret_cast<const uint4 *>(hist + i * nb);
+    int above = tb.above[i];
     uint4 v = make_uint4(0, 0, 0, 0);
     int c = (nb + 127) / 128 - 1, sum = 0;
     for (;; --c) { // 128 bins at a time from the top
-        const int i = c * 32 + lane;
-        v = i * 4 < nb ? h4[i] : make_uint4(0, 0, 0, 0);
+        const int k = c * 32 + lane;
+        v = k * 4 < nb ? h4[k] : make_uint4(0, 0, 0, 0);
         sum = (int)(v.x + v.y + v.z + v.w);
         above += warp_sum(sum);
         if (c == 0 || above >= q) break;
@@ -329,42 +456,40 @@ __device__ __forceinline__ void find_bin(SegTab &tb, const unsigned *hist, int n
         int run = before, bin = 0, m = 0;
         const int cnt[4] = {(int)v.w, (int)v.z, (int)v.y, (int)v.x};
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            if (run < q && q <= run + cnt[i]) { bin = c * 128 + lane * 4 + 3 - i; m = cnt[i]; above = run; }
-            run += cnt[i];
+        for (int j = 0; j < 4; ++j) {
+            if (run < q && q <= run + cnt[j]) { bin = c * 128 + lane * 4 + 3 - j; m = cnt[j]; above = run; }
+            run += cnt[j];
         }
-        const unsigned lo = tb.lo[s], hi = tb.hi[s], sft = tb.shift[s];
-        const unsigned L = lo + ((unsigned)bin << sft);
-        const unsigned U = (unsigned)bin == (hi - lo) >> sft ? hi + 1u : lo + ((unsigned)(bin + 1) << sft);
+        const unsigned sft = tb.shift[i], off = (unsigned)bin << sft;
+        const unsigned L = tb.lo[i] + off, w = min((1u << sft) - 1u, tb.w[i] - off);
         const int r = q - above;
-        tb.above[s] = above;
-        tb.r[s] = r;
-        tb.m[s] = m;
-        tb.U[s] = r == m ? L : U;
-        tb.L[s] = L;
-        tb.state[s] = r == m ? kDone : (U - L == 1u ? kTies : kSearch);
+        tb.above[i] = above;
+        tb.r[i] = r;
+        tb.m[i] = m;
+        tb.L[i] = L;
+        tb.U[i] = r == m ? L : L + w + 1u;
+        tb.state[i] = r == m ? kDone : (w == 0u ? kTies : kSearch);
     }
 }
 
-__device__ __forceinline__ int bin_shift(unsigned width_less_1, int nb) // smallest shift with width_less_1 >> shift < nb
+__device__ __forceinline__ int bin_shift(unsigned w, int nb) // smallest shift with w >> shift < nb
 {
-    const int bits = 32 - __clz(width_less_1), have = 31 - __clz(nb);
-    return max(0, bits - have);
+    return max(0, __clz(nb) + 1 - __clz(w)); // nb a power of two: log2(nb) = 31 - clz(nb)
 }
 
-// Top-q_i of the n <= kBatch segments at `bounds`: kept bits into mask, best rejected keys (must-keep positions apart)
-// into the chunk table.
+// Top-q_i of the n <= kBatch long segments of the table: kept bits into mask, best rejected keys (must-keep positions
+// apart) into `best`, pieces taking the slots from slot0 on.
 template <int NT>
-__device__ void select_batch(const float *g, const int *bounds, const int *quota, int n, unsigned *mask, SegTab &tb, unsigned *hist, uint2 *list,
-                             int ns, int t_last, int chunk_log, SelShared &sh)
+__device__ void select_long(const float *g, const int *bounds, const int *quota, int n, unsigned *mask, unsigned *best, int slot0, bool fine,
+                            SegTab &tb, unsigned *hist, uint2 *list, int ns, int t_last, SelShared &sh)
 {
     constexpr int NW = NT / 32, kList = Tune<NT>::kList;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int nb = Tune<NT>::kBins / n;
     nb = min(kMaxBins, 1 << (31 - __clz(nb)));
 
-    // ---- walk 1: range of keys
-    for (int i = tid; i < n; i += NT) { tb.lo[i] = kFull; tb.hi[i] = 0u; }
+    // ---- walk 1: range of keys (U holds the largest for now)
+    for (int i = tid; i < n; i += NT) { tb.lo[i] = kFull; tb.U[i] = 0u; }
     uint4 *h4 = reinterpret_cast<uint4 *>(hist);
     for (int i = tid; i < n * nb / 4; i += NT) h4[i] = make_uint4(0, 0, 0, 0);
     __syncthreads();
@@ -374,50 +499,56 @@ __device__ void select_batch(const float *g, const int *bounds, const int *quota
         auto flush = [&]() {
             mn = __reduce_min_sync(kFull, mn);
             mx = __reduce_max_sync(kFull, mx);
-            if (lane == 0 && mn <= mx) { atomicMin(&tb.lo[cur], mn); atomicMax(&tb.hi[cur], mx); }
+            if (lane == 0 && mn <= mx) { atomicMin(&tb.lo[cur], mn); atomicMax(&tb.U[cur], mx); }
             mn = kFull; mx = 0u;
         };
-        walk<NT>(g, bounds, n, 30, [&](int s) { flush(); cur = s; },
-                 [&](int, int s, bool in, unsigned key, bool crossing) {
-                     if (!crossing) { mn = min(mn, key); mx = max(mx, key); }
-                     else if (in) { atomicMin(&tb.lo[s], key); atomicMax(&tb.hi[s], key); }
-                 },
-                 [&](int) { flush(); });
+        walk_long<NT>(g, bounds, tb, n, [&](int i) { flush(); cur = i; },
+                      [&](int, int, int, int len, const float (&x)[kPer]) {
+#pragma unroll
+                          for (int j = 0; j < kPer; ++j) {
+                              const unsigned k = score_key(x[j]);
+                              mx = max(mx, k);
+                              mn = min(mn, j * 32 + lane < len ? k : kFull);
+                          }
+                      });
+        flush();
     }
     __syncthreads();
     for (int i = tid; i < n; i += NT) {
-        const int len = bounds[i + 1] - bounds[i], q = quota[i];
-        const unsigned lo = tb.lo[i], hi = tb.hi[i];
+        const int s = tb.seg[i], len = bounds[s + 1] - bounds[s], q = quota[s];
+        const unsigned lo = tb.lo[i], w = tb.U[i] - lo;
+        tb.w[i] = w;
         tb.above[i] = 0;
         tb.r[i] = q;
         tb.m[i] = len;
-        tb.state[i] = kSearch;
-        tb.L[i] = lo; tb.U[i] = hi + 1u;
-        tb.shift[i] = (unsigned char)bin_shift(hi - lo, nb);
-        if (q <= 0) { tb.state[i] = kDone; tb.L[i] = tb.U[i] = kFull; }
-        else if (q >= len) { tb.state[i] = kDone; tb.L[i] = tb.U[i] = 0u; }
-        else if (lo == hi) tb.state[i] = kTies;
-        if (tb.state[i] != kSearch) tb.shift[i] = 255;
+        tb.L[i] = lo; tb.U[i] = lo + w + 1u;
+        int state = kSearch, shift = bin_shift(w, nb);
+        if (q <= 0) { state = kDone; tb.L[i] = tb.U[i] = kFull; }
+        else if (q >= len) { state = kDone; tb.L[i] = tb.U[i] = 0u; }
+        else if (w == 0u) state = kTies;
+        tb.state[i] = (unsigned char)state;
+        tb.shift[i] = (unsigned char)(state == kSearch ? shift : 255);
     }
     __syncthreads();
 
     // ---- walk 2: histograms, and again over the threshold's bin where that is still crowded
     for (;;) {
         {
-            unsigned lo = 0u, hi = 0u, sft = 255u;
-            int cur = 0;
-            auto load = [&](int s) { cur = s; lo = tb.lo[s]; hi = tb.hi[s]; sft = tb.shift[s]; };
-            walk<NT>(g, bounds, n, 30, load,
-                     [&](int, int s, bool in, unsigned key, bool crossing) {
-                         unsigned l = lo, h = hi, f = sft;
-                         if (crossing && s != cur) { l = tb.lo[s]; h = tb.hi[s]; f = tb.shift[s]; }
-                         if (in && f < 32u && key >= l && key <= h) atomicAdd(&hist[s * nb + ((key - l) >> f)], 1u);
-                     },
-                     [](int) {});
+            unsigned lo = 0u, w = 0u, sft = 255u;
+            unsigned *mine = hist;
+            walk_long<NT>(g, bounds, tb, n, [&](int i) { lo = tb.lo[i]; w = tb.w[i]; sft = tb.shift[i]; mine = hist + i * nb; },
+                          [&](int, int, int, int len, const float (&x)[kPer]) {
+                              if (sft >= 32u) return;
+#pragma unroll
+                              for (int j = 0; j < kPer; ++j) {
+                                  const unsigned d = score_key(x[j]) - lo;
+                                  if (d <= w && j * 32 + lane < len) atomicAdd(&mine[d >> sft], 1u);
+                              }
+                          });
         }
         __syncthreads();
-        for (int s = warp; s < n; s += NW)
-            if (tb.shift[s] < 32) find_bin(tb, hist, nb, s, quota[s]);
+        for (int i = warp; i < n; i += NW)
+            if (tb.shift[i] < 32) find_long_bin(tb, hist, nb, i, quota[tb.seg[i]]);
         __syncthreads();
         // room in the list: segments in order, each with its m candidates
         if (warp == 0) {
@@ -431,73 +562,84 @@ __device__ void select_batch(const float *g, const int *bounds, const int *quota
             if (lane == 0) sh.total = tot;
         }
         __syncthreads();
-        const int limit = sh.total > kList ? kList / kBatch : 384; // most candidates of a segment that are ranked pairwise
+        const int limit = sh.total > kList ? kList / kBatch : 256; // most candidates of a segment that are ranked pairwise
         bool again = false;
         for (int i = tid; i < n; i += NT) {
             tb.shift[i] = 255;
             if (tb.state[i] == kSearch && tb.m[i] > limit) {
-                tb.lo[i] = tb.L[i]; tb.hi[i] = tb.U[i] - 1u;
-                tb.shift[i] = (unsigned char)bin_shift(tb.U[i] - 1u - tb.L[i], nb);
+                const unsigned w = tb.U[i] - 1u - tb.L[i];
+                tb.lo[i] = tb.L[i]; tb.w[i] = w;
+                tb.shift[i] = (unsigned char)bin_shift(w, nb);
                 again = true;
             }
         }
         if (!__syncthreads_or(again)) break;
-        for (int s = warp; s < n; s += NW)
-            if (tb.shift[s] < 32)
-                for (int i = lane; i < nb; i += 32) hist[s * nb + i] = 0u;
+        for (int i = warp; i < n; i += NW)
+            if (tb.shift[i] < 32)
+                for (int k = lane; k < nb; k += 32) hist[i * nb + k] = 0u;
         __syncthreads();
     }
 
     // ---- walk 3: kept bits, candidates, best rejected keys
     {
-        unsigned L = 0u, U = 0u, best = 0u;
-        int cur = 0;
-        walk<NT>(g, bounds, n, chunk_log, [&](int s) { cur = s; L = tb.L[s]; U = tb.U[s]; },
-                 [&](int t, int s, bool in, unsigned key, bool crossing) {
-                     unsigned l = L, u = U;
-                     if (crossing && s != cur) { l = tb.L[s]; u = tb.U[s]; }
-                     const unsigned bal = __ballot_sync(kFull, in && key >= u);
-                     if (lane == 0 && bal) atomicOr(&mask[t >> 5], bal);
-                     if (in && key < u) {
-                         if (key >= l) {
-                             if (tb.state[s] == kSearch) list[atomicAdd(&tb.cnt[s], 1)] = make_uint2(key, (unsigned)t | ((unsigned)s << 24));
-                         } else if (t >= ns && t < t_last) {
-                             best = max(best, key);
-                         }
-                     }
-                 },
-                 [&](int w) {
-                     best = __reduce_max_sync(kFull, best);
-                     if (lane == 0 && best) atomicMax(&sh.cmax[w >> chunk_log], best);
-                     best = 0u;
-                 });
+        unsigned L = 0u, U = 0u;
+        bool search = false;
+        walk_long<NT>(g, bounds, tb, n, [&](int i) { L = tb.L[i]; U = tb.U[i]; search = tb.state[i] == kSearch; },
+                      [&](int i, int pc, int a, int len, const float (&x)[kPer]) {
+                          const bool plain = a >= ns && a + len <= t_last; // no must-keep position in it
+                          unsigned word = 0, rej = 0, cand = 0;
+#pragma unroll
+                          for (int j = 0; j < kPer; ++j) {
+                              const bool in = j * 32 + lane < len;
+                              const unsigned k = score_key(x[j]);
+                              const unsigned bal = __ballot_sync(kFull, in && k >= U);
+                              if (lane == j) word = bal;
+                              if (k < L) {
+                                  if (plain || (a + j * 32 + lane >= ns && a + j * 32 + lane < t_last)) rej = max(rej, k);
+                              } else if (in && k < U) {
+                                  cand |= 1u << j;
+                              }
+                          }
+                          if (search && __any_sync(kFull, cand)) {
+#pragma unroll
+                              for (int j = 0; j < kPer; ++j)
+                                  if ((cand >> j) & 1u)
+                                      list[atomicAdd(&tb.cnt[i], 1)] = make_uint2(score_key(x[j]), (unsigned)(a + j * 32 + lane) | ((unsigned)i << 24));
+                          }
+                          mask_or(mask, a, word);
+                          note_best(best, slot0 + pc, fine, rej);
+                      });
     }
     __syncthreads();
-    for (int i = tid; i < sh.total; i += NT) { // every candidate ranks itself
-        const uint2 v = list[i];
-        const int s = (int)(v.y >> 24), t = (int)(v.y & 0xffffffu);
-        const int b = tb.base[s], e = b + tb.m[s];
+    auto rejected = [&](unsigned key, int i, int t) { // a candidate that did not make it
+        const int slot = slot0 + tb.piece0[i] + (t - bounds[tb.seg[i]]) / kPiece;
+        if (t >= ns && t < t_last) atomicMax(&best[fine ? slot * 4 : slot & (kBest - 1)], key);
+    };
+    for (int c = tid; c < sh.total; c += NT) { // every candidate ranks itself
+        const uint2 v = list[c];
+        const int i = (int)(v.y >> 24), t = (int)(v.y & 0xffffffu);
+        const int b = tb.base[i], e = b + tb.m[i];
         int rank = 0;
         for (int j = b; j < e; ++j) {
             const uint2 o = list[j];
             rank += o.x > v.x || (o.x == v.x && o.y < v.y); // (same segment: y orders by position)
         }
-        if (rank < tb.r[s]) atomicOr(&mask[t >> 5], 1u << (t & 31));
-        else if (t >= ns && t < t_last) atomicMax(&sh.cmax[(t >> 5) >> chunk_log], v.x);
+        if (rank < tb.r[i]) atomicOr(&mask[t >> 5], 1u << (t & 31));
+        else rejected(v.x, i, t);
     }
-    for (int s = warp; s < n; s += NW) { // ties across the threshold: the first r of them in position order
-        if (tb.state[s] != kTies) continue;
-        const unsigned key = tb.L[s];
-        const int a = bounds[s], e = bounds[s + 1], r = tb.r[s];
+    for (int i = warp; i < n; i += NW) { // ties across the threshold: the first r of them in position order
+        if (tb.state[i] != kTies) continue;
+        const unsigned key = tb.L[i];
+        const int s = tb.seg[i], a = bounds[s], e = bounds[s + 1], r = tb.r[i];
         int seen = 0;
-        for (int t0 = a & ~31; t0 < e; t0 += 32) {
+        for (int t0 = a; t0 < e; t0 += 32) {
             const int t = t0 + lane;
-            const bool tie = t >= a && t < e && score_key(g[t]) == key;
+            const bool tie = t < e && score_key(g[t]) == key;
             const unsigned bal = __ballot_sync(kFull, tie);
-            const bool kept = tie && seen + __popc(bal & ((1u << lane) - 1u)) < r;
-            const unsigned kb = __ballot_sync(kFull, kept);
-            if (lane == 0 && kb) atomicOr(&mask[t0 >> 5], kb);
-            if (__any_sync(kFull, tie && !kept && t >= ns && t < t_last) && lane == 0) atomicMax(&sh.cmax[(t0 >> 5) >> chunk_log], key);
+            if (tie) {
+                if (seen + __popc(bal & ((1u << lane) - 1u)) < r) atomicOr(&mask[t >> 5], 1u << (t & 31));
+                else rejected(key, i, t);
+            }
             seen += __popc(bal);
         }
     }
@@ -546,7 +688,7 @@ __device__ void block_select_stream(const float *g, int T, int q, SelShared &sh,
 // -------------------------------------------------------------------------------------- k_select_compact
 
 template <int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p)
+__global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, int longs)
 {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ SelShared sh;
@@ -556,13 +698,14 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p)
     const int T = p.seq_lens[bq];
     if (T <= p.Tk || T > p.T_cap) return;
     const int sc = p.seg_cap;
-    const SelSmem mp = sel_smem<NT>(p.T_cap, sc, p.S);
+    const SelSmem mp = sel_smem<NT>(p.T_cap, sc, p.S, longs != 0);
     unsigned *mask = reinterpret_cast<unsigned *>(dyn + mp.mask);
     int *bounds = reinterpret_cast<int *>(dyn + mp.bounds);
     int *quota = reinterpret_cast<int *>(dyn + mp.quota);
-    unsigned *hist = reinterpret_cast<unsigned *>(dyn + mp.hist);
-    SegTab &tb = *reinterpret_cast<SegTab *>(dyn + mp.tab);
+    unsigned *best = reinterpret_cast<unsigned *>(dyn + mp.best);
+    unsigned *hist = reinterpret_cast<unsigned *>(dyn + mp.hist) + warp * kWarpBins;
     uint2 *list = reinterpret_cast<uint2 *>(dyn + mp.list); // (key, position) of candidates
+    SegTab &tb = *reinterpret_cast<SegTab *>(dyn + mp.tab);
     const size_t row = (size_t)uid * p.T_cap;
     const float *g = p.scores + row;
     int *keep = p.keep_idx + (size_t)uid * p.Tk;
@@ -571,16 +714,13 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p)
     const int ns = max(0, min(p.n_sink, min(p.Tk, T)));           // must-keep prefix and suffix
     const int nl = max(0, min(p.n_last, min(p.Tk - ns, T - ns)));
     const int t_last = T - nl;
-    int chunk_log = 0; // chunks of 2^chunk_log windows, at most kMaxChunks of them
-    while ((n_words - 1) >> chunk_log >= kMaxChunks) ++chunk_log;
-    const int n_chunk = ((n_words - 1) >> chunk_log) + 1;
     int round = 0;
     for (int i = tid; i <= n_words; i += NT) mask[i] = 0u;
-    for (int i = tid; i < kMaxChunks; i += NT) sh.cmax[i] = 0u;
-    if (tid == 0) { sh.n_list = 0; sh.n_clist = 0; sh.bound = 0u; }
+    for (int i = tid; i < kBest; i += NT) best[i] = 0u;
+    if (tid == 0) { sh.n_list = 0; sh.bound = 0u; }
     wait_for_previous_kernel(); // prefix sums and cuts
     const int n_seg = segments_and_quotas<NT>(p, uid, T, p.Tk - ns - nl, reinterpret_cast<u64 *>(dyn + mp.ms), bounds, quota,
-                                              reinterpret_cast<int *>(hist), sh, round);
+                                              reinterpret_cast<int *>(list), sh, round);
     if (n_seg < 0) { // cannot happen with the capacity formula of the header; reported all the same
         if (tid == 0) { set_status(p.status, AMS_ERR_CAPACITY, uid, sh.n_seg, sc); p.n_seg[uid] = -1; p.seq_bad[bq] = 1; }
         return;
@@ -594,9 +734,52 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p)
         }
     }
 
-    // ---- per-segment top-q_i
-    for (int s0 = 0; s0 < n_seg; s0 += kBatch)
-        select_batch<NT>(g, bounds + s0, quota + s0, min(kBatch, n_seg - s0), mask, tb, hist, list, ns, t_last, chunk_log, sh);
+    // ---- per-segment top-q_i.  Slots of the table of best rejected keys: short segment sg takes sg, the pieces of long
+    //      ones those behind.  The next segment's scores are fetched before the current one is searched.
+    const bool fine = (longs ? 2 * n_seg + T / kPiece : n_seg) <= kBest / 4;
+    {
+        float xn[kPer];
+        auto fetch = [&](int sg) {
+            if (sg < n_seg) load_piece(g, bounds[sg], min(kPiece, bounds[sg + 1] - bounds[sg]), xn);
+        };
+        fetch(warp);
+        for (int sg = warp; sg < n_seg; sg += NW) {
+            const int a = bounds[sg], L = bounds[sg + 1] - a, q = quota[sg];
+            float x[kPer];
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) x[j] = xn[j];
+            fetch(sg + NW);
+            if (L <= kPiece) warp_segment(x, mask, best, hist, sg, fine, a, L, q, ns, t_last);
+        }
+    }
+    int n_slot = n_seg;
+    if (longs) {
+        for (int s0 = 0; s0 < n_seg;) { // batches of long segments
+            __syncthreads();
+            if (warp == 0) {
+                int n = 0, pc = 0, sg = s0;
+                for (; sg < n_seg && n <= kBatch - 32; sg += 32) {
+                    const int i = sg + lane, len = i < n_seg ? bounds[i + 1] - bounds[i] : 0;
+                    const bool is = len > kPiece;
+                    const unsigned bal = __ballot_sync(kFull, is);
+                    const int c = is ? (len + kPiece - 1) / kPiece : 0, inc = warp_incl_scan(c), at = n + __popc(bal & ((1u << lane) - 1u));
+                    if (is) { tb.seg[at] = (unsigned short)i; tb.piece0[at] = pc + inc - c; }
+                    n += __popc(bal);
+                    pc += __shfl_sync(kFull, inc, 31);
+                }
+                if (lane == 0) { tb.piece0[n] = pc; sh.n_long = n; sh.level = sg; }
+            }
+            __syncthreads();
+            s0 = sh.level;
+            const int n = sh.n_long;
+            if (n > 0) {
+                const int n_pc = tb.piece0[n];
+                select_long<NT>(g, bounds, quota, n, mask, best, n_slot, fine, tb, reinterpret_cast<unsigned *>(dyn + mp.lhist), list, ns, t_last, sh);
+                n_slot += n_pc;
+            }
+        }
+    }
+    __syncthreads();
 
     // ---- must-keep prefix and suffix; every must-keep position a segment already chose frees one slot,
     //      refilled by the best positions not yet kept (top r_fill of the unflagged tokens of the sequence)
@@ -607,41 +790,51 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p)
     }
     const int r_fill = block_count<NT>(already, round, sh);
     if (r_fill > 0) {
-        // At least r_fill unflagged tokens lie at or above the r_fill-th largest of the chunks' best rejected keys, so
-        // only chunks whose best key reaches that bound can hold a winner; their tokens at or above it go to a list.
-        for (int i = tid; i < n_chunk; i += NT) {
-            const unsigned v = sh.cmax[i];
-            int rank = 0;
-            for (int j = 0; j < n_chunk; ++j) {
-                const unsigned o = sh.cmax[j];
-                rank += o > v || (o == v && j < i);
-            }
-            if (rank == r_fill - 1) sh.bound = v; // (none, or 0: too few chunks with a candidate, everything is looked at)
+        // At least r_fill unflagged tokens lie at or above the r_fill-th largest entry of the table, so only pieces with an
+        // entry that reaches that bound can hold a winner; their tokens at or above it go to a list.
+        if (warp == 0) {
+            unsigned k[kBest / 32];
+            int c = 0;
+#pragma unroll
+            for (int j = 0; j < kBest / 32; ++j) { k[j] = best[j * 32 + lane]; c += k[j] > 0u; }
+            unsigned M = 0u; // (too few entries: every token is looked at)
+            if (warp_sum(c) >= r_fill) M = warp_cut<kBest / 32>(k, kBest, r_fill, hist).key;
+            if (lane == 0) sh.bound = M;
         }
         __syncthreads();
         const unsigned M = sh.bound;
         auto raise = [&](int t) { atomicOr(&mask[t >> 5], 1u << (t & 31)); };
         auto unflagged = [&](int t) { return ((mask[t >> 5] >> (t & 31)) & 1u) == 0u; };
-        for (int i = tid; i < n_chunk; i += NT)
-            if (sh.cmax[i] >= M) sh.clist[atomicAdd(&sh.n_clist, 1)] = (unsigned short)i;
-        __syncthreads();
-        const int n_w = sh.n_clist << chunk_log; // windows to look at
-        for (int i0 = warp; i0 < n_w; i0 += NW * 4) {
-            float x[4];
-            int tt[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int i = i0 + j * NW;
-                tt[j] = i < n_w ? (((int)sh.clist[i >> chunk_log] << chunk_log) + (i & ((1 << chunk_log) - 1))) * 32 + lane : T;
-                x[j] = tt[j] < T ? g[tt[j]] : 0.0f;
+        auto look = [&](int slot, int a, int len) { // a piece
+            unsigned b;
+            if (fine) {
+                const uint4 v = reinterpret_cast<const uint4 *>(best)[slot];
+                b = max(max(v.x, v.y), max(v.z, v.w));
+            } else {
+                b = best[slot & (kBest - 1)];
             }
+            if (b < M) return;
+            float x[kPer];
+            load_piece(g, a, len, x);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
+            for (int j = 0; j < kPer; ++j) {
+                const int t = a + j * 32 + lane;
                 const unsigned key = score_key(x[j]);
-                if (tt[j] < T && key >= M && unflagged(tt[j])) {
+                if (j * 32 + lane < len && key >= M && unflagged(t)) {
                     const int at = atomicAdd(&sh.n_list, 1);
-                    if (at < kList) list[at] = make_uint2(key, (unsigned)tt[j]);
+                    if (at < kList) list[at] = make_uint2(key, (unsigned)t);
                 }
+            }
+        };
+        int slot = n_seg;
+        for (int sg = 0; sg < n_seg; ++sg) {
+            const int a = bounds[sg], L = bounds[sg + 1] - a;
+            if (L <= kPiece) {
+                if (sg % NW == warp) look(sg, a, L);
+            } else {
+                const int n_pc = (L + kPiece - 1) / kPiece;
+                for (int i = (warp - slot % NW + NW) % NW; i < n_pc; i += NW) look(slot + i, a + i * kPiece, min(kPiece, L - i * kPiece));
+                slot += n_pc;
             }
         }
         __syncthreads();
@@ -667,39 +860,41 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p)
     int n_kept = 0;
     for (int w = w0 + lane; w < w1; w += 32) n_kept += __popc(mask[w]);
     n_kept = warp_sum(n_kept);
-    if (lane == 0) sh.cmax[warp] = (unsigned)n_kept;
+    if (lane == 0) sh.wc[0][warp] = n_kept;
     __syncthreads();
-    int pos = warp_sum(lane < warp ? (int)sh.cmax[lane] : 0);
-    const int total = warp_sum(lane < NW ? (int)sh.cmax[lane] : 0);
+    int pos = warp_sum(lane < warp ? sh.wc[0][lane] : 0);
+    const int total = warp_sum(lane < NW ? sh.wc[0][lane] : 0);
     if (total != p.Tk) {
         if (tid == 0) { set_status(p.status, AMS_ERR_INTERNAL, uid, total, p.Tk); p.seq_bad[bq] = 1; }
         return;
     }
     for (int g0 = w0; g0 < w1; g0 += 32) {
         const unsigned mine = g0 + lane < w1 ? mask[g0 + lane] : 0u;
-        const int n = min(32, w1 - g0);
-        for (int i = 0; i < n; ++i) {
+        const int inc = warp_incl_scan(__popc(mine)), at = pos + inc - __popc(mine);
+#pragma unroll 8
+        for (int i = 0; i < 32; ++i) { // (words past the end are 0)
             const unsigned m = __shfl_sync(kFull, mine, i);
-            if ((m >> lane) & 1u) keep[pos + __popc(m & ((1u << lane) - 1u))] = (g0 + i) * 32 + lane;
-            pos += __popc(m);
+            const int b = __shfl_sync(kFull, at, i);
+            if ((m >> lane) & 1u) keep[b + __popc(m & ((1u << lane) - 1u))] = (g0 + i) * 32 + lane;
         }
+        pos += __shfl_sync(kFull, inc, 31);
     }
     // ---- credit rows travel with their tokens, in place: kept positions ascend and keep[j] >= j, so what a tile
     //      writes is never read by a later one.  Rows beyond the budget start from zero.
     if (ema_on) {
         float *credit = p.ema + (((size_t)l * p.Bmax + bq) * p.H + h) * (size_t)p.T_cap;
-        constexpr int kPer = 8;
+        constexpr int kIn = 8; // rows in flight per thread
         __syncthreads();
-        for (int base = 0; base < p.Tk; base += NT * kPer) {
-            float c[kPer];
+        for (int base = 0; base < p.Tk; base += NT * kIn) {
+            float c[kIn];
 #pragma unroll
-            for (int i = 0; i < kPer; ++i) {
+            for (int i = 0; i < kIn; ++i) {
                 const int j = base + i * NT + tid;
                 c[i] = j < p.Tk ? credit[keep[j]] : 0.0f;
             }
             __syncthreads();
 #pragma unroll
-            for (int i = 0; i < kPer; ++i) {
+            for (int i = 0; i < kIn; ++i) {
                 const int j = base + i * NT + tid;
                 if (j < p.Tk) credit[j] = c[i];
             }
@@ -714,24 +909,27 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p)
 }
 
 template <int NT>
-cudaError_t launch_nt(const DevParams &p, int units, LaunchCtx &ctx)
+cudaError_t launch_nt(const DevParams &p, int units, bool longs, LaunchCtx &ctx)
 {
     static SmemGrant grant;
-    const size_t smem = sel_smem<NT>(p.T_cap, p.seg_cap, p.S).total;
+    const size_t smem = sel_smem<NT>(p.T_cap, p.seg_cap, p.S, longs).total;
     if (!grant_dynamic_smem(k_select_compact<NT>, smem, grant)) return cudaErrorInvalidValue;
-    return launch_after(k_select_compact<NT>, dim3((unsigned)units), dim3(NT), smem, ctx.s, p);
+    return launch_after(k_select_compact<NT>, dim3((unsigned)units), dim3(NT), smem, ctx.s, p, longs ? 1 : 0);
 }
+
+bool long_segments(const DevParams &p) { return p.l_max == 0 || p.l_max > kPiece; }
 
 } // namespace
 
-size_t select_smem_bytes(const DevParams &p) { return sel_smem<512>(p.T_cap, p.seg_cap, p.S).total; }
+size_t select_smem_bytes(const DevParams &p) { return sel_smem<1024>(p.T_cap, p.seg_cap, p.S, long_segments(p)).total; }
 
 int launch_select(const DevParams &p, LaunchCtx &ctx)
 {
     const int units = p.L * p.B * p.H, n_sm = sm_count();
     if (n_sm <= 0) return AMS_ERR_CUDA;
-    const cudaError_t e = units >= 6 * n_sm ? launch_nt<256>(p, units, ctx)
-                        : units > n_sm ? launch_nt<512>(p, units, ctx) : launch_nt<1024>(p, units, ctx);
+    const bool longs = long_segments(p);
+    const cudaError_t e = units >= 6 * n_sm ? launch_nt<256>(p, units, longs, ctx)
+                        : units > n_sm ? launch_nt<512>(p, units, longs, ctx) : launch_nt<1024>(p, units, longs, ctx);
     if (e != cudaSuccess) return AMS_ERR_CUDA;
     ctx.mark(kKernSelect);
     return AMS_OK;
