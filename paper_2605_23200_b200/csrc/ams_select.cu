@@ -6,16 +6,21 @@
 // Selection order is (score key descending, position ascending), a strict total order, so a segment and its quota have
 // exactly one answer however it is found.  Finding the q-th largest key is what costs.  It is bound by latency and issue
 // slots, not by memory (4 bytes per token, from L2):
-//   * a segment of at most 256 tokens lives in the registers of one warp.  A histogram of 128 bins over the segment's own
-//     range of keys leads to the bin of the q-th key, a second one over that bin usually ends the search: two short
-//     steps instead of 16 to 20 dependent warp-wide counts, one per key bit.
-//   * longer segments are searched together by the whole block, in three walks over their 256-token pieces: range of
-//     keys, histogram per segment, then keys above the threshold's bin are kept and the few inside it go to a list in which
-//     every entry counts the entries of its segment before it.  (A bin that is still crowded gets another histogram
-//     first; ties by the hundred end with a bin of one key.)  Every warp has the same share of the walks whatever the
-//     lengths of the segments.
+//   * a segment of at most 256 tokens lives in the registers of one warp.  A histogram over the 16 octaves below its largest
+//     key (256 bins, shared memory) leads to the bin of the q-th key, and the few keys in that bin are taken apart one by
+//     one; exact fallbacks take over for thresholds further down, ties, NaN.  Fixing key bits from the top instead is a
+//     chain of 16 to 20 dependent warp-wide counts: 74 segments of a 16384-token unit 38 k cycles, 15 k now.
+//   * longer segments are searched together by the whole block, in walks over their 256-token pieces: largest key (from a
+//     quarter of the tokens), histogram per segment over the octaves below it, then keys above the threshold's bin are
+//     kept and the few inside it go to a list in which every entry counts the entries of its segment before it.  (A bin
+//     that is still crowded gets another histogram first; ties by the hundred end with a bin of one key.)  Every warp has
+//     the same share of the walks whatever the lengths of the segments.
 // The backfill takes its bound from the best rejected key of every piece, which the searches leave behind, and looks only
 // at pieces that reach it, instead of walking the sequence twice.
+// Placing segments and quotas here, by the block that needs them, costs 5 k cycles of latency; a kernel of one-warp blocks
+// in front took 16 to 54 us.  Both together, us per event before / now: 256 units of 16384 tokens 76 / 39, 1792 ragged
+// units of 8192..32768 tokens 401 / 200, 1792 units of 4224 tokens 168 / 96, 2048 units of 32768 tokens in long segments
+// 528 / 330.
 #include "ams_common.cuh"
 #include "ams_select.cuh"
 
@@ -28,21 +33,23 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kPiece = 256;         // tokens a warp holds in registers, eight per lane
 constexpr int kPer = kPiece / 32;
-constexpr int kWarpBins = 128;      // bins of a warp's own histogram
-constexpr int kBatch = 256;         // long segments searched together
+constexpr int kWarpBins = 256;      // bins of a warp's own histogram, eight per lane
+constexpr int kBatch = 64;          // long segments searched together
 constexpr int kMaxBins = 1024;      // histogram bins per long segment
-constexpr int kBest = 1024;         // entries of the table of best rejected keys
+constexpr unsigned kOctaves = 12;   // octaves below a long segment's largest score that its histogram resolves
+constexpr int kBest = 512;          // entries of the table of best rejected keys
 
 // Working arrays of the search of long segments, one entry per segment of the batch.
 struct SegTab {
-    unsigned lo[kBatch], w[kBatch];  // the histogram covers the keys [lo, lo + w]
+    unsigned lo[kBatch];             // bin = (key - lo) >> shift, the first and last one taking what lies outside
+    unsigned rl[kBatch], rw[kBatch]; // only the keys [rl, rl + rw] are counted
     unsigned L[kBatch], U[kBatch];   // keys >= U win, keys < L lose
     int above[kBatch];               // keys above the range of the histogram
     int r[kBatch], m[kBatch];        // r of the m keys in [L, U) win
     int base[kBatch], cnt[kBatch];   // part of the list
     unsigned short seg[kBatch];
     int piece0[kBatch + 1];          // first piece
-    unsigned char shift[kBatch];     // bin = (key - lo) >> shift
+    unsigned char shift[kBatch];
     unsigned char state[kBatch];
 };
 enum { kDone = 0, kSearch = 1, kTies = 2 };
@@ -52,7 +59,7 @@ template <int NT> struct Tune {
     static constexpr int kList = NT <= 256 ? 1024 : 2048;  // candidates, of the long segments and then of the backfill
 };
 
-struct SelSmem { size_t mask, ms, bounds, quota, best, list, hist, lhist, tab, total; };
+struct SelSmem { size_t mask, ms, bounds, quota, best, list, hist, tab, total; };
 template <int NT>
 __host__ __device__ inline SelSmem sel_smem(int T_cap, int sc, int S, bool longs)
 {
@@ -65,20 +72,21 @@ __host__ __device__ inline SelSmem sel_smem(int T_cap, int sc, int S, bool longs
     m.quota = o;  o += (size_t)sc * 4;
     o = (o + 15) & ~(size_t)15;
     m.best = o;   o += (size_t)kBest * 4;
-    m.hist = o;   o += (size_t)(NT / 32) * kWarpBins * 4;
-    // the quota computation, which comes first, uses the list (and what follows) as scratch
-    const size_t q = (size_t)(S + 1) * 8 + (size_t)sc * 4, l = (size_t)Tune<NT>::kList * 8 + (longs ? (size_t)Tune<NT>::kBins * 4 + sizeof(SegTab) : 0);
-    m.list = o;
-    m.lhist = o + (size_t)Tune<NT>::kList * 8;
-    m.tab = m.lhist + (size_t)Tune<NT>::kBins * 4;
-    o += q > l ? q : l;
+    m.list = o;   o += (size_t)Tune<NT>::kList * 8;
+    // one area in turn for: the quota computation, the warps' histograms, those of the long segments, the backfill's bound
+    // and the pieces it looks at
+    m.hist = o;
+    const size_t q = (size_t)(S + 1) * 8 + (size_t)sc * 4, w = (size_t)(NT / 32) * kWarpBins * 4, l = longs ? (size_t)Tune<NT>::kBins * 4 : 0;
+    o += q > w ? (q > l ? q : l) : (w > l ? w : l);
+    o = (o + 15) & ~(size_t)15;
+    m.tab = o;    o += longs ? sizeof(SegTab) : 0;
     m.total = (o + 15) & ~(size_t)15;
     return m;
 }
 
 struct SelShared {
     int wc[2][32];   // per-warp counts of even / odd rounds of a block-wide count
-    int n_list, n_long, total;
+    int n_list, n_look, n_long, total;
     unsigned bound;
     int n_merged, n_seg, level, rem;
 };
@@ -121,8 +129,14 @@ __device__ int block_distribute(int sign, int D, const int *cap, int *quota, con
 {
     const int tid = threadIdx.x, lane = tid & 31;
     if (tid < 32) {
-        int cnt1 = 0, tot = 0, mx = 0;
-        for (int i = lane; i < n_seg; i += 32) { cnt1 += cap[i] >= 1; tot += cap[i]; mx = max(mx, cap[i]); }
+        constexpr int kC = 8; // room of the first 256 segments in registers
+        int c[kC], cnt1 = 0, tot = 0, mx = 0;
+#pragma unroll
+        for (int j = 0; j < kC; ++j) {
+            c[j] = j * 32 + lane < n_seg ? cap[j * 32 + lane] : 0;
+            cnt1 += c[j] >= 1; tot += c[j]; mx = max(mx, c[j]);
+        }
+        for (int i = kC * 32 + lane; i < n_seg; i += 32) { cnt1 += cap[i] >= 1; tot += cap[i]; mx = max(mx, cap[i]); }
         cnt1 = warp_sum(cnt1);
         tot = warp_sum(tot);
         mx = __reduce_max_sync(kFull, mx);
@@ -136,7 +150,9 @@ __device__ int block_distribute(int sign, int D, const int *cap, int *quota, con
             while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
                 int f = 0;
-                for (int i = lane; i < n_seg; i += 32) f += min(cap[i], mid);
+#pragma unroll
+                for (int j = 0; j < kC; ++j) f += min(c[j], mid);
+                for (int i = kC * 32 + lane; i < n_seg; i += 32) f += min(cap[i], mid);
                 f = warp_sum(f);
                 if (f <= D) { lo = mid; used = f; } else hi = mid;
             }
@@ -152,10 +168,10 @@ __device__ int block_distribute(int sign, int D, const int *cap, int *quota, con
         if (rem > 0 && ci > level) {
             const u64 Mi = M[i];
             int rank = 0;
-            for (int j = lane; j < n_seg; j += 32) {
-                const u64 Mj = M[j];
-                const bool before = sign > 0 ? (Mj > Mi || (Mj == Mi && j < i)) : (Mj < Mi || (Mj == Mi && j > i));
-                rank += cap[j] > level && before;
+#pragma unroll 4
+            for (int j = lane; j < n_seg; j += 32) { // (M, position) as one strict order; masses stay far below 2^63
+                const long long Mj = (long long)M[j], Mx = (long long)Mi;
+                rank += cap[j] > level && (sign > 0 ? Mj + (j < i) > Mx : Mj < Mx + (j > i));
             }
             g += warp_sum(rank) < rem;
         }
@@ -165,10 +181,11 @@ __device__ int block_distribute(int sign, int D, const int *cap, int *quota, con
     return left;
 }
 
-// floor(x / y) for a quotient below 2^20 and x < 2^62: the fp64 quotient is off by less than one, the remainder corrects it.
-__device__ __forceinline__ u64 quotient(u64 x, u64 y)
+// floor(x / y) for a quotient below 2^20 and x < 2^62, inv = 1 / y rounded: the product is off by less than one, the
+// remainder corrects it.
+__device__ __forceinline__ u64 quotient(u64 x, u64 y, double inv)
 {
-    u64 q = (u64)((double)x / (double)y);
+    u64 q = (u64)((double)x * inv);
     const long long rem = (long long)(x - q * y);
     if (rem < 0) --q;
     else if (rem >= (long long)y) ++q;
@@ -187,6 +204,8 @@ __device__ int segments_and_quotas(const DevParams &p, int uid, int T, int Bq, u
     int *merged = tmp, *poff = merged + p.S + 1, *cap = poff + p.S + 1;
     const u64 *C = p.cbuf + (size_t)uid * p.T_cap;
     const u64 SH = C[T - 1];
+    const u64 SHq = p.uniform_q ? (u64)T : SH; // total of what the quotas are proportional to
+    const double inv = 1.0 / (double)(2ull * SHq);
     if (warp == 0) {
         // raw cuts of the mass quantiles, ascending, found by the scan kernel (a cut at or beyond T means "none"); short raw
         // segments merge forward: the next boundary is the first cut at least l_min past the last one
@@ -232,7 +251,6 @@ __device__ int segments_and_quotas(const DevParams &p, int uid, int T, int Bq, u
     }
     __syncthreads();
     // quotas: q_i = q_i^min + round(T_rem M_i / sum M), clipped, then adjusted
-    const u64 SHq = p.uniform_q ? (u64)T : SH; // total of what the quotas are proportional to
     int smin = 0;
     for (int i = tid; i < n_seg; i += NT) {
         const int a = bounds[i], e = bounds[i + 1];
@@ -244,7 +262,7 @@ __device__ int segments_and_quotas(const DevParams &p, int uid, int T, int Bq, u
     for (int i = tid; i < n_seg; i += NT) {
         const int L = bounds[i + 1] - bounds[i];
         long long qi = max(0, min(p.q_min, L));
-        if (Trem >= 0) qi += (long long)quotient(2ull * (u64)Trem * Ms[i] + SHq, 2ull * SHq);
+        if (Trem >= 0) qi += (long long)quotient(2ull * (u64)Trem * Ms[i] + SHq, 2ull * SHq, inv);
         if (qi > L) qi = L;
         quota[i] = (int)qi;
         sq += (int)qi;
@@ -270,20 +288,34 @@ __device__ int segments_and_quotas(const DevParams &p, int uid, int T, int Bq, u
 
 struct Cut { unsigned key; int ties; }; // the keys above `key` win, and `ties` of those equal to it (-1: all of them)
 
-// Bin of a warp's histogram of kWarpBins bins that holds the q-th key from the top (1 <= q <= number of keys counted): bin,
+// *word += 1 where d <= w, as a predicated instruction (a branch around each of a lane's increments costs more than they do).
+__device__ __forceinline__ void count_if(unsigned *word, unsigned d, unsigned w)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.le.u32 p, %1, %2;\n\t@p red.shared.add.u32 [%0], 1;\n\t}"
+                 ::"r"((unsigned)__cvta_generic_to_shared(word)), "r"(d), "r"(w) : "memory");
+}
+
+// Bin of a warp's histogram that holds the q-th key from the top (1 <= q <= number of keys counted, at most 1023 keys): bin,
 // keys in it, keys above it.
 __device__ __forceinline__ void find_bin(const unsigned *hist, int q, int &bin, int &m, int &above)
 {
     const int lane = threadIdx.x & 31;
-    const uint4 v = reinterpret_cast<const uint4 *>(hist)[31 - lane]; // lane 0 has the top four bins
-    const int c0 = (int)v.w, c1 = c0 + (int)v.z, c2 = c1 + (int)v.y, c3 = c2 + (int)v.x;
-    const int inc = warp_incl_scan(c3), exc = inc - c3, rest = q - exc;
+    const uint4 *h4 = reinterpret_cast<const uint4 *>(hist) + 2 * (31 - lane); // lane 0 has the top eight bins
+    const uint4 a = h4[1], b = h4[0];
+    int c[8]; // keys in this lane's first 1 .. 8 bins from the top
+    c[0] = (int)a.w; c[1] = c[0] + (int)a.z; c[2] = c[1] + (int)a.y; c[3] = c[2] + (int)a.x;
+    c[4] = c[3] + (int)b.w; c[5] = c[4] + (int)b.z; c[6] = c[5] + (int)b.y; c[7] = c[6] + (int)b.x;
+    const int inc = warp_incl_scan(c[7]), exc = inc - c[7], rest = q - exc;
     const int src = __ffs(__ballot_sync(kFull, inc >= q)) - 1; // the first lane that covers q
-    const int i = (rest > c0) + (rest > c1) + (rest > c2);
-    const int below = i == 0 ? 0 : (i == 1 ? c0 : (i == 2 ? c1 : c2)), upto = i == 0 ? c0 : (i == 1 ? c1 : (i == 2 ? c2 : c3));
-    bin = __shfl_sync(kFull, (31 - lane) * 4 + 3 - i, src);
-    m = __shfl_sync(kFull, upto - below, src);
-    above = __shfl_sync(kFull, exc + below, src);
+    int i = 0, below = 0, upto = c[7];
+#pragma unroll
+    for (int j = 6; j >= 0; --j) {
+        if (rest > c[j]) { below = max(below, c[j]); ++i; }
+        else upto = c[j];
+    }
+    const unsigned mine = (unsigned)(255 - lane * 8 - i) | (unsigned)(upto - below) << 8 | (unsigned)(exc + below) << 18;
+    const unsigned got = __shfl_sync(kFull, mine, src);
+    bin = (int)(got & 255u); m = (int)((got >> 8) & 1023u); above = (int)(got >> 18);
 }
 
 // The q-th largest (0 < q < n) of n keys in a warp's registers, kPL per lane, key number j * 32 + lane in register j, unused
@@ -312,13 +344,14 @@ __device__ __forceinline__ Cut warp_cut(const unsigned (&k)[kPL], int n, int q, 
     }
     unsigned lo = mn, w = mx - mn;
     for (;;) {
-        const int shift = max(0, 25 - __clz(w)); // w >> shift < kWarpBins
+        const int shift = max(0, 24 - __clz(w)); // w >> shift < kWarpBins
         reinterpret_cast<uint4 *>(hist)[lane] = make_uint4(0, 0, 0, 0);
+        reinterpret_cast<uint4 *>(hist)[32 + lane] = make_uint4(0, 0, 0, 0);
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < kPL; ++j) {
             const unsigned d = k[j] - lo;
-            if (d <= w) atomicAdd(&hist[d >> shift], 1u);
+            count_if(&hist[d >> shift], d, w);
         }
         __syncwarp();
         int bin, m, above;
@@ -328,8 +361,71 @@ __device__ __forceinline__ Cut warp_cut(const unsigned (&k)[kPL], int n, int q, 
         if (q == m) return {lo, -1};
         w = min((1u << shift) - 1u, w - ((unsigned)bin << shift));
         if (w == 0u) return {lo, q};
+        if (m <= 4) break;
         __syncwarp();
     }
+    for (;;) { // few keys are left in [lo, lo + w]: from the largest down
+        unsigned v = 0u;
+#pragma unroll
+        for (int j = 0; j < kPL; ++j) { const unsigned d = k[j] - lo; v = max(v, d <= w ? d : 0u); }
+        v = __reduce_max_sync(kFull, v);
+        int c = 0;
+#pragma unroll
+        for (int j = 0; j < kPL; ++j) c += k[j] - lo == v;
+        c = warp_sum(c);
+        if (c >= q) return {lo + v, c == q ? -1 : q};
+        q -= c;
+        w = v - 1u;
+    }
+}
+
+// The usual case of the search in two short steps: bins of 2^19 keys over the 16 octaves below the largest key mx, then the
+// few keys of the threshold's bin from the largest down.  key: the q-th largest distinct key from there on, which is the
+// q-th largest unless some are equal (the caller counts).  False: the threshold lies further down.  Unused registers must
+// hold keys below mx - 2^27.
+template <int kPL>
+__device__ __forceinline__ bool warp_cut_fast(const unsigned (&k)[kPL], int q, unsigned mx, unsigned *hist, unsigned &key)
+{
+    const int lane = threadIdx.x & 31;
+    unsigned lo = mx - ((16u << 23) - 1u), w = (1u << 19) - 1u;
+    reinterpret_cast<uint4 *>(hist)[lane] = make_uint4(0, 0, 0, 0);
+    reinterpret_cast<uint4 *>(hist)[32 + lane] = make_uint4(0, 0, 0, 0);
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < kPL; ++j) atomicAdd(&hist[(max(k[j], lo) - lo) >> 19], 1u);
+    __syncwarp();
+    int bin, m, above;
+    find_bin(hist, q, bin, m, above);
+    if (bin == 0) return false;
+    lo += (unsigned)bin << 19;
+    q -= above;
+    key = lo;
+    while (m > 5 && q < m && w > 0u) { // crowded: another histogram over the bin
+        const int shift = max(0, 24 - __clz(w));
+        __syncwarp();
+        reinterpret_cast<uint4 *>(hist)[lane] = make_uint4(0, 0, 0, 0);
+        reinterpret_cast<uint4 *>(hist)[32 + lane] = make_uint4(0, 0, 0, 0);
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < kPL; ++j) { const unsigned d = k[j] - lo; count_if(&hist[d >> shift], d, w); }
+        __syncwarp();
+        find_bin(hist, q, bin, m, above);
+        lo += (unsigned)bin << shift;
+        q -= above;
+        key = lo;
+        w = min((1u << shift) - 1u, w - ((unsigned)bin << shift));
+    }
+    for (; q < m; --m) { // drop the smallest of the bin's keys, one at a time
+        unsigned v = kFull;
+#pragma unroll
+        for (int j = 0; j < kPL; ++j) { const unsigned d = k[j] - lo; v = min(v, d <= w ? d : kFull); }
+        v = __reduce_min_sync(kFull, v);
+        if (v >= w) break; // (equal keys)
+        lo += v + 1u;
+        w -= v + 1u;
+        key = lo;
+    }
+    return true;
 }
 
 // Kept bits of a piece of at most kPiece tokens from position a: lane j's word holds tokens a + 32 j .., shifted onto
@@ -361,7 +457,7 @@ __device__ __forceinline__ void load_piece(const float *g, int a, int len, float
     const float *src = g + a + (threadIdx.x & 31);
     const int room = len - (int)(threadIdx.x & 31);
 #pragma unroll
-    for (int j = 0; j < kPer; ++j) x[j] = j * 32 < room ? src[j * 32] : __uint_as_float(0x7fffffffu); // NaN: key 0
+    for (int j = 0; j < kPer; ++j) x[j] = j * 32 < room ? src[j * 32] : 0.0f;
 }
 
 // One segment of at most kPiece tokens.
@@ -369,27 +465,57 @@ __device__ __forceinline__ void warp_segment(const float (&x)[kPer], unsigned *m
                                              int a, int L, int q, int ns, int t_last)
 {
     const int lane = threadIdx.x & 31, room = L - lane;
-    unsigned k[kPer];
-#pragma unroll
-    for (int j = 0; j < kPer; ++j) k[j] = score_key(x[j]);
-    Cut cut = {kFull, 0};                    // none of it
-    if (q >= L) cut = {0u, -1};              // all of it
-    else if (q > 0) cut = warp_cut<kPer>(k, L, q, hist);
     const bool plain = a >= ns && a + L <= t_last; // no must-keep position in it
     auto may_fill = [&](int j) { return plain || (a + j * 32 + lane >= ns && a + j * 32 + lane < t_last); };
-    unsigned word = 0, rej = 0;
-    if (cut.ties < 0 && cut.key > 0u) {      // the usual end: the keys from cut.key on
+    unsigned k[kPer], word = 0, rej = 0, mx = 0u;
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            const bool kept = k[j] >= cut.key;
-            const unsigned bal = __ballot_sync(kFull, kept);
-            if (lane == j) word = bal;
-            if (!kept && may_fill(j)) rej = max(rej, k[j]);
+    for (int j = 0; j < kPer; ++j) { k[j] = __float_as_uint(x[j]); mx = max(mx, k[j]); }
+    mx = __reduce_max_sync(kFull, mx);
+    const bool pos = mx <= 0x7f800000u && mx > (17u << 23); // no negative score, no NaN (unused registers read as +0)
+    if (pos) {
+        mx |= 0x80000000u;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) k[j] |= 0x80000000u;
+    } else {
+        mx = 0u;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) { k[j] = j * 32 < room ? score_key(x[j]) : 0u; mx = max(mx, k[j]); }
+        mx = __reduce_max_sync(kFull, mx);
+    }
+    bool done = false;
+    if (q >= L) { // all of it
+        const int n = min(32, max(0, L - lane * 32));
+        word = n > 0 ? kFull >> (32 - n) : 0u;
+        done = true;
+    } else if (q > 0 && mx > (17u << 23)) {
+        unsigned key = 0u;
+        if (warp_cut_fast<kPer>(k, q, mx, hist, key)) {
+            unsigned b[kPer];
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+                const bool kept = k[j] >= key;
+                b[j] = __ballot_sync(kFull, kept);
+                if (!kept && may_fill(j)) rej = max(rej, k[j]);
+            }
+            const bool l0 = lane & 1, l1 = lane & 2, l2 = lane & 4;
+            const unsigned w0 = l0 ? b[1] : b[0], w1 = l0 ? b[3] : b[2], w2 = l0 ? b[5] : b[4], w3 = l0 ? b[7] : b[6];
+            const unsigned v0 = l1 ? w1 : w0, v1 = l1 ? w3 : w2;
+            word = lane < kPer ? (l2 ? v1 : v0) : 0u;
+            done = warp_sum(__popc(word)) == q;
+            if (pos && L < kPiece && rej == 0x80000000u) rej = 0u; // (may be an unused register; scores of 0 are not worth an entry)
         }
-    } else {                                 // the first ties in position order
-        int seen = 0;
+    }
+    if (!done) {
+        if (pos) {
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) {
+            for (int j = 0; j < kPer; ++j) if (j * 32 >= room) k[j] = 0u;
+        }
+        Cut cut = {kFull, 0};                // none of it
+        if (q > 0) cut = warp_cut<kPer>(k, L, q, hist);
+        int seen = 0;
+        word = 0; rej = 0;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) { // ties: the first ones in position order
             const bool in = j * 32 < room, tie = in && k[j] == cut.key;
             const unsigned tb = __ballot_sync(kFull, tie);
             const bool kept = in && (k[j] > cut.key || (tie && (cut.ties < 0 || seen + __popc(tb & ((1u << lane) - 1u)) < cut.ties)));
@@ -460,8 +586,8 @@ __device__ __forceinline__ void find_long_bin(SegTab &tb, const unsigned *hist, 
             if (run < q && q <= run + cnt[j]) { bin = c * 128 + lane * 4 + 3 - j; m = cnt[j]; above = run; }
             run += cnt[j];
         }
-        const unsigned sft = tb.shift[i], off = (unsigned)bin << sft;
-        const unsigned L = tb.lo[i] + off, w = min((1u << sft) - 1u, tb.w[i] - off);
+        const unsigned sft = tb.shift[i], rl = tb.rl[i], rh = rl + tb.rw[i], first = tb.lo[i] + ((unsigned)bin << sft);
+        const unsigned L = bin == 0 ? rl : first, w = bin == nb - 1 ? rh - L : min(rh - L, first - L + (1u << sft) - 1u);
         const int r = q - above;
         tb.above[i] = above;
         tb.r[i] = r;
@@ -488,61 +614,51 @@ __device__ void select_long(const float *g, const int *bounds, const int *quota,
     int nb = Tune<NT>::kBins / n;
     nb = min(kMaxBins, 1 << (31 - __clz(nb)));
 
-    // ---- walk 1: range of keys (U holds the largest for now)
-    for (int i = tid; i < n; i += NT) { tb.lo[i] = kFull; tb.U[i] = 0u; }
+    // ---- walk 1: the bins of a segment cover the kOctaves octaves (2^23 keys each) below its largest key, judged by a
+    //      quarter of the tokens: scores below that hardly ever hold the threshold, whatever their sign, and what does
+    //      lie outside falls into the first or the last bin
     uint4 *h4 = reinterpret_cast<uint4 *>(hist);
     for (int i = tid; i < n * nb / 4; i += NT) h4[i] = make_uint4(0, 0, 0, 0);
-    __syncthreads();
-    {
-        int cur = 0;
-        unsigned mn = kFull, mx = 0u;
-        auto flush = [&]() {
-            mn = __reduce_min_sync(kFull, mn);
-            mx = __reduce_max_sync(kFull, mx);
-            if (lane == 0 && mn <= mx) { atomicMin(&tb.lo[cur], mn); atomicMax(&tb.U[cur], mx); }
-            mn = kFull; mx = 0u;
-        };
-        walk_long<NT>(g, bounds, tb, n, [&](int i) { flush(); cur = i; },
-                      [&](int, int, int, int len, const float (&x)[kPer]) {
+    for (int i = warp; i < n; i += NW) { // (32 tokens of every 128, at most 64 such groups)
+        const int a = bounds[tb.seg[i]], len = bounds[tb.seg[i] + 1] - a, q = quota[tb.seg[i]], step = max(128, (len >> 6) & ~31);
+        unsigned hi = 0u;
+        for (int t0 = lane; t0 < len; t0 += 8 * step) {
+            float x[8];
 #pragma unroll
-                          for (int j = 0; j < kPer; ++j) {
-                              const unsigned k = score_key(x[j]);
-                              mx = max(mx, k);
-                              mn = min(mn, j * 32 + lane < len ? k : kFull);
-                          }
-                      });
-        flush();
-    }
-    __syncthreads();
-    for (int i = tid; i < n; i += NT) {
-        const int s = tb.seg[i], len = bounds[s + 1] - bounds[s], q = quota[s];
-        const unsigned lo = tb.lo[i], w = tb.U[i] - lo;
-        tb.w[i] = w;
-        tb.above[i] = 0;
-        tb.r[i] = q;
-        tb.m[i] = len;
-        tb.L[i] = lo; tb.U[i] = lo + w + 1u;
-        int state = kSearch, shift = bin_shift(w, nb);
-        if (q <= 0) { state = kDone; tb.L[i] = tb.U[i] = kFull; }
-        else if (q >= len) { state = kDone; tb.L[i] = tb.U[i] = 0u; }
-        else if (w == 0u) state = kTies;
-        tb.state[i] = (unsigned char)state;
-        tb.shift[i] = (unsigned char)(state == kSearch ? shift : 255);
+            for (int j = 0; j < 8; ++j) x[j] = t0 + j * step < len ? g[a + t0 + j * step] : __uint_as_float(0x7fffffffu);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) hi = max(hi, score_key(x[j]));
+        }
+        hi = __reduce_max_sync(kFull, hi);
+        if (lane == 0) {
+            constexpr unsigned span = kOctaves << 23;
+            const unsigned lo = hi > span ? hi - span : 0u;
+            int state = kSearch;
+            unsigned L = 0u, U = kFull; // (no key is as large as kFull)
+            if (q <= 0) { state = kDone; L = kFull; }
+            else if (q >= len) { state = kDone; U = 0u; }
+            tb.L[i] = L; tb.U[i] = U;
+            tb.lo[i] = lo; tb.rl[i] = 0u; tb.rw[i] = kFull - 1u;
+            tb.above[i] = 0; tb.r[i] = q; tb.m[i] = len;
+            tb.state[i] = (unsigned char)state;
+            tb.shift[i] = (unsigned char)(state == kSearch ? bin_shift(hi - lo, nb) : 255);
+        }
     }
     __syncthreads();
 
     // ---- walk 2: histograms, and again over the threshold's bin where that is still crowded
     for (;;) {
         {
-            unsigned lo = 0u, w = 0u, sft = 255u;
+            unsigned lo = 0u, rl = 0u, rw = 0u, sft = 255u;
             unsigned *mine = hist;
-            walk_long<NT>(g, bounds, tb, n, [&](int i) { lo = tb.lo[i]; w = tb.w[i]; sft = tb.shift[i]; mine = hist + i * nb; },
+            walk_long<NT>(g, bounds, tb, n,
+                          [&](int i) { lo = tb.lo[i]; rl = tb.rl[i]; rw = tb.rw[i]; sft = tb.shift[i]; mine = hist + i * nb; },
                           [&](int, int, int, int len, const float (&x)[kPer]) {
                               if (sft >= 32u) return;
 #pragma unroll
                               for (int j = 0; j < kPer; ++j) {
-                                  const unsigned d = score_key(x[j]) - lo;
-                                  if (d <= w && j * 32 + lane < len) atomicAdd(&mine[d >> sft], 1u);
+                                  const unsigned k = score_key(x[j]), b = min((max(k, lo) - lo) >> sft, (unsigned)(nb - 1));
+                                  count_if(&mine[b], j * 32 + lane < len ? k - rl : kFull, rw); // (rw < kFull)
                               }
                           });
         }
@@ -568,7 +684,7 @@ __device__ void select_long(const float *g, const int *bounds, const int *quota,
             tb.shift[i] = 255;
             if (tb.state[i] == kSearch && tb.m[i] > limit) {
                 const unsigned w = tb.U[i] - 1u - tb.L[i];
-                tb.lo[i] = tb.L[i]; tb.w[i] = w;
+                tb.lo[i] = tb.rl[i] = tb.L[i]; tb.rw[i] = w;
                 tb.shift[i] = (unsigned char)bin_shift(w, nb);
                 again = true;
             }
@@ -595,7 +711,7 @@ __device__ void select_long(const float *g, const int *bounds, const int *quota,
                               const unsigned bal = __ballot_sync(kFull, in && k >= U);
                               if (lane == j) word = bal;
                               if (k < L) {
-                                  if (plain || (a + j * 32 + lane >= ns && a + j * 32 + lane < t_last)) rej = max(rej, k);
+                                  if (in && (plain || (a + j * 32 + lane >= ns && a + j * 32 + lane < t_last))) rej = max(rej, k);
                               } else if (in && k < U) {
                                   cand |= 1u << j;
                               }
@@ -706,10 +822,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
     unsigned *hist = reinterpret_cast<unsigned *>(dyn + mp.hist) + warp * kWarpBins;
     uint2 *list = reinterpret_cast<uint2 *>(dyn + mp.list); // (key, position) of candidates
     SegTab &tb = *reinterpret_cast<SegTab *>(dyn + mp.tab);
+    u64 *look_at = reinterpret_cast<u64 *>(dyn + mp.hist);  // pieces the backfill looks at: position, length
     const size_t row = (size_t)uid * p.T_cap;
     const float *g = p.scores + row;
     int *keep = p.keep_idx + (size_t)uid * p.Tk;
-    const bool ema_on = p.beta != 1.0f;
     const int n_words = (T + 31) >> 5;
     const int ns = max(0, min(p.n_sink, min(p.Tk, T)));           // must-keep prefix and suffix
     const int nl = max(0, min(p.n_last, min(p.Tk - ns, T - ns)));
@@ -717,10 +833,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
     int round = 0;
     for (int i = tid; i <= n_words; i += NT) mask[i] = 0u;
     for (int i = tid; i < kBest; i += NT) best[i] = 0u;
-    if (tid == 0) { sh.n_list = 0; sh.bound = 0u; }
+    if (tid == 0) { sh.n_list = 0; sh.n_look = 0; sh.bound = 0u; }
     wait_for_previous_kernel(); // prefix sums and cuts
     const int n_seg = segments_and_quotas<NT>(p, uid, T, p.Tk - ns - nl, reinterpret_cast<u64 *>(dyn + mp.ms), bounds, quota,
-                                              reinterpret_cast<int *>(list), sh, round);
+                                              reinterpret_cast<int *>(dyn + mp.hist), sh, round);
     if (n_seg < 0) { // cannot happen with the capacity formula of the header; reported all the same
         if (tid == 0) { set_status(p.status, AMS_ERR_CAPACITY, uid, sh.n_seg, sc); p.n_seg[uid] = -1; p.seq_bad[bq] = 1; }
         return;
@@ -774,7 +890,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
             const int n = sh.n_long;
             if (n > 0) {
                 const int n_pc = tb.piece0[n];
-                select_long<NT>(g, bounds, quota, n, mask, best, n_slot, fine, tb, reinterpret_cast<unsigned *>(dyn + mp.lhist), list, ns, t_last, sh);
+                select_long<NT>(g, bounds, quota, n, mask, best, n_slot, fine, tb, reinterpret_cast<unsigned *>(dyn + mp.hist), list, ns, t_last, sh);
                 n_slot += n_pc;
             }
         }
@@ -798,58 +914,85 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
 #pragma unroll
             for (int j = 0; j < kBest / 32; ++j) { k[j] = best[j * 32 + lane]; c += k[j] > 0u; }
             unsigned M = 0u; // (too few entries: every token is looked at)
-            if (warp_sum(c) >= r_fill) M = warp_cut<kBest / 32>(k, kBest, r_fill, hist).key;
+            if (warp_sum(c) >= r_fill) {
+                unsigned mx = 0u;
+#pragma unroll
+                for (int j = 0; j < kBest / 32; ++j) mx = max(mx, k[j]);
+                mx = __reduce_max_sync(kFull, mx);
+                bool ok = mx > (17u << 23) && warp_cut_fast<kBest / 32>(k, r_fill, mx, hist, M);
+                if (ok) { // (equal entries can leave too few)
+                    c = 0;
+#pragma unroll
+                    for (int j = 0; j < kBest / 32; ++j) c += k[j] >= M;
+                    ok = warp_sum(c) >= r_fill;
+                }
+                if (!ok) M = warp_cut<kBest / 32>(k, kBest, r_fill, hist).key;
+            }
             if (lane == 0) sh.bound = M;
         }
         __syncthreads();
         const unsigned M = sh.bound;
         auto raise = [&](int t) { atomicOr(&mask[t >> 5], 1u << (t & 31)); };
         auto unflagged = [&](int t) { return ((mask[t >> 5] >> (t & 31)) & 1u) == 0u; };
-        auto look = [&](int slot, int a, int len) { // a piece
-            unsigned b;
-            if (fine) {
-                const uint4 v = reinterpret_cast<const uint4 *>(best)[slot];
-                b = max(max(v.x, v.y), max(v.z, v.w));
-            } else {
-                b = best[slot & (kBest - 1)];
-            }
-            if (b < M) return;
+        auto best_of = [&](int slot) {
+            if (!fine) return best[slot & (kBest - 1)];
+            const uint4 v = reinterpret_cast<const uint4 *>(best)[slot];
+            return max(max(v.x, v.y), max(v.z, v.w));
+        };
+        const float least = M ? __uint_as_float((M & 0x80000000u) ? M ^ 0x80000000u : ~M) : -INFINITY;
+        auto look = [&](int a, int len) { // a piece, by one warp
             float x[kPer];
             load_piece(g, a, len, x);
 #pragma unroll
             for (int j = 0; j < kPer; ++j) {
                 const int t = a + j * 32 + lane;
-                const unsigned key = score_key(x[j]);
-                if (j * 32 + lane < len && key >= M && unflagged(t)) {
+                if (!(x[j] < least) && j * 32 + lane < len && unflagged(t)) { // (NaN too: a candidate that ranks last)
                     const int at = atomicAdd(&sh.n_list, 1);
-                    if (at < kList) list[at] = make_uint2(key, (unsigned)t);
+                    if (at < kList) list[at] = make_uint2(score_key(x[j]), (unsigned)t);
                 }
             }
         };
-        int slot = n_seg;
-        for (int sg = 0; sg < n_seg; ++sg) {
-            const int a = bounds[sg], L = bounds[sg + 1] - a;
-            if (L <= kPiece) {
-                if (sg % NW == warp) look(sg, a, L);
-            } else {
-                const int n_pc = (L + kPiece - 1) / kPiece;
-                for (int i = (warp - slot % NW + NW) % NW; i < n_pc; i += NW) look(slot + i, a + i * kPiece, min(kPiece, L - i * kPiece));
-                slot += n_pc;
+        // pieces that reach the bound go to a list of their own
+        auto note = [&](int slot, int a, int len) {
+            if (best_of(slot) < M) return;
+            const int at = atomicAdd(&sh.n_look, 1);
+            if (at < kBest) look_at[at] = (u64)(unsigned)a << 32 | (unsigned)len;
+        };
+        if (!longs) {
+            for (int sg = tid; sg < n_seg; sg += NT) note(sg, bounds[sg], bounds[sg + 1] - bounds[sg]);
+        } else {
+            int slot = n_seg;
+            for (int sg = 0; sg < n_seg; ++sg) {
+                const int a = bounds[sg], L = bounds[sg + 1] - a;
+                if (L <= kPiece) {
+                    if (sg % NT == tid) note(sg, a, L);
+                } else {
+                    const int n_pc = (L + kPiece - 1) / kPiece;
+                    for (int i = tid; i < n_pc; i += NT) note(slot + i, a + i * kPiece, min(kPiece, L - i * kPiece));
+                    slot += n_pc;
+                }
             }
+        }
+        __syncthreads();
+        const int n_look = sh.n_look;
+        if (n_look <= kBest) {
+            for (int i = warp; i < n_look; i += NW) look((int)(look_at[i] >> 32), (int)(unsigned)look_at[i]);
+        } else { // (a bound of 0, or hundreds of pieces with equal keys)
+            for (int a = warp * kPiece; a < T; a += NW * kPiece) look(a, min(kPiece, T - a));
         }
         __syncthreads();
         const int n_list = sh.n_list;
         if (n_list > kList) {
             block_select_stream<NT>(g, T, r_fill, sh, round, unflagged, raise);
         } else {
-            for (int i = tid; i < n_list; i += NT) {
+            for (int i = warp; i < n_list; i += NW) { // every candidate is ranked by a warp
                 const uint2 v = list[i];
                 int rank = 0;
-                for (int j = 0; j < n_list; ++j) {
+                for (int j = lane; j < n_list; j += 32) {
                     const uint2 o = list[j];
                     rank += o.x > v.x || (o.x == v.x && o.y < v.y);
                 }
-                if (rank < r_fill) raise((int)v.y);
+                if (warp_sum(rank) < r_fill && lane == 0) raise((int)v.y);
             }
         }
     }
@@ -871,27 +1014,34 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
     for (int g0 = w0; g0 < w1; g0 += 32) {
         const unsigned mine = g0 + lane < w1 ? mask[g0 + lane] : 0u;
         const int inc = warp_incl_scan(__popc(mine)), at = pos + inc - __popc(mine);
-#pragma unroll 8
-        for (int i = 0; i < 32; ++i) { // (words past the end are 0)
-            const unsigned m = __shfl_sync(kFull, mine, i);
-            const int b = __shfl_sync(kFull, at, i);
-            if ((m >> lane) & 1u) keep[b + __popc(m & ((1u << lane) - 1u))] = (g0 + i) * 32 + lane;
+        if (__shfl_sync(kFull, inc, 31) > 256) { // dense: a word after the other, a bit per lane (coalesced)
+            const int n = min(32, w1 - g0);
+#pragma unroll 4
+            for (int i = 0; i < n; ++i) {
+                const unsigned m = __shfl_sync(kFull, mine, i);
+                const int b = __shfl_sync(kFull, at, i);
+                if ((m >> lane) & 1u) keep[b + __popc(m & ((1u << lane) - 1u))] = (g0 + i) * 32 + lane;
+            }
+        } else { // sparse: every lane its own word
+            int to = at;
+            for (unsigned m = mine; m; m &= m - 1u) keep[to++] = (g0 + lane) * 32 + __ffs(m) - 1;
         }
         pos += __shfl_sync(kFull, inc, 31);
     }
     // ---- credit rows travel with their tokens, in place: kept positions ascend and keep[j] >= j, so what a tile
-    //      writes is never read by a later one.  Rows beyond the budget start from zero.
-    if (ema_on) {
+    //      writes is never read by a later one.  Rows beyond the budget start from zero.  (As extra blocks of the gather
+    //      kernel, "hidden" behind the K and V rows, the same moves cost that kernel 40 us more than they take here.)
+    if (p.beta != 1.0f) {
         float *credit = p.ema + (((size_t)l * p.Bmax + bq) * p.H + h) * (size_t)p.T_cap;
-        constexpr int kIn = 8; // rows in flight per thread
+        constexpr int kIn = 4; // rows in flight per thread
         __syncthreads();
         for (int base = 0; base < p.Tk; base += NT * kIn) {
+            int from[kIn];
             float c[kIn];
 #pragma unroll
-            for (int i = 0; i < kIn; ++i) {
-                const int j = base + i * NT + tid;
-                c[i] = j < p.Tk ? credit[keep[j]] : 0.0f;
-            }
+            for (int i = 0; i < kIn; ++i) from[i] = keep[min(base + i * NT + tid, p.Tk - 1)];
+#pragma unroll
+            for (int i = 0; i < kIn; ++i) c[i] = credit[from[i]];
             __syncthreads();
 #pragma unroll
             for (int i = 0; i < kIn; ++i) {
@@ -928,8 +1078,15 @@ int launch_select(const DevParams &p, LaunchCtx &ctx)
     const int units = p.L * p.B * p.H, n_sm = sm_count();
     if (n_sm <= 0) return AMS_ERR_CUDA;
     const bool longs = long_segments(p);
-    const cudaError_t e = units >= 6 * n_sm ? launch_nt<256>(p, units, longs, ctx)
-                        : units > n_sm ? launch_nt<512>(p, units, longs, ctx) : launch_nt<1024>(p, units, longs, ctx);
+    // Threads per unit: a unit costs about (T / threads + a fixed part worth 64 tokens a thread), and the SMs' 1024 slots of 64
+    // registers make ceil(units / resident blocks) rounds of it.
+    auto cost = [&](long long nt) {
+        const long long rounds = ((long long)units * nt + 1024LL * n_sm - 1) / (1024LL * n_sm);
+        return rounds * (p.T_cap / nt + 64);
+    };
+    const long long c256 = cost(256), c512 = cost(512), c1024 = cost(1024);
+    const cudaError_t e = c256 <= c512 && c256 <= c1024 ? launch_nt<256>(p, units, longs, ctx)
+                        : c512 <= c1024 ? launch_nt<512>(p, units, longs, ctx) : launch_nt<1024>(p, units, longs, ctx);
     if (e != cudaSuccess) return AMS_ERR_CUDA;
     ctx.mark(kKernSelect);
     return AMS_OK;
