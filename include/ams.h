@@ -225,7 +225,7 @@ const char *ams_kernel_name(int32_t idx);
  * must-keep, backfill) on caller-supplied scores and writes the kept positions; there is
  * no EMA credit (the mass is that of the given scores alone), no K/V movement, no handle
  * and no workspace argument.  The scratch is a fixed device array inside the library
- * (about 2.4 MB, held by every GPU that loads the library until the process exits).
+ * (a status word and two flags per row, held by every GPU that loads the library until the process exits).
  *   scores   : DEVICE fp32 [n_units][score_stride], score_stride a multiple of 16, >= seq_len
  *   keep_idx : DEVICE int32 [n_units][budget], ascending positions
  *   cfg      : only l_min, l_max, q_min, n_sink, n_last and eps are read

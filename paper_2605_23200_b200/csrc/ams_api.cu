@@ -8,7 +8,7 @@
 namespace ams {
 
 struct Layout {
-    size_t status, eff_lens, seq_bad, scores, usage, logits, ex_logits, cbuf, n_seg, raw_cuts, seg_bounds, quotas, keep_idx, part, fin, total;
+    size_t status, eff_lens, seq_bad, scores, usage, logits, ex_logits, n_seg, seg_bounds, quotas, keep_idx, part, fin, total;
     int units, T_cap, seg_cap, n_slices, slice_len, rows_pad_cap;
 };
 
@@ -89,9 +89,7 @@ static Layout make_layout(const ams_config *c)
     y.scores = off;     off = align_up(off + U * T * 4, 256);
     // second per-token array: the usage when it is smoothed or comes from another scorer than the base scores
     y.usage = off;      off = align_up(off + ((c->pool_kernel > 1 || c->decoupled) ? U * T * 4 : 0), 256);
-    y.cbuf = off;       off = align_up(off + U * T * 8, 256);
     y.n_seg = off;      off = align_up(off + U * 4, 256);
-    y.raw_cuts = off;   off = align_up(off + U * (size_t)(c->max_segments + 1) * 4, 256);
     y.seg_bounds = off; off = align_up(off + U * (size_t)(y.seg_cap + 1) * 4, 256);
     y.quotas = off;     off = align_up(off + U * (size_t)y.seg_cap * 4, 256);
     y.keep_idx = off;   off = align_up(off + U * (size_t)c->max_budget * 4, 256);
@@ -188,7 +186,7 @@ int ams_init_state(const ams_config *cfg, void *ema_state, void *workspace, size
     // status word, effective lengths and error flags; kept positions and segment counts start from zero so that
     // nothing downstream ever indexes with an uninitialised value
     if (cudaMemsetAsync(workspace, 0, lay.scores, s) != cudaSuccess) return AMS_ERR_CUDA;
-    if (cudaMemsetAsync((unsigned char *)workspace + lay.n_seg, 0, lay.raw_cuts - lay.n_seg, s) != cudaSuccess) return AMS_ERR_CUDA;
+    if (cudaMemsetAsync((unsigned char *)workspace + lay.n_seg, 0, lay.seg_bounds - lay.n_seg, s) != cudaSuccess) return AMS_ERR_CUDA;
     if (cudaMemsetAsync((unsigned char *)workspace + lay.keep_idx, 0, lay.part - lay.keep_idx, s) != cudaSuccess) return AMS_ERR_CUDA;
     ams_state *st = new (std::nothrow) ams_state;
     if (!st) return AMS_ERR_INTERNAL;
@@ -259,10 +257,8 @@ int ams_compress(ams_state *st, void *k_pages, void *v_pages, int64_t num_pages,
         p.usage = ext_usage ? ext_usage : ext_scores;
     }
     float *usage_buf = (float *)(st->ws + y.usage);
-    p.cbuf = (u64 *)(st->ws + y.cbuf);
     p.n_seg = (int *)(st->ws + y.n_seg); p.seg_bounds = (int *)(st->ws + y.seg_bounds);
     p.quotas = (int *)(st->ws + y.quotas); p.keep_idx = (int *)(st->ws + y.keep_idx);
-    p.raw_cuts = (int *)(st->ws + y.raw_cuts);
     p.mass_dbg = dbg ? dbg->mass : nullptr;
     p.seg_out = dbg && (dbg->n_segments || dbg->seg_bounds || dbg->quotas || dbg->keep_idx);
     p.part = (float *)(st->ws + y.part); p.fin = (float *)(st->ws + y.fin);
@@ -309,11 +305,7 @@ int ams_compress(ams_state *st, void *k_pages, void *v_pages, int64_t num_pages,
     if (rc == AMS_OK) rc = segsel_supported(p) ? launch_segsel(p, ctx) : AMS_ERR_UNSUPPORTED;
     if (rc == AMS_OK && dbg) {
         // inspection copies are taken before the table is rewritten
-        const size_t U = (size_t)p.L * p.B * p.H;
-        cudaError_t e = cudaSuccess;
-        if (dbg->scores && e == cudaSuccess) e = cudaMemcpyAsync(dbg->scores, p.scores, U * p.T_cap * 4, cudaMemcpyDeviceToDevice, s);
-        if (dbg->usage && e == cudaSuccess) e = cudaMemcpyAsync(dbg->usage, p.usage, U * p.T_cap * 4, cudaMemcpyDeviceToDevice, s);
-        if (e != cudaSuccess) rc = AMS_ERR_CUDA;
+        if (dbg->scores || dbg->usage) rc = launch_inspect_scores(p, *dbg, ctx);
         if (rc == AMS_OK && p.seg_out) rc = launch_inspect(p, *dbg, ctx);
         if (rc == AMS_OK && dbg->prev_kept && dbg->retained_iou) rc = launch_retained_iou(p, dbg->prev_kept, dbg->retained_iou, ctx);
     }

@@ -32,6 +32,7 @@ struct DevParams {
     const int *seq_lens;              // effective lengths of this call ([B], workspace): the caller's length where the
                                       // sequence is compressed, 0 where it is skipped (within the budget) or was
                                       // reported (over capacity, window longer than the sequence, bad page id)
+    int fixed_len;                    // with seq_lens null: the length of every sequence
     int *seq_lens_out;                // the caller's lengths, rewritten by the table update
     const __nv_bfloat16 *q;           // [L][B][H*G][W][128]
     float *ema;                       // [L][Bmax][H][T_cap]
@@ -39,13 +40,10 @@ struct DevParams {
     // per-unit working arrays, [L*B*H][...]
     const float *usage;               // u: what the mass is built from
     float *scores;                    // g: what segments rank by (== usage unless external)
-    u64 *cbuf;                        // [T_cap]  integer mass, then its inclusive prefix sum
-    unsigned char *flags;             // [T_cap]  1 = kept
     int *n_seg;                       // [1]
     int *seg_bounds;                  // [seg_cap + 1]
     int *quotas;                      // [seg_cap]
     int *keep_idx;                    // [Tk]
-    int *raw_cuts;                    // [S + 1]  cut after the token that reaches mass quantile k (T: none)
     float *mass_dbg;                  // [T_cap] or null
     int seg_out;                      // segments and quotas are wanted by the caller: write n_seg, seg_bounds, quotas
     // scorer scratch
@@ -75,6 +73,8 @@ __device__ __forceinline__ void set_status(int *status, int code, int unit, int 
         status[3] = b;
     }
 }
+
+__device__ __forceinline__ int seq_len_of(const DevParams &p, int b) { return p.seq_lens ? p.seq_lens[b] : p.fixed_len; }
 
 // Element offset of the 128-wide row (layer, page, slot, head) in a page pool.
 __device__ __forceinline__ size_t row_offset(const DevParams &p, int layer, int page, int slot, int h)
@@ -263,9 +263,7 @@ int launch_score_keydiff(const DevParams &p, LaunchCtx &ctx);
 bool expected_supported(const DevParams &p);
 int launch_score_expected(const DevParams &p, LaunchCtx &ctx);
 bool segsel_supported(const DevParams &p);   // shared-memory need of the selection kernels fits (always, within the configuration limits)
-int launch_segsel(const DevParams &p, LaunchCtx &ctx); // Algorithm 1 steps 1-5: k_mass_scan, then launch_select
-size_t select_smem_bytes(const DevParams &p);
-int launch_select(const DevParams &p, LaunchCtx &ctx);
+int launch_segsel(const DevParams &p, LaunchCtx &ctx); // Algorithm 1 steps 1-5
 int launch_gather(const DevParams &p, LaunchCtx &ctx);
 int launch_smooth_usage(const DevParams &p, const float *src, float *dst, int k, LaunchCtx &ctx);
 // First kernel of an event: validates lengths and page ids, writes the effective lengths (lens_in: the caller's).
@@ -300,6 +298,7 @@ inline bool grant_dynamic_smem(K kernel, size_t smem, SmemGrant &g)
     }
     return true;
 }
+int launch_inspect_scores(const DevParams &p, const ams_debug_views &v, LaunchCtx &ctx); // scores, usage -> views
 int launch_inspect(const DevParams &p, const ams_debug_views &v, LaunchCtx &ctx); // segments, quotas, kept positions -> views
 int launch_retained_iou(const DevParams &p, const int *prev_kept, float *out, LaunchCtx &ctx); // before the lengths are rewritten
 

@@ -1,7 +1,18 @@
-// Algorithm 1 steps 3-5 of the paper for all (layer, sequence, KV head) units of an event, from the prefix sums and
-// mass-quantile cuts of k_mass_scan: segments (merge, split) and their quotas, per-segment top-q_i, must-keep prefix
-// and suffix, backfill to exactly the budget, ordered kept positions and the credit rows that travel with them.  One
-// block per unit, one kept bit per token in shared memory.
+// Algorithm 1 steps 1-5 of the paper for all (layer, sequence, KV head) units of an event, in one kernel with one block per
+// unit: Eq. 1 on fixed-point weights, the EMA credit update and the history-aware mass (Section 3.3, "EMA credit"; steps
+// 1-2), the mass-quantile cuts b_k = min{t : c(t) >= k / S} (step 3), segments (merge, split) and their quotas (steps 3-4),
+// per-segment top-q_i, must-keep prefix and suffix, backfill to exactly the budget, ordered kept positions and the credit
+// rows that travel with them (step 5).
+//
+// Every decision is integer arithmetic on fixed-point images of the mass (kFixBits fractional bits) and every
+// floating-point step a single round-to-nearest operation, so results do not depend on the order in which a block adds
+// things up.
+//
+// The mass takes one walk over the unit's row per reduction that the arithmetic needs (largest weight, sum of the images,
+// credit and its maximum, sum of the credit's images, mass), a warp taking 256-token pieces.  The last walk leaves one sum
+// per 32-token window in shared memory; the cuts and the masses of the segments need the mass at a hundred positions or
+// so, for which the tokens of one window are computed again.  (A prefix sum of every token in memory, 8 bytes each, cost
+// three times the instructions, 290 MB of traffic on the ragged batch, and a kernel of its own.)
 //
 // Selection order is (score key descending, position ascending), a strict total order, so a segment and its quota have
 // exactly one answer however it is found.  Finding the q-th largest key is what costs.  It is bound by latency and issue
@@ -17,10 +28,8 @@
 //     the same share of the walks whatever the lengths of the segments.
 // The backfill takes its bound from the best rejected key of every piece, which the searches leave behind, and looks only
 // at pieces that reach it, instead of walking the sequence twice.
-// Placing segments and quotas here, by the block that needs them, costs 5 k cycles of latency; a kernel of one-warp blocks
-// in front took 16 to 54 us.  Both together, us per event before / now: 256 units of 16384 tokens 76 / 39, 1792 ragged
-// units of 8192..32768 tokens 401 / 200, 1792 units of 4224 tokens 168 / 96, 2048 units of 32768 tokens in long segments
-// 528 / 330.
+#include <type_traits>
+
 #include "ams_common.cuh"
 #include "ams_select.cuh"
 
@@ -72,11 +81,14 @@ __host__ __device__ inline SelSmem sel_smem(int T_cap, int sc, int S, bool longs
     m.quota = o;  o += (size_t)sc * 4;
     o = (o + 15) & ~(size_t)15;
     m.best = o;   o += (size_t)kBest * 4;
-    m.list = o;   o += (size_t)Tune<NT>::kList * 8;
+    o = (o + 15) & ~(size_t)15;
+    const size_t wsum = (size_t)((T_cap + 31) / 32) * 8, list = (size_t)Tune<NT>::kList * 8;
+    m.list = o;   o += wsum > list ? wsum : list; // the windows' sums of the mass, then candidates
+    o = (o + 15) & ~(size_t)15;
     // one area in turn for: the quota computation, the warps' histograms, those of the long segments, the backfill's bound
     // and the pieces it looks at
     m.hist = o;
-    const size_t q = (size_t)(S + 1) * 8 + (size_t)sc * 4, w = (size_t)(NT / 32) * kWarpBins * 4, l = longs ? (size_t)Tune<NT>::kBins * 4 : 0;
+    const size_t q = (size_t)(S + 1) * 12 + (size_t)sc * 4, w = (size_t)(NT / 32) * kWarpBins * 4, l = longs ? (size_t)Tune<NT>::kBins * 4 : 0;
     o += q > w ? (q > l ? q : l) : (w > l ? w : l);
     o = (o + 15) & ~(size_t)15;
     m.tab = o;    o += longs ? sizeof(SegTab) : 0;
@@ -85,6 +97,7 @@ __host__ __device__ inline SelSmem sel_smem(int T_cap, int sc, int S, bool longs
 }
 
 struct SelShared {
+    u64 scratch[40];
     int wc[2][32];   // per-warp counts of even / odd rounds of a block-wide count
     int n_list, n_look, n_long, total;
     unsigned bound;
@@ -115,6 +128,233 @@ __device__ __forceinline__ int block_count(int c, int &round, SelShared &sh)
     if (lane == 0) mine[threadIdx.x >> 5] = c;
     __syncthreads();
     return warp_sum(lane < NT / 32 ? mine[lane] : 0);
+}
+
+// ------------------------------------------------------------------------------------------- the mass
+
+// Calls f(a, room, full) for the 256-token pieces of [0, T): the lane's tokens are a + lane + 32 j for 32 j < room; full
+// (a compile-time flag) says that all eight exist.
+template <int NT, typename F>
+__device__ __forceinline__ void walk_pieces(int T, F f)
+{
+    const int lane = threadIdx.x & 31;
+    for (int a = (threadIdx.x >> 5) * kPiece; a < T; a += NT / 32 * kPiece) {
+        if (a + kPiece <= T) f(a, kPiece, std::true_type{});
+        else f(a, T - a - lane, std::false_type{});
+    }
+}
+
+// Block-wide sum of doubles that are multiples of one unit and whose sum has fewer than 53 bits of it (exact, hence
+// independent of the order).
+__device__ __forceinline__ double block_sum_exact_f64(double v, u64 *scratch)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+    __syncthreads();
+    if (lane == 0) scratch[warp] = (u64)__double_as_longlong(v);
+    __syncthreads();
+    double x = lane < nw ? __longlong_as_double((long long)scratch[lane]) : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+    return x;
+}
+// Block-wide maximum of non-negative floats.
+__device__ __forceinline__ float block_max_pos(float v, u64 *scratch)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const unsigned m = __reduce_max_sync(kFull, __float_as_uint(v));
+    __syncthreads();
+    if (lane == 0) scratch[warp] = m;
+    __syncthreads();
+    return __uint_as_float(__reduce_max_sync(kFull, lane < nw ? (unsigned)scratch[lane] : 0u));
+}
+// Sum over a warp of 37-bit integers.
+__device__ __forceinline__ u64 warp_sum_mass(u64 h)
+{
+    const unsigned lo = __reduce_add_sync(kFull, (unsigned)h & 0xfffffu), hi = __reduce_add_sync(kFull, (unsigned)(h >> 20));
+    return ((u64)hi << 20) + lo;
+}
+
+// What the integer mass of a token is made of.
+struct Mass {
+    const float *u, *credit;
+    float eps, cut_w, cut_c;
+    double inv_sa_w, inv_sc_c, beta, omb; // 2^(36 - e_w) / SA, 2^(36 - e_c) / SC
+    bool ema, have_credit;
+
+    __device__ __forceinline__ double share(float x) const // Eq. 1 mass of a token with usage x
+    {
+        return __dmul_rn((double)fixed_trunc_by_add(weight_of(x, eps), cut_w), inv_sa_w);
+    }
+    // history-aware integer mass floor((beta m + (1 - beta) normalize(c)) 2^36)
+    __device__ __forceinline__ u64 of(float x, float c) const
+    {
+        double r = share(x);
+        if (ema) {
+            double hist = 0.0;
+            if (have_credit) hist = __dmul_rn(omb, __dmul_rn((double)fixed_trunc_by_add(c, cut_c), inv_sc_c));
+            r = __dadd_rn(__dmul_rn(beta, r), hist);
+        }
+        return floor_to_u64(__dmul_rn(r, (double)(1ull << kFixBits)));
+    }
+    __device__ __forceinline__ u64 at(int t) const { return of(u[t], have_credit ? credit[t] : 0.0f); }
+};
+
+// Eq. 1, credit update, integer mass: exclusive sums of the 32-token windows into wsum; returns the total.
+template <int NT>
+__device__ u64 mass_of_unit(const DevParams &p, int uid, int T, float *credit, u64 *wsum, Mass &ms, SelShared &sh)
+{
+    constexpr int NW = NT / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const size_t row = (size_t)uid * p.T_cap;
+    const float *u = p.usage + row;
+    float *mass_dbg = p.mass_dbg ? p.mass_dbg + row : nullptr;
+    ms.u = u; ms.credit = credit; ms.eps = p.eps;
+    ms.ema = p.beta != 1.0f;
+    ms.have_credit = false;
+    ms.cut_c = 0.0f; ms.inv_sc_c = 0.0;
+    ms.beta = (double)p.beta; ms.omb = __dsub_rn(1.0, ms.beta);
+    // ---- largest Eq. 1 weight (that of the largest usage) -> exponent of the fixed-point images
+    float umax = 0.0f;
+    walk_pieces<NT>(T, [&](int a, int room, auto full) {
+        float x[kPer];
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) x[j] = decltype(full)::value || j * 32 < room ? u[a + j * 32 + lane] : 0.0f;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) umax = fmaxf(umax, x[j]);
+    });
+    const int ew = fix_exponent(weight_of(block_max_pos(umax, sh.scratch), p.eps));
+    // ---- SA = sum of the images A_t = floor(w_t 2^(36 - ew)); the truncated weights are added unscaled (multiples of
+    //      2^(ew - 36) below 2^(ew + 17): exact)
+    const double scale_w = fix_scale_of(ew);
+    ms.cut_w = fixed_trunc_threshold(ew); // weights below it lose their bits under the image's last one
+    double sa = 0.0;
+    walk_pieces<NT>(T, [&](int a, int room, auto full) {
+        float x[kPer];
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) x[j] = decltype(full)::value || j * 32 < room ? u[a + j * 32 + lane] : 0.0f;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j)
+            if (decltype(full)::value || j * 32 < room) sa += (double)fixed_trunc_by_add(weight_of(x[j], p.eps), ms.cut_w);
+    });
+    const double SA = __dmul_rn(block_sum_exact_f64(sa, sh.scratch), scale_w);
+    ms.inv_sa_w = __dmul_rn(__ddiv_rn(1.0, SA), scale_w); // normalisations multiply by the rounded reciprocal; the scaling is exact
+
+    // ---- EMA credit: c <- lambda c + (1 - lambda) m, updated in place (the block-wide reductions that follow
+    //      make every thread's writes visible to the others before anybody reads them back)
+    if (ms.ema) {
+        const float oml = __fsub_rn(1.0f, p.lambda);
+        float cmax = 0.0f;
+        walk_pieces<NT>(T, [&](int a, int room, auto full) {
+            float x[kPer], c[kPer];
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+                x[j] = c[j] = 0.0f;
+                if (decltype(full)::value || j * 32 < room) { x[j] = u[a + j * 32 + lane]; c[j] = credit[a + j * 32 + lane]; }
+            }
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+                const float m = __double2float_rn(ms.share(x[j]));
+                c[j] = __fadd_rn(__fmul_rn(p.lambda, c[j]), __fmul_rn(oml, m));
+                if (decltype(full)::value || j * 32 < room) {
+                    cmax = fmaxf(cmax, c[j]);
+                    credit[a + j * 32 + lane] = c[j];
+                    if (mass_dbg) mass_dbg[a + j * 32 + lane] = m;
+                }
+            }
+        });
+        cmax = block_max_pos(cmax, sh.scratch);
+        if (cmax > 0.0f) {
+            const int ec = fix_exponent(cmax);
+            const double scale_c = fix_scale_of(ec);
+            ms.cut_c = fixed_trunc_threshold(ec);
+            double sc = 0.0;
+            walk_pieces<NT>(T, [&](int a, int room, auto full) {
+                float c[kPer];
+#pragma unroll
+                for (int j = 0; j < kPer; ++j) c[j] = decltype(full)::value || j * 32 < room ? credit[a + j * 32 + lane] : 0.0f;
+#pragma unroll
+                for (int j = 0; j < kPer; ++j) sc += (double)fixed_trunc_by_add(c[j], ms.cut_c);
+            });
+            const double SC = __dmul_rn(block_sum_exact_f64(sc, sh.scratch), scale_c);
+            ms.have_credit = SC > 0.0;
+            if (ms.have_credit) ms.inv_sc_c = __dmul_rn(__ddiv_rn(1.0, SC), scale_c);
+        }
+    } else if (mass_dbg) {
+        for (int t = tid; t < T; t += NT) mass_dbg[t] = __double2float_rn(ms.share(u[t]));
+    }
+
+    // ---- integer mass, summed per window, and the windows' exclusive sums
+    walk_pieces<NT>(T, [&](int a, int room, auto full) {
+        float x[kPer], c[kPer];
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            x[j] = c[j] = 0.0f;
+            if (decltype(full)::value || j * 32 < room) {
+                x[j] = u[a + j * 32 + lane];
+                if (ms.have_credit) c[j] = credit[a + j * 32 + lane];
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            u64 h = ms.of(x[j], c[j]);
+            if (!(decltype(full)::value || j * 32 < room)) h = 0;
+            const u64 sum = warp_sum_mass(h);
+            if (lane == j && (a >> 5) + j < (T + 31) >> 5) wsum[(a >> 5) + j] = sum;
+        }
+    });
+    __syncthreads();
+    // a warp takes a run of windows, a lane eight at a time
+    const int n_win = (T + 31) >> 5, per = (n_win + NW - 1) / NW, w0 = min(n_win, warp * per), w1 = min(n_win, w0 + per);
+    u64 mine = 0;
+    for (int w = w0 + lane; w < w1; w += 32) mine += wsum[w];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(kFull, mine, o);
+    if (lane == 0) sh.scratch[warp] = mine; // (the reductions above ended with reads of this table two barriers ago)
+    __syncthreads();
+    u64 run = lane < warp ? sh.scratch[lane] : 0ull, tot = lane < NW ? sh.scratch[lane] : 0ull;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) { run += __shfl_xor_sync(kFull, run, o); tot += __shfl_xor_sync(kFull, tot, o); }
+    for (int g = w0; g < w1; g += 32) {
+        const u64 v = g + lane < w1 ? wsum[g + lane] : 0ull;
+        u64 inc = v;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const u64 y = __shfl_up_sync(kFull, inc, d);
+            if (lane >= d) inc += y;
+        }
+        if (g + lane < w1) wsum[g + lane] = run + inc - v;
+        run += __shfl_sync(kFull, inc, 31);
+    }
+    __syncthreads();
+    return tot;
+}
+
+// Sum of the integer mass before position b (0 <= b < T), by one warp.
+__device__ __forceinline__ u64 mass_before(const Mass &ms, const u64 *wsum, int b)
+{
+    const int lane = threadIdx.x & 31;
+    return wsum[b >> 5] + warp_sum_mass(lane < (b & 31) ? ms.at((b & ~31) + lane) : 0ull);
+}
+
+// Boundary after the token that reaches `thr` (0 < thr <= total), by one warp.
+__device__ __forceinline__ int mass_cut(const Mass &ms, const u64 *wsum, int T, u64 thr)
+{
+    const int lane = threadIdx.x & 31;
+    int w = 0; // the last window that starts below thr
+    for (int hi = (T + 31) >> 5; hi - w > 1;) {
+        const int mid = (w + hi) >> 1;
+        if (wsum[mid] < thr) w = mid; else hi = mid;
+    }
+    const int t = w * 32 + lane;
+    u64 inc = t < T ? ms.at(t) : 0ull;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const u64 y = __shfl_up_sync(kFull, inc, d);
+        if (lane >= d) inc += y;
+    }
+    return w * 32 + __ffs(__ballot_sync(kFull, wsum[w] + inc >= thr));
 }
 
 // ------------------------------------------------------------------------------- segments and quotas
@@ -194,28 +434,30 @@ __device__ __forceinline__ u64 quotient(u64 x, u64 y, double inv)
 
 // Merge of short and split of long segments, quotas with their adjustment (Section 3.3 of the paper; Algorithm 1 steps
 // 3-4): bounds[0..n], quota[0..n).  Returns n, or -1 if the tables cannot hold the segments.  Bq: the budget less the
-// must-keep positions.  `tmp`: 2 (S + 1) + seg_cap ints.
+// must-keep positions.  SH: total of the integer mass.  `tmp`: 3 (S + 1) + seg_cap ints.
 template <int NT>
-__device__ int segments_and_quotas(const DevParams &p, int uid, int T, int Bq, u64 *Ms, int *bounds, int *quota, int *tmp,
-                                   SelShared &sh, int &round)
+__device__ int segments_and_quotas(const DevParams &p, int T, int Bq, const Mass &ms, const u64 *wsum, u64 SH, u64 *Ms, int *bounds,
+                                   int *quota, int *tmp, SelShared &sh, int &round)
 {
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    int *merged = tmp, *poff = merged + p.S + 1, *cap = poff + p.S + 1;
-    const u64 *C = p.cbuf + (size_t)uid * p.T_cap;
-    const u64 SH = C[T - 1];
+    int *merged = tmp, *poff = merged + p.S + 1, *raw = poff + p.S + 1, *cap = raw + p.S + 1;
     const u64 SHq = p.uniform_q ? (u64)T : SH; // total of what the quotas are proportional to
     const double inv = 1.0 / (double)(2ull * SHq);
+    // raw cuts, ascending: the token that reaches quantile k closes its segment, c(t) >= k / S <=> C(t) >= ceil(k SH / S)
+    for (int k = warp + 1; k < p.S; k += NW) {
+        const int e = p.fixed_seg ? (int)(((long long)k * T) / p.S) // component ablation: boundary k at floor(k T / S)
+                                  : mass_cut(ms, wsum, T, ((u64)k * SH + (u64)p.S - 1) / (u64)p.S);
+        if (lane == 0) raw[k] = e;
+    }
+    __syncthreads();
     if (warp == 0) {
-        // raw cuts of the mass quantiles, ascending, found by the scan kernel (a cut at or beyond T means "none"); short raw
-        // segments merge forward: the next boundary is the first cut at least l_min past the last one
+        // short raw segments merge forward: the next boundary is the first cut at least l_min past the last one
         int nm = 0, start = 0;
         if (lane == 0) merged[0] = 0;
         for (int k0 = 1; k0 < p.S; k0 += 32) {
             const int k = k0 + lane;
-            int e = T;
-            if (k < p.S) e = p.fixed_seg ? (int)(((long long)k * T) / p.S) // component ablation: boundary k at floor(k T / S)
-                                         : p.raw_cuts[(size_t)uid * (p.S + 1) + k];
+            const int e = k < p.S ? raw[k] : T;
             for (;;) {
                 const unsigned can = __ballot_sync(kFull, e < T && e - start >= p.l_min);
                 if (!can) break;
@@ -251,19 +493,37 @@ __device__ int segments_and_quotas(const DevParams &p, int uid, int T, int Bq, u
     }
     __syncthreads();
     // quotas: q_i = q_i^min + round(T_rem M_i / sum M), clipped, then adjusted
-    int smin = 0;
-    for (int i = tid; i < n_seg; i += NT) {
-        const int a = bounds[i], e = bounds[i + 1];
-        Ms[i] = p.uniform_q ? (u64)(e - a) : C[e - 1] - (a > 0 ? C[a - 1] : 0ull); // ablation: share by length
-        smin += max(0, min(p.q_min, e - a));
+    if (!p.uniform_q) {
+        for (int i = warp; i < n_seg; i += NW) { // mass before the segment
+            const u64 c = mass_before(ms, wsum, bounds[i]);
+            if (lane == 0) Ms[i] = c;
+        }
+        __syncthreads();
     }
+    int smin = 0;
+    for (int i = tid; i < n_seg; i += NT) smin += max(0, min(p.q_min, bounds[i + 1] - bounds[i]));
     const int Trem = Bq - block_count<NT>(smin, round, sh);
     int sq = 0;
-    for (int i = tid; i < n_seg; i += NT) {
+    constexpr int kIn = 4096 / NT; // (at most 4096 segments)
+    u64 M[kIn];
+#pragma unroll
+    for (int j = 0; j < kIn; ++j) {
+        const int i = j * NT + tid;
+        M[j] = 0;
+        if (j > 0 && j * NT >= n_seg) break;
+        if (i < n_seg) M[j] = p.uniform_q ? (u64)(bounds[i + 1] - bounds[i]) // ablation: share by length
+                                          : (i + 1 < n_seg ? Ms[i + 1] : SH) - Ms[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kIn; ++j) {
+        const int i = j * NT + tid;
+        if (i >= n_seg) break;
         const int L = bounds[i + 1] - bounds[i];
         long long qi = max(0, min(p.q_min, L));
-        if (Trem >= 0) qi += (long long)quotient(2ull * (u64)Trem * Ms[i] + SHq, 2ull * SHq, inv);
+        if (Trem >= 0) qi += (long long)quotient(2ull * (u64)Trem * M[j] + SHq, 2ull * SHq, inv);
         if (qi > L) qi = L;
+        Ms[i] = M[j];
         quota[i] = (int)qi;
         sq += (int)qi;
     }
@@ -811,7 +1071,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
     constexpr int NW = NT / 32, kList = Tune<NT>::kList;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, uid = blockIdx.x;
     const int h = uid % p.H, bq = (uid / p.H) % p.B, l = uid / (p.H * p.B);
-    const int T = p.seq_lens[bq];
+    wait_for_previous_kernel(); // scores, effective lengths
+    const int T = seq_len_of(p, bq);
     if (T <= p.Tk || T > p.T_cap) return;
     const int sc = p.seg_cap;
     const SelSmem mp = sel_smem<NT>(p.T_cap, sc, p.S, longs != 0);
@@ -834,8 +1095,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
     for (int i = tid; i <= n_words; i += NT) mask[i] = 0u;
     for (int i = tid; i < kBest; i += NT) best[i] = 0u;
     if (tid == 0) { sh.n_list = 0; sh.n_look = 0; sh.bound = 0u; }
-    wait_for_previous_kernel(); // prefix sums and cuts
-    const int n_seg = segments_and_quotas<NT>(p, uid, T, p.Tk - ns - nl, reinterpret_cast<u64 *>(dyn + mp.ms), bounds, quota,
+    float *credit = p.ema ? p.ema + (((size_t)l * p.Bmax + bq) * p.H + h) * (size_t)p.T_cap : nullptr;
+    Mass ms;
+    u64 *wsum = reinterpret_cast<u64 *>(dyn + mp.list);
+    const u64 SH = mass_of_unit<NT>(p, uid, T, credit, wsum, ms, sh);
+    const int n_seg = segments_and_quotas<NT>(p, T, p.Tk - ns - nl, ms, wsum, SH, reinterpret_cast<u64 *>(dyn + mp.ms), bounds, quota,
                                               reinterpret_cast<int *>(dyn + mp.hist), sh, round);
     if (n_seg < 0) { // cannot happen with the capacity formula of the header; reported all the same
         if (tid == 0) { set_status(p.status, AMS_ERR_CAPACITY, uid, sh.n_seg, sc); p.n_seg[uid] = -1; p.seq_bad[bq] = 1; }
@@ -1032,7 +1296,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
     //      writes is never read by a later one.  Rows beyond the budget start from zero.  (As extra blocks of the gather
     //      kernel, "hidden" behind the K and V rows, the same moves cost that kernel 40 us more than they take here.)
     if (p.beta != 1.0f) {
-        float *credit = p.ema + (((size_t)l * p.Bmax + bq) * p.H + h) * (size_t)p.T_cap;
         constexpr int kIn = 4; // rows in flight per thread
         __syncthreads();
         for (int base = 0; base < p.Tk; base += NT * kIn) {
@@ -1071,9 +1334,9 @@ bool long_segments(const DevParams &p) { return p.l_max == 0 || p.l_max > kPiece
 
 } // namespace
 
-size_t select_smem_bytes(const DevParams &p) { return sel_smem<1024>(p.T_cap, p.seg_cap, p.S, long_segments(p)).total; }
+bool segsel_supported(const DevParams &p) { return sel_smem<1024>(p.T_cap, p.seg_cap, p.S, long_segments(p)).total <= (size_t)224 * 1024; }
 
-int launch_select(const DevParams &p, LaunchCtx &ctx)
+int launch_segsel(const DevParams &p, LaunchCtx &ctx)
 {
     const int units = p.L * p.B * p.H, n_sm = sm_count();
     if (n_sm <= 0) return AMS_ERR_CUDA;

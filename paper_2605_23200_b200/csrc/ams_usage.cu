@@ -55,6 +55,17 @@ __global__ void __launch_bounds__(128) k_retained_iou(DevParams p, const int *pr
     out[uid] = either > 0 ? __fdiv_rn((float)both, (float)either) : 0.0f;
 }
 
+// Inspection views of the scores and the usage: whole rows, one block per unit.
+__global__ void __launch_bounds__(256) k_inspect_scores(DevParams p, ams_debug_views v)
+{
+    wait_for_previous_kernel();
+    const size_t row = (size_t)blockIdx.x * p.T_cap;
+    for (int t = threadIdx.x; t < p.T_cap; t += 256) {
+        if (v.scores) v.scores[row + t] = p.scores[row + t];
+        if (v.usage) v.usage[row + t] = p.usage[row + t];
+    }
+}
+
 // Inspection views of the selection, one block per unit: segments, quotas and kept positions go to the caller's arrays in
 // one launch.  Units that were skipped are left untouched.
 __global__ void __launch_bounds__(256) k_inspect(DevParams p, ams_debug_views v)
@@ -139,6 +150,13 @@ int launch_expire_wait(int *status, uint32_t polls, cudaStream_t s)
 {
     k_expire_wait<<<1, 1, 0, s>>>(status, polls);
     return cudaGetLastError() == cudaSuccess ? AMS_OK : AMS_ERR_CUDA;
+}
+
+int launch_inspect_scores(const DevParams &p, const ams_debug_views &v, LaunchCtx &ctx)
+{
+    if (launch_after(k_inspect_scores, dim3((unsigned)(p.L * p.B * p.H)), dim3(256), 0, ctx.s, p, v) != cudaSuccess) return AMS_ERR_CUDA;
+    ctx.mark(kKernSegmentSelect);
+    return AMS_OK;
 }
 
 int launch_inspect(const DevParams &p, const ams_debug_views &v, LaunchCtx &ctx)
