@@ -1341,11 +1341,11 @@ int launch_segsel(const DevParams &p, LaunchCtx &ctx)
     const int units = p.L * p.B * p.H, n_sm = sm_count();
     if (n_sm <= 0) return AMS_ERR_CUDA;
     const bool longs = long_segments(p);
-    // Threads per unit: a unit costs about (T / threads + a fixed part worth 64 tokens a thread), and the SMs' 1024 slots of 64
+    // Threads per unit: a unit costs about (T / threads + a fixed part worth 24 tokens a thread), and the SMs' 1024 slots of 64
     // registers make ceil(units / resident blocks) rounds of it.
     auto cost = [&](long long nt) {
         const long long rounds = ((long long)units * nt + 1024LL * n_sm - 1) / (1024LL * n_sm);
-        return rounds * (p.T_cap / nt + 64);
+        return rounds * (p.T_cap / nt + 24);
     };
     const long long c256 = cost(256), c512 = cost(512), c1024 = cost(1024);
     const cudaError_t e = c256 <= c512 && c256 <= c1024 ? launch_nt<256>(p, units, longs, ctx)
