@@ -47,165 +47,221 @@ __device__ __forceinline__ void lse_merge(float &m, float &z, float m2, float z2
 }
 
 constexpr int kTovaThreads = 128;
-constexpr int kQPitch = 136; // bf16 elements per staged query row: 272 bytes, conflict-free 16-byte reads
+constexpr int kQPitch = 136;   // bf16 elements per staged query row: 272 bytes, conflict-free 16-byte reads
+constexpr int kRing = 3;       // 16-token K tiles per warp in shared memory: one worked on, two on their way
+constexpr int kTileK = 16 * kRowBytes;
 
-// One block = one (unit, token slice).  Each warp walks 16-token tiles; a tile is one
-// page.  The tile is the M operand of m16n8k16 and eight query rows are the N
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+template <int NTB>
+__host__ __device__ constexpr size_t tova_smem(int slice_len)
+{
+    return (size_t)(kTovaThreads / 32) * kRing * kTileK + (NTB > 1 ? (size_t)NTB * 8 * kQPitch * 2 : 0) + (size_t)(slice_len / 16) * 4;
+}
+
+// A block takes (unit, token slice) pairs in turn, all units of a slice number before the next one: the blocks of
+// neighbouring KV heads read the same pages at the same time, and the slices past a sequence's end cost a look at its
+// length instead of a block.  Each warp walks 16-token tiles; a tile is one page.  Its K rows come through a ring of
+// tiles in shared memory (asynchronous copies, two tiles ahead; a chunk of 16 bytes lies at its number XOR 4 in odd rows,
+// so that reads are free of bank conflicts), and the slice's page ids are fetched once.  Bound by the K stream: a warp that
+// loaded a tile into registers and then worked on it reached 4.0 TB/s with 32 query rows.  The
+// tile is the M operand of m16n8k16 and eight query rows are the N
 // operand, both read as 16-byte pieces along d: lane (g, tq) loads d = 32 j + 8 tq
 // .. +7 of its rows, and those eight values feed k-steps 2j and 2j+1.  The same
 // assignment of d to k on both operands leaves the dot product unchanged.
 template <int NTB, int PHASE>
 __global__ void __launch_bounds__(kTovaThreads) k_tova(DevParams p)
 {
-    __shared__ __align__(16) __nv_bfloat16 Qs[NTB > 1 ? NTB * 8 * kQPitch : 8];
+    extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ float red[4][NTB * 8][2];
+    unsigned char *ring = dyn + (threadIdx.x >> 5) * (kRing * kTileK);
+    __nv_bfloat16 *Qs = reinterpret_cast<__nv_bfloat16 *>(dyn + (kTovaThreads / 32) * kRing * kTileK);
+    int *pages = reinterpret_cast<int *>(Qs + (NTB > 1 ? NTB * 8 * kQPitch : 0));
     if (PHASE == 2) wait_for_previous_kernel(); // merged statistics
-    const int uid = blockIdx.y;
-    const int h = uid % p.H, b = (uid / p.H) % p.B, l = uid / (p.H * p.B);
-    const int T = p.seq_lens[b];
-    if (T <= p.Tk || T > p.T_cap) return;
-    if (p.W > T) { if (PHASE == 1 && blockIdx.x == 0 && threadIdx.x == 0) set_status(p.status, AMS_ERR_INVALID_ARG, uid, p.W, T); return; }
-    const int slice = blockIdx.x;
-    const int t_begin = slice * p.slice_len;
-    if (t_begin >= T) return;
-    const int t_end = min(T, t_begin + p.slice_len);
-    const int n_tiles = (t_end - t_begin + 15) >> 4;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, tq = lane & 3;
-    const int *table = p.block_table + (size_t)b * p.bt_stride;
-    const __nv_bfloat16 *Q = p.q + ((((size_t)l * p.B + b) * p.H + h) * p.G) * (size_t)p.W * kHeadDim;
+    const int units = p.L * p.B * p.H, n_slices = (p.T_cap + p.slice_len - 1) / p.slice_len;
     const float c = kLog2e * 0.08838834764831845f; // log2(e) / sqrt(128)
-    const float *fin = p.fin + (size_t)uid * (p.rows_pad + 8);
-    float *u_out = p.scores + (size_t)uid * p.T_cap;
     const int n_rb = p.rows_pad / (NTB * 8);
-    float *lg = (PHASE == 1 && p.logits && n_rb == 1) ? p.logits + (size_t)uid * p.T_cap * (NTB * 8) : nullptr;
-    const float pmax = PHASE == 2 ? fin[p.rows_pad] : 0.0f;
     const float inv_rows = 1.0f / (float)p.rows;
+    const size_t row_stride = (size_t)p.H * kHeadDim; // elements between the slots of a page
 
-    for (int rb = 0; rb < n_rb; ++rb) {
-        const int row0 = rb * NTB * 8;
-        uint4 zq[4];
-        if (NTB > 1) {
-            __syncthreads();
-            for (int i = threadIdx.x; i < NTB * 8 * 16; i += kTovaThreads) {
-                const int r = i >> 4, cpos = i & 15;
-                uint4 v = make_uint4(0, 0, 0, 0);
-                if (row0 + r < p.rows) v = *reinterpret_cast<const uint4 *>(Q + (size_t)(row0 + r) * kHeadDim + cpos * 8);
-                *reinterpret_cast<uint4 *>(Qs + r * kQPitch + cpos * 8) = v;
-            }
-            __syncthreads();
-        } else {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                zq[j] = make_uint4(0, 0, 0, 0);
-                if (row0 + g < p.rows) zq[j] = *reinterpret_cast<const uint4 *>(Q + (size_t)(row0 + g) * kHeadDim + 32 * j + 8 * tq);
-            }
-        }
-        // per thread: rows (nt, e) = row0 + 8 nt + 2 tq + e
-        int lastv[NTB][2];
-        float st_a[NTB][2], st_b[NTB][2]; // phase 1: (m, z); phase 2: (b_r, unused)
-#pragma unroll
-        for (int nt = 0; nt < NTB; ++nt)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int r = row0 + nt * 8 + 2 * tq + e;
-                lastv[nt][e] = r < p.rows ? (p.causal ? T - p.W + (r % p.W) : T - 1) : -1;
-                if (PHASE == 1) { st_a[nt][e] = -INFINITY; st_b[nt][e] = 0.0f; }
-                else { st_a[nt][e] = fin[r]; st_b[nt][e] = 0.0f; }
-            }
+    for (long long item = blockIdx.x; item < (long long)units * n_slices; item += gridDim.x) {
+        const int uid = (int)(item % units), slice = (int)(item / units);
+        const int h = uid % p.H, b = (uid / p.H) % p.B, l = uid / (p.H * p.B);
+        const int T = p.seq_lens[b];
+        if (T <= p.Tk || T > p.T_cap) continue;
+        if (p.W > T) { if (PHASE == 1 && slice == 0 && threadIdx.x == 0) set_status(p.status, AMS_ERR_INVALID_ARG, uid, p.W, T); continue; }
+        const int t_begin = slice * p.slice_len;
+        if (t_begin >= T) continue;
+        const int t_end = min(T, t_begin + p.slice_len);
+        const int n_tiles = (t_end - t_begin + 15) >> 4;
+        const __nv_bfloat16 *Q = p.q + ((((size_t)l * p.B + b) * p.H + h) * p.G) * (size_t)p.W * kHeadDim;
+        const float *fin = p.fin + (size_t)uid * (p.rows_pad + 8);
+        float *u_out = p.scores + (size_t)uid * p.T_cap;
+        float *lg = (PHASE == 1 && NTB <= 2 && p.logits && n_rb == 1) ? p.logits + (size_t)uid * p.T_cap * (NTB * 8) : nullptr;
+        const float pmax = PHASE == 2 ? fin[p.rows_pad] : 0.0f;
+        __syncthreads(); // the previous slice's page ids and queries are no longer read
+        for (int i = threadIdx.x; i < n_tiles; i += kTovaThreads) pages[i] = p.block_table[(size_t)b * p.bt_stride + (t_begin >> 4) + i];
 
-        for (int tile = warp; tile < n_tiles; tile += 4) {
-            const int t0 = t_begin + tile * 16;
-            const int page = table[t0 >> 4];
-            const __nv_bfloat16 *ra = p.k_pages + row_offset(p, l, page, g, h) + 8 * tq;
-            const __nv_bfloat16 *rbp = ra + (size_t)8 * p.H * kHeadDim;
-            uint4 x[4], y[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) { x[j] = ld_stream16(ra + 32 * j); y[j] = ld_stream16(rbp + 32 * j); }
-            const int ta = t0 + g, tb = t0 + g + 8;
-            float acc_a = 0.0f, acc_b = 0.0f;
-#pragma unroll
-            for (int nt = 0; nt < NTB; ++nt) {
-                if (NTB > 1) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        zq[j] = *reinterpret_cast<const uint4 *>(Qs + (nt * 8 + g) * kQPitch + 32 * j + 8 * tq);
+        for (int rb = 0; rb < n_rb; ++rb) {
+            const int row0 = rb * NTB * 8;
+            uint4 zq[4];
+            if (NTB > 1) {
+                if (rb > 0) __syncthreads();
+                for (int i = threadIdx.x; i < NTB * 8 * 16; i += kTovaThreads) {
+                    const int r = i >> 4, cpos = i & 15;
+                    uint4 v = make_uint4(0, 0, 0, 0);
+                    if (row0 + r < p.rows) v = *reinterpret_cast<const uint4 *>(Q + (size_t)(row0 + r) * kHeadDim + cpos * 8);
+                    *reinterpret_cast<uint4 *>(Qs + r * kQPitch + cpos * 8) = v;
                 }
-                float d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            } else {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    mma_bf16(d, x[j].x, y[j].x, x[j].y, y[j].y, zq[j].x, zq[j].y);
-                    mma_bf16(d, x[j].z, y[j].z, x[j].w, y[j].w, zq[j].z, zq[j].w);
-                }
-                float keep_a[2], keep_b[2];
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int lv = min(lastv[nt][e], t_end - 1);
-                    const float va = ta <= lv ? d[e] * c : -INFINITY;
-                    const float vb = tb <= lv ? d[2 + e] * c : -INFINITY;
-                    if (PHASE == 1) {
-                        if (NTB <= 2) { keep_a[e] = va; keep_b[e] = vb; }
-                        const float mn = fmaxf(st_a[nt][e], fmaxf(va, vb));
-                        if (mn != -INFINITY) {
-                            st_b[nt][e] = st_b[nt][e] * ex2(st_a[nt][e] - mn) + ex2(va - mn) + ex2(vb - mn);
-                            st_a[nt][e] = mn;
-                        }
-                    } else {
-                        acc_a += ex2(va - st_a[nt][e]);
-                        acc_b += ex2(vb - st_a[nt][e]);
-                    }
-                }
-                if (PHASE == 1 && NTB <= 2 && lg) { // pairs the window hides are stored as -inf: they add nothing later
-                    if (ta < t_end) *reinterpret_cast<float2 *>(lg + (size_t)ta * (NTB * 8) + nt * 8 + 2 * tq) = make_float2(keep_a[0], keep_a[1]);
-                    if (tb < t_end) *reinterpret_cast<float2 *>(lg + (size_t)tb * (NTB * 8) + nt * 8 + 2 * tq) = make_float2(keep_b[0], keep_b[1]);
+                    zq[j] = make_uint4(0, 0, 0, 0);
+                    if (row0 + g < p.rows) zq[j] = *reinterpret_cast<const uint4 *>(Q + (size_t)(row0 + g) * kHeadDim + 32 * j + 8 * tq);
                 }
             }
-            if (PHASE == 2) {
-                acc_a += __shfl_xor_sync(0xffffffffu, acc_a, 1);
-                acc_a += __shfl_xor_sync(0xffffffffu, acc_a, 2);
-                acc_b += __shfl_xor_sync(0xffffffffu, acc_b, 1);
-                acc_b += __shfl_xor_sync(0xffffffffu, acc_b, 2);
-                if (tq == 0) {
+            __syncthreads();
+            auto fetch = [&](int tile, int slot) { // lane: 16 bytes of two rows at a time
+                if (tile < n_tiles) {
+                    const int r0 = lane >> 4, ch = lane & 15;
+                    const __nv_bfloat16 *src = p.k_pages + row_offset(p, l, pages[tile], r0, h) + ch * 8;
+                    unsigned char *dst = ring + slot * kTileK + r0 * kRowBytes + ((ch ^ (r0 << 2)) << 4);
 #pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int t = e ? tb : ta;
-                        if (t < t_end) {
-                            float v = e ? acc_b : acc_a;
-                            if (rb > 0) v += u_out[t];
-                            if (rb == n_rb - 1) {
-                                const int ninv = p.causal ? p.G * max(0, t - (T - p.W)) : 0;
-                                v = (v + (float)ninv * pmax) * inv_rows;
-                            }
-                            u_out[t] = v;
-                        }
-                    }
+                    for (int i = 0; i < 8; ++i) cp_async16(dst + i * 2 * kRowBytes, src + (size_t)(2 * i) * row_stride);
                 }
-            }
-        }
-
-        if (PHASE == 1) {
-            // rows live in the quad index; fold the eight token groups, then the four warps
+                cp_async_commit();
+            };
+            // per thread: rows (nt, e) = row0 + 8 nt + 2 tq + e
+            int lastv[NTB][2];
+            float st_a[NTB][2], st_b[NTB][2]; // phase 1: (reference, sum of 2^(x - reference)); phase 2: (-b_r, unused)
 #pragma unroll
             for (int nt = 0; nt < NTB; ++nt)
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
+                    const int r = row0 + nt * 8 + 2 * tq + e;
+                    lastv[nt][e] = r < p.rows ? (p.causal ? T - p.W + (r % p.W) : T - 1) : -1;
+                    if (PHASE == 1) { st_a[nt][e] = -INFINITY; st_b[nt][e] = 0.0f; }
+                    else { st_a[nt][e] = -fin[r]; st_b[nt][e] = 0.0f; }
+                }
+
+            fetch(warp, 0);
+            fetch(warp + 4, 1);
+            int slot = 0;
+            for (int tile = warp; tile < n_tiles; tile += 4) {
+                cp_async_wait<1>();
+                __syncwarp();
+                const unsigned char *ta_ = ring + slot * kTileK + g * kRowBytes;
+                uint4 x[4], y[4];
 #pragma unroll
-                    for (int o = 4; o < 32; o <<= 1) {
-                        const float m2 = __shfl_xor_sync(0xffffffffu, st_a[nt][e], o);
-                        const float z2 = __shfl_xor_sync(0xffffffffu, st_b[nt][e], o);
-                        lse_merge(st_a[nt][e], st_b[nt][e], m2, z2);
+                for (int j = 0; j < 4; ++j) {
+                    const int at = ((4 * j + tq) ^ ((g & 1) << 2)) << 4; // (rows g and g + 8 are both odd or both even)
+                    x[j] = *reinterpret_cast<const uint4 *>(ta_ + at);
+                    y[j] = *reinterpret_cast<const uint4 *>(ta_ + 8 * kRowBytes + at);
+                }
+                fetch(tile + 8, slot == 0 ? 2 : slot - 1); // the slot read in the round before
+                slot = slot == 2 ? 0 : slot + 1;
+                const int t0 = t_begin + tile * 16, ta = t0 + g, tb = t0 + g + 8;
+                // every row sees every token of the tile (padding rows are taken care of by their statistics or at the end)
+                const bool plain = t0 + 15 < t_end && t0 + 15 <= (p.causal ? T - p.W : T - 1);
+                float acc_a = 0.0f, acc_b = 0.0f;
+#pragma unroll
+                for (int nt = 0; nt < NTB; ++nt) {
+                    if (NTB > 1) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j)
+                            zq[j] = *reinterpret_cast<const uint4 *>(Qs + (nt * 8 + g) * kQPitch + 32 * j + 8 * tq);
                     }
-                    if (g == 0) {
-                        red[warp][nt * 8 + 2 * tq + e][0] = st_a[nt][e];
-                        red[warp][nt * 8 + 2 * tq + e][1] = st_b[nt][e];
+                    float d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        mma_bf16(d, x[j].x, y[j].x, x[j].y, y[j].y, zq[j].x, zq[j].y);
+                        mma_bf16(d, x[j].z, y[j].z, x[j].w, y[j].w, zq[j].z, zq[j].w);
+                    }
+                    float keep_a[2], keep_b[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        float da = d[e], db = d[2 + e];
+                        if (!plain || lg) { // pairs the window hides add nothing, now or (stored logits) later
+                            const int lv = min(lastv[nt][e], t_end - 1);
+                            da = ta <= lv ? da : -INFINITY;
+                            db = tb <= lv ? db : -INFINITY;
+                        }
+                        if (PHASE == 1) {
+                            if (NTB <= 2) { keep_a[e] = da * c; keep_b[e] = db * c; }
+                            // the reference follows the largest logit at a distance of at most 2^32 in the sum, so that
+                            // rescaling is rare
+                            const float mx = fmaxf(da, db) * c;
+                            if (mx > st_a[nt][e] + 32.0f || (st_a[nt][e] == -INFINITY && mx > -INFINITY)) {
+                                st_b[nt][e] *= ex2(st_a[nt][e] - mx);
+                                st_a[nt][e] = mx;
+                            }
+                            if (st_a[nt][e] > -INFINITY) st_b[nt][e] += ex2(fmaf(da, c, -st_a[nt][e])) + ex2(fmaf(db, c, -st_a[nt][e]));
+                        } else {
+                            acc_a += ex2(fmaf(da, c, st_a[nt][e]));
+                            acc_b += ex2(fmaf(db, c, st_a[nt][e]));
+                        }
+                    }
+                    if (PHASE == 1 && NTB <= 2 && lg) {
+                        if (ta < t_end) *reinterpret_cast<float2 *>(lg + (size_t)ta * (NTB * 8) + nt * 8 + 2 * tq) = make_float2(keep_a[0], keep_a[1]);
+                        if (tb < t_end) *reinterpret_cast<float2 *>(lg + (size_t)tb * (NTB * 8) + nt * 8 + 2 * tq) = make_float2(keep_b[0], keep_b[1]);
                     }
                 }
-            __syncthreads();
-            for (int r = threadIdx.x; r < NTB * 8; r += kTovaThreads) {
-                float m = red[0][r][0], z = red[0][r][1];
+                if (PHASE == 2) {
+                    acc_a += __shfl_xor_sync(0xffffffffu, acc_a, 1);
+                    acc_a += __shfl_xor_sync(0xffffffffu, acc_a, 2);
+                    acc_b += __shfl_xor_sync(0xffffffffu, acc_b, 1);
+                    acc_b += __shfl_xor_sync(0xffffffffu, acc_b, 2);
+                    if (tq == 0) {
 #pragma unroll
-                for (int w = 1; w < 4; ++w) lse_merge(m, z, red[w][r][0], red[w][r][1]);
-                float2 *out = reinterpret_cast<float2 *>(p.part) + ((size_t)uid * p.n_slices + slice) * p.rows_pad + row0 + r;
-                *out = make_float2(m, z);
+                        for (int e = 0; e < 2; ++e) {
+                            const int t = e ? tb : ta;
+                            if (t < t_end) {
+                                float v = e ? acc_b : acc_a;
+                                if (rb > 0) v += u_out[t];
+                                if (rb == n_rb - 1) {
+                                    const int ninv = p.causal ? p.G * max(0, t - (T - p.W)) : 0;
+                                    v = (v + (float)ninv * pmax) * inv_rows;
+                                }
+                                u_out[t] = v;
+                            }
+                        }
+                    }
+                }
+            }
+            cp_async_wait<0>();
+
+            if (PHASE == 1) {
+                // rows live in the quad index; fold the eight token groups, then the four warps
+#pragma unroll
+                for (int nt = 0; nt < NTB; ++nt)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+#pragma unroll
+                        for (int o = 4; o < 32; o <<= 1) {
+                            const float m2 = __shfl_xor_sync(0xffffffffu, st_a[nt][e], o);
+                            const float z2 = __shfl_xor_sync(0xffffffffu, st_b[nt][e], o);
+                            lse_merge(st_a[nt][e], st_b[nt][e], m2, z2);
+                        }
+                        if (g == 0) {
+                            red[warp][nt * 8 + 2 * tq + e][0] = st_a[nt][e];
+                            red[warp][nt * 8 + 2 * tq + e][1] = st_b[nt][e];
+                        }
+                    }
+                __syncthreads();
+                for (int r = threadIdx.x; r < NTB * 8; r += kTovaThreads) {
+                    float m = red[0][r][0], z = red[0][r][1];
+#pragma unroll
+                    for (int w = 1; w < 4; ++w) lse_merge(m, z, red[w][r][0], red[w][r][1]);
+                    float2 *out = reinterpret_cast<float2 *>(p.part) + ((size_t)uid * p.n_slices + slice) * p.rows_pad + row0 + r;
+                    *out = make_float2(m, z);
+                }
             }
         }
     }
