@@ -47,224 +47,459 @@ __device__ __forceinline__ void lse_merge(float &m, float &z, float m2, float z2
 }
 
 constexpr int kTovaThreads = 128;
-constexpr int kQPitch = 136;   // bf16 elements per staged query row: 272 bytes, conflict-free 16-byte reads
 constexpr int kRing = 3;       // 16-token K tiles per warp in shared memory: one worked on, two on their way
 constexpr int kTileK = 16 * kRowBytes;
+static_assert(kRing == 3, "the waits below count on two tiles in flight");
 
-__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+__device__ __forceinline__ void cp_async16(unsigned dst, const void *src)
 {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+// 16 bytes, or zeros without reading
+__device__ __forceinline__ void cp_async16_or_zero(unsigned dst, const void *src, bool read)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(read ? 16 : 0) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-template <int NTB>
-__host__ __device__ constexpr size_t tova_smem(int slice_len)
+__device__ __forceinline__ uint4 lds16(unsigned addr)
 {
-    return (size_t)(kTovaThreads / 32) * kRing * kTileK + (NTB > 1 ? (size_t)NTB * 8 * kQPitch * 2 : 0) + (size_t)(slice_len / 16) * 4;
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
 }
 
-// A block takes (unit, token slice) pairs in turn, all units of a slice number before the next one: the blocks of
-// neighbouring KV heads read the same pages at the same time, and the slices past a sequence's end cost a look at its
-// length instead of a block.  Each warp walks 16-token tiles; a tile is one page.  Its K rows come through a ring of
-// tiles in shared memory (asynchronous copies, two tiles ahead; a chunk of 16 bytes lies at its number XOR 4 in odd rows,
-// so that reads are free of bank conflicts), and the slice's page ids are fetched once.  Bound by the K stream: a warp that
-// loaded a tile into registers and then worked on it reached 4.0 TB/s with 32 query rows.  The
-// tile is the M operand of m16n8k16 and eight query rows are the N
-// operand, both read as 16-byte pieces along d: lane (g, tq) loads d = 32 j + 8 tq
-// .. +7 of its rows, and those eight values feed k-steps 2j and 2j+1.  The same
-// assignment of d to k on both operands leaves the dot product unchanged.
+// One (unit, token slice, block of query rows) of work, and the warp's share of it.
+struct TovaItem {
+    int uid, slice, rb, b, h, l, T, t_begin, t_end, mine; // mine: tiles of this warp (warp, warp + 4, ...)
+    int page[2];                                          // lane k: page ids of the warp's tiles k and 32 + k
+    const __nv_bfloat16 *k, *q;                           // this lane's 16 bytes of the layer's first page; first query row
+};
+
+// The stream of K tiles of one warp, and the query rows of the block, across all the work the block takes.  A block takes
+// (unit, token slice) pairs in turn, all units of a slice number before the next one: the blocks of neighbouring KV heads
+// read the same pages at the same time, and the slices past a sequence's end cost a look at its length instead of a block.
+// A tile is 16 tokens, one page.  Its rows come through a ring of tiles in shared memory (asynchronous copies, two
+// tiles ahead; a chunk of 16 bytes lies at its number XOR 4 in odd rows, so that reads are free of bank conflicts).  The
+// stream runs on across the ends of slices: the next slice's page ids, queries and first tiles are on their way while this
+// one's last tiles are worked on.
+template <int kQRows, int PHASE>
+struct TovaStream {
+    const DevParams &p;
+    unsigned ring, qbuf;     // shared addresses: this warp's tiles, the block's query rows [kQRows][256 bytes], one or two of them
+    int units, n_slices, n_rb, wslot, rslot;
+    long long item;
+    int next_rb;
+    size_t page_stride, row2; // elements between pages, between every other slot of a page
+
+    __device__ __forceinline__ TovaStream(const DevParams &p_, unsigned ring0, unsigned q0) : p(p_)
+    {
+        ring = ring0 + (threadIdx.x >> 5) * (kRing * kTileK);
+        qbuf = q0;
+        units = p.L * p.B * p.H;
+        n_slices = (p.T_cap + p.slice_len - 1) / p.slice_len;
+        n_rb = p.rows_pad / kQRows;
+        wslot = rslot = next_rb = 0;
+        item = blockIdx.x;
+        page_stride = (size_t)kPage * p.H * kHeadDim;
+        row2 = (size_t)2 * p.H * kHeadDim;
+    }
+    // the next piece of work; false at the end
+    __device__ __forceinline__ bool next(TovaItem &it)
+    {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        for (; item < (long long)units * n_slices; item += gridDim.x, next_rb = 0) {
+            it.uid = (int)(item % units);
+            it.slice = (int)(item / units);
+            it.h = it.uid % p.H; it.b = (it.uid / p.H) % p.B; it.l = it.uid / (p.H * p.B);
+            it.T = p.seq_lens[it.b];
+            it.t_begin = it.slice * p.slice_len;
+            if (it.T <= p.Tk || it.T > p.T_cap) continue;
+            if (p.W > it.T) { if (PHASE == 1 && it.slice == 0 && threadIdx.x == 0) set_status(p.status, AMS_ERR_INVALID_ARG, it.uid, p.W, it.T); continue; }
+            if (it.t_begin >= it.T) continue;
+            it.t_end = min(it.T, it.t_begin + p.slice_len);
+            it.rb = next_rb;
+            it.mine = max(0, (((it.t_end - it.t_begin + 15) >> 4) - warp + 3) >> 2);
+            const int *table = p.block_table + (size_t)it.b * p.bt_stride + (it.t_begin >> 4) + warp;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) it.page[j] = j * 32 + lane < it.mine ? table[4 * (j * 32 + lane)] : 0;
+            it.k = p.k_pages + row_offset(p, it.l, 0, lane >> 4, it.h) + (lane & 15) * 8;
+            it.q = p.q + ((((size_t)it.l * p.B + it.b) * p.H + it.h) * p.G) * (size_t)p.W * kHeadDim;
+            if (++next_rb >= n_rb) { next_rb = 0; item += gridDim.x; }
+            return true;
+        }
+        return false;
+    }
+    // starts the copy of the warp's tile k (none past the end) and with the first one that of the queries, as one group
+    __device__ __forceinline__ void fetch(const TovaItem &it, bool live, int k, int buf)
+    {
+        if (live && k < it.mine) {
+            const int lane = threadIdx.x & 31, page = __shfl_sync(0xffffffffu, k < 32 ? it.page[0] : it.page[1], k & 31);
+            const __nv_bfloat16 *src = it.k + (size_t)page * page_stride;
+            const unsigned dst = ring + wslot * kTileK + (lane >> 4) * kRowBytes + (((lane & 15) ^ ((lane >> 4) << 2)) << 4);
+#pragma unroll
+            for (int i = 0; i < 8; ++i, src += row2) cp_async16(dst + i * 2 * kRowBytes, src);
+            wslot = wslot == kRing - 1 ? 0 : wslot + 1;
+        }
+        if (live && k == 0) {
+#pragma unroll
+            for (int j = 0; j < kQRows / 8; ++j) {
+                const int i = j * kTovaThreads + threadIdx.x, r = i >> 4, ch = i & 15, row = it.rb * kQRows + r;
+                cp_async16_or_zero(qbuf + (buf * kQRows + r) * kRowBytes + ((ch ^ ((r & 1) << 2)) << 4),
+                                   it.q + (size_t)min(row, p.rows - 1) * kHeadDim + ch * 8, row < p.rows);
+            }
+        }
+        cp_async_commit();
+    }
+    // waits for the stream's next tile and reads it: lane (g, tq) gets 16-byte pieces 4 j + tq of its rows g and g + 8
+    __device__ __forceinline__ void read(uint4 (&x)[4], uint4 (&y)[4])
+    {
+        const int lane = threadIdx.x & 31, g = lane >> 2, tq = lane & 3;
+        cp_async_wait<1>();
+        __syncwarp();
+        const unsigned at = ring + rslot * kTileK + g * kRowBytes;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const unsigned ch = ((4 * j + tq) ^ ((g & 1) << 2)) << 4; // (rows g and g + 8 are both odd or both even)
+            x[j] = lds16(at + ch);
+            y[j] = lds16(at + 8 * kRowBytes + ch);
+        }
+        rslot = rslot == kRing - 1 ? 0 : rslot + 1;
+    }
+};
+
+// Narrow windows (8 or 16 padded rows).  The tile is the M operand of m16n8k16 and eight query rows are the N operand, both
+// read as 16-byte pieces along d: lane (g, tq) holds d = 32 j + 8 tq .. +7 of its rows, and those eight values feed k-steps
+// 2j and 2j+1.  The same assignment of d to k on both operands leaves the dot product unchanged.  Bound by the K
+// stream: 9.4 GB of K at 7 query rows 1.81 -> 1.67 ms with the asynchronous ring (logits included 6.2 TB/s).
 template <int NTB, int PHASE>
 __global__ void __launch_bounds__(kTovaThreads) k_tova(DevParams p)
 {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ float red[4][NTB * 8][2];
-    unsigned char *ring = dyn + (threadIdx.x >> 5) * (kRing * kTileK);
-    __nv_bfloat16 *Qs = reinterpret_cast<__nv_bfloat16 *>(dyn + (kTovaThreads / 32) * kRing * kTileK);
-    int *pages = reinterpret_cast<int *>(Qs + (NTB > 1 ? NTB * 8 * kQPitch : 0));
+    const unsigned smem = (unsigned)__cvta_generic_to_shared(dyn);
+    const unsigned Qb = smem + (kTovaThreads / 32) * kRing * kTileK;
     if (PHASE == 2) wait_for_previous_kernel(); // merged statistics
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, tq = lane & 3;
-    const int units = p.L * p.B * p.H, n_slices = (p.T_cap + p.slice_len - 1) / p.slice_len;
     const float c = kLog2e * 0.08838834764831845f; // log2(e) / sqrt(128)
-    const int n_rb = p.rows_pad / (NTB * 8);
     const float inv_rows = 1.0f / (float)p.rows;
-    const size_t row_stride = (size_t)p.H * kHeadDim; // elements between the slots of a page
+    TovaStream<NTB * 8, PHASE> st(p, smem, Qb);
+    const int n_rb = st.n_rb;
 
-    for (long long item = blockIdx.x; item < (long long)units * n_slices; item += gridDim.x) {
-        const int uid = (int)(item % units), slice = (int)(item / units);
-        const int h = uid % p.H, b = (uid / p.H) % p.B, l = uid / (p.H * p.B);
-        const int T = p.seq_lens[b];
-        if (T <= p.Tk || T > p.T_cap) continue;
-        if (p.W > T) { if (PHASE == 1 && slice == 0 && threadIdx.x == 0) set_status(p.status, AMS_ERR_INVALID_ARG, uid, p.W, T); continue; }
-        const int t_begin = slice * p.slice_len;
-        if (t_begin >= T) continue;
-        const int t_end = min(T, t_begin + p.slice_len);
-        const int n_tiles = (t_end - t_begin + 15) >> 4;
-        const __nv_bfloat16 *Q = p.q + ((((size_t)l * p.B + b) * p.H + h) * p.G) * (size_t)p.W * kHeadDim;
+    TovaItem cur, nxt;
+    bool live = st.next(cur);
+    int qsel = 0;
+    st.fetch(cur, live, 0, 0);
+    st.fetch(cur, live, 1, 0);
+    while (live) {
+        const bool more = st.next(nxt);
+        int ahead = 0; // tiles of the next piece of work whose copy has been started
+        const int uid = cur.uid, T = cur.T, t_begin = cur.t_begin, t_end = cur.t_end, rb = cur.rb, row0 = rb * NTB * 8;
         const float *fin = p.fin + (size_t)uid * (p.rows_pad + 8);
         float *u_out = p.scores + (size_t)uid * p.T_cap;
-        float *lg = (PHASE == 1 && NTB <= 2 && p.logits && n_rb == 1) ? p.logits + (size_t)uid * p.T_cap * (NTB * 8) : nullptr;
+        float *lg = (PHASE == 1 && p.logits && n_rb == 1) ? p.logits + (size_t)uid * p.T_cap * (NTB * 8) : nullptr;
         const float pmax = PHASE == 2 ? fin[p.rows_pad] : 0.0f;
-        __syncthreads(); // the previous slice's page ids and queries are no longer read
-        for (int i = threadIdx.x; i < n_tiles; i += kTovaThreads) pages[i] = p.block_table[(size_t)b * p.bt_stride + (t_begin >> 4) + i];
+        cp_async_wait<1>(); // the queries and the first tile
+        __syncthreads();
+        uint4 zq[NTB][4];
+#pragma unroll
+        for (int nt = 0; nt < NTB; ++nt)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) zq[nt][j] = lds16(Qb + (qsel * NTB * 8 + nt * 8 + g) * kRowBytes + (((4 * j + tq) ^ ((g & 1) << 2)) << 4));
+        // per thread: rows (nt, e) = row0 + 8 nt + 2 tq + e
+        int lastv[NTB][2];
+        float st_a[NTB][2], st_b[NTB][2], st_m[NTB][2]; // phase 1: reference, sum of 2^(x - reference), largest unscaled
+                                                        // logit; phase 2: -b_r in the first
+#pragma unroll
+        for (int nt = 0; nt < NTB; ++nt)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int r = row0 + nt * 8 + 2 * tq + e;
+                lastv[nt][e] = r < p.rows ? (p.causal ? T - p.W + (r % p.W) : T - 1) : -1;
+                st_a[nt][e] = PHASE == 1 ? -1e30f : -fin[r];
+                st_b[nt][e] = 0.0f;
+                st_m[nt][e] = -INFINITY;
+            }
 
-        for (int rb = 0; rb < n_rb; ++rb) {
-            const int row0 = rb * NTB * 8;
-            uint4 zq[4];
-            if (NTB > 1) {
-                if (rb > 0) __syncthreads();
-                for (int i = threadIdx.x; i < NTB * 8 * 16; i += kTovaThreads) {
-                    const int r = i >> 4, cpos = i & 15;
-                    uint4 v = make_uint4(0, 0, 0, 0);
-                    if (row0 + r < p.rows) v = *reinterpret_cast<const uint4 *>(Q + (size_t)(row0 + r) * kHeadDim + cpos * 8);
-                    *reinterpret_cast<uint4 *>(Qs + r * kQPitch + cpos * 8) = v;
-                }
-            } else {
+        for (int kt = 0; kt < cur.mine; ++kt) {
+            uint4 x[4], y[4];
+            st.read(x, y);
+            if (kt + 2 < cur.mine) st.fetch(cur, true, kt + 2, qsel); // into the slot read in the round before
+            else { st.fetch(nxt, more, ahead, qsel ^ 1); ++ahead; }
+            const int t0 = t_begin + (warp + 4 * kt) * 16, ta = t0 + g, tb = t0 + g + 8;
+            // every row sees every token of the tile (padding rows are taken care of by their statistics or at the end)
+            const bool plain = t0 + 15 < t_end && t0 + 15 <= (p.causal ? T - p.W : T - 1);
+            float acc_a = 0.0f, acc_b = 0.0f;
+#pragma unroll
+            for (int nt = 0; nt < NTB; ++nt) {
+                float d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    zq[j] = make_uint4(0, 0, 0, 0);
-                    if (row0 + g < p.rows) zq[j] = *reinterpret_cast<const uint4 *>(Q + (size_t)(row0 + g) * kHeadDim + 32 * j + 8 * tq);
+                    mma_bf16(d, x[j].x, y[j].x, x[j].y, y[j].y, zq[nt][j].x, zq[nt][j].y);
+                    mma_bf16(d, x[j].z, y[j].z, x[j].w, y[j].w, zq[nt][j].z, zq[nt][j].w);
+                }
+                if (!plain) { // pairs the window hides add nothing, now or (stored logits) later
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int lv = min(lastv[nt][e], t_end - 1);
+                        d[e] = ta <= lv ? d[e] : -INFINITY;
+                        d[2 + e] = tb <= lv ? d[2 + e] : -INFINITY;
+                    }
+                }
+                if (PHASE == 1) {
+                    // The sum's reference follows the largest logit at a distance of up to 2^32, so that rescaling is rare;
+                    // the sum is put on the maximum at the end.
+                    bool far = false;
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        st_m[nt][e] = fmaxf(st_m[nt][e], fmaxf(d[e], d[2 + e]));
+                        far |= fmaf(st_m[nt][e], c, -32.0f) > st_a[nt][e];
+                    }
+                    if (far) {
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            const float mx = st_m[nt][e] * c;
+                            if (mx > st_a[nt][e]) { st_b[nt][e] *= ex2(st_a[nt][e] - mx); st_a[nt][e] = mx; }
+                        }
+                    }
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) st_b[nt][e] += ex2(fmaf(d[e], c, -st_a[nt][e])) + ex2(fmaf(d[2 + e], c, -st_a[nt][e]));
+                    if (lg) {
+                        if (ta < t_end) *reinterpret_cast<float2 *>(lg + (size_t)ta * (NTB * 8) + nt * 8 + 2 * tq) = make_float2(d[0] * c, d[1] * c);
+                        if (tb < t_end) *reinterpret_cast<float2 *>(lg + (size_t)tb * (NTB * 8) + nt * 8 + 2 * tq) = make_float2(d[2] * c, d[3] * c);
+                    }
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        acc_a += ex2(fmaf(d[e], c, st_a[nt][e]));
+                        acc_b += ex2(fmaf(d[2 + e], c, st_a[nt][e]));
+                    }
                 }
             }
-            __syncthreads();
-            auto fetch = [&](int tile, int slot) { // lane: 16 bytes of two rows at a time
-                if (tile < n_tiles) {
-                    const int r0 = lane >> 4, ch = lane & 15;
-                    const __nv_bfloat16 *src = p.k_pages + row_offset(p, l, pages[tile], r0, h) + ch * 8;
-                    unsigned char *dst = ring + slot * kTileK + r0 * kRowBytes + ((ch ^ (r0 << 2)) << 4);
+            if (PHASE == 2) {
+                acc_a += __shfl_xor_sync(0xffffffffu, acc_a, 1);
+                acc_a += __shfl_xor_sync(0xffffffffu, acc_a, 2);
+                acc_b += __shfl_xor_sync(0xffffffffu, acc_b, 1);
+                acc_b += __shfl_xor_sync(0xffffffffu, acc_b, 2);
+                if (tq == 0) {
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) cp_async16(dst + i * 2 * kRowBytes, src + (size_t)(2 * i) * row_stride);
+                    for (int e = 0; e < 2; ++e) {
+                        const int t = e ? tb : ta;
+                        if (t < t_end) {
+                            float v = e ? acc_b : acc_a;
+                            if (rb > 0) v += u_out[t];
+                            if (rb == n_rb - 1) {
+                                const int ninv = p.causal ? p.G * max(0, t - (T - p.W)) : 0;
+                                v = (v + (float)ninv * pmax) * inv_rows;
+                            }
+                            u_out[t] = v;
+                        }
+                    }
                 }
-                cp_async_commit();
-            };
-            // per thread: rows (nt, e) = row0 + 8 nt + 2 tq + e
-            int lastv[NTB][2];
-            float st_a[NTB][2], st_b[NTB][2]; // phase 1: (reference, sum of 2^(x - reference)); phase 2: (-b_r, unused)
+            }
+        }
+        for (; ahead < 2; ++ahead) st.fetch(nxt, more, ahead, qsel ^ 1); // (fewer than two tiles for this warp)
+
+        if (PHASE == 1) {
+            // rows live in the quad index; fold the eight token groups, then the four warps
 #pragma unroll
             for (int nt = 0; nt < NTB; ++nt)
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    const int r = row0 + nt * 8 + 2 * tq + e;
-                    lastv[nt][e] = r < p.rows ? (p.causal ? T - p.W + (r % p.W) : T - 1) : -1;
-                    if (PHASE == 1) { st_a[nt][e] = -INFINITY; st_b[nt][e] = 0.0f; }
-                    else { st_a[nt][e] = -fin[r]; st_b[nt][e] = 0.0f; }
+                    const float mx = st_m[nt][e] * c;
+                    st_b[nt][e] = mx > -INFINITY ? st_b[nt][e] * ex2(st_a[nt][e] - mx) : 0.0f;
+                    st_a[nt][e] = mx;
+#pragma unroll
+                    for (int o = 4; o < 32; o <<= 1) {
+                        const float m2 = __shfl_xor_sync(0xffffffffu, st_a[nt][e], o);
+                        const float z2 = __shfl_xor_sync(0xffffffffu, st_b[nt][e], o);
+                        lse_merge(st_a[nt][e], st_b[nt][e], m2, z2);
+                    }
+                    if (g == 0) {
+                        red[warp][nt * 8 + 2 * tq + e][0] = st_a[nt][e];
+                        red[warp][nt * 8 + 2 * tq + e][1] = st_b[nt][e];
+                    }
                 }
+            __syncthreads();
+            for (int r = threadIdx.x; r < NTB * 8; r += kTovaThreads) {
+                float m = red[0][r][0], z = red[0][r][1];
+#pragma unroll
+                for (int w = 1; w < 4; ++w) lse_merge(m, z, red[w][r][0], red[w][r][1]);
+                float2 *out = reinterpret_cast<float2 *>(p.part) + ((size_t)uid * p.n_slices + cur.slice) * p.rows_pad + row0 + r;
+                *out = make_float2(m, z);
+            }
+        }
+        cur = nxt;
+        live = more;
+        qsel ^= 1;
+    }
+    cp_async_wait<0>();
+}
 
-            fetch(warp, 0);
-            fetch(warp + 4, 1);
-            int slot = 0;
-            for (int tile = warp; tile < n_tiles; tile += 4) {
-                cp_async_wait<1>();
-                __syncwarp();
-                const unsigned char *ta_ = ring + slot * kTileK + g * kRowBytes;
-                uint4 x[4], y[4];
+// Middle-sized windows (32 or 64 padded rows; blocks of 128 rows where the tcgen05 form does not apply): 16 query rows are the
+// M operand, the tile's tokens two N operands.  A token's piece of 16 bytes is then two consecutive registers per k-step,
+// as the instruction wants them (with the tile as M operand every k-step interleaves two rows' pieces: 380 of 546
+// instructions per tile were moves and their like), and a thread sees four logits of a row per tile.  The queries are laid
+// out in shared
+// memory as the fragments the lanes read.  3.0 GB of K at 32 query rows: statistics 0.70 -> 0.52 ms, usage 0.69 -> 0.51 ms (5.9
+// TB/s).
+template <int MT, int PHASE>
+__global__ void __launch_bounds__(kTovaThreads) k_tova_wide(DevParams p)
+{
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ float red[4][MT * 16][2];
+    const unsigned smem = (unsigned)__cvta_generic_to_shared(dyn);
+    const unsigned Qb = smem + (kTovaThreads / 32) * kRing * kTileK;    // [MT * 16 rows][256 bytes] as they come
+    const unsigned Fr = Qb + MT * 16 * kRowBytes;                   // [MT][8 k-steps][32 lanes] fragments of the current rows
+    if (PHASE == 2) wait_for_previous_kernel(); // merged statistics
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, tq = lane & 3;
+    const float c = kLog2e * 0.08838834764831845f; // log2(e) / sqrt(128)
+    const float inv_rows = 1.0f / (float)p.rows;
+    TovaStream<MT * 16, PHASE> st(p, smem, Qb);
+    const int n_rb = st.n_rb;
+
+    TovaItem cur, nxt;
+    bool live = st.next(cur);
+    st.fetch(cur, live, 0, 0);
+    st.fetch(cur, live, 1, 0);
+    while (live) {
+        const bool more = st.next(nxt);
+        int ahead = 0; // tiles of the next piece of work whose copy has been started
+        const int uid = cur.uid, T = cur.T, t_begin = cur.t_begin, t_end = cur.t_end, rb = cur.rb, row0 = rb * MT * 16;
+        const float *fin = p.fin + (size_t)uid * (p.rows_pad + 8);
+        float *u_out = p.scores + (size_t)uid * p.T_cap;
+        const float pmax = PHASE == 2 ? fin[p.rows_pad] : 0.0f;
+        // per thread: rows (mt, e) = row0 + 16 mt + g + 8 e
+        float st_a[MT][2], st_b[MT][2], st_m[MT][2]; // phase 1: reference, sum of 2^(x - reference), largest unscaled logit;
+                                                     // phase 2: -b_r in the first
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                st_a[mt][e] = PHASE == 1 ? -1e30f : -fin[row0 + mt * 16 + 8 * e + g];
+                st_b[mt][e] = 0.0f;
+                st_m[mt][e] = -INFINITY;
+            }
+        cp_async_wait<1>(); // the queries and the first tile
+        __syncthreads();
+        // fragments: k-step 2 j takes words 0 and 1 of piece 4 j + tq, k-step 2 j + 1 words 2 and 3 (the tiles' pieces alike)
+        for (int i = threadIdx.x; i < MT * 4 * 32; i += kTovaThreads) {
+            const int ln = i & 31, j = (i >> 5) & 3, mt = i >> 7, gg = ln >> 2, ch = ((4 * j + (ln & 3)) ^ ((gg & 1) << 2)) << 4;
+            const unsigned row = Qb + (mt * 16 + gg) * kRowBytes + ch;
+            const uint4 lo = lds16(row), hi = lds16(row + 8 * kRowBytes);
+            const unsigned f = Fr + ((mt * 8 + 2 * j) * 32 + ln) * 16;
+            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(f), "r"(lo.x), "r"(hi.x), "r"(lo.y), "r"(hi.y) : "memory");
+            asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(f + 512), "r"(lo.z), "r"(hi.z), "r"(lo.w), "r"(hi.w) : "memory");
+        }
+        __syncthreads();
+
+        for (int kt = 0; kt < cur.mine; ++kt) {
+            uint4 x[4], y[4];
+            st.read(x, y);
+            if (kt + 2 < cur.mine) st.fetch(cur, true, kt + 2, 0); // into the slot read in the round before
+            else { st.fetch(nxt, more, ahead, 0); ++ahead; }
+            const int t0 = t_begin + (warp + 4 * kt) * 16;
+            // every row sees every token of the tile (padding rows are taken care of by their statistics)
+            const bool plain = t0 + 15 < t_end && t0 + 15 <= (p.causal ? T - p.W : T - 1);
+            float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f}; // tokens 2 tq, 2 tq + 1, 8 + 2 tq, 9 + 2 tq
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt) {
+                float da[4] = {0.0f, 0.0f, 0.0f, 0.0f}, db[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const int at = ((4 * j + tq) ^ ((g & 1) << 2)) << 4; // (rows g and g + 8 are both odd or both even)
-                    x[j] = *reinterpret_cast<const uint4 *>(ta_ + at);
-                    y[j] = *reinterpret_cast<const uint4 *>(ta_ + 8 * kRowBytes + at);
+                    const uint4 f0 = lds16(Fr + ((mt * 8 + 2 * j) * 32 + lane) * 16), f1 = lds16(Fr + ((mt * 8 + 2 * j + 1) * 32 + lane) * 16);
+                    mma_bf16(da, f0.x, f0.y, f0.z, f0.w, x[j].x, x[j].y);
+                    mma_bf16(db, f0.x, f0.y, f0.z, f0.w, y[j].x, y[j].y);
+                    mma_bf16(da, f1.x, f1.y, f1.z, f1.w, x[j].z, x[j].w);
+                    mma_bf16(db, f1.x, f1.y, f1.z, f1.w, y[j].z, y[j].w);
                 }
-                fetch(tile + 8, slot == 0 ? 2 : slot - 1); // the slot read in the round before
-                slot = slot == 2 ? 0 : slot + 1;
-                const int t0 = t_begin + tile * 16, ta = t0 + g, tb = t0 + g + 8;
-                // every row sees every token of the tile (padding rows are taken care of by their statistics or at the end)
-                const bool plain = t0 + 15 < t_end && t0 + 15 <= (p.causal ? T - p.W : T - 1);
-                float acc_a = 0.0f, acc_b = 0.0f;
 #pragma unroll
-                for (int nt = 0; nt < NTB; ++nt) {
-                    if (NTB > 1) {
+                for (int e = 0; e < 2; ++e) {
+                    float v[4] = {da[2 * e], da[2 * e + 1], db[2 * e], db[2 * e + 1]};
+                    if (!plain) { // pairs the window hides add nothing
+                        const int r = row0 + mt * 16 + 8 * e + g;
+                        const int lv = min(r < p.rows ? (p.causal ? T - p.W + (r % p.W) : T - 1) : -1, t_end - 1) - t0 - 2 * tq;
 #pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            zq[j] = *reinterpret_cast<const uint4 *>(Qs + (nt * 8 + g) * kQPitch + 32 * j + 8 * tq);
+                        for (int i = 0; i < 4; ++i) v[i] = (i >> 1) * 8 + (i & 1) <= lv ? v[i] : -INFINITY;
                     }
-                    float d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        mma_bf16(d, x[j].x, y[j].x, x[j].y, y[j].y, zq[j].x, zq[j].y);
-                        mma_bf16(d, x[j].z, y[j].z, x[j].w, y[j].w, zq[j].z, zq[j].w);
-                    }
-                    float keep_a[2], keep_b[2];
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        float da = d[e], db = d[2 + e];
-                        if (!plain || lg) { // pairs the window hides add nothing, now or (stored logits) later
-                            const int lv = min(lastv[nt][e], t_end - 1);
-                            da = ta <= lv ? da : -INFINITY;
-                            db = tb <= lv ? db : -INFINITY;
+                    if (PHASE == 1) {
+                        // The sum's reference follows the largest logit at a distance of up to 2^32, so that rescaling is
+                        // rare; the sum is put on the maximum at the end.
+                        st_m[mt][e] = fmaxf(fmaxf(st_m[mt][e], fmaxf(v[0], v[1])), fmaxf(v[2], v[3]));
+                        if (fmaf(st_m[mt][e], c, -32.0f) > st_a[mt][e]) {
+                            const float mx = st_m[mt][e] * c;
+                            st_b[mt][e] *= ex2(st_a[mt][e] - mx);
+                            st_a[mt][e] = mx;
                         }
-                        if (PHASE == 1) {
-                            if (NTB <= 2) { keep_a[e] = da * c; keep_b[e] = db * c; }
-                            // the reference follows the largest logit at a distance of at most 2^32 in the sum, so that
-                            // rescaling is rare
-                            const float mx = fmaxf(da, db) * c;
-                            if (mx > st_a[nt][e] + 32.0f || (st_a[nt][e] == -INFINITY && mx > -INFINITY)) {
-                                st_b[nt][e] *= ex2(st_a[nt][e] - mx);
-                                st_a[nt][e] = mx;
-                            }
-                            if (st_a[nt][e] > -INFINITY) st_b[nt][e] += ex2(fmaf(da, c, -st_a[nt][e])) + ex2(fmaf(db, c, -st_a[nt][e]));
-                        } else {
-                            acc_a += ex2(fmaf(da, c, st_a[nt][e]));
-                            acc_b += ex2(fmaf(db, c, st_a[nt][e]));
-                        }
-                    }
-                    if (PHASE == 1 && NTB <= 2 && lg) {
-                        if (ta < t_end) *reinterpret_cast<float2 *>(lg + (size_t)ta * (NTB * 8) + nt * 8 + 2 * tq) = make_float2(keep_a[0], keep_a[1]);
-                        if (tb < t_end) *reinterpret_cast<float2 *>(lg + (size_t)tb * (NTB * 8) + nt * 8 + 2 * tq) = make_float2(keep_b[0], keep_b[1]);
-                    }
-                }
-                if (PHASE == 2) {
-                    acc_a += __shfl_xor_sync(0xffffffffu, acc_a, 1);
-                    acc_a += __shfl_xor_sync(0xffffffffu, acc_a, 2);
-                    acc_b += __shfl_xor_sync(0xffffffffu, acc_b, 1);
-                    acc_b += __shfl_xor_sync(0xffffffffu, acc_b, 2);
-                    if (tq == 0) {
+                        float s[4];
 #pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const int t = e ? tb : ta;
-                            if (t < t_end) {
-                                float v = e ? acc_b : acc_a;
-                                if (rb > 0) v += u_out[t];
-                                if (rb == n_rb - 1) {
-                                    const int ninv = p.causal ? p.G * max(0, t - (T - p.W)) : 0;
-                                    v = (v + (float)ninv * pmax) * inv_rows;
-                                }
-                                u_out[t] = v;
-                            }
-                        }
+                        for (int i = 0; i < 4; ++i) s[i] = ex2(fmaf(v[i], c, -st_a[mt][e]));
+                        st_b[mt][e] += (s[0] + s[1]) + (s[2] + s[3]);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) acc[i] += ex2(fmaf(v[i], c, st_a[mt][e]));
                     }
                 }
             }
-            cp_async_wait<0>();
-
-            if (PHASE == 1) {
-                // rows live in the quad index; fold the eight token groups, then the four warps
-#pragma unroll
-                for (int nt = 0; nt < NTB; ++nt)
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-#pragma unroll
-                        for (int o = 4; o < 32; o <<= 1) {
-                            const float m2 = __shfl_xor_sync(0xffffffffu, st_a[nt][e], o);
-                            const float z2 = __shfl_xor_sync(0xffffffffu, st_b[nt][e], o);
-                            lse_merge(st_a[nt][e], st_b[nt][e], m2, z2);
-                        }
-                        if (g == 0) {
-                            red[warp][nt * 8 + 2 * tq + e][0] = st_a[nt][e];
-                            red[warp][nt * 8 + 2 * tq + e][1] = st_b[nt][e];
-                        }
+            if (PHASE == 2) {
+                // sums over the eight lanes of a tq, four tokens at once: at each step a lane hands half of its values over
+                const bool up = lane & 16, odd = lane & 8;
+                float k0 = up ? acc[2] : acc[0], k1 = up ? acc[3] : acc[1];
+                k0 += __shfl_xor_sync(0xffffffffu, up ? acc[0] : acc[2], 16);
+                k1 += __shfl_xor_sync(0xffffffffu, up ? acc[1] : acc[3], 16);
+                float v = (odd ? k1 : k0) + __shfl_xor_sync(0xffffffffu, odd ? k0 : k1, 8);
+                v += __shfl_xor_sync(0xffffffffu, v, 4);
+                const int t = t0 + (up ? 8 : 0) + 2 * tq + (odd ? 1 : 0);
+                if (!(lane & 4) && t < t_end) {
+                    if (rb > 0) v += u_out[t];
+                    if (rb == n_rb - 1) {
+                        const int ninv = p.causal ? p.G * max(0, t - (T - p.W)) : 0;
+                        v = (v + (float)ninv * pmax) * inv_rows;
                     }
-                __syncthreads();
-                for (int r = threadIdx.x; r < NTB * 8; r += kTovaThreads) {
-                    float m = red[0][r][0], z = red[0][r][1];
-#pragma unroll
-                    for (int w = 1; w < 4; ++w) lse_merge(m, z, red[w][r][0], red[w][r][1]);
-                    float2 *out = reinterpret_cast<float2 *>(p.part) + ((size_t)uid * p.n_slices + slice) * p.rows_pad + row0 + r;
-                    *out = make_float2(m, z);
+                    u_out[t] = v;
                 }
             }
         }
+        for (; ahead < 2; ++ahead) st.fetch(nxt, more, ahead, 0); // (fewer than two tiles for this warp)
+
+        if (PHASE == 1) {
+            // fold the four lanes of a row, then the four warps
+#pragma unroll
+            for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    float m = st_m[mt][e] * c, z = m > -INFINITY ? st_b[mt][e] * ex2(st_a[mt][e] - m) : 0.0f;
+#pragma unroll
+                    for (int o = 1; o < 4; o <<= 1) {
+                        const float m2 = __shfl_xor_sync(0xffffffffu, m, o), z2 = __shfl_xor_sync(0xffffffffu, z, o);
+                        lse_merge(m, z, m2, z2);
+                    }
+                    if (tq == 0) {
+                        red[warp][mt * 16 + 8 * e + g][0] = m;
+                        red[warp][mt * 16 + 8 * e + g][1] = z;
+                    }
+                }
+            __syncthreads();
+            for (int r = threadIdx.x; r < MT * 16; r += kTovaThreads) {
+                float m = red[0][r][0], z = red[0][r][1];
+#pragma unroll
+                for (int w = 1; w < 4; ++w) lse_merge(m, z, red[w][r][0], red[w][r][1]);
+                float2 *out = reinterpret_cast<float2 *>(p.part) + ((size_t)uid * p.n_slices + cur.slice) * p.rows_pad + row0 + r;
+                *out = make_float2(m, z);
+            }
+        }
+        cur = nxt;
+        live = more;
     }
+    cp_async_wait<0>();
+}
+
+template <int NTB, int PHASE> // NTB: padded query rows / 8
+constexpr auto tova_kernel()
+{
+    if constexpr (NTB >= 4) return k_tova_wide<NTB / 2, PHASE>;
+    else return k_tova<NTB, PHASE>;
 }
 
 // Per unit: merge the slices' (max, sum) in slice order; b_r = M_r + log2 Z_r in the
@@ -490,26 +725,39 @@ __global__ void __launch_bounds__(kKdThreads) k_keydiff_score(DevParams p)
 }
 
 template <int NTB>
-void launch_tova_ntb(const DevParams &p_in, LaunchCtx &ctx)
+int launch_tova_ntb(const DevParams &p_in, LaunchCtx &ctx)
 {
     DevParams p = p_in;
-    const dim3 grid(p.n_slices, p.L * p.B * p.H);
-    k_tova<NTB, 1><<<grid, kTovaThreads, 0, ctx.s>>>(p);
+    constexpr size_t smem = (size_t)(kTovaThreads / 32) * kRing * kTileK + (size_t)2 * NTB * 8 * kRowBytes;
+    const auto k1 = tova_kernel<NTB, 1>(), k2 = tova_kernel<NTB, 2>();
+    static SmemGrant grant1, grant2;
+    static int resident[2][kMaxDevices]; // blocks per SM
+    const int dev = current_device(), n_sm = sm_count();
+    if (dev < 0 || n_sm <= 0 || !grant_dynamic_smem(k1, smem, grant1) || !grant_dynamic_smem(k2, smem, grant2)) return AMS_ERR_CUDA;
+    if (!resident[0][dev] && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident[1][dev], k2, kTovaThreads, smem) != cudaSuccess ||
+                              cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident[0][dev], k1, kTovaThreads, smem) != cudaSuccess))
+        return AMS_ERR_CUDA;
+    const long long units = (long long)p.L * p.B * p.H, items = units * ((p.T_cap + p.slice_len - 1) / p.slice_len);
+    auto blocks = [&](int phase) {
+        const long long r = (long long)n_sm * (resident[phase][dev] > 0 ? resident[phase][dev] : 1);
+        return dim3((unsigned)(items < r ? items : r));
+    };
+    k1<<<blocks(0), kTovaThreads, smem, ctx.s>>>(p);
     ctx.mark(kKernScore1);
     const bool from_logits = NTB <= 2 && p.logits && p.rows_pad == NTB * 8;
-    p.merge_in_usage = from_logits && p.L * p.B * p.H <= 2 * sm_count();
+    p.merge_in_usage = from_logits && units <= 2 * n_sm;
     if (!p.merge_in_usage) {
-        launch_after(k_tova_combine, dim3((unsigned)(p.L * p.B * p.H)), dim3(128), 0, ctx.s, p);
+        launch_after(k_tova_combine, dim3((unsigned)units), dim3(128), 0, ctx.s, p);
         ctx.mark(kKernScoreCombine);
     }
-    if (from_logits) {
+    if constexpr (NTB <= 2) if (from_logits) {
         const int n256 = (p.T_cap + 255) / 256, per = n256 >= 128 ? 8 : (n256 >= 32 ? n256 / 16 : 1); // tiles per block
-        const dim3 g2(p.L * p.B * p.H, (n256 + per - 1) / per);
+        const dim3 g2((unsigned)units, (n256 + per - 1) / per);
         launch_after(k_tova_usage_from_logits<NTB * 8>, g2, dim3(256), 0, ctx.s, p);
-    } else {
-        launch_after(k_tova<NTB, 2>, grid, dim3(kTovaThreads), 0, ctx.s, p);
     }
+    if (!from_logits) launch_after(k2, blocks(1), dim3(kTovaThreads), smem, ctx.s, p);
     ctx.mark(kKernScore2);
+    return cudaGetLastError() == cudaSuccess ? AMS_OK : AMS_ERR_CUDA;
 }
 
 } // namespace
@@ -525,13 +773,12 @@ int launch_score_tova(const DevParams &p, LaunchCtx &ctx)
 {
     if (tova_tc_supported(p)) return launch_score_tova_tc(p, ctx);
     switch (tova_rows_block(p.rows) / 8) {
-    case 1: launch_tova_ntb<1>(p, ctx); break;
-    case 2: launch_tova_ntb<2>(p, ctx); break;
-    case 4: launch_tova_ntb<4>(p, ctx); break;
-    case 8: launch_tova_ntb<8>(p, ctx); break;
-    default: launch_tova_ntb<16>(p, ctx); break;
+    case 1: return launch_tova_ntb<1>(p, ctx);
+    case 2: return launch_tova_ntb<2>(p, ctx);
+    case 4: return launch_tova_ntb<4>(p, ctx);
+    case 8: return launch_tova_ntb<8>(p, ctx);
+    default: return launch_tova_ntb<16>(p, ctx);
     }
-    return cudaGetLastError() == cudaSuccess ? AMS_OK : AMS_ERR_CUDA;
 }
 
 int launch_score_keydiff(const DevParams &p, LaunchCtx &ctx)
