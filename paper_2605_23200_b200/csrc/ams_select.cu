@@ -17,17 +17,21 @@
 // Selection order is (score key descending, position ascending), a strict total order, so a segment and its quota have
 // exactly one answer however it is found.  Finding the q-th largest key is what costs.  It is bound by latency and issue
 // slots, not by memory (4 bytes per token, from L2):
-//   * a segment of at most 256 tokens lives in the registers of one warp.  A histogram over the 16 octaves below its largest
-//     key (256 bins, shared memory) leads to the bin of the q-th key, and the few keys in that bin are taken apart one by
-//     one; exact fallbacks take over for thresholds further down, ties, NaN.  Fixing key bits from the top instead is a
-//     chain of 16 to 20 dependent warp-wide counts: 74 segments of a 16384-token unit 38 k cycles, 15 k now.
+//   * a segment of at most 256 tokens lives in the registers of one warp.  The lanes' extreme keys give a narrow range that
+//     holds the q-th key; a histogram over it (128 bins, shared memory) leads to its bin, and the few keys in that bin are
+//     taken apart one by one.  Exact fallbacks take over for ties, NaN and short segments.  Fixing key bits from the top
+//     instead is a chain of 16 to 20 dependent warp-wide counts.
 //   * longer segments are searched together by the whole block, in walks over their 256-token pieces: largest key (from a
 //     quarter of the tokens), histogram per segment over the octaves below it, then keys above the threshold's bin are
 //     kept and the few inside it go to a list in which every entry counts the entries of its segment before it.  (A bin
 //     that is still crowded gets another histogram first; ties by the hundred end with a bin of one key.)  Every warp has
 //     the same share of the walks whatever the lengths of the segments.
-// The backfill takes its bound from the best rejected key of every piece, which the searches leave behind, and looks only
-// at pieces that reach it, instead of walking the sequence twice.
+// The backfill takes its bound from the best keys that groups of lanes have seen rejected, and looks only at pieces whose best
+// rejected key reaches it, instead of walking the sequence twice.
+//
+// us per event, three kernels of the mass, the quotas and the selection before / this one: 256 units of 16384 tokens
+// 118 / 59, 1792 ragged units of 8192..32768 tokens 683 / 379, 1792 units of 4224 tokens 253 / 145, 2048 units of 32768 tokens in
+// long segments 922 / 480, 640 units of 131072 tokens 1684 / 1130, 512 units of 7001..8191 tokens 127 / 54.
 #include <type_traits>
 
 #include "ams_common.cuh"
@@ -42,11 +46,11 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kPiece = 256;         // tokens a warp holds in registers, eight per lane
 constexpr int kPer = kPiece / 32;
-constexpr int kWarpBins = 256;      // bins of a warp's own histogram, eight per lane
+constexpr int kWarpBins = 128;      // bins of a warp's own histogram, four per lane
 constexpr int kBatch = 64;          // long segments searched together
 constexpr int kMaxBins = 1024;      // histogram bins per long segment
 constexpr unsigned kOctaves = 12;   // octaves below a long segment's largest score that its histogram resolves
-constexpr int kBest = 512;          // entries of the table of best rejected keys
+constexpr int kBest = 512;          // entries of the table of the pieces' best rejected keys
 
 // Working arrays of the search of long segments, one entry per segment of the batch.
 struct SegTab {
@@ -100,7 +104,7 @@ struct SelShared {
     u64 scratch[40];
     int wc[2][32];   // per-warp counts of even / odd rounds of a block-wide count
     int n_list, n_look, n_long, total;
-    unsigned bound;
+    unsigned bound, gbest[128];
     int n_merged, n_seg, level, rem;
 };
 
@@ -380,48 +384,50 @@ __device__ int block_distribute(int sign, int D, const int *cap, int *quota, con
         cnt1 = warp_sum(cnt1);
         tot = warp_sum(tot);
         mx = __reduce_max_sync(kFull, mx);
-        int level = 0, used = 0;
+        int level = 0, used = 0; // F(k) = sum of min(cap, k) <= D < F(k + 1)
         if (tot <= D) {
             level = mx;
             used = tot;
-        } else if (cnt1 <= D) {
-            int lo = 1, hi = mx; // F(lo) <= D < F(hi), F(k) = sum of min(cap, k)
-            used = cnt1;
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                int f = 0;
+        } else {
+            // from F(level) <= D: as many whole rounds as the rest pays for if nobody else fills up, until it pays for none
+            for (int n = cnt1; D - used >= n;) {
+                level += (D - used) / n;
+                int f = 0, o = 0;
 #pragma unroll
-                for (int j = 0; j < kC; ++j) f += min(c[j], mid);
-                for (int i = kC * 32 + lane; i < n_seg; i += 32) f += min(cap[i], mid);
-                f = warp_sum(f);
-                if (f <= D) { lo = mid; used = f; } else hi = mid;
+                for (int j = 0; j < kC; ++j) { f += min(c[j], level); o += c[j] > level; }
+                for (int i = kC * 32 + lane; i < n_seg; i += 32) { f += min(cap[i], level); o += cap[i] > level; }
+                used = warp_sum(f);
+                n = warp_sum(o);
             }
-            level = lo;
         }
         if (lane == 0) { sh.level = level; sh.rem = D - used; sh.total = tot <= D ? D - tot : 0; }
     }
     __syncthreads();
     const int level = sh.level, rem = sh.rem, left = sh.total;
-    for (int i = tid >> 5; i < n_seg; i += NT / 32) { // a warp per segment: its rank in visiting order among those with room
-        const int ci = cap[i];
+    for (int i0 = 0; i0 < n_seg; i0 += NT / 8) { // eight lanes per segment: its rank in visiting order among those with room
+        const int i = i0 + (tid >> 3);
+        const bool in = i < n_seg;
+        const int ci = in ? cap[i] : 0;
         int g = min(ci, level);
-        if (rem > 0 && ci > level) {
-            const u64 Mi = M[i];
+        if (rem > 0) {
+            const long long Mx = in ? (long long)M[i] : 0ll;
             int rank = 0;
 #pragma unroll 4
-            for (int j = lane; j < n_seg; j += 32) { // (M, position) as one strict order; masses stay far below 2^63
-                const long long Mj = (long long)M[j], Mx = (long long)Mi;
+            for (int j = tid & 7; j < n_seg; j += 8) { // (M, position) as one strict order; masses stay far below 2^63
+                const long long Mj = (long long)M[j];
                 rank += cap[j] > level && (sign > 0 ? Mj + (j < i) > Mx : Mj < Mx + (j > i));
             }
-            g += warp_sum(rank) < rem;
+#pragma unroll
+            for (int d = 1; d < 8; d <<= 1) rank += __shfl_xor_sync(kFull, rank, d);
+            g += ci > level && rank < rem;
         }
-        if (lane == 0) quota[i] += sign * g;
+        if (in && (tid & 7) == 0) quota[i] += sign * g;
     }
     __syncthreads();
     return left;
 }
 
-// floor(x / y) for a quotient below 2^20 and x < 2^62, inv = 1 / y rounded: the product is off by less than one, the
+// floor(x / y) for a quotient below 2^50 and x < 2^62, inv = 1 / y rounded: the product is off by less than one, the
 // remainder corrects it.
 __device__ __forceinline__ u64 quotient(u64 x, u64 y, double inv)
 {
@@ -444,10 +450,11 @@ __device__ int segments_and_quotas(const DevParams &p, int T, int Bq, const Mass
     int *merged = tmp, *poff = merged + p.S + 1, *raw = poff + p.S + 1, *cap = raw + p.S + 1;
     const u64 SHq = p.uniform_q ? (u64)T : SH; // total of what the quotas are proportional to
     const double inv = 1.0 / (double)(2ull * SHq);
+    const double inv_s = 1.0 / (double)p.S;
     // raw cuts, ascending: the token that reaches quantile k closes its segment, c(t) >= k / S <=> C(t) >= ceil(k SH / S)
     for (int k = warp + 1; k < p.S; k += NW) {
         const int e = p.fixed_seg ? (int)(((long long)k * T) / p.S) // component ablation: boundary k at floor(k T / S)
-                                  : mass_cut(ms, wsum, T, ((u64)k * SH + (u64)p.S - 1) / (u64)p.S);
+                                  : mass_cut(ms, wsum, T, quotient((u64)k * SH + (u64)p.S - 1, (u64)p.S, inv_s));
         if (lane == 0) raw[k] = e;
     }
     __syncthreads();
@@ -560,20 +567,13 @@ __device__ __forceinline__ void count_if(unsigned *word, unsigned d, unsigned w)
 __device__ __forceinline__ void find_bin(const unsigned *hist, int q, int &bin, int &m, int &above)
 {
     const int lane = threadIdx.x & 31;
-    const uint4 *h4 = reinterpret_cast<const uint4 *>(hist) + 2 * (31 - lane); // lane 0 has the top eight bins
-    const uint4 a = h4[1], b = h4[0];
-    int c[8]; // keys in this lane's first 1 .. 8 bins from the top
-    c[0] = (int)a.w; c[1] = c[0] + (int)a.z; c[2] = c[1] + (int)a.y; c[3] = c[2] + (int)a.x;
-    c[4] = c[3] + (int)b.w; c[5] = c[4] + (int)b.z; c[6] = c[5] + (int)b.y; c[7] = c[6] + (int)b.x;
-    const int inc = warp_incl_scan(c[7]), exc = inc - c[7], rest = q - exc;
+    const uint4 v = reinterpret_cast<const uint4 *>(hist)[31 - lane]; // lane 0 has the top four bins
+    const int c0 = (int)v.w, c1 = c0 + (int)v.z, c2 = c1 + (int)v.y, c3 = c2 + (int)v.x;
+    const int inc = warp_incl_scan(c3), exc = inc - c3, rest = q - exc;
     const int src = __ffs(__ballot_sync(kFull, inc >= q)) - 1; // the first lane that covers q
-    int i = 0, below = 0, upto = c[7];
-#pragma unroll
-    for (int j = 6; j >= 0; --j) {
-        if (rest > c[j]) { below = max(below, c[j]); ++i; }
-        else upto = c[j];
-    }
-    const unsigned mine = (unsigned)(255 - lane * 8 - i) | (unsigned)(upto - below) << 8 | (unsigned)(exc + below) << 18;
+    const int i = (rest > c0) + (rest > c1) + (rest > c2);
+    const int below = rest > c2 ? c2 : (rest > c1 ? c1 : (rest > c0 ? c0 : 0)), upto = rest > c2 ? c3 : (rest > c1 ? c2 : (rest > c0 ? c1 : c0));
+    const unsigned mine = (unsigned)(127 - lane * 4 - i) | (unsigned)(upto - below) << 8 | (unsigned)(exc + below) << 18;
     const unsigned got = __shfl_sync(kFull, mine, src);
     bin = (int)(got & 255u); m = (int)((got >> 8) & 1023u); above = (int)(got >> 18);
 }
@@ -604,9 +604,8 @@ __device__ __forceinline__ Cut warp_cut(const unsigned (&k)[kPL], int n, int q, 
     }
     unsigned lo = mn, w = mx - mn;
     for (;;) {
-        const int shift = max(0, 24 - __clz(w)); // w >> shift < kWarpBins
+        const int shift = max(0, 25 - __clz(w)); // w >> shift < kWarpBins
         reinterpret_cast<uint4 *>(hist)[lane] = make_uint4(0, 0, 0, 0);
-        reinterpret_cast<uint4 *>(hist)[32 + lane] = make_uint4(0, 0, 0, 0);
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < kPL; ++j) {
@@ -639,32 +638,18 @@ __device__ __forceinline__ Cut warp_cut(const unsigned (&k)[kPL], int n, int q, 
     }
 }
 
-// The usual case of the search in two short steps: bins of 2^19 keys over the 16 octaves below the largest key mx, then the
-// few keys of the threshold's bin from the largest down.  key: the q-th largest distinct key from there on, which is the
-// q-th largest unless some are equal (the caller counts).  False: the threshold lies further down.  Unused registers must
-// hold keys below mx - 2^27.
+// The usual case of the search: at least q keys are known to lie in [lo, lo + w], the range is narrow, and a histogram over it
+// leaves few keys in the bin of the q-th one, of which the smallest are dropped one by one.  Returns the key from which on
+// q keys lie, unless some are equal (the caller counts).  Unused registers must lie outside the range.
 template <int kPL>
-__device__ __forceinline__ bool warp_cut_fast(const unsigned (&k)[kPL], int q, unsigned mx, unsigned *hist, unsigned &key)
+__device__ __forceinline__ unsigned warp_cut_fast(const unsigned (&k)[kPL], int q, unsigned lo, unsigned w, unsigned *hist)
 {
     const int lane = threadIdx.x & 31;
-    unsigned lo = mx - ((16u << 23) - 1u), w = (1u << 19) - 1u;
-    reinterpret_cast<uint4 *>(hist)[lane] = make_uint4(0, 0, 0, 0);
-    reinterpret_cast<uint4 *>(hist)[32 + lane] = make_uint4(0, 0, 0, 0);
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < kPL; ++j) atomicAdd(&hist[(max(k[j], lo) - lo) >> 19], 1u);
-    __syncwarp();
     int bin, m, above;
-    find_bin(hist, q, bin, m, above);
-    if (bin == 0) return false;
-    lo += (unsigned)bin << 19;
-    q -= above;
-    key = lo;
-    while (m > 5 && q < m && w > 0u) { // crowded: another histogram over the bin
-        const int shift = max(0, 24 - __clz(w));
+    do {
+        const int shift = max(0, 25 - __clz(w)); // w >> shift < kWarpBins
         __syncwarp();
         reinterpret_cast<uint4 *>(hist)[lane] = make_uint4(0, 0, 0, 0);
-        reinterpret_cast<uint4 *>(hist)[32 + lane] = make_uint4(0, 0, 0, 0);
         __syncwarp();
 #pragma unroll
         for (int j = 0; j < kPL; ++j) { const unsigned d = k[j] - lo; count_if(&hist[d >> shift], d, w); }
@@ -672,10 +657,9 @@ __device__ __forceinline__ bool warp_cut_fast(const unsigned (&k)[kPL], int q, u
         find_bin(hist, q, bin, m, above);
         lo += (unsigned)bin << shift;
         q -= above;
-        key = lo;
         w = min((1u << shift) - 1u, w - ((unsigned)bin << shift));
-    }
-    for (; q < m; --m) { // drop the smallest of the bin's keys, one at a time
+    } while (m - q > 4 && w > 0u); // crowded: another histogram over the bin
+    for (; q < m; --m) {
         unsigned v = kFull;
 #pragma unroll
         for (int j = 0; j < kPL; ++j) { const unsigned d = k[j] - lo; v = min(v, d <= w ? d : kFull); }
@@ -683,9 +667,8 @@ __device__ __forceinline__ bool warp_cut_fast(const unsigned (&k)[kPL], int q, u
         if (v >= w) break; // (equal keys)
         lo += v + 1u;
         w -= v + 1u;
-        key = lo;
     }
-    return true;
+    return lo;
 }
 
 // Kept bits of a piece of at most kPiece tokens from position a: lane j's word holds tokens a + 32 j .., shifted onto
@@ -698,18 +681,12 @@ __device__ __forceinline__ void mask_or(unsigned *mask, int a, unsigned word)
     if (lane <= kPer && w) atomicOr(&mask[(a >> 5) + lane], w);
 }
 
-// Best rejected key of a piece (slot): one entry per eight lanes while there are few pieces, one per piece otherwise.
-__device__ __forceinline__ void note_best(unsigned *best, int slot, bool fine, unsigned key)
+// Best rejected key of a piece (slots beyond the table share entries), and of all that this lane has seen.
+__device__ __forceinline__ void note_best(unsigned *best, int slot, unsigned key, unsigned &lane_best)
 {
-    const int lane = threadIdx.x & 31;
-    if (fine) {
-#pragma unroll
-        for (int d = 1; d < 8; d <<= 1) key = max(key, __shfl_xor_sync(kFull, key, d));
-        if ((lane & 7) == 0) best[slot * 4 + (lane >> 3)] = key;
-    } else {
-        key = __reduce_max_sync(kFull, key);
-        if (lane == 0) atomicMax(&best[slot & (kBest - 1)], key);
-    }
+    lane_best = max(lane_best, key);
+    key = __reduce_max_sync(kFull, key);
+    if ((threadIdx.x & 31) == 0) atomicMax(&best[slot & (kBest - 1)], key);
 }
 
 __device__ __forceinline__ void load_piece(const float *g, int a, int len, float (&x)[kPer])
@@ -721,35 +698,57 @@ __device__ __forceinline__ void load_piece(const float *g, int a, int len, float
 }
 
 // One segment of at most kPiece tokens.
-__device__ __forceinline__ void warp_segment(const float (&x)[kPer], unsigned *mask, unsigned *best, unsigned *hist, int slot, bool fine,
+__device__ __forceinline__ void warp_segment(const float (&x)[kPer], unsigned *mask, unsigned *best, unsigned *hist, int slot, unsigned &lane_best,
                                              int a, int L, int q, int ns, int t_last)
 {
     const int lane = threadIdx.x & 31, room = L - lane;
     const bool plain = a >= ns && a + L <= t_last; // no must-keep position in it
     auto may_fill = [&](int j) { return plain || (a + j * 32 + lane >= ns && a + j * 32 + lane < t_last); };
-    unsigned k[kPer], word = 0, rej = 0, mx = 0u;
+    unsigned k[kPer], word = 0, rej = 0, mine = 0u;
 #pragma unroll
-    for (int j = 0; j < kPer; ++j) { k[j] = __float_as_uint(x[j]); mx = max(mx, k[j]); }
-    mx = __reduce_max_sync(kFull, mx);
-    const bool pos = mx <= 0x7f800000u && mx > (17u << 23); // no negative score, no NaN (unused registers read as +0)
-    if (pos) {
-        mx |= 0x80000000u;
+    for (int j = 0; j < kPer; ++j) { k[j] = __float_as_uint(x[j]); mine = max(mine, k[j]); }
+    const bool pos = __reduce_max_sync(kFull, mine) <= 0x7f800000u; // no negative score, no NaN: the bit patterns ascend
+    if (!pos) {
+        mine = 0u;
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) k[j] |= 0x80000000u;
-    } else {
-        mx = 0u;
-#pragma unroll
-        for (int j = 0; j < kPer; ++j) { k[j] = j * 32 < room ? score_key(x[j]) : 0u; mx = max(mx, k[j]); }
-        mx = __reduce_max_sync(kFull, mx);
+        for (int j = 0; j < kPer; ++j) { k[j] = j * 32 < room ? score_key(x[j]) : 0u; mine = max(mine, k[j]); }
     }
     bool done = false;
     if (q >= L) { // all of it
         const int n = min(32, max(0, L - lane * 32));
         word = n > 0 ? kFull >> (32 - n) : 0u;
         done = true;
-    } else if (q > 0 && mx > (17u << 23)) {
-        unsigned key = 0u;
-        if (warp_cut_fast<kPer>(k, q, mx, hist, key)) {
+    } else if (q > 0 && L >= 2 * 32) {
+        // A narrow range that holds the q-th key: 32 (64) keys lie at or above the smallest of the lanes' largest (second
+        // largest) keys, and as many at or below the largest of their smallest (second smallest) ones.
+        unsigned top = mine, lo, hi;
+        int q_in = q; // its number from the top within the range
+        if (q <= 2 * 32) {
+            if (q > 32) {
+                unsigned first = 0u;
+                top = 0u;
+#pragma unroll
+                for (int j = 0; j < kPer; ++j) { top = max(top, min(first, k[j])); first = max(first, k[j]); }
+            }
+            lo = __reduce_min_sync(kFull, top);
+            hi = __reduce_max_sync(kFull, mine);
+        } else {
+            unsigned first = kFull, second = kFull;
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+                const unsigned v = j * 32 < room ? k[j] : kFull;
+                second = min(second, max(first, v));
+                first = min(first, v);
+            }
+            lo = __reduce_min_sync(kFull, first);
+            hi = __reduce_max_sync(kFull, L - q < 32 ? first : (L - q < 2 * 32 ? second : mine));
+            int above = 0;
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) above += k[j] > hi;
+            q_in = q - warp_sum(above);
+        }
+        if (lo > 0u && lo < hi) {
+            const unsigned key = warp_cut_fast<kPer>(k, q_in, lo, hi - lo, hist);
             unsigned b[kPer];
 #pragma unroll
             for (int j = 0; j < kPer; ++j) {
@@ -762,13 +761,22 @@ __device__ __forceinline__ void warp_segment(const float (&x)[kPer], unsigned *m
             const unsigned v0 = l1 ? w1 : w0, v1 = l1 ? w3 : w2;
             word = lane < kPer ? (l2 ? v1 : v0) : 0u;
             done = warp_sum(__popc(word)) == q;
-            if (pos && L < kPiece && rej == 0x80000000u) rej = 0u; // (may be an unused register; scores of 0 are not worth an entry)
+            if (pos) {
+                if (__any_sync(kFull, rej == 0u)) { // nothing rejected, or scores of 0, which unused registers look like
+                    bool zero = false;
+#pragma unroll
+                    for (int j = 0; j < kPer; ++j) zero |= j * 32 < room && k[j] == 0u && may_fill(j);
+                    rej = rej | (rej || zero ? 0x80000000u : 0u);
+                } else {
+                    rej |= 0x80000000u;
+                }
+            }
         }
     }
     if (!done) {
         if (pos) {
 #pragma unroll
-            for (int j = 0; j < kPer; ++j) if (j * 32 >= room) k[j] = 0u;
+            for (int j = 0; j < kPer; ++j) k[j] = j * 32 < room ? k[j] | 0x80000000u : 0u;
         }
         Cut cut = {kFull, 0};                // none of it
         if (q > 0) cut = warp_cut<kPer>(k, L, q, hist);
@@ -786,7 +794,7 @@ __device__ __forceinline__ void warp_segment(const float (&x)[kPer], unsigned *m
         }
     }
     mask_or(mask, a, word);
-    note_best(best, slot, fine, rej);
+    note_best(best, slot, rej, lane_best);
 }
 
 // Walks the pieces of the batch's long segments, a run of consecutive pieces per warp, the next piece's scores on their way
@@ -866,7 +874,7 @@ __device__ __forceinline__ int bin_shift(unsigned w, int nb) // smallest shift w
 // Top-q_i of the n <= kBatch long segments of the table: kept bits into mask, best rejected keys (must-keep positions
 // apart) into `best`, pieces taking the slots from slot0 on.
 template <int NT>
-__device__ void select_long(const float *g, const int *bounds, const int *quota, int n, unsigned *mask, unsigned *best, int slot0, bool fine,
+__device__ void select_long(const float *g, const int *bounds, const int *quota, int n, unsigned *mask, unsigned *best, int slot0, unsigned &lane_best,
                             SegTab &tb, unsigned *hist, uint2 *list, int ns, int t_last, SelShared &sh)
 {
     constexpr int NW = NT / 32, kList = Tune<NT>::kList;
@@ -983,13 +991,16 @@ __device__ void select_long(const float *g, const int *bounds, const int *quota,
                                       list[atomicAdd(&tb.cnt[i], 1)] = make_uint2(score_key(x[j]), (unsigned)(a + j * 32 + lane) | ((unsigned)i << 24));
                           }
                           mask_or(mask, a, word);
-                          note_best(best, slot0 + pc, fine, rej);
+                          note_best(best, slot0 + pc, rej, lane_best);
                       });
     }
     __syncthreads();
     auto rejected = [&](unsigned key, int i, int t) { // a candidate that did not make it
         const int slot = slot0 + tb.piece0[i] + (t - bounds[tb.seg[i]]) / kPiece;
-        if (t >= ns && t < t_last) atomicMax(&best[fine ? slot * 4 : slot & (kBest - 1)], key);
+        if (t >= ns && t < t_last) {
+            atomicMax(&best[slot & (kBest - 1)], key);
+            lane_best = max(lane_best, key);
+        }
     };
     for (int c = tid; c < sh.total; c += NT) { // every candidate ranks itself
         const uint2 v = list[c];
@@ -1116,7 +1127,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
 
     // ---- per-segment top-q_i.  Slots of the table of best rejected keys: short segment sg takes sg, the pieces of long
     //      ones those behind.  The next segment's scores are fetched before the current one is searched.
-    const bool fine = (longs ? 2 * n_seg + T / kPiece : n_seg) <= kBest / 4;
+    unsigned lane_best = 0u; // best key this lane has seen rejected
     {
         float xn[kPer];
         auto fetch = [&](int sg) {
@@ -1129,7 +1140,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
 #pragma unroll
             for (int j = 0; j < kPer; ++j) x[j] = xn[j];
             fetch(sg + NW);
-            if (L <= kPiece) warp_segment(x, mask, best, hist, sg, fine, a, L, q, ns, t_last);
+            if (L <= kPiece) warp_segment(x, mask, best, hist, sg, lane_best, a, L, q, ns, t_last);
         }
     }
     int n_slot = n_seg;
@@ -1154,11 +1165,15 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
             const int n = sh.n_long;
             if (n > 0) {
                 const int n_pc = tb.piece0[n];
-                select_long<NT>(g, bounds, quota, n, mask, best, n_slot, fine, tb, reinterpret_cast<unsigned *>(dyn + mp.hist), list, ns, t_last, sh);
+                select_long<NT>(g, bounds, quota, n, mask, best, n_slot, lane_best, tb, reinterpret_cast<unsigned *>(dyn + mp.hist), list, ns, t_last, sh);
                 n_slot += n_pc;
             }
         }
     }
+    // groups of eight lanes: the tokens they have seen
+#pragma unroll
+    for (int d = 1; d < 8; d <<= 1) lane_best = max(lane_best, __shfl_xor_sync(kFull, lane_best, d));
+    if ((lane & 7) == 0) sh.gbest[warp * 4 + (lane >> 3)] = lane_best;
     __syncthreads();
 
     // ---- must-keep prefix and suffix; every must-keep position a segment already chose frees one slot,
@@ -1170,39 +1185,20 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
     }
     const int r_fill = block_count<NT>(already, round, sh);
     if (r_fill > 0) {
-        // At least r_fill unflagged tokens lie at or above the r_fill-th largest entry of the table, so only pieces with an
-        // entry that reaches that bound can hold a winner; their tokens at or above it go to a list.
+        // At least r_fill unflagged tokens lie at or above the r_fill-th largest of the groups' best rejected keys, so
+        // only pieces whose best one reaches that bound can hold a winner; their tokens at or above it go to a list.
         if (warp == 0) {
-            unsigned k[kBest / 32];
+            unsigned k[NW / 8], M = 0u; // (0: too few groups, every token is looked at)
             int c = 0;
 #pragma unroll
-            for (int j = 0; j < kBest / 32; ++j) { k[j] = best[j * 32 + lane]; c += k[j] > 0u; }
-            unsigned M = 0u; // (too few entries: every token is looked at)
-            if (warp_sum(c) >= r_fill) {
-                unsigned mx = 0u;
-#pragma unroll
-                for (int j = 0; j < kBest / 32; ++j) mx = max(mx, k[j]);
-                mx = __reduce_max_sync(kFull, mx);
-                bool ok = mx > (17u << 23) && warp_cut_fast<kBest / 32>(k, r_fill, mx, hist, M);
-                if (ok) { // (equal entries can leave too few)
-                    c = 0;
-#pragma unroll
-                    for (int j = 0; j < kBest / 32; ++j) c += k[j] >= M;
-                    ok = warp_sum(c) >= r_fill;
-                }
-                if (!ok) M = warp_cut<kBest / 32>(k, kBest, r_fill, hist).key;
-            }
+            for (int j = 0; j < NW / 8; ++j) { k[j] = sh.gbest[j * 32 + lane]; c += k[j] > 0u; }
+            if (warp_sum(c) >= r_fill) M = warp_cut<NW / 8>(k, NW * 4, r_fill, hist).key;
             if (lane == 0) sh.bound = M;
         }
         __syncthreads();
         const unsigned M = sh.bound;
         auto raise = [&](int t) { atomicOr(&mask[t >> 5], 1u << (t & 31)); };
         auto unflagged = [&](int t) { return ((mask[t >> 5] >> (t & 31)) & 1u) == 0u; };
-        auto best_of = [&](int slot) {
-            if (!fine) return best[slot & (kBest - 1)];
-            const uint4 v = reinterpret_cast<const uint4 *>(best)[slot];
-            return max(max(v.x, v.y), max(v.z, v.w));
-        };
         const float least = M ? __uint_as_float((M & 0x80000000u) ? M ^ 0x80000000u : ~M) : -INFINITY;
         auto look = [&](int a, int len) { // a piece, by one warp
             float x[kPer];
@@ -1218,7 +1214,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
         };
         // pieces that reach the bound go to a list of their own
         auto note = [&](int slot, int a, int len) {
-            if (best_of(slot) < M) return;
+            if (best[slot & (kBest - 1)] < M) return;
             const int at = atomicAdd(&sh.n_look, 1);
             if (at < kBest) look_at[at] = (u64)(unsigned)a << 32 | (unsigned)len;
         };
