@@ -213,6 +213,10 @@ __device__ __forceinline__ void st_stream16(void *ptr, uint4 v)
 // A kernel launched with launch_after may start (prologue, loads that depend on nothing the previous kernel of
 // the stream writes) while that kernel's last blocks are still running; it calls wait_for_previous_kernel() before
 // it first touches anything the previous kernel wrote, or anything that kernel still reads and this one writes.
+// All kernels of an event are launched this way, its first ones too (one layer of 4096 tokens, six kernels: 43.4 ->
+// 40.0 us).  None lets the next one in any earlier than at its end (griddepcontrol.launch_dependents): blocks that sit and
+// wait hold slots that the running kernel's later blocks need (16 sequences just above a budget of 4096: 1829 ->
+// 2127 us), and at one to 32 layers of 4096 tokens it gave -4 to +12 us.
 __device__ __forceinline__ void wait_for_previous_kernel() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>

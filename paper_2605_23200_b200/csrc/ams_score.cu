@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kTovaThreads) k_tova(DevParams p)
     __shared__ float red[4][NTB * 8][2];
     const unsigned smem = (unsigned)__cvta_generic_to_shared(dyn);
     const unsigned Qb = smem + (kTovaThreads / 32) * kRing * kTileK;
-    if (PHASE == 2) wait_for_previous_kernel(); // merged statistics
+    wait_for_previous_kernel(); // effective lengths; merged statistics
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, tq = lane & 3;
     const float c = kLog2e * 0.08838834764831845f; // log2(e) / sqrt(128)
     const float inv_rows = 1.0f / (float)p.rows;
@@ -352,7 +352,7 @@ __global__ void __launch_bounds__(kTovaThreads) k_tova_wide(DevParams p)
     const unsigned smem = (unsigned)__cvta_generic_to_shared(dyn);
     const unsigned Qb = smem + (kTovaThreads / 32) * kRing * kTileK;    // [MT * 16 rows][256 bytes] as they come
     const unsigned Fr = Qb + MT * 16 * kRowBytes;                   // [MT][8 k-steps][32 lanes] fragments of the current rows
-    if (PHASE == 2) wait_for_previous_kernel(); // merged statistics
+    wait_for_previous_kernel(); // effective lengths; merged statistics
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, tq = lane & 3;
     const float c = kLog2e * 0.08838834764831845f; // log2(e) / sqrt(128)
     const float inv_rows = 1.0f / (float)p.rows;
@@ -607,6 +607,7 @@ constexpr int kKdThreads = 256; // 16 token rows x 16 lanes of 16 bytes
 __global__ void __launch_bounds__(kKdThreads) k_keydiff_sum(DevParams p)
 {
     __shared__ float red[16][kHeadDim];
+    wait_for_previous_kernel(); // effective lengths
     const int uid = blockIdx.y, slice = blockIdx.x;
     const int h = uid % p.H, b = (uid / p.H) % p.B, l = uid / (p.H * p.B);
     const int T = p.seq_lens[b];
@@ -742,7 +743,7 @@ int launch_tova_ntb(const DevParams &p_in, LaunchCtx &ctx)
         const long long r = (long long)n_sm * (resident[phase][dev] > 0 ? resident[phase][dev] : 1);
         return dim3((unsigned)(items < r ? items : r));
     };
-    k1<<<blocks(0), kTovaThreads, smem, ctx.s>>>(p);
+    launch_after(k1, blocks(0), dim3(kTovaThreads), smem, ctx.s, p);
     ctx.mark(kKernScore1);
     const bool from_logits = NTB <= 2 && p.logits && p.rows_pad == NTB * 8;
     p.merge_in_usage = from_logits && units <= 2 * n_sm;
@@ -784,7 +785,7 @@ int launch_score_tova(const DevParams &p, LaunchCtx &ctx)
 int launch_score_keydiff(const DevParams &p, LaunchCtx &ctx)
 {
     const dim3 grid(p.n_slices, p.L * p.B * p.H);
-    k_keydiff_sum<<<grid, kKdThreads, 0, ctx.s>>>(p);
+    launch_after(k_keydiff_sum, grid, dim3(kKdThreads), 0, ctx.s, p);
     ctx.mark(kKernScore1);
     launch_after(k_keydiff_combine, dim3((unsigned)(p.L * p.B * p.H)), dim3(kHeadDim), 0, ctx.s, p);
     ctx.mark(kKernScoreCombine);

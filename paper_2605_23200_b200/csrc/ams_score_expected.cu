@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_expected_tc(DevParams p, cons
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
+    wait_for_previous_kernel(); // effective lengths
     const int hpb = p.tc_hpb, my_hs = p.H / hpb;
     const int my_h0 = blockIdx.x % my_hs, my_group = blockIdx.x / my_hs;
     tc_partition(p, gridDim.x / my_hs, prefix, &sh.tiles_lh, &sh.n_tiles, &sh.tpc);
@@ -488,7 +489,7 @@ int launch_score_expected(const DevParams &p_in, LaunchCtx &ctx)
         p.tc_stages = p.ex_gc <= 2 ? 4 : 2;
         const size_t smem = 1024 + (size_t)(p.ex_gc + p.tc_stages) * kTileBytes + 256;
         if (!grant_dynamic_smem(k_expected_tc, smem, grant)) return AMS_ERR_CUDA;
-        k_expected_tc<<<tg.grid, kTcThreads, smem, ctx.s>>>(p, k_map, c_map);
+        if (launch_after(k_expected_tc, dim3((unsigned)tg.grid), dim3(kTcThreads), smem, ctx.s, p, k_map, c_map) != cudaSuccess) return AMS_ERR_CUDA;
         ctx.mark(kKernScore1);
     }
     const dim3 grid((unsigned)((p.T_cap + kFinSlice - 1) / kFinSlice), (unsigned)U);

@@ -76,6 +76,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
     // the SM count well: 148 SMs and 8 heads give 18 groups of 8 blocks, or 37 groups of 4 with two heads each).
     const int hpb = p.tc_hpb, my_hs = p.H / hpb;
     const int my_h0 = blockIdx.x % my_hs, my_group = blockIdx.x / my_hs;
+    if (PHASE == 1) wait_for_previous_kernel(); // effective lengths
     tc_partition(p, gridDim.x / my_hs, prefix, &sh.tiles_lh, &sh.n_tiles, &sh.tpc);
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem_base)), "r"(512) : "memory");
@@ -424,7 +425,7 @@ int launch_score_tova_tc(const DevParams &p_in, LaunchCtx &ctx)
     const TcGrid tg = tc_grid(p, n_sm);
     const int hpb = tg.hpb, grid = tg.grid;
     p.tc_hpb = hpb;
-    k_tova_tc<1><<<grid, kTcThreads, smem, ctx.s>>>(p, k_map, q_map);
+    if (launch_after(k_tova_tc<1>, dim3((unsigned)grid), dim3(kTcThreads), smem, ctx.s, p, k_map, q_map) != cudaSuccess) return AMS_ERR_CUDA;
     ctx.mark(kKernScore1);
     if (launch_after(k_tova_tc<2>, dim3((unsigned)grid), dim3(kTcThreads), smem, ctx.s, p, k_map, q_map) != cudaSuccess) return AMS_ERR_CUDA;
     ctx.mark(kKernScore2);

@@ -14,6 +14,7 @@ constexpr int kSmoothThreads = 256;
 
 __global__ void __launch_bounds__(kSmoothThreads) k_smooth_usage(DevParams p, const float *src, float *dst, int k)
 {
+    wait_for_previous_kernel(); // the usage
     const int uid = blockIdx.x;
     const int b = (uid / p.H) % p.B;
     const int T = p.seq_lens[b];
@@ -92,6 +93,7 @@ __global__ void __launch_bounds__(256) k_inspect(DevParams p, ams_debug_views v)
 // skipped as well, so that no kernel ever forms an address from a bad page id.
 __global__ void __launch_bounds__(256) k_prepare(DevParams p, const int *lens_in, int *eff_lens)
 {
+    wait_for_previous_kernel(); // the caller's table and lengths
     const int b = blockIdx.x;
     const int T = lens_in[b];
     int eff = 0;
@@ -141,9 +143,9 @@ __global__ void k_expire_wait(int *status, uint32_t polls)
 
 int launch_prepare(const DevParams &p, const int *lens_in, int *eff_lens, LaunchCtx &ctx)
 {
-    k_prepare<<<p.B, 256, 0, ctx.s>>>(p, lens_in, eff_lens);
+    if (launch_after(k_prepare, dim3((unsigned)p.B), dim3(256), 0, ctx.s, p, lens_in, eff_lens) != cudaSuccess) return AMS_ERR_CUDA;
     ctx.mark(kKernPrepare);
-    return cudaGetLastError() == cudaSuccess ? AMS_OK : AMS_ERR_CUDA;
+    return AMS_OK;
 }
 
 int launch_expire_wait(int *status, uint32_t polls, cudaStream_t s)
@@ -177,9 +179,9 @@ int launch_retained_iou(const DevParams &p, const int *prev_kept, float *out, La
 int launch_smooth_usage(const DevParams &p, const float *src, float *dst, int k, LaunchCtx &ctx)
 {
     const dim3 grid((unsigned)(p.L * p.B * p.H), (unsigned)((p.T_cap + kSmoothThreads - 1) / kSmoothThreads));
-    k_smooth_usage<<<grid, kSmoothThreads, 0, ctx.s>>>(p, src, dst, k);
+    if (launch_after(k_smooth_usage, grid, dim3(kSmoothThreads), 0, ctx.s, p, src, dst, k) != cudaSuccess) return AMS_ERR_CUDA;
     ctx.mark(kKernUsage);
-    return cudaGetLastError() == cudaSuccess ? AMS_OK : AMS_ERR_CUDA;
+    return AMS_OK;
 }
 
 } // namespace ams
