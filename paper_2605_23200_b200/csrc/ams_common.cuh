@@ -16,6 +16,10 @@ constexpr int kRowBytes = kHeadDim * 2;
 
 typedef unsigned long long u64;
 
+constexpr int kGroupBlocks = 256; // most blocks of a launch that work in groups,
+constexpr int kGroupSlot = 128;   // floats in one slot of their exchange
+constexpr int kGroupCounters = kGroupBlocks * 4 * 8;
+
 // Everything a kernel of one ams_compress call needs; passed by value.
 struct DevParams {
     // geometry of the call
@@ -61,6 +65,8 @@ struct DevParams {
     float score_eps;                  // added to the group-mean attention weight before the value norm multiplies
     float *ex_logits;                 // [units][G][T_cap] logits in log2 units, or null
     int ex_g0, ex_gc;                 // query heads [g0, g0 + gc) of the group handled by one launch (set by the launcher)
+    int *group_count;                 // blocks that work on a unit together: counters, cleared by the first kernel of an event,
+    float *group_part;                // and the slots of what they exchange
     int *seq_bad;                     // [B]: set when a unit of the sequence reported a device-side error (its rows stay)
     int *status;                      // [4]: code, unit, a, b
 };
@@ -186,11 +192,47 @@ __device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, un
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
 }
+__device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack_f32x2(unsigned long long a, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a)); }
 __device__ __forceinline__ float sum_f32x2(unsigned long long a)
 {
     float lo, hi;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
+    unpack_f32x2(a, lo, hi);
     return lo + hi;
+}
+
+__device__ __forceinline__ void mma_bf16(float (&d)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3,
+                                         unsigned b0, unsigned b1)
+{
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+                 "{%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// Asynchronous 16-byte copies into shared memory.
+__device__ __forceinline__ void cp_async16(unsigned dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+// 16 bytes, or zeros without reading
+__device__ __forceinline__ void cp_async16_or_zero(unsigned dst, const void *src, bool read)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(read ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ uint4 lds16(unsigned addr)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
 }
 
 // 16-byte global load that does not pollute L1 (streamed once per phase).

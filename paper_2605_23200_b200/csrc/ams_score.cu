@@ -1,4 +1,4 @@
-// Base scorers of the AMS compression step.
+// Window scorer of the AMS compression step.
 //
 // TOVA-style usage (Section 3.2 / Algorithm 1 step 1 of the paper): every query row
 // r = (head of the GQA group, window query j) is a softmax of q_r.k_t/sqrt(D) over the
@@ -10,9 +10,6 @@
 // maximum is 1/min_r Z_r and needs no third pass.  With at most 16 (padded) query rows
 // phase 1 also stores the scaled logits (at most 64 bytes per token against the 256
 // bytes of its key), and phase 2 is a per-token kernel over those instead of K.
-//
-// KeyDiff-style score: negative cosine similarity of each key to the mean key of its
-// (sequence, KV head) cache.
 #include "ams_common.cuh"
 
 namespace ams {
@@ -28,15 +25,6 @@ __device__ __forceinline__ float ex2(float x)
     return y;
 }
 
-__device__ __forceinline__ void mma_bf16(float (&d)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3,
-                                         unsigned b0, unsigned b1)
-{
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-                 "{%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-
 // (m, z) <- log-sum-exp merge of (m, z) and (m2, z2) in the base-2 domain.
 __device__ __forceinline__ void lse_merge(float &m, float &z, float m2, float z2)
 {
@@ -50,25 +38,6 @@ constexpr int kTovaThreads = 128;
 constexpr int kRing = 3;       // 16-token K tiles per warp in shared memory: one worked on, two on their way
 constexpr int kTileK = 16 * kRowBytes;
 static_assert(kRing == 3, "the waits below count on two tiles in flight");
-
-__device__ __forceinline__ void cp_async16(unsigned dst, const void *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-// 16 bytes, or zeros without reading
-__device__ __forceinline__ void cp_async16_or_zero(unsigned dst, const void *src, bool read)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(read ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ uint4 lds16(unsigned addr)
-{
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
-    return v;
-}
 
 // One (unit, token slice, block of query rows) of work, and the warp's share of it.
 struct TovaItem {
@@ -600,131 +569,6 @@ __global__ void __launch_bounds__(256) k_tova_usage_from_logits(DevParams p)
     }
 }
 
-// ---------------------------------------------------------------------------- KeyDiff
-
-constexpr int kKdThreads = 256; // 16 token rows x 16 lanes of 16 bytes
-
-__global__ void __launch_bounds__(kKdThreads) k_keydiff_sum(DevParams p)
-{
-    __shared__ float red[16][kHeadDim];
-    wait_for_previous_kernel(); // effective lengths
-    const int uid = blockIdx.y, slice = blockIdx.x;
-    const int h = uid % p.H, b = (uid / p.H) % p.B, l = uid / (p.H * p.B);
-    const int T = p.seq_lens[b];
-    if (T <= p.Tk || T > p.T_cap) return;
-    const int t_begin = slice * p.slice_len;
-    if (t_begin >= T) return;
-    const int t_end = min(T, t_begin + p.slice_len);
-    const int lane = threadIdx.x & 15, r = threadIdx.x >> 4;
-    const int *table = p.block_table + (size_t)b * p.bt_stride;
-    float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int t = t_begin + r; t < t_end; t += 16) {
-        const uint4 v = ld_stream16(p.k_pages + row_offset(p, l, table[t >> 4], t & 15, h) + lane * 8);
-        acc[0] += bf16_lo(v.x); acc[1] += bf16_hi(v.x); acc[2] += bf16_lo(v.y); acc[3] += bf16_hi(v.y);
-        acc[4] += bf16_lo(v.z); acc[5] += bf16_hi(v.z); acc[6] += bf16_lo(v.w); acc[7] += bf16_hi(v.w);
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) red[r][lane * 8 + i] = acc[i];
-    __syncthreads();
-    if (threadIdx.x < kHeadDim) {
-        float s = 0.0f;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) s += red[i][threadIdx.x];
-        p.part[((size_t)uid * p.n_slices + slice) * kHeadDim + threadIdx.x] = s;
-    }
-}
-
-__global__ void __launch_bounds__(kHeadDim) k_keydiff_combine(DevParams p)
-{
-    __shared__ float sq[kHeadDim];
-    wait_for_previous_kernel(); // the slices' sums
-    const int uid = blockIdx.x;
-    const int b = (uid / p.H) % p.B;
-    const int T = p.seq_lens[b];
-    if (T <= p.Tk || T > p.T_cap) return;
-    const int ns = (T + p.slice_len - 1) / p.slice_len;
-    float s = 0.0f;
-    for (int i = 0; i < ns; ++i) s += p.part[((size_t)uid * p.n_slices + i) * kHeadDim + threadIdx.x];
-    const float mu = s / (float)T;
-    float *fin = p.fin + (size_t)uid * (p.rows_pad + 8);
-    fin[threadIdx.x] = mu;
-    sq[threadIdx.x] = mu * mu;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float tot = 0.0f;
-        for (int i = 0; i < kHeadDim; ++i) tot += sq[i];
-        fin[kHeadDim] = sqrtf(tot);
-    }
-}
-
-__global__ void __launch_bounds__(kKdThreads) k_keydiff_score(DevParams p)
-{
-    wait_for_previous_kernel(); // the mean key
-    const int uid = blockIdx.y, slice = blockIdx.x;
-    const int h = uid % p.H, b = (uid / p.H) % p.B, l = uid / (p.H * p.B);
-    const int T = p.seq_lens[b];
-    if (T <= p.Tk || T > p.T_cap) return;
-    const int t_begin = slice * p.slice_len;
-    if (t_begin >= T) return;
-    const int t_end = min(T, t_begin + p.slice_len);
-    const int lane = threadIdx.x & 15, r = threadIdx.x >> 4;
-    const int *table = p.block_table + (size_t)b * p.bt_stride;
-    const float *fin = p.fin + (size_t)uid * (p.rows_pad + 8);
-    unsigned long long mu2[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) mu2[i] = pack_f32x2(fin[lane * 8 + 2 * i], fin[lane * 8 + 2 * i + 1]);
-    const float mu_norm = fin[kHeadDim];
-    float *g_out = p.scores + (size_t)uid * p.T_cap;
-    // four tokens per thread and round: their loads are issued together, so that enough bytes are in flight
-    constexpr int kU = 4;
-    const int n_iter = (t_end - t_begin + 16 * kU - 1) / (16 * kU);
-    for (int it = 0; it < n_iter; ++it) {
-        uint4 v[kU];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int t = t_begin + (it * kU + u) * 16 + r;
-            v[u] = make_uint4(0, 0, 0, 0);
-            if (t < t_end) v[u] = ld_stream16(p.k_pages + row_offset(p, l, table[t >> 4], t & 15, h) + lane * 8);
-        }
-        // a[2u] = this lane's part of k_t . mu, a[2u + 1] of |k_t|^2, for the four tokens u
-        float a[2 * kU];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            // two dimensions per instruction: a bf16 pair widens to a packed fp32 pair (low half shifted up, high half
-            // masked), and both running sums take packed multiply-adds
-            const unsigned w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-            unsigned long long dot2 = 0ull, sq2 = 0ull; // (0.0f, 0.0f)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const unsigned long long k2 = pack_f32x2(bf16_lo(w[i]), bf16_hi(w[i]));
-                dot2 = fma_f32x2(k2, mu2[i], dot2);
-                sq2 = fma_f32x2(k2, k2, sq2);
-            }
-            a[2 * u] = sum_f32x2(dot2); a[2 * u + 1] = sum_f32x2(sq2);
-        }
-        // sums over the 16 lanes of a token row, all eight values at once: at each step a lane hands half of
-        // its values to its partner and keeps the other half (9 shuffles instead of 32)
-#pragma unroll
-        for (int o = 8, n = 2 * kU; o >= 2; o >>= 1, n >>= 1) {
-            const bool up = (lane & o) != 0;
-#pragma unroll
-            for (int i = 0; i < n / 2; ++i) {
-                const float send = up ? a[i] : a[i + n / 2];
-                const float keep = up ? a[i + n / 2] : a[i];
-                a[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-            }
-        }
-        a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
-        // lane holds value index 4 * bit3 + 2 * bit2 + bit1: even = dot of token (index / 2), odd = its |k|^2
-        const float other = __shfl_xor_sync(0xffffffffu, a[0], 2);
-        if ((lane & 3) == 0) {
-            const int u = lane >> 2;
-            const int t = t_begin + (it * kU + u) * 16 + r;
-            if (t < t_end) g_out[t] = -a[0] / fmaxf(sqrtf(other) * mu_norm, 1e-30f);
-        }
-    }
-}
-
 template <int NTB>
 int launch_tova_ntb(const DevParams &p_in, LaunchCtx &ctx)
 {
@@ -780,18 +624,6 @@ int launch_score_tova(const DevParams &p, LaunchCtx &ctx)
     case 8: return launch_tova_ntb<8>(p, ctx);
     default: return launch_tova_ntb<16>(p, ctx);
     }
-}
-
-int launch_score_keydiff(const DevParams &p, LaunchCtx &ctx)
-{
-    const dim3 grid(p.n_slices, p.L * p.B * p.H);
-    launch_after(k_keydiff_sum, grid, dim3(kKdThreads), 0, ctx.s, p);
-    ctx.mark(kKernScore1);
-    launch_after(k_keydiff_combine, dim3((unsigned)(p.L * p.B * p.H)), dim3(kHeadDim), 0, ctx.s, p);
-    ctx.mark(kKernScoreCombine);
-    launch_after(k_keydiff_score, grid, dim3(kKdThreads), 0, ctx.s, p);
-    ctx.mark(kKernScore2);
-    return cudaGetLastError() == cudaSuccess ? AMS_OK : AMS_ERR_CUDA;
 }
 
 } // namespace ams
