@@ -8,7 +8,7 @@
 namespace ams {
 
 struct Layout {
-    size_t status, eff_lens, seq_bad, scores, usage, logits, ex_logits, n_seg, seg_bounds, quotas, keep_idx, part, fin, group_count, group_part, total;
+    size_t status, eff_lens, seq_bad, scores, usage, ex_logits, n_seg, seg_bounds, quotas, keep_idx, part, fin, group_count, group_part, total;
     int units, T_cap, seg_cap, n_slices, slice_len, rows_pad_cap;
 };
 
@@ -97,13 +97,10 @@ static Layout make_layout(const ams_config *c)
     y.part = off;       off = align_up(off + U * part_per, 256);
     const size_t fin_per = (size_t)((y.rows_pad_cap > kHeadDim ? y.rows_pad_cap : kHeadDim) + 8) * 4;
     y.fin = off;        off = align_up(off + U * fin_per, 256);
-    // narrow query blocks keep their logits (rows_pad floats per token, at most 1/4 of the K bytes) so that
-    // the usage pass need not read K again
-    y.logits = off;     off = align_up(off + (y.rows_pad_cap <= 16 && c->max_window > 0 ? U * T * (size_t)y.rows_pad_cap * 4 : 0), 256);
     // expected-attention scorer: one logit per (query head, token), so that K is read once
     y.ex_logits = off;  off = align_up(off + (c->expected_scorer ? U * T * (size_t)(c->n_q_heads / c->n_kv_heads) * 4 : 0), 256);
-    y.group_count = off; off = align_up(off + (size_t)kGroupCounters * 4, 256);
-    y.group_part = off;  off = align_up(off + (size_t)kGroupBlocks * 4 * kGroupSlot * 4, 256);
+    y.group_count = off; off = align_up(off + (size_t)2 * kGroupCounters * kGroupCounterPad * 4, 256);
+    y.group_part = off;  off = align_up(off + (size_t)kGroupBlocks * 4 * kGroupSlot, 256);
     y.total = off;
     return y;
 }
@@ -264,13 +261,12 @@ int ams_compress(ams_state *st, void *k_pages, void *v_pages, int64_t num_pages,
     p.mass_dbg = dbg ? dbg->mass : nullptr;
     p.seg_out = dbg && (dbg->n_segments || dbg->seg_bounds || dbg->quotas || dbg->keep_idx);
     p.part = (float *)(st->ws + y.part); p.fin = (float *)(st->ws + y.fin);
-    p.group_count = (int *)(st->ws + y.group_count); p.group_part = (float *)(st->ws + y.group_part);
+    p.group_count = (int *)(st->ws + y.group_count); p.group_part = st->ws + y.group_part;
     p.slice_len = y.slice_len; p.n_slices = y.n_slices;
     p.rows_pad = scorer_id == AMS_SCORER_TOVA ? rows_padded(p.rows) : kHeadDim;
     p.tc_tpc_min = tc_tiles_per_block_min(y.T_cap);
     p.tc_stages = p.rows_pad <= 256 ? 4 : 2; // even: each stage then belongs to one of the two MMA issuers
     p.status = (int *)(st->ws + y.status);
-    p.logits = (y.rows_pad_cap <= 16 && c.max_window > 0) ? (float *)(st->ws + y.logits) : nullptr;
     p.q_mean = st->q_mean; p.q_cov = (const __nv_bfloat16 *)st->q_cov; p.score_eps = st->score_eps;
     p.ex_logits = c.expected_scorer ? (float *)(st->ws + y.ex_logits) : nullptr;
 

@@ -17,8 +17,9 @@ constexpr int kRowBytes = kHeadDim * 2;
 typedef unsigned long long u64;
 
 constexpr int kGroupBlocks = 256; // most blocks of a launch that work in groups,
-constexpr int kGroupSlot = 128;   // floats in one slot of their exchange
-constexpr int kGroupCounters = kGroupBlocks * 4 * 8;
+constexpr int kGroupSlot = 512;   // bytes in one slot of their exchange
+constexpr int kGroupCounterPad = 32; // words from one counter to the next: a cache line each
+constexpr int kGroupCounters = kGroupBlocks * 4; // of one launch; an event has room for two
 
 // Everything a kernel of one ams_compress call needs; passed by value.
 struct DevParams {
@@ -56,9 +57,6 @@ struct DevParams {
     int slice_len, n_slices, rows_pad;
     int tc_tpc_min, tc_stages;        // tensor-core scorer: least tiles per block, K stages in shared memory
     int tc_hpb;                       // tensor-core scorer: KV heads a block takes one after the other (set by its launcher)
-    int merge_in_usage;               // narrow query blocks: the pass over the stored logits merges the slices' statistics itself
-                                      // (set by the launcher when there are too few units for a kernel of its own to pay)
-    float *logits;                    // narrow query blocks (rows_pad <= 16): scaled logits [units][T_cap][rows_pad], or null
     // expected-attention scorer
     const float *q_mean;              // [L][B][H*G][128] mean of the future queries per query head
     const __nv_bfloat16 *q_cov;       // [L][B][H*G][128][128] their covariance
@@ -66,7 +64,7 @@ struct DevParams {
     float *ex_logits;                 // [units][G][T_cap] logits in log2 units, or null
     int ex_g0, ex_gc;                 // query heads [g0, g0 + gc) of the group handled by one launch (set by the launcher)
     int *group_count;                 // blocks that work on a unit together: counters, cleared by the first kernel of an event,
-    float *group_part;                // and the slots of what they exchange
+    unsigned char *group_part;        // and the slots of what they exchange
     int *seq_bad;                     // [B]: set when a unit of the sequence reported a device-side error (its rows stay)
     int *status;                      // [4]: code, unit, a, b
 };
@@ -302,6 +300,7 @@ struct LaunchCtx {
 };
 
 int launch_score_tova(const DevParams &p, LaunchCtx &ctx);
+int launch_score_window(const DevParams &p, LaunchCtx &ctx); // up to 32 query rows
 bool tova_tc_supported(const DevParams &p);
 size_t tova_tc_smem_bytes(const DevParams &p);
 int launch_score_tova_tc(const DevParams &p, LaunchCtx &ctx);

@@ -1,19 +1,19 @@
-// Units of work shared by groups of resident blocks: the two-pass scorers that read K twice in one launch.
+// Units of work shared by groups of resident blocks: scorers that need a statistic over all keys of a unit before they can score
+// any of them, in one launch.
 //
-// A unit is one (layer, sequence, KV head).  Its scores need a statistic of all of its keys first, so K is read twice.
-// The blocks of a cooperative launch (one per SM, all resident) are split into groups; each group takes a unit at a
-// time, each block a share of its pages.  A block works on "pass 1 of unit n, pass 2 of unit n - 1" in turn: while the blocks
-// exchange the statistics of a unit they read the next one, and the second pass finds its keys in L2.  The groups are made as
-// wide as that takes: their units together hold kGroupWindow bytes.  Measured without the exchange, one head of 32768
-// tokens per group, 8.6 GB of K: read once 1.24 ms; twice with 17 / 25 / 34 / 42 MB of units 1.33 / 1.35 / 1.38 / 1.50 ms
-// with the second read marked evict-first, 1.33 / 1.58 / 2.00 / 2.34 ms without the mark.  With the exchange, key scores of
-// 512 units of 4096 tokens at a window of 26 / 34 / 42 / 50 / 64 MB: 131 / 136 / 148 / 149 / 175 us.
+// A unit is one (layer, sequence, KV head).  The blocks of a cooperative launch (one per SM, all resident) are split into
+// groups; each group takes a unit at a time, each block a share of its pages.  A block works on "pass 1 of unit n, pass 2
+// of unit n - 1" in turn: while the blocks exchange the statistics of a unit they read the next one, and the second pass
+// finds its keys in L2, or what it needs of them in shared memory.  The groups are made as wide as it takes for their
+// units together to hold a window of so many bytes: small enough to be still there, large enough to hide the exchange.
+// Measured without the exchange, one head of 32768 tokens per group, 8.6 GB of K: read once 1.24 ms; twice with 17 / 25 / 34 / 42
+// MB of units 1.33 / 1.35 / 1.38 / 1.50 ms with the second read marked evict-first, 1.33 / 1.58 / 2.00 / 2.34 ms without.
 #pragma once
 #include "ams_common.cuh"
+#include "ams_tc_ptx.cuh"
+#include "ams_tc_tiles.cuh"
 
 namespace ams {
-
-constexpr long long kGroupWindow = 26ll << 20;
 
 struct Groups {
     int g, n;    // blocks per group, groups
@@ -22,26 +22,30 @@ struct Groups {
     int dh, db, dl;    // n as a number of heads, sequences and layers: the step from a unit of the group to the next
 };
 
-// The split for the lengths of this call; the same in every block, computed by each warp for itself.
-__device__ __forceinline__ Groups split_groups(const DevParams &p, int warps)
+// The split for the lengths of this call; the same in every block, computed by each warp for itself.  most_pages: of a unit that
+// a block can hold.
+__device__ __forceinline__ Groups split_groups(const DevParams &p, int warps, long long window, int most_pages)
 {
     const int lane = threadIdx.x & 31, nb = gridDim.x;
     int longest = 0, active = 0;
+    u64 total = 0;
     for (int b = lane; b < p.B; b += 32) {
         const int T = p.seq_lens[b];
-        if (T > p.Tk && T <= p.T_cap) { longest = max(longest, T); ++active; }
+        if (T > p.Tk && T <= p.T_cap) { longest = max(longest, T); total += (u64)T; ++active; }
     }
     longest = __reduce_max_sync(0xffffffffu, longest);
     active = __reduce_add_sync(0xffffffffu, active);
+    total = warp_sum_u64(total);
     const int units = active * p.L * p.H, pages = (longest + kPage - 1) / kPage;
     Groups r;
     r.g = 1; r.n = 0; r.id = 1; r.me = 0;
     if (units <= 0) return r;
-    const long long bytes = (long long)pages * kPage * kRowBytes;
+    const long long bytes = (long long)(total / active) * kRowBytes; // of a unit, on the average
     // two groups at least, so that one reads while the other waits (K of 80000 tokens, 32 units: 222 -> 132 us; of 131072,
     // where two units no longer fit L2: 388 -> 324 us); no group without work; no fewer units in the last round than need be
-    int n = min(min(nb, units), (int)max(2ll, kGroupWindow / bytes));
+    int n = min(min(nb, units), (int)max(2ll, window / bytes));
     n = (units + (units + n - 1) / n - 1) / ((units + n - 1) / n);
+    n = max(1, min(n, nb / ((pages + most_pages - 2) / (most_pages - 1)))); // no share above what a block can hold (its ends are rounded)
     const int g = min(nb / n, (pages + warps - 1) / warps); // no warp without a page
     r.g = g;
     r.n = min(nb / g, units);
@@ -86,30 +90,41 @@ __device__ __forceinline__ bool next_group_unit(const DevParams &p, const Groups
     return false;
 }
 
-// Exchange of a block's statistics with its group.  Four slots in turn: a block publishes unit n + 4 only after its
-// pass 2 of unit n + 2, which waited until every block of the group had published unit n + 2 and so was through with unit n.
-// The counters only grow during a launch (the first kernel of the event clears them).
-__device__ __forceinline__ int *group_counter(const DevParams &p, const Groups &gr, int n) { return p.group_count + (gr.id * 4 + (n & 3)) * 8; }
-__device__ __forceinline__ float *group_slot(const DevParams &p, const Groups &gr, int member, int n)
+// Exchange of a block's statistics with its group: slots of data, and a counter of the blocks that have filled theirs.  Four of
+// each in turn: a block publishes unit n + 4 only after its pass 2 of unit n + 2, which waited until every block of the group
+// had published unit n + 2 and so was through with unit n.  The counters only grow during a launch (the first kernel of the event
+// clears them).  One lane waits for one word: a flag per block, or tags in the data themselves, cost more than the
+// counter's extra trips, because a warp's acquiring loads of many words are not pipelined (2048 units of 32768 tokens in
+// groups of 49 blocks: 3.47 ms with the counter, 5.84 with flags, 6.05 with tags).
+constexpr int kGroupCollectors = 2; // warps that read a group's slots
+template <typename T>
+__device__ __forceinline__ T *group_slot(const DevParams &p, const Groups &gr, int member, int n)
 {
-    return p.group_part + (size_t)((gr.id * gr.g + member) * 4 + (n & 3)) * kGroupSlot;
+    return reinterpret_cast<T *>(p.group_part + (size_t)((n & 3) * kGroupBlocks + gr.id * gr.g + member) * kGroupSlot);
 }
-// one lane, after the warp's stores to the slot and a __syncwarp
-__device__ __forceinline__ void group_publish(int *counter)
+__device__ __forceinline__ int *group_counter(const DevParams &p, const Groups &gr, int n) { return p.group_count + (gr.id * 4 + (n & 3)) * kGroupCounterPad; }
+// after the warp's stores to the block's slot
+__device__ __forceinline__ void group_publish(const DevParams &p, const Groups &gr, int n)
 {
-    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(counter) : "memory");
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(group_counter(p, gr, n)) : "memory");
 }
-// one lane, before the warp's reads of the group's slots; false when the wait ran out or another role gave up
-__device__ __forceinline__ bool group_wait(const int *counter, int want, volatile int *abort_flag)
+// before a warp's reads of the group's slots; false when the wait ran out or another role gave up
+__device__ __forceinline__ bool group_await(const DevParams &p, const Groups &gr, int n, volatile int *abort_flag)
 {
-    for (int i = 0; i < (1 << 21); ++i) {
-        int have;
-        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(have) : "l"(counter) : "memory");
-        if (have >= want) return true;
-        if ((i & 255) == 255 && *abort_flag) return false;
+    bool ok = true;
+    if ((threadIdx.x & 31) == 0) {
+        const int *counter = group_counter(p, gr, n);
+        const int want = (n / 4 + 1) * gr.g;
+        for (int i = 0;; ++i) {
+            int have;
+            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(have) : "l"(counter) : "memory");
+            if (have >= want) break;
+            if (i == (1 << 21)) *abort_flag = 1;
+            if ((i & 255) == 255 && *abort_flag) { ok = false; break; }
+        }
     }
-    *abort_flag = 1;
-    return false;
+    return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
 }
 // barrier over the first `threads` that arrive at it: true if `ok` holds in all
 __device__ __forceinline__ bool named_barrier_all(int id, int threads, bool ok)
@@ -133,11 +148,186 @@ __device__ __forceinline__ unsigned long long l2_done()
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
     return pol;
 }
-// Cooperative launch, one block per SM (fewer where the context does not have all of the device's SMs).
-template <typename... KArgs, typename... Args>
-inline cudaError_t launch_groups(void (*kernel)(KArgs...), int blocks, int threads, size_t smem, cudaStream_t s, Args... args)
+// ------------------------------------------------------------------ the stream of pages
+// kFeeders warps feed pages of 16 tokens by TMA to kWarps streaming warps, in turn and on across the ends of passes and
+// units, into a ring of kRing pages per warp.  Page number q of this walk (pass 1 of unit 0, pass 1 of unit 1, pass 2 of unit
+// 0, pass 1 of unit 2, ...) goes to streaming warp q % kWarps.
+constexpr int kPageBytes = kPage * kRowBytes;
+constexpr int kFeeders = 2;
+constexpr uint32_t kFeedLimit = 1u << 25;
+constexpr int kHeldIds = 128; // page ids of a unit that are fetched a unit ahead
+
+// A unit as the streaming warps need it
+struct GroupShare {
+    float *scores;     // of the block's first page
+    int tokens, pages; // of the sequence from there on; of the block's share, < 0: no more units
+};
+
+template <int kWarps, int kRing, int kUnits> // kUnits: units whose description is held
+struct GroupPipe {
+    unsigned char ring[kWarps * kRing * kPageBytes];              // first: aligned to 1024 bytes with the whole
+    GroupShare unit[kUnits];
+    int ids[kFeeders][2][kHeldIds];                               // page ids of a feeder's unit and the one before
+    unsigned long long full[kWarps * kRing], empty[kWarps * kRing]; // page is there; page is used
+    unsigned long long unit_full[kUnits], unit_empty[kUnits];       // unit is known; unit is done
+    unsigned long long summed[2], ready[2];                         // statistics of the warps are there; of the group
+    int abort_flag;
+};
+
+template <int kWarps, int kRing, int kUnits>
+__device__ __forceinline__ void pipe_init(GroupPipe<kWarps, kRing, kUnits> &pipe)
 {
-    for (;; blocks /= 2) {
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < kWarps * kRing; ++i) { tc::mbar_init(tc::smem_u32(&pipe.full[i]), 1); tc::mbar_init(tc::smem_u32(&pipe.empty[i]), 1); }
+        for (int i = 0; i < kUnits; ++i) { tc::mbar_init(tc::smem_u32(&pipe.unit_full[i]), 1); tc::mbar_init(tc::smem_u32(&pipe.unit_empty[i]), kWarps); }
+        for (int i = 0; i < 2; ++i) { tc::mbar_init(tc::smem_u32(&pipe.summed[i]), kWarps); tc::mbar_init(tc::smem_u32(&pipe.ready[i]), 1); }
+        pipe.abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+}
+
+// bounded, the same result in all lanes
+__device__ __forceinline__ bool warp_wait(const unsigned long long *bar, uint32_t parity, volatile int *abort_flag)
+{
+    return __all_sync(0xffffffffu, tc::mbar_wait(tc::smem_u32(bar), parity, abort_flag));
+}
+
+// A feeder warp.  announce(n, u) is called by one lane with each unit's description in place and completes unit_full[n % kUnits]'s
+// arrival.  A lane feeds one streaming warp throughout, so that the places of a ring are filled in turn by the same lane
+// and no wait for a place can be a round of the ring off.  False after a wait that ran out, with the copies on their
+// way landed.
+template <int kPasses, int kWarps, int kRing, int kUnits, typename Announce>
+__device__ __forceinline__ bool feed_pages(const DevParams &p, const Groups &gr, const CUtensorMap &k_map, GroupPipe<kWarps, kRing, kUnits> &pipe,
+                                           int feeder, Announce announce)
+{
+    constexpr int kShare = kWarps / kFeeders, kSlots = kWarps * kRing;
+    static_assert(kWarps % kFeeders == 0 && kShare <= 32, "a lane per streaming warp");
+    const int lane = threadIdx.x & 31;
+    const unsigned long long keep = l2_keep(), done = l2_done();
+    const uint32_t ring = tc::smem_u32(pipe.ring), full = tc::smem_u32(pipe.full), empty = tc::smem_u32(pipe.empty);
+    volatile int *abort_flag = &pipe.abort_flag;
+    const bool feeds = lane < kShare;
+    const int fed = feeder * kShare + (feeds ? lane : 0);
+    GroupWalk walk = group_walk(p, gr);
+    GroupUnit cur, old, nxt;
+    cur.pages = old.pages = 0;
+    unsigned at = 0; // walk number of the pass's first page
+    bool ok = true;
+    // page ids come a unit ahead, so that no copy waits for one
+    int ahead[kHeldIds / 32] = {};
+    auto fetch_ids = [&]() {
+#pragma unroll
+        for (int i = 0; i < kHeldIds / 32; ++i)
+            ahead[i] = lane + 32 * i < nxt.pages ? p.block_table[(size_t)nxt.b * p.bt_stride + nxt.first + lane + 32 * i] : 0;
+    };
+    bool more = next_group_unit(p, gr, walk, nxt);
+    if (more) fetch_ids();
+    int announced = 0;
+    for (int n = 0, last = 0; !last && ok; ++n) {
+        last = !more;
+        cur = nxt;
+        if (last) cur.pages = 0;
+#pragma unroll
+        for (int i = 0; i < kHeldIds / 32; ++i) pipe.ids[feeder][n & 1][lane + 32 * i] = ahead[i];
+        __syncwarp();
+        if (more) more = next_group_unit(p, gr, walk, nxt);
+        if (more) fetch_ids();
+        if (feeder == 0) {
+            ok = warp_wait(&pipe.unit_empty[n % kUnits], (uint32_t)(((n / kUnits) & 1) ^ 1), abort_flag);
+            if (!ok) break;
+            if (lane == 0) {
+                GroupShare &u = pipe.unit[n % kUnits];
+                u.pages = last ? -1 : cur.pages;
+                u.tokens = last ? 0 : cur.T - cur.first * kPage;
+                u.scores = !last ? p.scores + (size_t)((cur.l * p.B + cur.b) * p.H + cur.h) * p.T_cap + (size_t)cur.first * kPage : nullptr;
+                if (!last) announce(n, cur);
+                else tc::mbar_arrive(tc::smem_u32(&pipe.unit_full[n % kUnits]));
+            }
+            ++announced;
+            __syncwarp();
+        }
+#pragma unroll 1
+        for (int pass = 0; pass < kPasses && ok; ++pass) {
+            const GroupUnit u = pass ? old : cur;
+            const int *ids = pipe.ids[feeder][(n - pass) & 1];
+            const int layer = u.l * (int)p.num_pages;
+            for (int k0 = -(int)(at % kWarps); k0 < u.pages && ok; k0 += kWarps) {
+                const int k = k0 + fed;
+                const bool mine = feeds && k >= 0 && k < u.pages;
+                const int page = layer + (!mine ? 0 : k < kHeldIds ? ids[k] : p.block_table[(size_t)u.b * p.bt_stride + u.first + k]);
+                const unsigned q = at + k;
+                const int s = (int)(q % kSlots);
+                bool todo = mine;
+                for (uint32_t i = 0; ok; ++i) { // each page goes out as soon as its place is free
+                    if (todo && tc::mbar_test_wait(empty + 8 * s, ((q / kSlots) & 1) ^ 1)) {
+                        tc::mbar_expect_tx(full + 8 * s, kPageBytes);
+                        tc::tma_load_5d_policy(ring + s * kPageBytes, &k_map, full + 8 * s, 0, 0, 2 * u.h, 0, page, pass == kPasses - 1 ? done : keep);
+                        todo = false;
+                    }
+                    if (!__any_sync(0xffffffffu, todo)) break;
+                    if (i == kFeedLimit) *abort_flag = 1;
+                    if ((i & 1023u) == 1023u) ok = __all_sync(0xffffffffu, !*abort_flag);
+                }
+            }
+            at += u.pages;
+        }
+        old = cur;
+    }
+    if (!ok) {
+        for (int u = max(0, announced - kUnits); u < announced; ++u) // (a unit's description may come with a copy)
+            for (int i = 0; i < (1 << 16) && !tc::mbar_try_wait(tc::smem_u32(&pipe.unit_full[u % kUnits]), (u / kUnits) & 1); ++i) {}
+        for (int s = lane; s < kSlots; s += 32) {
+            // the last walk number of this place below `at` (its copy may not have been started: the wait is bounded)
+            if (at <= (unsigned)s) continue;
+            const unsigned turns = (at - 1 - s) / kSlots;
+            for (int i = 0; i < (1 << 16) && !tc::mbar_try_wait(full + 8 * s, turns & 1); ++i) {}
+        }
+    }
+    return ok;
+}
+
+// A streaming warp's place in the stream.
+template <int kWarps, int kRing, int kUnits>
+struct PipeReader {
+    GroupPipe<kWarps, kRing, kUnits> &pipe;
+    int warp, slot, turn; // place in the ring; pages from the start of the pass until the warp's next one
+    uint32_t phase;
+    __device__ __forceinline__ PipeReader(GroupPipe<kWarps, kRing, kUnits> &pipe_, int warp_) : pipe(pipe_), warp(warp_), slot(0), turn(warp_), phase(0) {}
+    __device__ __forceinline__ bool wait() { return warp_wait(&pipe.full[slot * kWarps + warp], phase, &pipe.abort_flag); }
+    // Matrix loads of the page: ldsm of chunk pair s (dimensions 16 s .. 16 s + 15), each lane from token 8 rows8 + lane % 8 and
+    // chunk 2 s + chunk.  Tokens in eights lie at 2048, halves of a row at 1024, a 16-byte chunk of a half at its
+    // number XOR the token, which leaves the loads free of bank conflicts.
+    __device__ __forceinline__ uint32_t at(int rows8) const
+    {
+        return tc::smem_u32(pipe.ring) + (slot * kWarps + warp) * kPageBytes + rows8 * 2048 + (threadIdx.x & 7) * 128;
+    }
+    static __device__ __forceinline__ uint32_t chunk(int s, int chunk) { return (s >> 2) * 1024 + (((2 * (s & 3) + chunk) ^ (threadIdx.x & 7)) << 4); }
+    __device__ __forceinline__ void release()
+    {
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) tc::mbar_arrive(tc::smem_u32(&pipe.empty[slot * kWarps + warp]));
+        if (++slot == kRing) { slot = 0; phase ^= 1; }
+    }
+};
+
+__device__ __forceinline__ void ldsm4(unsigned (&r)[4], unsigned addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+__device__ __forceinline__ void ldsm4_trans(unsigned (&r)[4], unsigned addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
+}
+
+// Cooperative launch, one block per SM (fewer, but not below `least`, where the context does not have all of the device's SMs).
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_groups(void (*kernel)(KArgs...), int least, int threads, size_t smem, cudaStream_t s, Args... args)
+{
+    int blocks = sm_count() < kGroupBlocks ? sm_count() : kGroupBlocks;
+    for (;; blocks = (blocks + 1) / 2) {
+        if (blocks < least || blocks < 1) return cudaErrorCooperativeLaunchTooLarge;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)blocks);
         cfg.blockDim = dim3((unsigned)threads);

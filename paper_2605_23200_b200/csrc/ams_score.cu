@@ -7,9 +7,7 @@
 // window.  Two phases over K: phase 1 finds each row's (max, sum of exponentials),
 // phase 2 recomputes the logits and sums the normalised probabilities over rows.
 // The largest probability of a row is 1/Z_r (its arg-max token), so the window
-// maximum is 1/min_r Z_r and needs no third pass.  With at most 16 (padded) query rows
-// phase 1 also stores the scaled logits (at most 64 bytes per token against the 256
-// bytes of its key), and phase 2 is a per-token kernel over those instead of K.
+// maximum is 1/min_r Z_r and needs no third pass.  Up to 32 rows: ams_score_window.cu; from 64: ams_score_tc.cu; the rest here.
 #include "ams_common.cuh"
 
 namespace ams {
@@ -138,175 +136,7 @@ struct TovaStream {
     }
 };
 
-// Narrow windows (8 or 16 padded rows).  The tile is the M operand of m16n8k16 and eight query rows are the N operand, both
-// read as 16-byte pieces along d: lane (g, tq) holds d = 32 j + 8 tq .. +7 of its rows, and those eight values feed k-steps
-// 2j and 2j+1.  The same assignment of d to k on both operands leaves the dot product unchanged.  Bound by the K
-// stream: 9.4 GB of K at 7 query rows 1.81 -> 1.67 ms with the asynchronous ring (logits included 6.2 TB/s).
-template <int NTB, int PHASE>
-__global__ void __launch_bounds__(kTovaThreads) k_tova(DevParams p)
-{
-    extern __shared__ __align__(16) unsigned char dyn[];
-    __shared__ float red[4][NTB * 8][2];
-    const unsigned smem = (unsigned)__cvta_generic_to_shared(dyn);
-    const unsigned Qb = smem + (kTovaThreads / 32) * kRing * kTileK;
-    wait_for_previous_kernel(); // effective lengths; merged statistics
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, tq = lane & 3;
-    const float c = kLog2e * 0.08838834764831845f; // log2(e) / sqrt(128)
-    const float inv_rows = 1.0f / (float)p.rows;
-    TovaStream<NTB * 8, PHASE> st(p, smem, Qb);
-    const int n_rb = st.n_rb;
-
-    TovaItem cur, nxt;
-    bool live = st.next(cur);
-    int qsel = 0;
-    st.fetch(cur, live, 0, 0);
-    st.fetch(cur, live, 1, 0);
-    while (live) {
-        const bool more = st.next(nxt);
-        int ahead = 0; // tiles of the next piece of work whose copy has been started
-        const int uid = cur.uid, T = cur.T, t_begin = cur.t_begin, t_end = cur.t_end, rb = cur.rb, row0 = rb * NTB * 8;
-        const float *fin = p.fin + (size_t)uid * (p.rows_pad + 8);
-        float *u_out = p.scores + (size_t)uid * p.T_cap;
-        float *lg = (PHASE == 1 && p.logits && n_rb == 1) ? p.logits + (size_t)uid * p.T_cap * (NTB * 8) : nullptr;
-        const float pmax = PHASE == 2 ? fin[p.rows_pad] : 0.0f;
-        cp_async_wait<1>(); // the queries and the first tile
-        __syncthreads();
-        uint4 zq[NTB][4];
-#pragma unroll
-        for (int nt = 0; nt < NTB; ++nt)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) zq[nt][j] = lds16(Qb + (qsel * NTB * 8 + nt * 8 + g) * kRowBytes + (((4 * j + tq) ^ ((g & 1) << 2)) << 4));
-        // per thread: rows (nt, e) = row0 + 8 nt + 2 tq + e
-        int lastv[NTB][2];
-        float st_a[NTB][2], st_b[NTB][2], st_m[NTB][2]; // phase 1: reference, sum of 2^(x - reference), largest unscaled
-                                                        // logit; phase 2: -b_r in the first
-#pragma unroll
-        for (int nt = 0; nt < NTB; ++nt)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int r = row0 + nt * 8 + 2 * tq + e;
-                lastv[nt][e] = r < p.rows ? (p.causal ? T - p.W + (r % p.W) : T - 1) : -1;
-                st_a[nt][e] = PHASE == 1 ? -1e30f : -fin[r];
-                st_b[nt][e] = 0.0f;
-                st_m[nt][e] = -INFINITY;
-            }
-
-        for (int kt = 0; kt < cur.mine; ++kt) {
-            uint4 x[4], y[4];
-            st.read(x, y);
-            if (kt + 2 < cur.mine) st.fetch(cur, true, kt + 2, qsel); // into the slot read in the round before
-            else { st.fetch(nxt, more, ahead, qsel ^ 1); ++ahead; }
-            const int t0 = t_begin + (warp + 4 * kt) * 16, ta = t0 + g, tb = t0 + g + 8;
-            // every row sees every token of the tile (padding rows are taken care of by their statistics or at the end)
-            const bool plain = t0 + 15 < t_end && t0 + 15 <= (p.causal ? T - p.W : T - 1);
-            float acc_a = 0.0f, acc_b = 0.0f;
-#pragma unroll
-            for (int nt = 0; nt < NTB; ++nt) {
-                float d[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    mma_bf16(d, x[j].x, y[j].x, x[j].y, y[j].y, zq[nt][j].x, zq[nt][j].y);
-                    mma_bf16(d, x[j].z, y[j].z, x[j].w, y[j].w, zq[nt][j].z, zq[nt][j].w);
-                }
-                if (!plain) { // pairs the window hides add nothing, now or (stored logits) later
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int lv = min(lastv[nt][e], t_end - 1);
-                        d[e] = ta <= lv ? d[e] : -INFINITY;
-                        d[2 + e] = tb <= lv ? d[2 + e] : -INFINITY;
-                    }
-                }
-                if (PHASE == 1) {
-                    // The sum's reference follows the largest logit at a distance of up to 2^32, so that rescaling is rare;
-                    // the sum is put on the maximum at the end.
-                    bool far = false;
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        st_m[nt][e] = fmaxf(st_m[nt][e], fmaxf(d[e], d[2 + e]));
-                        far |= fmaf(st_m[nt][e], c, -32.0f) > st_a[nt][e];
-                    }
-                    if (far) {
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const float mx = st_m[nt][e] * c;
-                            if (mx > st_a[nt][e]) { st_b[nt][e] *= ex2(st_a[nt][e] - mx); st_a[nt][e] = mx; }
-                        }
-                    }
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) st_b[nt][e] += ex2(fmaf(d[e], c, -st_a[nt][e])) + ex2(fmaf(d[2 + e], c, -st_a[nt][e]));
-                    if (lg) {
-                        if (ta < t_end) *reinterpret_cast<float2 *>(lg + (size_t)ta * (NTB * 8) + nt * 8 + 2 * tq) = make_float2(d[0] * c, d[1] * c);
-                        if (tb < t_end) *reinterpret_cast<float2 *>(lg + (size_t)tb * (NTB * 8) + nt * 8 + 2 * tq) = make_float2(d[2] * c, d[3] * c);
-                    }
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        acc_a += ex2(fmaf(d[e], c, st_a[nt][e]));
-                        acc_b += ex2(fmaf(d[2 + e], c, st_a[nt][e]));
-                    }
-                }
-            }
-            if (PHASE == 2) {
-                acc_a += __shfl_xor_sync(0xffffffffu, acc_a, 1);
-                acc_a += __shfl_xor_sync(0xffffffffu, acc_a, 2);
-                acc_b += __shfl_xor_sync(0xffffffffu, acc_b, 1);
-                acc_b += __shfl_xor_sync(0xffffffffu, acc_b, 2);
-                if (tq == 0) {
-#pragma unroll
-                    for (int e = 0; e < 2; ++e) {
-                        const int t = e ? tb : ta;
-                        if (t < t_end) {
-                            float v = e ? acc_b : acc_a;
-                            if (rb > 0) v += u_out[t];
-                            if (rb == n_rb - 1) {
-                                const int ninv = p.causal ? p.G * max(0, t - (T - p.W)) : 0;
-                                v = (v + (float)ninv * pmax) * inv_rows;
-                            }
-                            u_out[t] = v;
-                        }
-                    }
-                }
-            }
-        }
-        for (; ahead < 2; ++ahead) st.fetch(nxt, more, ahead, qsel ^ 1); // (fewer than two tiles for this warp)
-
-        if (PHASE == 1) {
-            // rows live in the quad index; fold the eight token groups, then the four warps
-#pragma unroll
-            for (int nt = 0; nt < NTB; ++nt)
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const float mx = st_m[nt][e] * c;
-                    st_b[nt][e] = mx > -INFINITY ? st_b[nt][e] * ex2(st_a[nt][e] - mx) : 0.0f;
-                    st_a[nt][e] = mx;
-#pragma unroll
-                    for (int o = 4; o < 32; o <<= 1) {
-                        const float m2 = __shfl_xor_sync(0xffffffffu, st_a[nt][e], o);
-                        const float z2 = __shfl_xor_sync(0xffffffffu, st_b[nt][e], o);
-                        lse_merge(st_a[nt][e], st_b[nt][e], m2, z2);
-                    }
-                    if (g == 0) {
-                        red[warp][nt * 8 + 2 * tq + e][0] = st_a[nt][e];
-                        red[warp][nt * 8 + 2 * tq + e][1] = st_b[nt][e];
-                    }
-                }
-            __syncthreads();
-            for (int r = threadIdx.x; r < NTB * 8; r += kTovaThreads) {
-                float m = red[0][r][0], z = red[0][r][1];
-#pragma unroll
-                for (int w = 1; w < 4; ++w) lse_merge(m, z, red[w][r][0], red[w][r][1]);
-                float2 *out = reinterpret_cast<float2 *>(p.part) + ((size_t)uid * p.n_slices + cur.slice) * p.rows_pad + row0 + r;
-                *out = make_float2(m, z);
-            }
-        }
-        cur = nxt;
-        live = more;
-        qsel ^= 1;
-    }
-    cp_async_wait<0>();
-}
-
-// Middle-sized windows (32 or 64 padded rows; blocks of 128 rows where the tcgen05 form does not apply): 16 query rows are the
+// Windows of 33 to 63 rows (blocks of 128 rows where the tcgen05 form does not apply): 16 query rows are the
 // M operand, the tile's tokens two N operands.  A token's piece of 16 bytes is then two consecutive registers per k-step,
 // as the instruction wants them (with the tile as M operand every k-step interleaves two rows' pieces: 380 of 546
 // instructions per tile were moves and their like), and a thread sees four logits of a row per tile.  The queries are laid
@@ -464,13 +294,6 @@ __global__ void __launch_bounds__(kTovaThreads) k_tova_wide(DevParams p)
     cp_async_wait<0>();
 }
 
-template <int NTB, int PHASE> // NTB: padded query rows / 8
-constexpr auto tova_kernel()
-{
-    if constexpr (NTB >= 4) return k_tova_wide<NTB / 2, PHASE>;
-    else return k_tova<NTB, PHASE>;
-}
-
 // Per unit: merge the slices' (max, sum) in slice order; b_r = M_r + log2 Z_r in the
 // base-2 domain, and the window maximum 1 / min_r Z_r.
 __global__ void __launch_bounds__(128) k_tova_combine(DevParams p)
@@ -501,80 +324,11 @@ __global__ void __launch_bounds__(128) k_tova_combine(DevParams p)
     if (threadIdx.x == 0) fin[p.rows_pad] = best;
 }
 
-// Usage pass over stored logits (RP = padded query rows, 8 or 16): one thread per token sums
-// 2^(x_r - b_r) over the rows; pairs the window hides were stored as -inf, padding rows have
-// b_r = +inf; the hidden pairs count as the window maximum.
-template <int RP>
-__global__ void __launch_bounds__(256) k_tova_usage_from_logits(DevParams p)
+template <int MT>
+int launch_tova_wide(const DevParams &p, LaunchCtx &ctx)
 {
-    __shared__ float bs[RP + 1], zinv[RP];
-    wait_for_previous_kernel(); // the slices' statistics and the logits
-    const int uid = blockIdx.x;
-    const int b = (uid / p.H) % p.B;
-    const int T = p.seq_lens[b];
-    if (T <= p.Tk || T > p.T_cap || p.W > T) return;
-    if (!p.merge_in_usage) {
-        const float *fin = p.fin + (size_t)uid * (p.rows_pad + 8);
-        if (threadIdx.x <= RP) bs[threadIdx.x] = fin[threadIdx.x]; // b_r of the rows, then the window maximum
-        __syncthreads();
-    } else {
-        // With few units (a launch-bound event) every block merges the slices' (max, sum) of its unit itself (a warp per
-        // row, a slice per lane, then a fixed tree over the lanes: the same result in every block): b_r = M_r + log2 Z_r,
-        // and the window maximum 1 / min_r Z_r.  With many units a kernel of its own does it once per unit.
-        const int ns = (T + p.slice_len - 1) / p.slice_len, lane = threadIdx.x & 31;
-        for (int r = threadIdx.x >> 5; r < RP; r += 8) {
-            float m = -INFINITY, z = 0.0f;
-            for (int sl = lane; sl < ns; sl += 32) {
-                const float2 v = __ldcg(reinterpret_cast<const float2 *>(p.part) + ((size_t)uid * p.n_slices + sl) * RP + r);
-                lse_merge(m, z, v.x, v.y);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float m2 = __shfl_xor_sync(0xffffffffu, m, o), z2 = __shfl_xor_sync(0xffffffffu, z, o);
-                lse_merge(m, z, m2, z2);
-            }
-            if (lane == 0) {
-                const bool live = r < p.rows && z > 0.0f;
-                bs[r] = live ? m + log2f(z) : INFINITY; // padding rows contribute nothing
-                zinv[r] = live ? 1.0f / z : 0.0f;
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float best = 0.0f;
-#pragma unroll
-            for (int r = 0; r < RP; ++r) best = fmaxf(best, zinv[r]);
-            bs[RP] = best;
-        }
-        __syncthreads();
-    }
-    // a block takes several tiles of 256 tokens (up to eight at large capacities), so that the statistics above are
-    // fetched once per 2048 tokens and a sequence far below the capacity costs few idle blocks
-    const int tiles = ((p.T_cap + 255) / 256 + gridDim.y - 1) / gridDim.y;
-    for (int tile = 0; tile < tiles; ++tile) {
-        const int t = (blockIdx.y * tiles + tile) * 256 + threadIdx.x;
-        if (t >= T) return;
-        const float4 *x = reinterpret_cast<const float4 *>(p.logits + ((size_t)uid * p.T_cap + t) * RP);
-        float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-        for (int q = 0; q < RP / 4; ++q) {
-            const float4 v = __ldcs(x + q);
-            acc[0] += ex2(v.x - bs[4 * q]);
-            acc[1] += ex2(v.y - bs[4 * q + 1]);
-            acc[2] += ex2(v.z - bs[4 * q + 2]);
-            acc[3] += ex2(v.w - bs[4 * q + 3]);
-        }
-        const int ninv = p.causal ? p.G * max(0, t - (T - p.W)) : 0;
-        p.scores[(size_t)uid * p.T_cap + t] = ((acc[0] + acc[1]) + (acc[2] + acc[3]) + (float)ninv * bs[RP]) * (1.0f / (float)p.rows);
-    }
-}
-
-template <int NTB>
-int launch_tova_ntb(const DevParams &p_in, LaunchCtx &ctx)
-{
-    DevParams p = p_in;
-    constexpr size_t smem = (size_t)(kTovaThreads / 32) * kRing * kTileK + (size_t)2 * NTB * 8 * kRowBytes;
-    const auto k1 = tova_kernel<NTB, 1>(), k2 = tova_kernel<NTB, 2>();
+    constexpr size_t smem = (size_t)(kTovaThreads / 32) * kRing * kTileK + (size_t)2 * MT * 16 * kRowBytes;
+    const auto k1 = k_tova_wide<MT, 1>, k2 = k_tova_wide<MT, 2>;
     static SmemGrant grant1, grant2;
     static int resident[2][kMaxDevices]; // blocks per SM
     const int dev = current_device(), n_sm = sm_count();
@@ -589,18 +343,9 @@ int launch_tova_ntb(const DevParams &p_in, LaunchCtx &ctx)
     };
     launch_after(k1, blocks(0), dim3(kTovaThreads), smem, ctx.s, p);
     ctx.mark(kKernScore1);
-    const bool from_logits = NTB <= 2 && p.logits && p.rows_pad == NTB * 8;
-    p.merge_in_usage = from_logits && units <= 2 * n_sm;
-    if (!p.merge_in_usage) {
-        launch_after(k_tova_combine, dim3((unsigned)units), dim3(128), 0, ctx.s, p);
-        ctx.mark(kKernScoreCombine);
-    }
-    if constexpr (NTB <= 2) if (from_logits) {
-        const int n256 = (p.T_cap + 255) / 256, per = n256 >= 128 ? 8 : (n256 >= 32 ? n256 / 16 : 1); // tiles per block
-        const dim3 g2((unsigned)units, (n256 + per - 1) / per);
-        launch_after(k_tova_usage_from_logits<NTB * 8>, g2, dim3(256), 0, ctx.s, p);
-    }
-    if (!from_logits) launch_after(k2, blocks(1), dim3(kTovaThreads), smem, ctx.s, p);
+    launch_after(k_tova_combine, dim3((unsigned)units), dim3(128), 0, ctx.s, p);
+    ctx.mark(kKernScoreCombine);
+    launch_after(k2, blocks(1), dim3(kTovaThreads), smem, ctx.s, p);
     ctx.mark(kKernScore2);
     return cudaGetLastError() == cudaSuccess ? AMS_OK : AMS_ERR_CUDA;
 }
@@ -617,13 +362,8 @@ int tova_rows_block(int rows)
 int launch_score_tova(const DevParams &p, LaunchCtx &ctx)
 {
     if (tova_tc_supported(p)) return launch_score_tova_tc(p, ctx);
-    switch (tova_rows_block(p.rows) / 8) {
-    case 1: return launch_tova_ntb<1>(p, ctx);
-    case 2: return launch_tova_ntb<2>(p, ctx);
-    case 4: return launch_tova_ntb<4>(p, ctx);
-    case 8: return launch_tova_ntb<8>(p, ctx);
-    default: return launch_tova_ntb<16>(p, ctx);
-    }
+    if (p.rows <= 32) return launch_score_window(p, ctx);
+    return tova_rows_block(p.rows) == 64 ? launch_tova_wide<4>(p, ctx) : launch_tova_wide<8>(p, ctx);
 }
 
 } // namespace ams

@@ -98,12 +98,12 @@ inline int make_k_map(const DevParams &p, EncodeTiledFn enc, CUtensorMap *map)
                ? AMS_OK : AMS_ERR_CUDA;
 }
 
-// Tensor map over `rows` contiguous 128-wide bf16 rows; a box is one 64-wide half of 128 rows.
-inline int make_rows_map(const void *ptr, unsigned long long rows, EncodeTiledFn enc, CUtensorMap *map)
+// Tensor map over `rows` contiguous 128-wide bf16 rows; a box is one 64-wide half of 128 rows (or of `box_rows`).
+inline int make_rows_map(const void *ptr, unsigned long long rows, EncodeTiledFn enc, CUtensorMap *map, int box_rows = 128)
 {
     const cuuint64_t dims[2] = {kHeadDim, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {kRowBytes};
-    const cuuint32_t box[2] = {64, 128};
+    const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
