@@ -24,35 +24,38 @@ struct Groups {
 
 // The split for the lengths of this call; the same in every block, computed by each warp for itself.  most_pages: of a unit that
 // a block can hold.
-__device__ __forceinline__ Groups split_groups(const DevParams &p, int warps, long long window, int most_pages)
+__device__ __forceinline__ Groups split_groups(const DevParams &p, int warps, float window, int most_pages)
 {
     const int lane = threadIdx.x & 31, nb = gridDim.x;
     int longest = 0, active = 0;
-    u64 total = 0;
+    float total = 0.0f;
     for (int b = lane; b < p.B; b += 32) {
         const int T = p.seq_lens[b];
-        if (T > p.Tk && T <= p.T_cap) { longest = max(longest, T); total += (u64)T; ++active; }
+        if (T > p.Tk && T <= p.T_cap) { longest = max(longest, T); total += (float)T; ++active; }
     }
     longest = __reduce_max_sync(0xffffffffu, longest);
     active = __reduce_add_sync(0xffffffffu, active);
-    total = warp_sum_u64(total);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
     const int units = active * p.L * p.H, pages = (longest + kPage - 1) / kPage;
     Groups r;
     r.g = 1; r.n = 0; r.id = 1; r.me = 0;
     if (units <= 0) return r;
-    const long long bytes = (long long)(total / active) * kRowBytes; // of a unit, on the average
+    const float fit = window * (float)active / (total * kRowBytes); // units in the window, of the average size
     // two groups at least, so that one reads while the other waits (K of 80000 tokens, 32 units: 222 -> 132 us; of 131072,
     // where two units no longer fit L2: 388 -> 324 us); no group without work; no fewer units in the last round than need be
-    int n = min(min(nb, units), (int)max(2ll, window / bytes));
+    int n = min(min(nb, units), (int)fmaxf(2.0f, fit));
     n = (units + (units + n - 1) / n - 1) / ((units + n - 1) / n);
     n = max(1, min(n, nb / ((pages + most_pages - 2) / (most_pages - 1)))); // no share above what a block can hold (its ends are rounded)
-    const int g = min(nb / n, (pages + warps - 1) / warps); // no warp without a page
+    int g = min(nb / n, (pages + warps - 1) / warps); // no warp without a page
+    if (p.group_size) g = p.group_size;
     r.g = g;
     r.n = min(nb / g, units);
     r.id = blockIdx.x / g;
     r.me = blockIdx.x % g;
-    r.from = (unsigned)(((unsigned long long)r.me << 32) / g);
-    r.to = (unsigned)(((unsigned long long)(r.me + 1) << 32) / g); // (0 for the last block: wraps)
+    const unsigned share = g > 1 ? 0xffffffffu / g + 1 : 0u;
+    r.from = r.me * share;
+    r.to = r.from + share; // (the last block takes what is left)
     r.dh = r.n % p.H;
     r.db = (r.n / p.H) % p.B;
     r.dl = r.n / (p.H * p.B);
@@ -177,13 +180,13 @@ struct GroupPipe {
 template <int kWarps, int kRing, int kUnits>
 __device__ __forceinline__ void pipe_init(GroupPipe<kWarps, kRing, kUnits> &pipe)
 {
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < kWarps * kRing; ++i) { tc::mbar_init(tc::smem_u32(&pipe.full[i]), 1); tc::mbar_init(tc::smem_u32(&pipe.empty[i]), 1); }
-        for (int i = 0; i < kUnits; ++i) { tc::mbar_init(tc::smem_u32(&pipe.unit_full[i]), 1); tc::mbar_init(tc::smem_u32(&pipe.unit_empty[i]), kWarps); }
-        for (int i = 0; i < 2; ++i) { tc::mbar_init(tc::smem_u32(&pipe.summed[i]), kWarps); tc::mbar_init(tc::smem_u32(&pipe.ready[i]), 1); }
-        pipe.abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
+    static_assert(kWarps * kRing <= 64, "a thread per barrier");
+    const int i = threadIdx.x;
+    if (i < kWarps * kRing) { tc::mbar_init(tc::smem_u32(&pipe.full[i]), 1); tc::mbar_init(tc::smem_u32(&pipe.empty[i]), 1); }
+    if (i < kUnits) { tc::mbar_init(tc::smem_u32(&pipe.unit_full[i]), 1); tc::mbar_init(tc::smem_u32(&pipe.unit_empty[i]), kWarps); }
+    if (i < 2) { tc::mbar_init(tc::smem_u32(&pipe.summed[i]), kWarps); tc::mbar_init(tc::smem_u32(&pipe.ready[i]), 1); }
+    if (i == 0) pipe.abort_flag = 0;
+    if (i < 64) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     __syncthreads();
 }
 
@@ -321,10 +324,34 @@ __device__ __forceinline__ void ldsm4_trans(unsigned (&r)[4], unsigned addr)
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
 }
 
-// Cooperative launch, one block per SM (fewer, but not below `least`, where the context does not have all of the device's SMs).
-template <typename... KArgs, typename... Args>
-inline cudaError_t launch_groups(void (*kernel)(KArgs...), int least, int threads, size_t smem, cudaStream_t s, Args... args)
+// Cooperative launch, one block per SM (fewer, but not below `least`, the blocks that can hold a unit, where the context does not have
+// all of the device's SMs).
+template <typename... Maps>
+inline cudaError_t launch_groups(void (*kernel)(DevParams, Maps...), int least, int threads, size_t smem, cudaStream_t s, DevParams p, Maps... maps)
 {
+    const long long units = (long long)p.L * p.B * p.H;
+    // The blocks of a cluster are resident together as well, and unlike a cooperative launch one of clusters comes in behind the kernel
+    // before it: few short units take a cluster each (one layer of 4096 tokens, event: 43.3 -> 41.1 us; 32 units of 4096 tokens at 32
+    // rows 66.6 -> 63.5).  16 units in clusters of eight no longer fit at once (56 -> 63 us).
+    const int cluster = units <= 8 && p.T_cap <= 8192 ? 8 : units <= 32 && p.T_cap <= 4096 ? 4 : 0;
+    if (cluster && least <= cluster) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(units * cluster));
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = cluster; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 2;
+        p.group_size = cluster;
+        if (cudaLaunchKernelEx(&cfg, kernel, p, maps...) == cudaSuccess) return cudaSuccess;
+        (void)cudaGetLastError();
+        p.group_size = 0;
+    }
     int blocks = sm_count() < kGroupBlocks ? sm_count() : kGroupBlocks;
     for (;; blocks = (blocks + 1) / 2) {
         if (blocks < least || blocks < 1) return cudaErrorCooperativeLaunchTooLarge;
@@ -338,7 +365,7 @@ inline cudaError_t launch_groups(void (*kernel)(KArgs...), int least, int thread
         attr[0].val.cooperative = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, p, maps...);
         if (e != cudaErrorCooperativeLaunchTooLarge || blocks == 1) return e;
         (void)cudaGetLastError();
     }

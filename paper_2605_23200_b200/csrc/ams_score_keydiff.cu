@@ -19,7 +19,7 @@ using namespace tc;
 
 constexpr int kKdWarps = 16, kKdRing = 3, kKdUnits = 4;
 // 512 units of 4096 tokens at 26 / 34 / 42 / 50 / 64 MB: 131 / 136 / 148 / 149 / 175 us
-constexpr long long kKdWindow = 26ll << 20;
+constexpr float kKdWindow = 26.0f * (1 << 20);
 constexpr int kKdThreads = (kKdWarps + kFeeders + kGroupCollectors) * 32;
 
 struct KdShared {
@@ -39,7 +39,9 @@ __global__ void __launch_bounds__(kKdThreads, 1) k_keydiff(DevParams p, const __
     KdShared &sh = *reinterpret_cast<KdShared *>(smem);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gq = lane >> 2, tq = lane & 3;
     volatile int *abort_flag = &sh.pipe.abort_flag;
+    if (threadIdx.x == 0) tma_prefetch_map(&k_map);
     pipe_init(sh.pipe);
+    wait_for_previous_kernel(); // effective lengths; the exchange's counters
     const Groups gr = split_groups(p, kKdWarps, kKdWindow, 1 << 20);
     if (gr.id >= gr.n) return;
     bool ok = true;

@@ -39,7 +39,7 @@ struct WideTraits {
     static constexpr int threads = (warps + kFeeders + kGroupCollectors) * 32;
 };
 // 2048 units of 1900 to 9001 tokens at 26 / 34 / 42 MB: 773 / 738 / 767 us
-constexpr long long kWideWindow = 34ll << 20;
+constexpr float kWideWindow = 34.0f * (1 << 20);
 
 struct WideShared {
     using T = WideTraits;
@@ -136,7 +136,9 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
     WideShared &sh = *reinterpret_cast<WideShared *>(smem);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, tq = lane & 3;
     volatile int *abort_flag = &sh.pipe.abort_flag;
+    if (threadIdx.x == 0) { tma_prefetch_map(&k_map); tma_prefetch_map(&q_map); }
     pipe_init(sh.pipe);
+    wait_for_previous_kernel(); // effective lengths; the exchange's counters
     const Groups gr = split_groups(p, kWarps, kWideWindow, 1 << 20);
     if (gr.id >= gr.n) return;
     bool ok = true;
@@ -347,7 +349,7 @@ struct OnceTraits {
     static constexpr int threads = (warps + kFeeders + kGroupCollectors) * 32;
 };
 // (no second read: as much as the places hold; 256 units of 20000 tokens at 36 / 44 MB: 249 / 225 us)
-constexpr long long kOnceWindow = 44ll << 20;
+constexpr float kOnceWindow = 44.0f * (1 << 20);
 
 template <int NB>
 struct OnceShared {
@@ -372,7 +374,9 @@ __global__ void __launch_bounds__(OnceTraits<NB>::threads, 1) k_window_once(DevP
     OnceShared<NB> &sh = *reinterpret_cast<OnceShared<NB> *>(smem);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, tq = lane & 3;
     volatile int *abort_flag = &sh.pipe.abort_flag;
+    if (threadIdx.x == 0) { tma_prefetch_map(&k_map); tma_prefetch_map(&q_map); }
     pipe_init(sh.pipe);
+    wait_for_previous_kernel(); // effective lengths; the exchange's counters
     const Groups gr = split_groups(p, kWarps, kOnceWindow, T::pages);
     if (gr.id >= gr.n) return;
     bool ok = true;
