@@ -6,7 +6,7 @@
 // hide the exchange, and pass 2 recomputes them with K from L2.  Before, 7 rows over 9.4 GB of K (1792 units of 8192 to
 // 32768 tokens) took 1.87 ms in three launches, with the logits through HBM, now 1.66 (5.7 TB/s, bound by the K stream and by
 // the spread of a group's blocks at each exchange); 16 rows, 256 units of 3000 tokens, 76 -> 49 us; 32 rows over 2.9 GB, with K
-// twice from HBM, 1.04 ms, now 0.74 (bound by the latency of a page in a warp: loads, eight dependent products, exponentials).
+// twice from HBM, 1.04 ms, now 0.77 (bound by the latency of a page in a warp: loads, eight dependent products, exponentials).
 #include "ams_common.cuh"
 #include "ams_groups.cuh"
 
@@ -38,7 +38,7 @@ struct WideTraits {
     static constexpr int warps = 12, ring = 3, units = 3;
     static constexpr int threads = (warps + kFeeders + kGroupCollectors) * 32;
 };
-// 2048 units of 1900 to 9001 tokens at 26 / 34 / 42 MB: 773 / 738 / 767 us
+// 2048 units of 1900 to 9001 tokens at 26 / 34 / 42 MB: 773 / 738 / 767 us (with other code around it; 769 at 34 as it is)
 constexpr float kWideWindow = 34.0f * (1 << 20);
 
 struct WideShared {
@@ -144,16 +144,7 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
     bool ok = true;
     if (warp < kWarps) {
         const float c = kLog2e * 0.08838834764831845f; // log2(e) / sqrt(128)
-        const float inv_rows = 1.0f / (float)p.rows;
         PipeReader<T::warps, T::ring, T::units> in(sh.pipe, warp);
-        int see[MT][E]; // row 16 mt + 8 e + g: the last token it sees, from the end of the sequence
-#pragma unroll
-        for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const int r = mt * 16 + 8 * e + g;
-                see[mt][e] = r < p.rows ? (p.causal ? (r % p.W) - p.W : -1) : -(1 << 30);
-            }
         unsigned q[MT][8][4];
         auto load_queries = [&](int n) {
             const uint32_t at = smem_u32(sh.q[n % T::units]) + (lane & 7) * 128;
@@ -181,14 +172,17 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
                 for (int i = 0; i < 4; ++i) da[mt][i] = db[mt][i] = 0.0f;
             const uint32_t at = in.at(lane >> 4);
 #pragma unroll
-            for (int s = 0; s < 8; ++s) {
-                unsigned k[4];
-                ldsm4(k, at + in.chunk(s, (lane >> 3) & 1));
+            for (int s = 0; s < 8; s += 2) {
+                unsigned k[2][4];
+                ldsm4(k[0], at + in.chunk(s, (lane >> 3) & 1));
+                ldsm4(k[1], at + in.chunk(s + 1, (lane >> 3) & 1));
 #pragma unroll
-                for (int mt = 0; mt < MT; ++mt) {
-                    mma_bf16(da[mt], q[mt][s][0], q[mt][s][1], q[mt][s][2], q[mt][s][3], k[0], k[1]);
-                    mma_bf16(db[mt], q[mt][s][0], q[mt][s][1], q[mt][s][2], q[mt][s][3], k[2], k[3]);
-                }
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int mt = 0; mt < MT; ++mt) {
+                        mma_bf16(da[mt], q[mt][s + i][0], q[mt][s + i][1], q[mt][s + i][2], q[mt][s + i][3], k[i][0], k[i][1]);
+                        mma_bf16(db[mt], q[mt][s + i][0], q[mt][s + i][1], q[mt][s + i][2], q[mt][s + i][3], k[i][2], k[i][3]);
+                    }
             }
         };
         // pairs the window hides add nothing
@@ -197,7 +191,8 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
             for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
-                    const int last = min(tokens + see[mt][e], tokens - 1) - t0 - 2 * tq;
+                    const int r = mt * 16 + 8 * e + g;
+                    const int last = (r < p.rows ? tokens - (p.causal ? p.W - r % p.W : 1) : -1) - t0 - 2 * tq; // that the row sees
 #pragma unroll
                     for (int i = 0; i < 2; ++i) {
                         if (i > last) da[mt][2 * e + i] = -INFINITY;
@@ -314,7 +309,7 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
                     const int t = t0 + (up ? 8 : 0) + 2 * tq + (odd ? 1 : 0);
                     if (!(lane & 4) && t < old.tokens) {
                         const int ninv = p.causal ? p.G * max(0, t - (old.tokens - p.W)) : 0;
-                        old.scores[t] = (v + (float)ninv * pmax) * inv_rows;
+                        old.scores[t] = (v + (float)ninv * pmax) * p.inv_rows;
                     }
                 }
                 if (!ok) break;
@@ -382,7 +377,6 @@ __global__ void __launch_bounds__(OnceTraits<NB>::threads, 1) k_window_once(DevP
     bool ok = true;
     if (warp < kWarps) {
         const float c = kLog2e * 0.08838834764831845f; // log2(e) / sqrt(128)
-        const float inv_rows = 1.0f / (float)p.rows;
         PipeReader<T::warps, T::ring, T::units> in(sh.pipe, warp);
         int see[NB][2]; // row 8 nb + 2 tq + e: the last token it sees, from the end of the sequence
 #pragma unroll
@@ -518,7 +512,7 @@ __global__ void __launch_bounds__(OnceTraits<NB>::threads, 1) k_window_once(DevP
                     const int t = k * kPage + g + (tq & 1 ? 8 : 0);
                     if (tq < 2 && t < old.tokens) {
                         const int ninv = p.causal ? p.G * max(0, t - (old.tokens - p.W)) : 0;
-                        old.scores[t] = (v + (float)ninv * pmax) * inv_rows;
+                        old.scores[t] = (v + (float)ninv * pmax) * p.inv_rows;
                     }
                 }
             }
@@ -540,6 +534,7 @@ template <int RP, typename Shared, typename Kernel>
 int launch_window(Kernel kernel, int least, int threads, const DevParams &p_in, LaunchCtx &ctx)
 {
     DevParams p = p_in;
+    p.inv_rows = 1.0f / (float)p.rows;
     p.group_count += kGroupCounters * kGroupCounterPad; // (the event's other launch of this kind scores keys)
     const EncodeTiledFn enc = encode_fn();
     if (!enc) return AMS_ERR_CUDA;
