@@ -72,9 +72,8 @@ NCU_TRAFFIC_BYTES: dict = {
     "cfg1_llama8b_L32_T16384_k2048_w32": {"score_phase1": 1_089_513_472 + 14_958_336,
                                           "score_phase2": 1_090_619_136 + 20_133_632,
                                           "gather": 270_614_528 + 219_303_168},
-    # one-layer capture x 4 resident layers (profiles/keydiff_cfg3_1layer_ncu_full.md)
-    "cfg3_qwen3_8b_L36_B64_T32768_k2048_keydiff": {"score_phase1": 4 * (4_295_511_552 + 7_466_752),
-                                                   "score_phase2": 4 * (4_296_070_144 + 16_274_688)},
+    # capture of one layer and half of the sequences x 8 (profiles/group_scorers_ncu.md)
+    "cfg3_qwen3_8b_L36_B64_T32768_k2048_keydiff": {"score_phase1": 8 * (2_159_701_504 + 37_753_856)},
     # four-layer capture x 8 (profiles/expected_attention_cfg5_4layers_ncu_full.md)
     "cfg5_llama8b_L32_T16384_k2048_expected": {"score_phase1": 8 * (138_547_456 + 6_842_624),
                                                "score_phase2": 8 * (142_662_656 + 4_295_936)},
@@ -240,7 +239,7 @@ class Bench:
 
 SCORER_NAMES = {0: "tova", 1: "keydiff", 2: "external", 3: "expected_attention"}
 SCORE_SLOTS = ("score_phase1", "score_combine", "score_phase2")
-SELECT_SLOTS = ("segment_select", "segments_quotas", "select_compact")
+SELECT_SLOTS = ("select_compact",)
 
 
 def roofline_of(wl, kern_ms, k_read, moved, lens, peaks, traffic=None):
