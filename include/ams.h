@@ -204,6 +204,11 @@ int ams_get_status(ams_state *st, void *stream, int32_t *detail);
  * out.  The next ams_get_status returns that code; nothing else is touched. */
 int ams_debug_expire_wait(ams_state *st, uint32_t polls, void *stream);
 
+/* The same inside an event: in the next ams_compress on this handle the scorer waits for something that never comes (an arrival
+ * from one block more than share the work, or a free place that nobody frees) and gives up after `polls` polls (1 .. 2^20).  A
+ * scorer without such waits runs as usual. */
+int ams_debug_expire_event(ams_state *st, uint32_t polls);
+
 /* Number of kernels the last ams_compress on this handle launched. */
 int32_t ams_last_launch_count(const ams_state *st);
 

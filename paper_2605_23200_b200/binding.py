@@ -25,7 +25,7 @@ AMS_SCORER_TOVA, AMS_SCORER_KEYDIFF, AMS_SCORER_EXTERNAL, AMS_SCORER_EXPECTED = 
 EXPORTS = ["ams_config_default", "ams_ema_state_bytes", "ams_workspace_bytes", "ams_segment_capacity",
            "ams_init_state", "ams_compress", "ams_get_status", "ams_last_launch_count", "ams_free",
            "ams_strerror", "ams_set_profiling", "ams_get_kernel_times", "ams_kernel_name", "ams_select_static",
-           "ams_select_static_status", "ams_debug_expire_wait", "ams_set_query_stats"]
+           "ams_select_static_status", "ams_debug_expire_wait", "ams_debug_expire_event", "ams_set_query_stats"]
 KERNEL_SLOTS = 10
 
 
@@ -89,6 +89,8 @@ def lib() -> ctypes.CDLL:
         L.ams_select_static_status.restype = ctypes.c_int
         L.ams_debug_expire_wait.argtypes = [ctypes.c_void_p, ctypes.c_uint32, ctypes.c_void_p]
         L.ams_debug_expire_wait.restype = ctypes.c_int
+        L.ams_debug_expire_event.argtypes = [ctypes.c_void_p, ctypes.c_uint32]
+        L.ams_debug_expire_event.restype = ctypes.c_int
         L.ams_set_query_stats.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_float]
         L.ams_set_query_stats.restype = ctypes.c_int
         L.ams_strerror.argtypes = [ctypes.c_int]
@@ -221,6 +223,12 @@ class AmsCompressor:
         rc = lib().ams_debug_expire_wait(self._h, polls, ctypes.c_void_p(s.cuda_stream))
         if rc != AMS_OK:
             raise AmsError(rc, "ams_debug_expire_wait")
+
+    def expire_event(self, polls: int = 1000) -> None:
+        """Failure-handling check: a wait inside the next event's scorer runs out after `polls` polls."""
+        rc = lib().ams_debug_expire_event(self._h, polls)
+        if rc != AMS_OK:
+            raise AmsError(rc, "ams_debug_expire_event")
 
     def set_profiling(self, enable: bool) -> None:
         rc = lib().ams_set_profiling(self._h, 1 if enable else 0)

@@ -119,6 +119,7 @@ struct ams_state {
     const float *q_mean; // query statistics of the expected-attention scorer (ams_set_query_stats)
     const void *q_cov;
     float score_eps;
+    uint32_t expire_polls; // of the next event (ams_debug_expire_event)
     bool profiling;
     int n_ev;
     int ev_ids[32];
@@ -197,6 +198,7 @@ int ams_init_state(const ams_config *cfg, void *ema_state, void *workspace, size
     st->q_mean = nullptr;
     st->q_cov = nullptr;
     st->score_eps = 0.0f;
+    st->expire_polls = 0;
     st->profiling = false;
     st->n_ev = 0;
     *out = st;
@@ -268,6 +270,8 @@ int ams_compress(ams_state *st, void *k_pages, void *v_pages, int64_t num_pages,
     p.tc_stages = p.rows_pad <= 256 ? 4 : 2; // even: each stage then belongs to one of the two MMA issuers
     p.status = (int *)(st->ws + y.status);
     p.q_mean = st->q_mean; p.q_cov = (const __nv_bfloat16 *)st->q_cov; p.score_eps = st->score_eps;
+    p.expire_polls = st->expire_polls;
+    st->expire_polls = 0;
     p.ex_logits = c.expected_scorer ? (float *)(st->ws + y.ex_logits) : nullptr;
 
     int rc = AMS_OK;
@@ -341,6 +345,13 @@ int ams_debug_expire_wait(ams_state *st, uint32_t polls, void *stream)
 {
     if (!st || polls < 1 || polls > (1u << 20)) return AMS_ERR_INVALID_ARG;
     return launch_expire_wait((int *)(st->ws + st->lay.status), polls, (cudaStream_t)stream);
+}
+
+int ams_debug_expire_event(ams_state *st, uint32_t polls)
+{
+    if (!st || polls < 1 || polls > (1u << 20)) return AMS_ERR_INVALID_ARG;
+    st->expire_polls = polls;
+    return AMS_OK;
 }
 
 int32_t ams_last_launch_count(const ams_state *st) { return st ? st->last_launches : 0; }

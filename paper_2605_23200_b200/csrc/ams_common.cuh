@@ -69,6 +69,8 @@ struct DevParams {
     unsigned char *group_part;        // and the slots of what they exchange
     int *seq_bad;                     // [B]: set when a unit of the sequence reported a device-side error (its rows stay)
     int *status;                      // [4]: code, unit, a, b
+    uint32_t expire_polls;            // test hook: a wait of this event's scorer is for something that never comes, and gives up
+                                      // after so many polls (0: off)
 };
 
 __device__ __forceinline__ void set_status(int *status, int code, int unit, int a, int b)

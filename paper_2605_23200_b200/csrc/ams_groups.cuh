@@ -118,12 +118,12 @@ __device__ __forceinline__ bool group_await(const DevParams &p, const Groups &gr
     bool ok = true;
     if ((threadIdx.x & 31) == 0) {
         const int *counter = group_counter(p, gr, n);
-        const int want = (n / 4 + 1) * gr.g;
+        const int want = (n / 4 + 1) * gr.g + (p.expire_polls ? 1 : 0), limit = p.expire_polls ? (int)p.expire_polls : 1 << 21;
         for (int i = 0;; ++i) {
             int have;
             asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(have) : "l"(counter) : "memory");
             if (have >= want) break;
-            if (i == (1 << 21)) *abort_flag = 1;
+            if (i == limit) *abort_flag = 1;
             if ((i & 255) == 255 && *abort_flag) { ok = false; break; }
         }
     }
@@ -216,6 +216,7 @@ __device__ __forceinline__ bool feed_pages(const DevParams &p, const Groups &gr,
     GroupUnit cur, old, nxt;
     cur.pages = old.pages = 0;
     unsigned at = 0; // walk number of the pass's first page
+    int sent = 0;    // copies that this lane has started: all the pages of its streaming warp, in turn
     bool ok = true;
     // page ids come a unit ahead, so that no copy waits for one
     int ahead[kHeldIds / 32] = {};
@@ -267,6 +268,7 @@ __device__ __forceinline__ bool feed_pages(const DevParams &p, const Groups &gr,
                         tc::mbar_expect_tx(full + 8 * s, kPageBytes);
                         tc::tma_load_5d_policy(ring + s * kPageBytes, &k_map, full + 8 * s, 0, 0, 2 * u.h, 0, page, pass == kPasses - 1 ? done : keep);
                         todo = false;
+                        ++sent;
                     }
                     if (!__any_sync(0xffffffffu, todo)) break;
                     if (i == kFeedLimit) *abort_flag = 1;
@@ -280,12 +282,8 @@ __device__ __forceinline__ bool feed_pages(const DevParams &p, const Groups &gr,
     if (!ok) {
         for (int u = max(0, announced - kUnits); u < announced; ++u) // (a unit's description may come with a copy)
             for (int i = 0; i < (1 << 16) && !tc::mbar_try_wait(tc::smem_u32(&pipe.unit_full[u % kUnits]), (u / kUnits) & 1); ++i) {}
-        for (int s = lane; s < kSlots; s += 32) {
-            // the last walk number of this place below `at` (its copy may not have been started: the wait is bounded)
-            if (at <= (unsigned)s) continue;
-            const unsigned turns = (at - 1 - s) / kSlots;
-            for (int i = 0; i < (1 << 16) && !tc::mbar_try_wait(full + 8 * s, turns & 1); ++i) {}
-        }
+        for (int k = max(0, sent - kRing); k < sent; ++k) // (by what was started: a wait for a turn that was not would pass at once)
+            for (int i = 0; i < (1 << 16) && !tc::mbar_try_wait(full + 8 * (k % kRing * kWarps + fed), (k / kRing) & 1); ++i) {}
     }
     return ok;
 }

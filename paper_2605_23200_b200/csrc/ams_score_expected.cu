@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_expected_tc(DevParams p, cons
     if (tiles_lh > 0 && g_begin < g_end) {
         if (warp == 0) {
             // ------------------------------------------------------------ TMA producer
-            int kit = 0, seg = 0, issued = 0;
+            int kit = 0, seg = 0, issued = 0, blocks_issued = 0;
             bool ok = true;
             for (long long gv = 0; gv < g_span * hpb && ok;) {
                 const int my_h = my_h0 + (int)(gv / g_span) * my_hs;
@@ -112,11 +112,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_expected_tc(DevParams p, cons
                             tma_load_2d(smem_u32(Cs + (size_t)rb * kTileBytes + hf * kHalfBytes), &c_map, smem_u32(&sh.cfull),
                                         hf * 64, crow0 + rb * kHeadDim);
                 }
+                blocks_issued = seg + 1;
                 const int *table = p.block_table + (size_t)s.b * p.bt_stride;
                 const int last_page = (s.T - 1) >> 4;
                 for (int i = 0; i < s.n && ok; ++i, ++kit) {
                     const int st = kit % NS;
-                    ok = mbar_wait(smem_u32(&sh.kempty[st]), (uint32_t)(((kit / NS) & 1) ^ 1), abort_flag);
+                    ok = mbar_wait(smem_u32(&sh.kempty[st]), (uint32_t)(((kit / NS) & 1) ^ (p.expire_polls ? 0 : 1)), abort_flag,
+                                   p.expire_polls ? p.expire_polls : kWaitLimit);
                     if (!ok) break;
                     if (lane == 0) mbar_expect_tx(smem_u32(&sh.kfull[st]), (uint32_t)kTileBytes);
                     __syncwarp();
@@ -137,6 +139,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_expected_tc(DevParams p, cons
                     for (uint32_t i = 0; i < kWaitLimit; ++i)
                         if (mbar_try_wait(smem_u32(&sh.kfull[k % NS]), (uint32_t)((k / NS) & 1))) break;
                 }
+                for (uint32_t i = 0; blocks_issued && i < kWaitLimit; ++i)
+                    if (mbar_try_wait(smem_u32(&sh.cfull), (uint32_t)((blocks_issued - 1) & 1))) break;
             }
         } else if (warp == 1 || warp == 3) {
             // ------------------------------------------------------------ MMA issuers (two heads of every tile each)

@@ -1,0 +1,50 @@
+"""A wait inside a scorer that runs out: every role of every block returns with its copies landed, the event reports AMS_ERR_TIMEOUT,
+and the next event on the handle is exact.  The wait is made to run out by construction (for an arrival that nobody makes)."""
+import pytest
+import torch
+
+from helpers import HostSnapshot, compare_event, gpu_event
+from paper_2605_23200_b200 import binding, inputs
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+CASES = [
+    dict(cfg=3, n_layers=1, batch=1, seq_len_min=4096, seq_len_max=4096),                                          # key-only, a cluster per unit
+    dict(cfg=3, n_layers=3, batch=4, seq_len_min=9000, seq_len_max=9001),                                          # key-only, groups over the whole device
+    dict(cfg=2, n_q_heads=32, n_kv_heads=8, window=1, n_layers=1, batch=1, seq_len_min=4096, seq_len_max=4096),    # 4 rows, a cluster per unit
+    dict(cfg=2, n_q_heads=28, n_kv_heads=4, window=1, n_layers=2, batch=5, seq_len_min=3000, seq_len_max=9001),    # 7 rows, whole device
+    dict(cfg=2, n_q_heads=28, n_kv_heads=4, window=2, n_layers=2, batch=5, seq_len_min=3000, seq_len_max=9001),    # 14 rows
+    dict(cfg=2, n_q_heads=32, n_kv_heads=8, window=8, n_layers=2, batch=3, seq_len_min=3000, seq_len_max=9001),    # 32 rows
+    dict(cfg=2, n_q_heads=32, n_kv_heads=8, window=32, n_layers=2, batch=2, seq_len_min=3000, seq_len_max=5000),   # 128 rows
+    dict(cfg=1, n_q_heads=32, n_kv_heads=8, window=0, n_layers=2, batch=2, seq_len_min=3000, seq_len_max=5000, scorer_id=inputs.SCORER_EXPECTED),
+]
+
+
+@pytest.mark.parametrize("polls", [1, 300])
+@pytest.mark.parametrize("kw", CASES)
+def test_a_wait_that_runs_out_inside_a_scorer(kw, polls):
+    kw = dict(kw)
+    wl = inputs.CONFIGS[kw.pop("cfg")].scaled(budget=512, resident_layers=0, **kw)
+    cache = inputs.make_cache(wl, DEV)
+    comp = binding.AmsCompressor(binding.config_for(wl), DEV)
+    if wl.scorer_id == inputs.SCORER_EXPECTED:
+        mean, cov = inputs.make_query_stats(cache)
+        comp.set_query_stats(mean, cov, 1e-2)
+    comp.ema_state.uniform_(0.0, 1e-3)
+    dst = inputs.alloc_dst_pages(cache)
+    own = [cache.k_pages, cache.v_pages, cache.block_table, cache.seq_lens, comp.ema_state]
+    before = [t.clone() for t in own]
+    comp.expire_event(polls)
+    comp.compress(cache.k_pages, cache.v_pages, cache.block_table, cache.seq_lens, cache.obs_queries if wl.window else None, wl.budget,
+                  wl.n_segments, wl.scorer_id, torch.from_numpy(dst).to(DEV))
+    assert comp.status(check=False)[0] == binding.AMS_ERR_TIMEOUT
+    for t, b in zip(own, before):
+        t.copy_(b)
+    snap = HostSnapshot(cache)
+    credit0 = comp.ema_state.cpu().numpy()
+    dbg = gpu_event(comp, cache, dst)
+    units = [(l, b, h) for l in {0, wl.n_layers - 1} for b in {0, wl.batch - 1} for h in {0, wl.n_kv_heads - 1}]
+    compare_event(snap, cache, comp, dbg, dst, credit0, dbg.scores.cpu().numpy(), units=units)
+    with pytest.raises(binding.AmsError):
+        comp.expire_event(0)
