@@ -127,6 +127,7 @@ __device__ __forceinline__ bool group_await(const DevParams &p, const Groups &gr
             if ((i & 255) == 255 && *abort_flag) { ok = false; break; }
         }
     }
+    __syncwarp(); // (a shuffle orders no memory: this makes the acquire one of the other lanes' reads too)
     return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
 }
 // barrier over the first `threads` that arrive at it: true if `ok` holds in all
