@@ -96,7 +96,7 @@ __device__ __forceinline__ bool next_group_unit(const DevParams &p, const Groups
 // Exchange of a block's statistics with its group: slots of data, and a counter of the blocks that have filled theirs.  Four of
 // each in turn: a block publishes unit n + 4 only after its pass 2 of unit n + 2, which waited until every block of the group
 // had published unit n + 2 and so was through with unit n.  The counters only grow during a launch (the first kernel of the event
-// clears them).  One lane waits for one word: a flag per block, or tags in the data themselves, cost more than the
+// clears them).  A warp waits for one word: a flag per block, or tags in the data themselves, cost more than the
 // counter's extra trips, because a warp's acquiring loads of many words are not pipelined (2048 units of 32768 tokens in
 // groups of 49 blocks: 3.47 ms with the counter, 5.84 with flags, 6.05 with tags).
 constexpr int kGroupCollectors = 2; // warps that read a group's slots
@@ -112,23 +112,20 @@ __device__ __forceinline__ void group_publish(const DevParams &p, const Groups &
     __syncwarp();
     if ((threadIdx.x & 31) == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(group_counter(p, gr, n)) : "memory");
 }
-// before a warp's reads of the group's slots; false when the wait ran out or another role gave up
+// before a warp's reads of the group's slots; false when the wait ran out or another role gave up.  All lanes load the one word, a
+// single request: each has then acquired what it reads next.  (One lane for all needs a __syncwarp to pass its acquire on and is
+// slower: 1792 units of 8192 to 32768 tokens at 16 rows, event 3531 us, this 3499; 2048 units of 6400 tokens, key scores, 1124 and 1109.)
 __device__ __forceinline__ bool group_await(const DevParams &p, const Groups &gr, int n, volatile int *abort_flag)
 {
-    bool ok = true;
-    if ((threadIdx.x & 31) == 0) {
-        const int *counter = group_counter(p, gr, n);
-        const int want = (n / 4 + 1) * gr.g + (p.expire_polls ? 1 : 0), limit = p.expire_polls ? (int)p.expire_polls : 1 << 21;
-        for (int i = 0;; ++i) {
-            int have;
-            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(have) : "l"(counter) : "memory");
-            if (have >= want) break;
-            if (i == limit) *abort_flag = 1;
-            if ((i & 255) == 255 && *abort_flag) { ok = false; break; }
-        }
+    const int *counter = group_counter(p, gr, n);
+    const int want = (n / 4 + 1) * gr.g + (p.expire_polls ? 1 : 0), limit = p.expire_polls ? (int)p.expire_polls : 1 << 21;
+    for (int i = 0;; ++i) {
+        int have;
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(have) : "l"(counter) : "memory");
+        if (__all_sync(0xffffffffu, have >= want)) return true;
+        if (i == limit) *abort_flag = 1;
+        if ((i & 255) == 255 && __any_sync(0xffffffffu, *abort_flag)) return false;
     }
-    __syncwarp(); // (a shuffle orders no memory: this makes the acquire one of the other lanes' reads too)
-    return __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
 }
 // barrier over the first `threads` that arrive at it: true if `ok` holds in all
 __device__ __forceinline__ bool named_barrier_all(int id, int threads, bool ok)
