@@ -47,7 +47,8 @@
  * one whose block-table row or replacement pages name a page outside [0, num_pages)
  * (AMS_ERR_INVALID_ARG, detail = sequence, index in the row, page id) is skipped
  * entirely: its pages, table row, length and credit stay as they were.  A bounded
- * wait that ran out is AMS_ERR_TIMEOUT.  The library serves any number of devices
+ * wait that ran out is AMS_ERR_TIMEOUT; the scores are then incomplete, and no sequence
+ * of the event is compressed: all pages, table rows, lengths and credit stay as they were.  The library serves any number of devices
  * per process (launch state is kept per device); a handle belongs to the device that
  * was current when it was created.
  */

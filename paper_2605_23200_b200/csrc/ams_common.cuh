@@ -67,7 +67,8 @@ struct DevParams {
     int group_size;                   // blocks that work on a unit together: their number if the launcher sets it (a cluster);
     int *group_count;                 // counters, cleared by the first kernel of an event,
     unsigned char *group_part;        // and the slots of what they exchange
-    int *seq_bad;                     // [B]: set when a unit of the sequence reported a device-side error (its rows stay)
+    int *seq_bad;                     // [B]: set when a unit of the sequence, or for all of them a scorer, reported a device-side
+                                      // error: what follows leaves the sequence as it is
     int *status;                      // [4]: code, unit, a, b
     uint32_t expire_polls;            // test hook: a wait of this event's scorer is for something that never comes, and gives up
                                       // after so many polls (0: off)
@@ -80,6 +81,13 @@ __device__ __forceinline__ void set_status(int *status, int code, int unit, int 
         status[2] = a;
         status[3] = b;
     }
+}
+
+// A wait of a scorer ran out: its scores are not all there, so the later kernels leave every sequence of the event alone.
+__device__ __forceinline__ void report_timeout(const DevParams &p, int a, int b)
+{
+    set_status(p.status, AMS_ERR_TIMEOUT, blockIdx.x, a, b);
+    for (int i = 0; i < p.B; ++i) p.seq_bad[i] = 1;
 }
 
 __device__ __forceinline__ int seq_len_of(const DevParams &p, int b) { return p.seq_lens ? p.seq_lens[b] : p.fixed_len; }

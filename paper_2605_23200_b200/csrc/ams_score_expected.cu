@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_expected_tc(DevParams p, cons
             }
         }
     }
-    if (*abort_flag && tid == 0) set_status(p.status, AMS_ERR_TIMEOUT, blockIdx.x, 3, 0);
+    if (*abort_flag && tid == 0) report_timeout(p, 3, 0);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();

@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kKdThreads, 1) k_keydiff(DevParams p, const __
             }
         }
     }
-    if (!ok && lane == 0) set_status(p.status, AMS_ERR_TIMEOUT, blockIdx.x, 4, 0);
+    if (!ok && lane == 0) report_timeout(p, 4, 0);
 }
 
 } // namespace

@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
             }
         }
     }
-    if (*abort_flag && tid == 0) set_status(p.status, AMS_ERR_TIMEOUT, blockIdx.x, PHASE, 0);
+    if (*abort_flag && tid == 0) report_timeout(p, PHASE, 0);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();

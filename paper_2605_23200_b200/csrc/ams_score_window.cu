@@ -326,7 +326,7 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
     } else {
         ok = exchange_stats<RP, kWarps>(p, gr, sh, warp - kWarps - kFeeders);
     }
-    if (!ok && lane == 0) set_status(p.status, AMS_ERR_TIMEOUT, blockIdx.x, 5, 0);
+    if (!ok && lane == 0) report_timeout(p, 5, 0);
 }
 
 // Up to sixteen query rows: a page's logits are an eighth or a quarter of its keys, so they stay in shared memory until the unit's
@@ -527,7 +527,7 @@ __global__ void __launch_bounds__(OnceTraits<NB>::threads, 1) k_window_once(DevP
     } else {
         ok = exchange_stats<T::rows, kWarps>(p, gr, sh, warp - kWarps - kFeeders);
     }
-    if (!ok && lane == 0) set_status(p.status, AMS_ERR_TIMEOUT, blockIdx.x, 5, 0);
+    if (!ok && lane == 0) report_timeout(p, 5, 0);
 }
 
 template <int RP, typename Shared, typename Kernel>

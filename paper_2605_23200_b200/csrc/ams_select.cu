@@ -1085,6 +1085,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
     wait_for_previous_kernel(); // scores, effective lengths
     const int T = seq_len_of(p, bq);
     if (T <= p.Tk || T > p.T_cap) return;
+    if (p.seq_lens && p.seq_bad[bq]) return; // no scores to go by (the allocation-free entry point has no scorer and keeps its flags)
     const int sc = p.seg_cap;
     const SelSmem mp = sel_smem<NT>(p.T_cap, sc, p.S, longs != 0);
     unsigned *mask = reinterpret_cast<unsigned *>(dyn + mp.mask);

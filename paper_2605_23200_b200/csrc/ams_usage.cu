@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(128) k_retained_iou(DevParams p, const int *pr
     if (uid >= p.L * p.B * p.H) return;
     const int b = (uid / p.H) % p.B;
     const int T = p.seq_lens[b];
-    if (T <= p.Tk || T > p.T_cap) return;
+    if (T <= p.Tk || T > p.T_cap || p.seq_bad[b]) return;
     const int prev = max(0, min(prev_kept[b], T));
     const int *keep = p.keep_idx + (size_t)uid * p.Tk;
     int lo = 0, hi = p.Tk; // first kept position that is not below prev
@@ -68,13 +68,13 @@ __global__ void __launch_bounds__(256) k_inspect_scores(DevParams p, ams_debug_v
 }
 
 // Inspection views of the selection, one block per unit: segments, quotas and kept positions go to the caller's arrays in
-// one launch.  Units that were skipped are left untouched.
+// one launch.  Units that were skipped or reported are left untouched.
 __global__ void __launch_bounds__(256) k_inspect(DevParams p, ams_debug_views v)
 {
     wait_for_previous_kernel(); // the selection
-    const int uid = blockIdx.x, tid = threadIdx.x;
-    const int T = p.seq_lens[(uid / p.H) % p.B];
-    if (T <= p.Tk || T > p.T_cap) return;
+    const int uid = blockIdx.x, tid = threadIdx.x, b = (uid / p.H) % p.B;
+    const int T = p.seq_lens[b];
+    if (T <= p.Tk || T > p.T_cap || p.seq_bad[b]) return;
     const int n = p.n_seg[uid];
     const size_t sc = (size_t)p.seg_cap, u = (size_t)uid;
     if (v.n_segments && tid == 0) v.n_segments[uid] = n;

@@ -1,5 +1,5 @@
-"""A wait inside a scorer that runs out: every role of every block returns with its copies landed, the event reports AMS_ERR_TIMEOUT,
-and the next event on the handle is exact.  The wait is made to run out by construction (for an arrival that nobody makes)."""
+"""A wait inside a scorer that runs out: every role of every block returns with its copies landed, the event reports AMS_ERR_TIMEOUT
+and leaves pages, table, lengths and credit alone, and the next event on the handle is exact.  The wait is made to run out by construction (for an arrival that nobody makes)."""
 import pytest
 import torch
 
@@ -35,12 +35,17 @@ def test_a_wait_that_runs_out_inside_a_scorer(kw, polls):
     dst = inputs.alloc_dst_pages(cache)
     own = [cache.k_pages, cache.v_pages, cache.block_table, cache.seq_lens, comp.ema_state]
     before = [t.clone() for t in own]
+    views = comp.make_debug_views(wl.batch, wl.budget)
+    views.prev_kept = torch.full((wl.batch,), 64, dtype=torch.int32, device=DEV)
+    views.retained_iou = iou = torch.zeros((wl.n_layers, wl.batch, wl.n_kv_heads), device=DEV)
     comp.expire_event(polls)
     comp.compress(cache.k_pages, cache.v_pages, cache.block_table, cache.seq_lens, cache.obs_queries if wl.window else None, wl.budget,
-                  wl.n_segments, wl.scorer_id, torch.from_numpy(dst).to(DEV))
+                  wl.n_segments, wl.scorer_id, torch.from_numpy(dst).to(DEV), dbg=views)
     assert comp.status(check=False)[0] == binding.AMS_ERR_TIMEOUT
     for t, b in zip(own, before):
-        t.copy_(b)
+        raw = torch.int16 if t.element_size() == 2 else torch.int32
+        assert torch.equal(t.view(raw), b.view(raw))
+    assert not bool(views.keep_idx.any()) and not bool(views.n_segments.any()) and not bool(iou.any())
     snap = HostSnapshot(cache)
     credit0 = comp.ema_state.cpu().numpy()
     dbg = gpu_event(comp, cache, dst)
