@@ -19,7 +19,10 @@ struct Groups {
     int g, n;    // blocks per group, groups
     int id, me;  // this block's group (>= n: none) and its place in it
     unsigned from, to; // the block's share of a unit's pages, in 2^-32
-    int dh, db, dl;    // n as a number of heads, sequences and layers: the step from a unit of the group to the next
+    bool all;          // every sequence has something to evict
+    int T;             // length of the lane's sequence, of the first 32
+    int dh, db, dl;    // n as a number of heads, sequences with something to evict and layers: the step from a unit of the group to
+                       // the next
 };
 
 // The split for the lengths of this call; the same in every block, computed by each warp for itself.  most_pages: of a unit that
@@ -29,8 +32,11 @@ __device__ __forceinline__ Groups split_groups(const DevParams &p, int warps, fl
     const int lane = threadIdx.x & 31, nb = gridDim.x;
     int longest = 0, active = 0;
     float total = 0.0f;
+    Groups r;
+    r.T = 0;
     for (int b = lane; b < p.B; b += 32) {
         const int T = p.seq_lens[b];
+        if (b == lane) r.T = T;
         if (T > p.Tk && T <= p.T_cap) { longest = max(longest, T); total += (float)T; ++active; }
     }
     longest = __reduce_max_sync(0xffffffffu, longest);
@@ -38,7 +44,6 @@ __device__ __forceinline__ Groups split_groups(const DevParams &p, int warps, fl
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
     const int units = active * p.L * p.H, pages = (longest + kPage - 1) / kPage;
-    Groups r;
     r.g = 1; r.n = 0; r.id = 1; r.me = 0;
     if (units <= 0) return r;
     const float fit = window * (float)active / (total * kRowBytes); // units in the window, of the average size
@@ -56,41 +61,79 @@ __device__ __forceinline__ Groups split_groups(const DevParams &p, int warps, fl
     const unsigned share = g > 1 ? 0xffffffffu / g + 1 : 0u;
     r.from = r.me * share;
     r.to = r.from + share; // (the last block takes what is left)
+    r.all = active == p.B;
     r.dh = r.n % p.H;
-    r.db = (r.n / p.H) % p.B;
-    r.dl = r.n / (p.H * p.B);
+    r.db = (r.n / p.H) % active;
+    r.dl = r.n / (p.H * active);
     return r;
 }
 
-// The walk over a group's units: one after the other those that have something to evict, and the block's share of their
-// pages.
+// The walk over a group's units, each with the block's share of their pages.  Only what has something to evict is dealt out: in
+// the numbers of all sequences, a stride of whole sequences can miss the active ones for half of the groups (32 layers of 16
+// sequences of 6400 tokens, every other one within the budget, key scores: 1236 us, now 650, as for the eight alone).  The
+// lengths of 32 sequences stay in the warp's registers: the exchange's acquiring loads empty L1, and a trip to L2 per unit shows
+// (the eight alone 660 us, with two trips 676).  Called by whole warps.
 struct GroupWalk {
-    int l, b, h;
+    int l, b, h;   // the next unit; l >= L: none
+    int base, T;   // first of the sequences at hand, the length of the lane's
+    unsigned live; // which of them have something to evict
 };
 struct GroupUnit {
     int l, b, h, T, first, pages;
 };
+__device__ __forceinline__ void walk_lengths(const DevParams &p, const Groups &gr, GroupWalk &w, int base)
+{
+    const int b = base + (threadIdx.x & 31);
+    w.base = base;
+    w.T = base == 0 ? gr.T : b < p.B ? p.seq_lens[b] : 0;
+    w.live = __ballot_sync(0xffffffffu, w.T > p.Tk && w.T <= p.T_cap);
+}
+// `count` sequences with something to evict further on, round the batch into the next layers
+__device__ __forceinline__ void walk_sequences(const DevParams &p, const Groups &gr, GroupWalk &w, int count)
+{
+    if (gr.all) {
+        for (w.b += count; w.b >= p.B; w.b -= p.B) ++w.l;
+        const int base = w.b & ~31;
+        if (base != w.base && w.l < p.L) walk_lengths(p, gr, w, base);
+        return;
+    }
+    if (count <= 0 || w.l >= p.L) return;
+    unsigned rest = w.b < w.base ? w.live : w.live & ~((2u << (w.b - w.base)) - 1u); // those after b
+    for (int found; (found = __popc(rest)) < count;) {
+        count -= found;
+        int base = w.base + 32;
+        if (base >= p.B) {
+            base = 0;
+            if (++w.l >= p.L) return;
+        }
+        if (base != w.base) walk_lengths(p, gr, w, base);
+        rest = w.live;
+    }
+    const int lane = threadIdx.x & 31;
+    w.b = w.base - 1 + __ffs(__ballot_sync(0xffffffffu, (rest >> lane & 1u) && __popc(rest & ((1u << lane) - 1u)) == count - 1));
+}
 __device__ __forceinline__ GroupWalk group_walk(const DevParams &p, const Groups &gr)
 {
-    return GroupWalk{gr.id / (p.H * p.B), (gr.id / p.H) % p.B, gr.id % p.H};
+    GroupWalk w;
+    w.l = 0; w.b = -1; w.h = gr.id % p.H;
+    walk_lengths(p, gr, w, 0);
+    walk_sequences(p, gr, w, gr.id / p.H + 1);
+    return w;
 }
 __device__ __forceinline__ bool next_group_unit(const DevParams &p, const Groups &gr, GroupWalk &w, GroupUnit &u)
 {
-    while (w.l < p.L) {
-        u.l = w.l; u.b = w.b; u.h = w.h;
-        u.T = p.seq_lens[w.b];
-        w.h += gr.dh;
-        w.b += gr.db;
-        w.l += gr.dl;
-        if (w.h >= p.H) { w.h -= p.H; ++w.b; }
-        if (w.b >= p.B) { w.b -= p.B; ++w.l; }
-        if (u.T <= p.Tk || u.T > p.T_cap) continue;
-        const int pages = (u.T + kPage - 1) / kPage;
-        u.first = (int)__umulhi((unsigned)pages, gr.from);
-        u.pages = (gr.me == gr.g - 1 ? pages : (int)__umulhi((unsigned)pages, gr.to)) - u.first;
-        return true;
-    }
-    return false;
+    if (w.l >= p.L) return false;
+    u.l = w.l; u.b = w.b; u.h = w.h;
+    u.T = __shfl_sync(0xffffffffu, w.T, w.b - w.base);
+    const int pages = (u.T + kPage - 1) / kPage;
+    u.first = (int)__umulhi((unsigned)pages, gr.from);
+    u.pages = (gr.me == gr.g - 1 ? pages : (int)__umulhi((unsigned)pages, gr.to)) - u.first;
+    w.h += gr.dh;
+    w.l += gr.dl;
+    const bool carry = w.h >= p.H;
+    if (carry) w.h -= p.H;
+    walk_sequences(p, gr, w, gr.db + (carry ? 1 : 0));
+    return true;
 }
 
 // Exchange of a block's statistics with its group: slots of data, and a counter of the blocks that have filled theirs.  Four of
@@ -294,14 +337,15 @@ struct PipeReader {
     uint32_t phase;
     __device__ __forceinline__ PipeReader(GroupPipe<kWarps, kRing, kUnits> &pipe_, int warp_) : pipe(pipe_), warp(warp_), slot(0), turn(warp_), phase(0) {}
     __device__ __forceinline__ bool wait() { return warp_wait(&pipe.full[slot * kWarps + warp], phase, &pipe.abort_flag); }
-    // Matrix loads of the page: ldsm of chunk pair s (dimensions 16 s .. 16 s + 15), each lane from token 8 rows8 + lane % 8 and
-    // chunk 2 s + chunk.  Tokens in eights lie at 2048, halves of a row at 1024, a 16-byte chunk of a half at its
-    // number XOR the token, which leaves the loads free of bank conflicts.
-    __device__ __forceinline__ uint32_t at(int rows8) const
+    // Matrix loads of the page: chunk pair s (dimensions 16 s .. 16 s + 15), each lane from token 8 rows8 + lane % 8 and chunk 2 s + odd
+    // at chunk(at(rows8, odd), s).  Tokens in eights lie at 2048, halves of a row at 1024, a 16-byte chunk of a half at its
+    // number XOR the token, which leaves the loads free of bank conflicts (rows are 128 bytes, so the XOR can be taken of the address).
+    __device__ __forceinline__ uint32_t at(int rows8, int odd) const
     {
-        return tc::smem_u32(pipe.ring) + (slot * kWarps + warp) * kPageBytes + rows8 * 2048 + (threadIdx.x & 7) * 128;
+        const int r = threadIdx.x & 7;
+        return tc::smem_u32(pipe.ring) + (slot * kWarps + warp) * kPageBytes + (rows8 * 2048 + r * 128 + ((odd ^ r) << 4));
     }
-    static __device__ __forceinline__ uint32_t chunk(int s, int chunk) { return (s >> 2) * 1024 + (((2 * (s & 3) + chunk) ^ (threadIdx.x & 7)) << 4); }
+    static __device__ __forceinline__ uint32_t chunk(uint32_t at, int s) { return (at ^ ((s & 3) << 5)) + (s >> 2) * 1024; }
     __device__ __forceinline__ void release()
     {
         __syncwarp();

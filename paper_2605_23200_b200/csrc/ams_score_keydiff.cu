@@ -63,8 +63,9 @@ __global__ void __launch_bounds__(kKdThreads, 1) k_keydiff(DevParams p, const __
                     if (!ok) break;
                     // dimensions as rows, tokens as the contraction, against a matrix of ones
                     unsigned a[8][4];
+                    const uint32_t at = in.at(lane >> 4, (lane >> 3) & 1);
 #pragma unroll
-                    for (int s = 0; s < 8; ++s) ldsm4_trans(a[s], in.at(lane >> 4) + in.chunk(s, (lane >> 3) & 1));
+                    for (int s = 0; s < 8; ++s) ldsm4_trans(a[s], in.chunk(at, s));
                     // the last page's rows past the end hold anything: they are taken as zeros
                     const int left = cur.tokens - k * kPage;
                     if (left < kPage) {
@@ -102,8 +103,9 @@ __global__ void __launch_bounds__(kKdThreads, 1) k_keydiff(DevParams p, const __
                     ok = in.wait();
                     if (!ok) break;
                     unsigned a[8][4];
+                    const uint32_t at = in.at((lane >> 3) & 1, lane >> 4);
 #pragma unroll
-                    for (int s = 0; s < 8; ++s) ldsm4(a[s], in.at((lane >> 3) & 1) + in.chunk(s, lane >> 4));
+                    for (int s = 0; s < 8; ++s) ldsm4(a[s], in.chunk(at, s));
                     float dot[4] = {0.0f, 0.0f, 0.0f, 0.0f}, lo[4] = {0.0f, 0.0f, 0.0f, 0.0f}, hi[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
                     for (int s = 0; s < 8; ++s) {

@@ -170,12 +170,12 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
             for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                 for (int i = 0; i < 4; ++i) da[mt][i] = db[mt][i] = 0.0f;
-            const uint32_t at = in.at(lane >> 4);
+            const uint32_t at = in.at(lane >> 4, (lane >> 3) & 1);
 #pragma unroll
             for (int s = 0; s < 8; s += 2) {
                 unsigned k[2][4];
-                ldsm4(k[0], at + in.chunk(s, (lane >> 3) & 1));
-                ldsm4(k[1], at + in.chunk(s + 1, (lane >> 3) & 1));
+                ldsm4(k[0], in.chunk(at, s));
+                ldsm4(k[1], in.chunk(at, s + 1));
 #pragma unroll
                 for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -185,6 +185,8 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
                     }
             }
         };
+        // the last page start from which every row sees every token (padding rows are taken care of by their statistics)
+        auto last_whole = [&](int tokens) { return tokens - (p.causal ? p.W : 1) - 15; };
         // pairs the window hides add nothing
         auto hide = [&](float (&da)[MT][4], float (&db)[MT][4], int tokens, int t0) {
 #pragma unroll
@@ -208,6 +210,7 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
             cur = sh.pipe.unit[n % T::units];
             if (cur.pages >= 0) {
                 load_queries(n);
+                const int whole = last_whole(cur.tokens);
                 float st_a[MT][E], st_b[MT][E], st_m[MT][E]; // reference, sum of 2^(x - reference), largest unscaled logit
 #pragma unroll
                 for (int mt = 0; mt < MT; ++mt)
@@ -221,8 +224,7 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
                     logits(da, db);
                     in.release();
                     const int t0 = k * kPage;
-                    // (else every row sees every token of the page; padding rows are taken care of by their statistics)
-                    if (t0 + 15 >= cur.tokens || (p.causal && t0 + 15 > cur.tokens - p.W)) hide(da, db, cur.tokens, t0);
+                    if (t0 > whole) hide(da, db, cur.tokens, t0);
                     // The sum's reference follows the largest logit at a distance of up to 2^32, so that rescaling is rare; the
                     // sum is put on the maximum at the end.  One branch for all rows: their exponentials then overlap.
                     bool far = false;
@@ -230,7 +232,7 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
                     for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                         for (int e = 0; e < E; ++e) {
-                            st_m[mt][e] = fmaxf(fmaxf(st_m[mt][e], fmaxf(da[mt][2 * e], da[mt][2 * e + 1])), fmaxf(db[mt][2 * e], db[mt][2 * e + 1]));
+                            st_m[mt][e] = max3(max3(st_m[mt][e], da[mt][2 * e], da[mt][2 * e + 1]), db[mt][2 * e], db[mt][2 * e + 1]);
                             far |= fmaf(st_m[mt][e], c, -32.0f) > st_a[mt][e];
                         }
                     if (far) {
@@ -274,6 +276,7 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
                 ok = warp_wait(&sh.pipe.ready[m & 1], (uint32_t)((m >> 1) & 1), abort_flag);
                 if (!ok) break;
                 load_queries(m);
+                const int whole = last_whole(old.tokens);
                 float b[MT][E];
 #pragma unroll
                 for (int mt = 0; mt < MT; ++mt)
@@ -288,7 +291,7 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
                     logits(da, db);
                     in.release();
                     const int t0 = k * kPage;
-                    if (t0 + 15 >= old.tokens || (p.causal && t0 + 15 > old.tokens - p.W)) hide(da, db, old.tokens, t0);
+                    if (t0 > whole) hide(da, db, old.tokens, t0);
                     float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f}; // tokens 2 tq, 2 tq + 1, 8 + 2 tq, 9 + 2 tq
 #pragma unroll
                     for (int mt = 0; mt < MT; ++mt)
@@ -422,11 +425,11 @@ __global__ void __launch_bounds__(OnceTraits<NB>::threads, 1) k_window_once(DevP
                     float d[NB][4];
 #pragma unroll
                     for (int nb = 0; nb < NB; ++nb) d[nb][0] = d[nb][1] = d[nb][2] = d[nb][3] = 0.0f;
-                    const uint32_t at = in.at((lane >> 3) & 1);
+                    const uint32_t at = in.at((lane >> 3) & 1, lane >> 4);
 #pragma unroll
                     for (int s = 0; s < 8; ++s) {
                         unsigned a[4];
-                        ldsm4(a, at + in.chunk(s, lane >> 4));
+                        ldsm4(a, in.chunk(at, s));
 #pragma unroll
                         for (int nb = 0; nb < NB; ++nb) mma_bf16(d[nb], a[0], a[1], a[2], a[3], q[nb][s][0], q[nb][s][1]);
                     }
@@ -448,7 +451,7 @@ __global__ void __launch_bounds__(OnceTraits<NB>::threads, 1) k_window_once(DevP
                     for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
                         for (int e = 0; e < 2; ++e) {
-                            st_m[nb][e] = fmaxf(st_m[nb][e], fmaxf(d[nb][e], d[nb][2 + e]));
+                            st_m[nb][e] = max3(st_m[nb][e], d[nb][e], d[nb][2 + e]);
                             far |= fmaf(st_m[nb][e], c, -32.0f) > st_a[nb][e];
                         }
                     if (far) {
