@@ -8,29 +8,16 @@
 // phase 2 recomputes the logits and sums the normalised probabilities over rows.
 // The largest probability of a row is 1/Z_r (its arg-max token), so the window
 // maximum is 1/min_r Z_r and needs no third pass.  Up to 32 rows: ams_score_window.cu; from 64: ams_score_tc.cu; the rest here.
+#include <float.h>
+
 #include "ams_common.cuh"
+#include "ams_tc_ptx.cuh"
 
 namespace ams {
 
 namespace {
 
-constexpr float kLog2e = 1.4426950408889634f;
-
-__device__ __forceinline__ float ex2(float x)
-{
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// (m, z) <- log-sum-exp merge of (m, z) and (m2, z2) in the base-2 domain.
-__device__ __forceinline__ void lse_merge(float &m, float &z, float m2, float z2)
-{
-    const float mn = fmaxf(m, m2);
-    if (mn == -INFINITY) return;
-    z = z * ex2(m - mn) + z2 * ex2(m2 - mn);
-    m = mn;
-}
+using namespace tc;
 
 constexpr int kTovaThreads = 128;
 constexpr int kRing = 3;       // 16-token K tiles per warp in shared memory: one worked on, two on their way
@@ -153,7 +140,7 @@ __global__ void __launch_bounds__(kTovaThreads) k_tova_wide(DevParams p)
     const unsigned Fr = Qb + MT * 16 * kRowBytes;                   // [MT][8 k-steps][32 lanes] fragments of the current rows
     wait_for_previous_kernel(); // effective lengths; merged statistics
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, tq = lane & 3;
-    const float c = kLog2e * 0.08838834764831845f; // log2(e) / sqrt(128)
+    constexpr float c = kLogitScale;
     const float inv_rows = 1.0f / (float)p.rows;
     TovaStream<MT * 16, PHASE> st(p, smem, Qb);
     const int n_rb = st.n_rb;
@@ -170,13 +157,13 @@ __global__ void __launch_bounds__(kTovaThreads) k_tova_wide(DevParams p)
         float *u_out = p.scores + (size_t)uid * p.T_cap;
         const float pmax = PHASE == 2 ? fin[p.rows_pad] : 0.0f;
         // per thread: rows (mt, e) = row0 + 16 mt + g + 8 e
-        float st_a[MT][2], st_b[MT][2], st_m[MT][2]; // phase 1: reference, sum of 2^(x - reference), largest unscaled logit;
-                                                     // phase 2: -b_r in the first
+        float st_a[MT][2], st_b[MT][2], st_m[MT][2]; // phase 1: reference, sum of 2^(c (x - reference)), largest logit;
+                                                     // phase 2: the row's reference in the first
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
-                st_a[mt][e] = PHASE == 1 ? -1e30f : -fin[row0 + mt * 16 + 8 * e + g];
+                st_a[mt][e] = PHASE == 1 ? -FLT_MAX : fin[row0 + mt * 16 + 8 * e + g];
                 st_b[mt][e] = 0.0f;
                 st_m[mt][e] = -INFINITY;
             }
@@ -225,19 +212,19 @@ __global__ void __launch_bounds__(kTovaThreads) k_tova_wide(DevParams p)
                     if (PHASE == 1) {
                         // The sum's reference follows the largest logit at a distance of up to 2^32, so that rescaling is
                         // rare; the sum is put on the maximum at the end.
-                        st_m[mt][e] = fmaxf(fmaxf(st_m[mt][e], fmaxf(v[0], v[1])), fmaxf(v[2], v[3]));
-                        if (fmaf(st_m[mt][e], c, -32.0f) > st_a[mt][e]) {
-                            const float mx = st_m[mt][e] * c;
-                            st_b[mt][e] *= ex2(st_a[mt][e] - mx);
+                        st_m[mt][e] = max3(max3(st_m[mt][e], v[0], v[1]), v[2], v[3]);
+                        if (st_m[mt][e] - st_a[mt][e] > 32.0f / c) {
+                            const float mx = st_m[mt][e];
+                            st_b[mt][e] *= ex2((st_a[mt][e] - mx) * c);
                             st_a[mt][e] = mx;
                         }
-                        float s[4];
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) s[i] = ex2(fmaf(v[i], c, -st_a[mt][e]));
-                        st_b[mt][e] += (s[0] + s[1]) + (s[2] + s[3]);
+                        const float n = -st_a[mt][e];
+                        const float2 s = ex2_from(v[0], v[1], n, n), t = ex2_from(v[2], v[3], n, n);
+                        st_b[mt][e] += (s.x + s.y) + (t.x + t.y);
                     } else {
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) acc[i] += ex2(fmaf(v[i], c, st_a[mt][e]));
+                        const float n = st_a[mt][e];
+                        const float2 s = ex2_from(v[0], v[1], n, n), t = ex2_from(v[2], v[3], n, n);
+                        acc[0] += s.x; acc[1] += s.y; acc[2] += t.x; acc[3] += t.y;
                     }
                 }
             }
@@ -268,11 +255,11 @@ __global__ void __launch_bounds__(kTovaThreads) k_tova_wide(DevParams p)
             for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    float m = st_m[mt][e] * c, z = m > -INFINITY ? st_b[mt][e] * ex2(st_a[mt][e] - m) : 0.0f;
+                    float m = st_m[mt][e], z = m > -INFINITY ? st_b[mt][e] * ex2((st_a[mt][e] - m) * c) : 0.0f;
 #pragma unroll
                     for (int o = 1; o < 4; o <<= 1) {
                         const float m2 = __shfl_xor_sync(0xffffffffu, m, o), z2 = __shfl_xor_sync(0xffffffffu, z, o);
-                        lse_merge(m, z, m2, z2);
+                        stat_merge(m, z, m2, z2);
                     }
                     if (tq == 0) {
                         red[warp][mt * 16 + 8 * e + g][0] = m;
@@ -283,7 +270,7 @@ __global__ void __launch_bounds__(kTovaThreads) k_tova_wide(DevParams p)
             for (int r = threadIdx.x; r < MT * 16; r += kTovaThreads) {
                 float m = red[0][r][0], z = red[0][r][1];
 #pragma unroll
-                for (int w = 1; w < 4; ++w) lse_merge(m, z, red[w][r][0], red[w][r][1]);
+                for (int w = 1; w < 4; ++w) stat_merge(m, z, red[w][r][0], red[w][r][1]);
                 float2 *out = reinterpret_cast<float2 *>(p.part) + ((size_t)uid * p.n_slices + cur.slice) * p.rows_pad + row0 + r;
                 *out = make_float2(m, z);
             }
@@ -294,8 +281,7 @@ __global__ void __launch_bounds__(kTovaThreads) k_tova_wide(DevParams p)
     cp_async_wait<0>();
 }
 
-// Per unit: merge the slices' (max, sum) in slice order; b_r = M_r + log2 Z_r in the
-// base-2 domain, and the window maximum 1 / min_r Z_r.
+// Per unit: merge the slices' (max, sum) in slice order; the rows' references, and the window maximum 1 / min_r Z_r.
 __global__ void __launch_bounds__(128) k_tova_combine(DevParams p)
 {
     __shared__ u64 scratch[40];
@@ -311,14 +297,11 @@ __global__ void __launch_bounds__(128) k_tova_combine(DevParams p)
         float m = -INFINITY, z = 0.0f;
         for (int s = 0; s < ns; ++s) {
             const float2 v = reinterpret_cast<const float2 *>(p.part)[((size_t)uid * p.n_slices + s) * p.rows_pad + r];
-            lse_merge(m, z, v.x, v.y);
+            stat_merge(m, z, v.x, v.y);
         }
-        if (r < p.rows && z > 0.0f) {
-            fin[r] = m + log2f(z);
-            best = fmaxf(best, 1.0f / z);
-        } else {
-            fin[r] = INFINITY; // padding rows contribute nothing
-        }
+        const bool live = r < p.rows && z > 0.0f;
+        set_reference(fin[r], live, m, z); // padding rows contribute nothing
+        if (live) best = fmaxf(best, 1.0f / z);
     }
     best = block_max_f32(best, scratch);
     if (threadIdx.x == 0) fin[p.rows_pad] = best;

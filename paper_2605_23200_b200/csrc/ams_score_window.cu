@@ -7,6 +7,8 @@
 // 32768 tokens) took 1.87 ms in three launches, with the logits through HBM, now 1.66 (5.7 TB/s, bound by the K stream and by
 // the spread of a group's blocks at each exchange); 16 rows, 256 units of 3000 tokens, 76 -> 49 us; 32 rows over 2.9 GB, with K
 // twice from HBM, 1.04 ms, now 0.77 (bound by the latency of a page in a warp: loads, eight dependent products, exponentials).
+#include <float.h>
+
 #include "ams_common.cuh"
 #include "ams_groups.cuh"
 
@@ -16,17 +18,17 @@ namespace {
 
 using namespace tc;
 
-// (m, z) <- log-sum-exp merge of (m, z) and all of v, base 2, with one maximum
+// (m, z) <- merge of (m, z) and all of v, with one maximum
 template <int N>
-__device__ __forceinline__ void lse_merge_all(float &m, float &z, const float2 (&v)[N])
+__device__ __forceinline__ void stat_merge_all(float &m, float &z, const float2 (&v)[N])
 {
     float mx = m;
 #pragma unroll
     for (int i = 0; i < N; ++i) mx = fmaxf(mx, v[i].x);
     if (mx == -INFINITY) return;
-    z *= ex2(m - mx);
+    z *= ex2((m - mx) * kLogitScale);
 #pragma unroll
-    for (int i = 0; i < N; ++i) z += v[i].y * ex2(v[i].x - mx);
+    for (int i = 0; i < N; ++i) z += v[i].y * ex2((v[i].x - mx) * kLogitScale);
     m = mx;
 }
 
@@ -47,7 +49,7 @@ struct WideShared {
     alignas(1024) unsigned char q[T::units][T::rows * kRowBytes]; // the units' query rows, halves of 128 bytes, swizzled
     float2 stat[2][T::warps][T::rows];                            // the warps' (max, sum)
     float2 part[2][32];                                           // the second collector's share of the group's
-    float b[2][T::rows];                                          // -b_r
+    float b[2][T::rows];                                          // the rows' references
     float pmax[2];                                                // largest probability of the window
 };
 static_assert(sizeof(WideShared) <= 227 * 1024, "shared memory of a block");
@@ -81,7 +83,7 @@ __device__ __forceinline__ bool exchange_stats(const DevParams &p, const Groups 
 #pragma unroll
                     for (int i = 0; i < kWarps; ++i) v[i] = sh.stat[n & 1][i][lane];
                     float m = -INFINITY, z = 0.0f;
-                    lse_merge_all(m, z, v);
+                    stat_merge_all(m, z, v);
                     __stcg(group_slot<float2>(p, gr, gr.me, n) + lane, make_float2(m, z));
                 }
                 group_publish(p, gr, n);
@@ -100,25 +102,25 @@ __device__ __forceinline__ bool exchange_stats(const DevParams &p, const Groups 
                     const int member = i0 + i * kSub * kGroupCollectors;
                     v[i] = member < gr.g ? __ldcg(src + (size_t)member * (kGroupSlot / 8)) : make_float2(-INFINITY, 0.0f);
                 }
-                lse_merge_all(m, z, v);
+                stat_merge_all(m, z, v);
             }
         }
 #pragma unroll
         for (int o = RP; o < 32; o <<= 1) {
             const float m2 = __shfl_xor_sync(0xffffffffu, m, o), z2 = __shfl_xor_sync(0xffffffffu, z, o);
-            lse_merge(m, z, m2, z2);
+            stat_merge(m, z, m2, z2);
         }
         if (w == 1) sh.part[n & 1][lane] = make_float2(m, z);
         ok = named_barrier_all(1, kGroupCollectors * 32, ok);
         if (!ok) break;
         if (w == 0) {
             const float2 v = sh.part[n & 1][lane];
-            lse_merge(m, z, v.x, v.y);
+            stat_merge(m, z, v.x, v.y);
             const bool live = lane < p.rows && z > 0.0f;
             float best = live ? 1.0f / z : 0.0f;
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-            if (lane < RP) sh.b[n & 1][lane] = live ? -(m + log2f(z)) : -INFINITY; // padding rows contribute nothing
+            if (lane < RP) set_reference(sh.b[n & 1][lane], live, m, z); // padding rows contribute nothing
             if (lane == 0) sh.pmax[n & 1] = best;
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&sh.pipe.ready[n & 1]));
@@ -143,7 +145,7 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
     if (gr.id >= gr.n) return;
     bool ok = true;
     if (warp < kWarps) {
-        const float c = kLog2e * 0.08838834764831845f; // log2(e) / sqrt(128)
+        constexpr float c = kLogitScale;
         PipeReader<T::warps, T::ring, T::units> in(sh.pipe, warp);
         unsigned q[MT][8][4];
         auto load_queries = [&](int n) {
@@ -211,11 +213,11 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
             if (cur.pages >= 0) {
                 load_queries(n);
                 const int whole = last_whole(cur.tokens);
-                float st_a[MT][E], st_b[MT][E], st_m[MT][E]; // reference, sum of 2^(x - reference), largest unscaled logit
+                float st_a[MT][E], st_b[MT][E], st_m[MT][E]; // reference, sum of 2^(c (x - reference)), largest logit
 #pragma unroll
                 for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-                    for (int e = 0; e < E; ++e) { st_a[mt][e] = -1e30f; st_b[mt][e] = 0.0f; st_m[mt][e] = -INFINITY; }
+                    for (int e = 0; e < E; ++e) { st_a[mt][e] = -FLT_MAX; st_b[mt][e] = 0.0f; st_m[mt][e] = -INFINITY; }
                 int k = in.turn;
                 for (; k < cur.pages; k += kWarps) {
                     ok = in.wait();
@@ -233,24 +235,24 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
 #pragma unroll
                         for (int e = 0; e < E; ++e) {
                             st_m[mt][e] = max3(max3(st_m[mt][e], da[mt][2 * e], da[mt][2 * e + 1]), db[mt][2 * e], db[mt][2 * e + 1]);
-                            far |= fmaf(st_m[mt][e], c, -32.0f) > st_a[mt][e];
+                            far |= st_m[mt][e] - st_a[mt][e] > 32.0f / c;
                         }
                     if (far) {
 #pragma unroll
                         for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                             for (int e = 0; e < E; ++e) {
-                                const float mx = st_m[mt][e] * c;
-                                if (mx > st_a[mt][e]) { st_b[mt][e] *= ex2(st_a[mt][e] - mx); st_a[mt][e] = mx; }
+                                const float mx = st_m[mt][e];
+                                if (mx > st_a[mt][e]) { st_b[mt][e] *= ex2((st_a[mt][e] - mx) * c); st_a[mt][e] = mx; }
                             }
                     }
 #pragma unroll
                     for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                         for (int e = 0; e < E; ++e) {
-                            const float a = st_a[mt][e];
-                            st_b[mt][e] += (ex2(fmaf(da[mt][2 * e], c, -a)) + ex2(fmaf(da[mt][2 * e + 1], c, -a))) +
-                                           (ex2(fmaf(db[mt][2 * e], c, -a)) + ex2(fmaf(db[mt][2 * e + 1], c, -a)));
+                            const float n = -st_a[mt][e];
+                            const float2 s = ex2_from(da[mt][2 * e], da[mt][2 * e + 1], n, n), t = ex2_from(db[mt][2 * e], db[mt][2 * e + 1], n, n);
+                            st_b[mt][e] += (s.x + s.y) + (t.x + t.y);
                         }
                 }
                 if (!ok) break;
@@ -260,11 +262,11 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
                 for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
                     for (int e = 0; e < E; ++e) {
-                        float m = st_m[mt][e] * c, z = m > -INFINITY ? st_b[mt][e] * ex2(st_a[mt][e] - m) : 0.0f;
+                        float m = st_m[mt][e], z = m > -INFINITY ? st_b[mt][e] * ex2((st_a[mt][e] - m) * c) : 0.0f;
 #pragma unroll
                         for (int o = 1; o < 4; o <<= 1) {
                             const float m2 = __shfl_xor_sync(0xffffffffu, m, o), z2 = __shfl_xor_sync(0xffffffffu, z, o);
-                            lse_merge(m, z, m2, z2);
+                            stat_merge(m, z, m2, z2);
                         }
                         if (tq == 0) sh.stat[n & 1][warp][mt * 16 + 8 * e + g] = make_float2(m, z);
                     }
@@ -296,12 +298,11 @@ __global__ void __launch_bounds__(WideTraits::threads, 1) k_window(DevParams p, 
 #pragma unroll
                     for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-                        for (int e = 0; e < E; ++e)
-#pragma unroll
-                            for (int i = 0; i < 2; ++i) {
-                                acc[i] += ex2(fmaf(da[mt][2 * e + i], c, b[mt][e]));
-                                acc[2 + i] += ex2(fmaf(db[mt][2 * e + i], c, b[mt][e]));
-                            }
+                        for (int e = 0; e < E; ++e) {
+                            const float n = b[mt][e];
+                            const float2 s = ex2_from(da[mt][2 * e], da[mt][2 * e + 1], n, n), t = ex2_from(db[mt][2 * e], db[mt][2 * e + 1], n, n);
+                            acc[0] += s.x; acc[1] += s.y; acc[2] += t.x; acc[3] += t.y;
+                        }
                     // sums over the eight lanes of a tq, four tokens at once: at each step a lane hands half of its values over
                     const bool up = lane & 16, odd = lane & 8;
                     float k0 = up ? acc[2] : acc[0], k1 = up ? acc[3] : acc[1];
@@ -357,7 +358,7 @@ struct OnceShared {
     float4 logits[T::warps][T::held][NB][32];
     float2 stat[2][T::warps][T::rows];                            // the warps' (max, sum)
     float2 part[2][32];                                           // the second collector's share of the group's
-    float b[2][T::rows];                                          // -b_r
+    float2 b[2][T::rows];                                         // the rows' references
     float pmax[2];                                                // largest probability of the window
 };
 static_assert(sizeof(OnceShared<1>) <= 227 * 1024 && sizeof(OnceShared<2>) <= 227 * 1024, "shared memory of a block");
@@ -379,7 +380,7 @@ __global__ void __launch_bounds__(OnceTraits<NB>::threads, 1) k_window_once(DevP
     if (gr.id >= gr.n) return;
     bool ok = true;
     if (warp < kWarps) {
-        const float c = kLog2e * 0.08838834764831845f; // log2(e) / sqrt(128)
+        constexpr float c = kLogitScale;
         PipeReader<T::warps, T::ring, T::units> in(sh.pipe, warp);
         int see[NB][2]; // row 8 nb + 2 tq + e: the last token it sees, from the end of the sequence
 #pragma unroll
@@ -412,11 +413,11 @@ __global__ void __launch_bounds__(OnceTraits<NB>::threads, 1) k_window_once(DevP
                     }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&sh.pipe.unit_empty[n % T::units]));
-                float st_a[NB][2], st_b[NB][2], st_m[NB][2]; // reference, sum of 2^(x - reference), largest unscaled logit
+                float st_a[NB][2], st_b[NB][2], st_m[NB][2]; // reference, sum of 2^(c (x - reference)), largest logit
 #pragma unroll
                 for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
-                    for (int e = 0; e < 2; ++e) { st_a[nb][e] = -1e30f; st_b[nb][e] = 0.0f; st_m[nb][e] = -INFINITY; }
+                    for (int e = 0; e < 2; ++e) { st_a[nb][e] = -FLT_MAX; st_b[nb][e] = 0.0f; st_m[nb][e] = -INFINITY; }
                 int k = in.turn;
                 k_cur = k;
                 for (; k < cur.pages; k += kWarps) {
@@ -452,21 +453,23 @@ __global__ void __launch_bounds__(OnceTraits<NB>::threads, 1) k_window_once(DevP
 #pragma unroll
                         for (int e = 0; e < 2; ++e) {
                             st_m[nb][e] = max3(st_m[nb][e], d[nb][e], d[nb][2 + e]);
-                            far |= fmaf(st_m[nb][e], c, -32.0f) > st_a[nb][e];
+                            far |= st_m[nb][e] - st_a[nb][e] > 32.0f / c;
                         }
                     if (far) {
 #pragma unroll
                         for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
                             for (int e = 0; e < 2; ++e) {
-                                const float mx = st_m[nb][e] * c;
-                                if (mx > st_a[nb][e]) { st_b[nb][e] *= ex2(st_a[nb][e] - mx); st_a[nb][e] = mx; }
+                                const float mx = st_m[nb][e];
+                                if (mx > st_a[nb][e]) { st_b[nb][e] *= ex2((st_a[nb][e] - mx) * c); st_a[nb][e] = mx; }
                             }
                     }
 #pragma unroll
                     for (int nb = 0; nb < NB; ++nb) {
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) st_b[nb][e] += ex2(fmaf(d[nb][e], c, -st_a[nb][e])) + ex2(fmaf(d[nb][2 + e], c, -st_a[nb][e]));
+                        const float2 s = ex2_from(d[nb][0], d[nb][1], -st_a[nb][0], -st_a[nb][1]);
+                        const float2 t = ex2_from(d[nb][2], d[nb][3], -st_a[nb][0], -st_a[nb][1]);
+                        st_b[nb][0] += s.x + t.x;
+                        st_b[nb][1] += s.y + t.y;
                         sh.logits[warp][kept][nb][lane] = make_float4(d[nb][0], d[nb][1], d[nb][2], d[nb][3]);
                     }
                     kept = kept == T::held - 1 ? 0 : kept + 1;
@@ -478,11 +481,11 @@ __global__ void __launch_bounds__(OnceTraits<NB>::threads, 1) k_window_once(DevP
                 for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
-                        float m = st_m[nb][e] * c, z = m > -INFINITY ? st_b[nb][e] * ex2(st_a[nb][e] - m) : 0.0f;
+                        float m = st_m[nb][e], z = m > -INFINITY ? st_b[nb][e] * ex2((st_a[nb][e] - m) * c) : 0.0f;
 #pragma unroll
                         for (int o = 4; o < 32; o <<= 1) {
                             const float m2 = __shfl_xor_sync(0xffffffffu, m, o), z2 = __shfl_xor_sync(0xffffffffu, z, o);
-                            lse_merge(m, z, m2, z2);
+                            stat_merge(m, z, m2, z2);
                         }
                         if (g == 0) sh.stat[n & 1][warp][8 * nb + 2 * tq + e] = make_float2(m, z);
                     }
@@ -493,7 +496,7 @@ __global__ void __launch_bounds__(OnceTraits<NB>::threads, 1) k_window_once(DevP
                 const int m = n - 1;
                 ok = warp_wait(&sh.pipe.ready[m & 1], (uint32_t)((m >> 1) & 1), abort_flag);
                 if (!ok) break;
-                float b[NB][2];
+                float2 b[NB][2];
 #pragma unroll
                 for (int nb = 0; nb < NB; ++nb)
 #pragma unroll
@@ -505,8 +508,9 @@ __global__ void __launch_bounds__(OnceTraits<NB>::threads, 1) k_window_once(DevP
 #pragma unroll
                     for (int nb = 0; nb < NB; ++nb) {
                         const float4 d = sh.logits[warp][at][nb][lane];
-                        lo += ex2(fmaf(d.x, c, b[nb][0])) + ex2(fmaf(d.y, c, b[nb][1]));
-                        hi += ex2(fmaf(d.z, c, b[nb][0])) + ex2(fmaf(d.w, c, b[nb][1]));
+                        const float2 s = ex2_from(d.x, d.y, b[nb][0], b[nb][1]), t = ex2_from(d.z, d.w, b[nb][0], b[nb][1]);
+                        lo += s.x + s.y;
+                        hi += t.x + t.y;
                     }
                     at = at == T::held - 1 ? 0 : at + 1;
                     // sums over the four lanes of a token, both tokens at once
