@@ -38,7 +38,8 @@
  * on fixed-point images of the mass, so they do not depend on summation order.
  *
  * Scorer selection is automatic (query rows per KV head >= 64: tensor-core path, otherwise the
- * mma.sync path) and depends on the arguments only: no environment variable changes what runs.
+ * mma.sync path) and depends on the arguments and ams_set_independent_blocks only: no environment variable changes what
+ * runs.
  *
  * Errors: every function returns AMS_OK (0) or a negative code.  Calls are
  * asynchronous on `stream`; conditions found on the device are reported by
@@ -170,7 +171,13 @@ int ams_init_state(const ams_config *cfg, void *ema_state, void *workspace, size
  * nothing and never synchronises; after one direct call (which sets kernel attributes) it can be captured
  * into a CUDA graph.  Its kernels follow one another on `stream` as dependent launches (a kernel may start
  * while its predecessor's last blocks run and waits before touching that kernel's output); work enqueued
- * on `stream` before or after the call is ordered as usual. */
+ * on `stream` before or after the call is ordered as usual.
+ * Key-only scores and windows of up to 32 query rows per KV head come from one cooperative launch (of one block of some
+ * 200 KB of shared memory per SM; of clusters for a few short units): it starts once all of its blocks fit at the same time, so a
+ * kernel of another stream that holds SMs delays it, and one that waits for this event would wait for ever.
+ * How a sequence is shared among the blocks depends on the other sequences of the call: its scores are the same in
+ * another batch up to the rounding of fp32 sums (1e-6 relative), the same call's are the same bits.  See
+ * ams_set_independent_blocks for neither. */
 int ams_compress(ams_state *st, void *k_pages, void *v_pages, int64_t num_pages, int32_t *block_table,
                  int32_t block_table_stride, int32_t *seq_lens, int32_t batch, const void *obs_queries,
                  int32_t window, void *ema_state, int32_t budget, int32_t n_segments, int32_t scorer_id,
@@ -193,6 +200,13 @@ int ams_compress(ams_state *st, void *k_pages, void *v_pages, int64_t num_pages,
  * this score ranks the tokens inside the segments (the runtime section's "decoupled mass and selection
  * scores, including TOVA-style and expected-attention selection"). */
 int ams_set_query_stats(ams_state *st, const float *q_mean, const void *q_cov, float score_eps);
+
+/* With `enable` non-zero, later events of the handle score with kernels whose blocks do not wait for one another wherever there
+ * are such (key-only scores, windows below 64 query rows per KV head): they run on whatever SMs are free, beside kernels that
+ * never leave theirs, and a sequence's scores do not depend on the other sequences of the call.  They read K twice and
+ * take up to 1.7 times as long.  Default: off.  Wider windows and the expected-attention scorer need no two blocks
+ * at the same time either way. */
+int ams_set_independent_blocks(ams_state *st, int enable);
 
 /* Synchronises `stream`, then returns and clears the device status: AMS_OK or the
  * first device-side error.  detail[0..3] (host, may be NULL) receive the code, the

@@ -25,7 +25,8 @@ AMS_SCORER_TOVA, AMS_SCORER_KEYDIFF, AMS_SCORER_EXTERNAL, AMS_SCORER_EXPECTED = 
 EXPORTS = ["ams_config_default", "ams_ema_state_bytes", "ams_workspace_bytes", "ams_segment_capacity",
            "ams_init_state", "ams_compress", "ams_get_status", "ams_last_launch_count", "ams_free",
            "ams_strerror", "ams_set_profiling", "ams_get_kernel_times", "ams_kernel_name", "ams_select_static",
-           "ams_select_static_status", "ams_debug_expire_wait", "ams_debug_expire_event", "ams_set_query_stats"]
+           "ams_select_static_status", "ams_debug_expire_wait", "ams_debug_expire_event", "ams_set_query_stats",
+           "ams_set_independent_blocks"]
 KERNEL_SLOTS = 10
 
 
@@ -91,6 +92,8 @@ def lib() -> ctypes.CDLL:
         L.ams_debug_expire_wait.restype = ctypes.c_int
         L.ams_debug_expire_event.argtypes = [ctypes.c_void_p, ctypes.c_uint32]
         L.ams_debug_expire_event.restype = ctypes.c_int
+        L.ams_set_independent_blocks.argtypes = [ctypes.c_void_p, ctypes.c_int]
+        L.ams_set_independent_blocks.restype = ctypes.c_int
         L.ams_set_query_stats.argtypes = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_float]
         L.ams_set_query_stats.restype = ctypes.c_int
         L.ams_strerror.argtypes = [ctypes.c_int]
@@ -208,6 +211,12 @@ class AmsCompressor:
         if rc != AMS_OK:
             raise AmsError(rc, "ams_set_query_stats")
         self._query_stats = (q_mean, q_cov)
+
+    def set_independent_blocks(self, enable: bool) -> None:
+        """Scorers that need no two blocks at the same time and whose scores do not depend on the rest of the batch (slower)."""
+        rc = lib().ams_set_independent_blocks(self._h, 1 if enable else 0)
+        if rc != AMS_OK:
+            raise AmsError(rc, "ams_set_independent_blocks")
 
     def status(self, stream: torch.cuda.Stream | None = None, check: bool = True):
         s = stream or torch.cuda.current_stream(self.device)

@@ -119,6 +119,7 @@ struct ams_state {
     const float *q_mean; // query statistics of the expected-attention scorer (ams_set_query_stats)
     const void *q_cov;
     float score_eps;
+    bool independent;      // ams_set_independent_blocks
     uint32_t expire_polls; // of the next event (ams_debug_expire_event)
     bool profiling;
     int n_ev;
@@ -198,6 +199,7 @@ int ams_init_state(const ams_config *cfg, void *ema_state, void *workspace, size
     st->q_mean = nullptr;
     st->q_cov = nullptr;
     st->score_eps = 0.0f;
+    st->independent = false;
     st->expire_polls = 0;
     st->profiling = false;
     st->n_ev = 0;
@@ -270,6 +272,7 @@ int ams_compress(ams_state *st, void *k_pages, void *v_pages, int64_t num_pages,
     p.tc_stages = p.rows_pad <= 256 ? 4 : 2; // even: each stage then belongs to one of the two MMA issuers
     p.status = (int *)(st->ws + y.status);
     p.q_mean = st->q_mean; p.q_cov = (const __nv_bfloat16 *)st->q_cov; p.score_eps = st->score_eps;
+    p.independent = st->independent ? 1 : 0;
     p.expire_polls = st->expire_polls;
     st->expire_polls = 0;
     p.ex_logits = c.expected_scorer ? (float *)(st->ws + y.ex_logits) : nullptr;
@@ -326,6 +329,13 @@ int ams_set_query_stats(ams_state *st, const float *q_mean, const void *q_cov, f
     st->q_mean = q_mean;
     st->q_cov = q_cov;
     st->score_eps = score_eps;
+    return AMS_OK;
+}
+
+int ams_set_independent_blocks(ams_state *st, int enable)
+{
+    if (!st) return AMS_ERR_INVALID_ARG;
+    st->independent = enable != 0;
     return AMS_OK;
 }
 

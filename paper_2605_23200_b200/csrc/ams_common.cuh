@@ -64,6 +64,7 @@ struct DevParams {
     float *ex_logits;                 // [units][G][T_cap] logits in log2 units, or null
     int ex_g0, ex_gc;                 // query heads [g0, g0 + gc) of the group handled by one launch (set by the launcher)
     float inv_rows;                   // window scorer in groups: 1 / rows, from the constant bank
+    int independent;                  // the caller wants scorers whose blocks do not wait for one another (ams_set_independent_blocks)
     int group_size;                   // blocks that work on a unit together: their number if the launcher sets it (a cluster);
     int *group_count;                 // counters, cleared by the first kernel of an event,
     unsigned char *group_part;        // and the slots of what they exchange

@@ -7,7 +7,8 @@
 // window.  Two phases over K: phase 1 finds each row's (max, sum of exponentials),
 // phase 2 recomputes the logits and sums the normalised probabilities over rows.
 // The largest probability of a row is 1/Z_r (its arg-max token), so the window
-// maximum is 1/min_r Z_r and needs no third pass.  Up to 32 rows: ams_score_window.cu; from 64: ams_score_tc.cu; the rest here.
+// maximum is 1/min_r Z_r and needs no third pass.  Up to 32 rows: ams_score_window.cu (here where the caller wants
+// independent blocks); from 64: ams_score_tc.cu; the rest here.
 #include <float.h>
 
 #include "ams_common.cuh"
@@ -345,7 +346,12 @@ int tova_rows_block(int rows)
 int launch_score_tova(const DevParams &p, LaunchCtx &ctx)
 {
     if (tova_tc_supported(p)) return launch_score_tova_tc(p, ctx);
-    if (p.rows <= 32) return launch_score_window(p, ctx);
+    if (p.rows <= 32 && !p.independent) return launch_score_window(p, ctx);
+    if (p.rows <= 32) {
+        DevParams q = p;
+        q.rows_pad = 32; // (the workspace has room for 128 floats per slice and 136 per unit at least)
+        return launch_tova_wide<2>(q, ctx);
+    }
     return tova_rows_block(p.rows) == 64 ? launch_tova_wide<4>(p, ctx) : launch_tova_wide<8>(p, ctx);
 }
 

@@ -199,10 +199,149 @@ __global__ void __launch_bounds__(kKdThreads, 1) k_keydiff(DevParams p, const __
     if (!ok && lane == 0) report_timeout(p, 4, 0);
 }
 
+// The same score by blocks that never wait for one another, both passes from HBM, a kernel each (5.7 ms where k_keydiff takes 3.5):
+// for callers that cannot give an event the whole device at once.  A sequence is cut by the capacity alone, so its scores do
+// not depend on the others of the batch.
+constexpr int kApartThreads = 256; // 16 token rows x 16 lanes of 16 bytes
+
+__global__ void __launch_bounds__(kApartThreads) k_keydiff_sum(DevParams p)
+{
+    __shared__ float red[16][kHeadDim];
+    wait_for_previous_kernel(); // effective lengths
+    const int uid = blockIdx.y, slice = blockIdx.x;
+    const int h = uid % p.H, b = (uid / p.H) % p.B, l = uid / (p.H * p.B);
+    const int T = p.seq_lens[b];
+    if (T <= p.Tk || T > p.T_cap) return;
+    const int t_begin = slice * p.slice_len;
+    if (t_begin >= T) return;
+    const int t_end = min(T, t_begin + p.slice_len);
+    const int lane = threadIdx.x & 15, r = threadIdx.x >> 4;
+    const int *table = p.block_table + (size_t)b * p.bt_stride;
+    float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    for (int t = t_begin + r; t < t_end; t += 16) {
+        const uint4 v = ld_stream16(p.k_pages + row_offset(p, l, table[t >> 4], t & 15, h) + lane * 8);
+        acc[0] += bf16_lo(v.x); acc[1] += bf16_hi(v.x); acc[2] += bf16_lo(v.y); acc[3] += bf16_hi(v.y);
+        acc[4] += bf16_lo(v.z); acc[5] += bf16_hi(v.z); acc[6] += bf16_lo(v.w); acc[7] += bf16_hi(v.w);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) red[r][lane * 8 + i] = acc[i];
+    __syncthreads();
+    if (threadIdx.x < kHeadDim) {
+        float s = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) s += red[i][threadIdx.x];
+        p.part[((size_t)uid * p.n_slices + slice) * kHeadDim + threadIdx.x] = s;
+    }
+}
+
+__global__ void __launch_bounds__(kHeadDim) k_keydiff_combine(DevParams p)
+{
+    __shared__ float sq[kHeadDim];
+    wait_for_previous_kernel(); // the slices' sums
+    const int uid = blockIdx.x;
+    const int b = (uid / p.H) % p.B;
+    const int T = p.seq_lens[b];
+    if (T <= p.Tk || T > p.T_cap) return;
+    const int ns = (T + p.slice_len - 1) / p.slice_len;
+    float s = 0.0f;
+    for (int i = 0; i < ns; ++i) s += p.part[((size_t)uid * p.n_slices + i) * kHeadDim + threadIdx.x];
+    const float mu = s / (float)T;
+    float *fin = p.fin + (size_t)uid * (p.rows_pad + 8);
+    fin[threadIdx.x] = mu;
+    sq[threadIdx.x] = mu * mu;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float tot = 0.0f;
+        for (int i = 0; i < kHeadDim; ++i) tot += sq[i];
+        fin[kHeadDim] = sqrtf(tot);
+    }
+}
+
+__global__ void __launch_bounds__(kApartThreads) k_keydiff_score(DevParams p)
+{
+    wait_for_previous_kernel(); // the mean key
+    const int uid = blockIdx.y, slice = blockIdx.x;
+    const int h = uid % p.H, b = (uid / p.H) % p.B, l = uid / (p.H * p.B);
+    const int T = p.seq_lens[b];
+    if (T <= p.Tk || T > p.T_cap) return;
+    const int t_begin = slice * p.slice_len;
+    if (t_begin >= T) return;
+    const int t_end = min(T, t_begin + p.slice_len);
+    const int lane = threadIdx.x & 15, r = threadIdx.x >> 4;
+    const int *table = p.block_table + (size_t)b * p.bt_stride;
+    const float *fin = p.fin + (size_t)uid * (p.rows_pad + 8);
+    unsigned long long mu2[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) mu2[i] = pack_f32x2(fin[lane * 8 + 2 * i], fin[lane * 8 + 2 * i + 1]);
+    const float mu_norm = fin[kHeadDim];
+    float *g_out = p.scores + (size_t)uid * p.T_cap;
+    // four tokens per thread and round: their loads are issued together, so that enough bytes are in flight
+    constexpr int kU = 4;
+    const int n_iter = (t_end - t_begin + 16 * kU - 1) / (16 * kU);
+    for (int it = 0; it < n_iter; ++it) {
+        uint4 v[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int t = t_begin + (it * kU + u) * 16 + r;
+            v[u] = make_uint4(0, 0, 0, 0);
+            if (t < t_end) v[u] = ld_stream16(p.k_pages + row_offset(p, l, table[t >> 4], t & 15, h) + lane * 8);
+        }
+        // a[2u] = this lane's part of k_t . mu, a[2u + 1] of |k_t|^2, for the four tokens u
+        float a[2 * kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            // two dimensions per instruction: a bf16 pair widens to a packed fp32 pair (low half shifted up, high half
+            // masked), and both running sums take packed multiply-adds
+            const unsigned w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+            unsigned long long dot2 = 0ull, sq2 = 0ull; // (0.0f, 0.0f)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const unsigned long long k2 = pack_f32x2(bf16_lo(w[i]), bf16_hi(w[i]));
+                dot2 = fma_f32x2(k2, mu2[i], dot2);
+                sq2 = fma_f32x2(k2, k2, sq2);
+            }
+            a[2 * u] = sum_f32x2(dot2); a[2 * u + 1] = sum_f32x2(sq2);
+        }
+        // sums over the 16 lanes of a token row, all eight values at once: at each step a lane hands half of
+        // its values to its partner and keeps the other half (9 shuffles instead of 32)
+#pragma unroll
+        for (int o = 8, n = 2 * kU; o >= 2; o >>= 1, n >>= 1) {
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int i = 0; i < n / 2; ++i) {
+                const float send = up ? a[i] : a[i + n / 2];
+                const float keep = up ? a[i + n / 2] : a[i];
+                a[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+            }
+        }
+        a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+        // lane holds value index 4 * bit3 + 2 * bit2 + bit1: even = dot of token (index / 2), odd = its |k|^2
+        const float other = __shfl_xor_sync(0xffffffffu, a[0], 2);
+        if ((lane & 3) == 0) {
+            const int u = lane >> 2;
+            const int t = t_begin + (it * kU + u) * 16 + r;
+            if (t < t_end) g_out[t] = -a[0] / fmaxf(sqrtf(other) * mu_norm, 1e-30f);
+        }
+    }
+}
+
+int launch_apart(const DevParams &p, LaunchCtx &ctx)
+{
+    const dim3 grid((unsigned)p.n_slices, (unsigned)(p.L * p.B * p.H));
+    launch_after(k_keydiff_sum, grid, dim3(kApartThreads), 0, ctx.s, p);
+    ctx.mark(kKernScore1);
+    launch_after(k_keydiff_combine, dim3((unsigned)(p.L * p.B * p.H)), dim3(kHeadDim), 0, ctx.s, p);
+    ctx.mark(kKernScoreCombine);
+    launch_after(k_keydiff_score, grid, dim3(kApartThreads), 0, ctx.s, p);
+    ctx.mark(kKernScore2);
+    return cudaGetLastError() == cudaSuccess ? AMS_OK : AMS_ERR_CUDA;
+}
+
 } // namespace
 
 int launch_score_keydiff(const DevParams &p, LaunchCtx &ctx)
 {
+    if (p.independent) return launch_apart(p, ctx);
     const EncodeTiledFn enc = encode_fn();
     if (!enc) return AMS_ERR_CUDA;
     CUtensorMap k_map;
