@@ -32,6 +32,7 @@
 // us per event, three kernels of the mass, the quotas and the selection before / this one: 256 units of 16384 tokens
 // 118 / 59, 1792 ragged units of 8192..32768 tokens 683 / 379, 1792 units of 4224 tokens 253 / 145, 2048 units of 32768 tokens in
 // long segments 922 / 480, 640 units of 131072 tokens 1684 / 1130, 512 units of 7001..8191 tokens 127 / 54.
+#include <algorithm>
 #include <type_traits>
 
 #include "ams_common.cuh"
@@ -1327,6 +1328,8 @@ cudaError_t launch_nt(const DevParams &p, int units, bool longs, LaunchCtx &ctx)
     return launch_after(k_select_compact<NT>, dim3((unsigned)units), dim3(NT), smem, ctx.s, p, longs ? 1 : 0);
 }
 
+constexpr size_t kSmShared = 228 * 1024, kBlockReserve = 1024; // shared memory of an SM; what each block takes besides its own
+
 bool long_segments(const DevParams &p) { return p.l_max == 0 || p.l_max > kPiece; }
 
 } // namespace
@@ -1339,12 +1342,16 @@ int launch_segsel(const DevParams &p, LaunchCtx &ctx)
     if (n_sm <= 0) return AMS_ERR_CUDA;
     const bool longs = long_segments(p);
     // Threads per unit: a unit costs about (T / threads + a fixed part worth 24 tokens a thread), and the SMs' 1024 slots of 64
-    // registers make ceil(units / resident blocks) rounds of it.
-    auto cost = [&](long long nt) {
-        const long long rounds = ((long long)units * nt + 1024LL * n_sm - 1) / (1024LL * n_sm);
-        return rounds * (p.T_cap / nt + 24);
+    // registers and their shared memory (which grows with the capacity: 121 KB for 512 threads at 131072 tokens in long segments) make
+    // ceil(units / resident blocks) rounds of it.  160 units of 125840 tokens, l_max 4096: 512 threads by the registers alone 500 us,
+    // 1024 by both 384; 640 of 131072 take 1024 either way, since one block of 512 fits as well.  The host knows the
+    // capacity, not the lengths: rows far below it take the capacity's size (640 of 8704 tokens under 131072: 230 us).
+    auto cost = [&](int nt, size_t smem) {
+        const long long fit = std::max(1LL, std::min(1024LL / nt, (long long)(kSmShared / (smem + sizeof(SelShared) + kBlockReserve))));
+        return (units + fit * n_sm - 1) / (fit * n_sm) * (p.T_cap / nt + 24);
     };
-    const long long c256 = cost(256), c512 = cost(512), c1024 = cost(1024);
+    const long long c256 = cost(256, sel_smem<256>(p.T_cap, p.seg_cap, p.S, longs).total), c512 = cost(512, sel_smem<512>(p.T_cap, p.seg_cap, p.S, longs).total),
+                    c1024 = cost(1024, sel_smem<1024>(p.T_cap, p.seg_cap, p.S, longs).total);
     const cudaError_t e = c256 <= c512 && c256 <= c1024 ? launch_nt<256>(p, units, longs, ctx)
                         : c512 <= c1024 ? launch_nt<512>(p, units, longs, ctx) : launch_nt<1024>(p, units, longs, ctx);
     if (e != cudaSuccess) return AMS_ERR_CUDA;
