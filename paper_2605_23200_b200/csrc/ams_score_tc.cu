@@ -5,18 +5,16 @@
 // takes the contiguous tile range [g * tpc, (g + 1) * tpc) for all KV heads (one or more heads per block).  Inside a block:
 //   warp 0      TMA producer: query block of the current unit, then one 32 KB K tile per
 //               stage (eight 16-token pages, one 4 KB copy each, 128-byte swizzle);
-//   warps 1, 3  MMA issuers (one lane each, one per pair of consumer warpgroups, tiles in
-//               turn): per (tile, 128-row query block) eight tcgen05.mma m128 n128 k16 into
-//               one of four 128-column TMEM slots (two per pair, used in turn);
-//   warps 4-19  four consumer warpgroups in two pairs, the pairs alternating tiles; thread i
-//               of either warpgroup of a pair owns TMEM lane i of the pair's slots, the
-//               first warpgroup taking columns [0, 64) and the second [64, 128).  (Two
-//               warpgroups alone left each scheduler with two dependent instruction streams
-//               and the accumulators waiting for them; four hide that latency.)
+//   warps 1, 3  MMA issuers (one lane each, one per parity of the products): per product of a tile and a 128-row
+//               query block eight tcgen05.mma m128 n128 k16 into one of four 128-column TMEM slots, used in turn;
+//   warps 4-19  four consumer warpgroups, one per slot: thread i of a warpgroup owns TMEM lane i and takes all 128 columns, the next
+//               16 or 32 of them on their way while it works on the last.  (Two warpgroups to a slot with half of the columns each spent
+//               more on waits and hand-over, and had no registers left to fetch ahead: 512 rows, 640 units of 8704 tokens.
+//               statistics 963, now 875 us; usage 887, now 900; the event 2865, now 2782.)
 // Phase 1 puts query rows on the TMEM lanes (A = Q, B = K), so a thread folds its row's
 // logits into a running (max, sum of 2^x) without leaving registers; phase 2 puts tokens
 // on the lanes (A = K, B = Q), so a thread sums 2^(x - b_r) over the query rows of its
-// token (the two halves of the rows meet through shared memory).  Both operands are K-major 128-byte-swizzled tiles, so the same shared-memory
+// token (a tile's query blocks meet through shared memory).  Both operands are K-major 128-byte-swizzled tiles, so the same shared-memory
 // tiles serve either role.  Every wait is bounded; on expiry the block reports
 // AMS_ERR_TIMEOUT, drains its copies, frees its TMEM and returns.
 #include <cuda.h>
@@ -34,8 +32,8 @@ namespace {
 struct TcShared {
     unsigned long long kfull[kMaxStages], kempty[kMaxStages], tfull[kSlots], tempty[kSlots];
     unsigned long long qfull, qempty, done[2];
-    unsigned long long pfull[2][2];                  // usage pass: second half's partial sums are in pacc[pair][slot bit]
-    float pacc[2][2][128];
+    unsigned long long pfull[2], pempty[2];          // usage pass: the sums of a tile's earlier query blocks are in pacc; are used
+    float pacc[2][3][128];
     uint32_t tmem_base;
     int abort_flag;
     float wmax[2][16];
@@ -43,6 +41,7 @@ struct TcShared {
     long long n_tiles;
 };
 
+constexpr int kConsumerWarp = 4; // first warp of the consumers
 template <int PHASE>
 __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __grid_constant__ CUtensorMap k_map,
                                                            const __grid_constant__ CUtensorMap q_map)
@@ -60,9 +59,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
     volatile int *abort_flag = &sh.abort_flag;
 
     if (tid == 0) {
-        for (int i = 0; i < kMaxStages; ++i) { mbar_init(smem_u32(&sh.kfull[i]), 1); mbar_init(smem_u32(&sh.kempty[i]), 1); }
-        for (int i = 0; i < kSlots; ++i) { mbar_init(smem_u32(&sh.tfull[i]), 1); mbar_init(smem_u32(&sh.tempty[i]), 8); }
-        for (int i = 0; i < 4; ++i) mbar_init(smem_u32(&sh.pfull[i >> 1][i & 1]), 4);
+        for (int i = 0; i < kMaxStages; ++i) { mbar_init(smem_u32(&sh.kfull[i]), 1); mbar_init(smem_u32(&sh.kempty[i]), n_rb > 1 ? 2 : 1); }
+        for (int i = 0; i < kSlots; ++i) { mbar_init(smem_u32(&sh.tfull[i]), 1); mbar_init(smem_u32(&sh.tempty[i]), 4); }
+        for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&sh.pfull[i]), (uint32_t)(n_rb > 1 ? 4 * (n_rb - 1) : 1)); mbar_init(smem_u32(&sh.pempty[i]), 4); }
         mbar_init(smem_u32(&sh.qfull), 1);
         mbar_init(smem_u32(&sh.qempty), 2); // both MMA issuers release the query block
         mbar_init(smem_u32(&sh.done[0]), 1);
@@ -150,26 +149,25 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
             }
         } else if (warp == 1 || warp == 3) {
             // ------------------------------------------------------------ MMA issuers
-            // One thread per consumer pair, taking the tiles in turn: a tile costs its issuer a
-            // chain of long waits (two barriers, eight MMAs, two commits) that is longer than the
-            // tile's share of the HBM stream, so a single issuer would be the bottleneck.
+            // One thread per parity of the (tile, query block) products: a product costs its issuer a chain of long waits (two
+            // barriers, eight MMAs, two commits) that is longer than its share of the HBM stream, so a single issuer
+            // would be the bottleneck.
             if (lane == 0) {
-                const int wg = warp >> 1; // issuer 0 feeds consumer pair 0 (even tiles), issuer 1 pair 1
-                int kit = 0, seg = 0, wsit = 0; // wsit: accumulator slots handed to the warpgroup so far
+                const int wg = warp >> 1;
+                int kit = 0, seg = 0;
                 bool ok = true;
                 for (long long gv = 0; gv < g_span * hpb && ok;) {
-                const int my_h = my_h0 + (int)(gv / g_span) * my_hs;
-                const long long g = g_begin + gv % g_span;
+                    const int my_h = my_h0 + (int)(gv / g_span) * my_hs;
+                    const long long g = g_begin + gv % g_span;
                     const Segment s = decode_segment(p, prefix, tiles_lh, tpc, g, g_end, my_h);
                     ok = mbar_wait(smem_u32(&sh.qfull), (uint32_t)(seg & 1), abort_flag);
                     for (int i = 0; i < s.n && ok; ++i, ++kit) {
-                        if ((kit & 1) != wg) continue;
+                        if (n_rb == 1 && (kit & 1) != wg) continue;
                         const int st = kit % NS;
                         ok = mbar_wait(smem_u32(&sh.kfull[st]), (uint32_t)((kit / NS) & 1), abort_flag);
-                        for (int rb = 0; rb < n_rb && ok; ++rb, ++wsit) {
-                            // warpgroup wg owns slots 2 wg and 2 wg + 1, used in turn
-                            const int slot = 2 * wg + (wsit & 1);
-                            ok = mbar_wait(smem_u32(&sh.tempty[slot]), (uint32_t)(((wsit >> 1) & 1) ^ 1), abort_flag);
+                        for (int rb = (kit * n_rb + wg) & 1; rb < n_rb && ok; rb += 2) {
+                            const int q = kit * n_rb + rb, slot = q & 3;
+                            ok = mbar_wait(smem_u32(&sh.tempty[slot]), (uint32_t)(((q >> 2) & 1) ^ 1), abort_flag);
                             if (!ok) break;
                             tc_fence_after();
                             const uint32_t qa = smem_u32(Qs + (size_t)rb * kTileBytes), ka = smem_u32(Ks + (size_t)st * kTileBytes);
@@ -194,13 +192,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
                     if (mbar_try_wait(smem_u32(&sh.done[wg]), 0)) break;
             }
             __syncwarp();
-        } else if (warp >= 4) {
+        } else if (warp >= kConsumerWarp) {
             // ------------------------------------------------------------ consumers
-            // Four warpgroups.  Warpgroups (pair, 0) and (pair, 1) share the tiles of one pair (tiles in
-            // turn between the two pairs): thread li of either owns TMEM lane li, the first takes
-            // columns [0, 64) of the slot and the second columns [64, 128).
-            const int wgq = (warp - 4) >> 2, pair = wgq & 1, half = wgq >> 1, quad = warp & 3, li = quad * 32 + lane;
-            int kit = 0, wsit = 0, seg = 0, pc0 = 0, pc1 = 0; // pc*: uses so far of this pair's two hand-over barriers
+            // Product number q = tile * n_rb + query block goes to warpgroup and slot q % 4: thread li of it owns TMEM lane li and
+            // all 128 columns.
+            const int wgq = (warp - kConsumerWarp) >> 2, quad = warp & 3, li = quad * 32 + lane;
+            int kit = 0, seg = 0;
             bool ok = true;
             // a thread whose wait ran out keeps walking the segments without touching the pipeline, so that
             // the consumers' named barriers stay matched
@@ -231,140 +228,142 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
                     const long long ustart = g - s.tile0;
                     const int n_parts = (int)((ustart + nt_u - 1) / tpc) - (int)(ustart / tpc) + 1;
                     float best = 0.0f;
-                    for (int r = (warp - 4) * 32 + lane; r < p.rows_pad; r += kConsumerThreads) {
+                    for (int r = (warp - kConsumerWarp) * 32 + lane; r < p.rows_pad; r += kConsumerThreads) {
                         float mm = -INFINITY, zz = 0.0f;
                         for (int q = 0; q < n_parts; ++q) {
                             const float2 v = __ldcg(reinterpret_cast<const float2 *>(p.part) + ((size_t)s.uid * p.n_slices + q) * p.rows_pad + r);
                             lse_merge(mm, zz, v.x, v.y);
                         }
                         const bool live = r < p.rows && zz > 0.0f;
-                        fs[r] = live ? mm + log2f(zz) : INFINITY; // padding rows contribute nothing
+                        fs[r] = live ? -(mm + log2f(zz)) : -INFINITY; // padding rows contribute nothing
                         if (live) best = fmaxf(best, 1.0f / zz);
                     }
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-                    if (lane == 0) sh.wmax[seg & 1][warp - 4] = best;
+                    if (lane == 0) sh.wmax[seg & 1][warp - kConsumerWarp] = best;
                     asm volatile("bar.sync 1, %0;" ::"n"(kConsumerThreads) : "memory");
 #pragma unroll
                     for (int w = 0; w < kConsumerThreads / 32; ++w) pmax = fmaxf(pmax, sh.wmax[seg & 1][w]);
                 }
                 for (int i = 0; i < s.n && ok; ++i, ++kit) {
-                    if ((kit & 1) != pair) continue;
                     const int t0 = (s.tile0 + i) * kTileTokens;
-                    float acc = 0.0f;
-                    int last_slot = 0;
-                    for (int rb = 0; rb < n_rb && ok; ++rb, ++wsit) {
-                        const int slot = 2 * pair + (wsit & 1);
-                        last_slot = slot;
-                        ok = mbar_wait(smem_u32(&sh.tfull[slot]), (uint32_t)((wsit >> 1) & 1), abort_flag);
+                    for (int rb = (wgq - kit * n_rb) & 3; rb < n_rb && ok; rb += 4) {
+                        const int slot = wgq;
+                        const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(slot * 128);
+                        ok = mbar_wait(smem_u32(&sh.tfull[slot]), (uint32_t)(((kit * n_rb + rb) >> 2) & 1), abort_flag);
+                        ok = __all_sync(0xffffffffu, ok) != 0; // one answer per warp: what follows is warp-wide
                         if (!ok) break;
                         tc_fence_after();
-                        const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(slot * 128 + half * 64);
+                        // the slot is free again as soon as its last columns are in registers
+                        auto release = [&]() {
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(smem_u32(&sh.tempty[slot]));
+                        };
                         if (PHASE == 1) {
-                            // 32 columns at a time: one running-maximum update (one rescaling exponential) per 32 logits, and
-                            // the maximum tree of one half can overlap the exponentials of the other
+                            // 32 columns at a time, the next 32 on their way meanwhile: one running-maximum update (one rescaling
+                            // exponential) per 32 logits
                             const int lv = min(lastv[rb], T - 1);
                             float mr = m[rb], zr = z[rb];
-                            uint32_t d[32];
-                            tc_ld32_issue(taddr, d);
+                            uint32_t d[2][32];
+                            tc_ld32_issue(taddr, d[0]);
 #pragma unroll
-                            for (int ch = 0; ch < 2; ++ch) {
-                                tc_ld_wait(d);
-                                float v[32];
-#pragma unroll
-                                for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(d[j]);
-                                if (ch == 0) tc_ld32_issue(taddr + 32, d);
-                                const int tc0 = t0 + half * 64 + ch * 32;
+                            for (int ch = 0; ch < 4; ++ch) {
+                                uint32_t (&x)[32] = d[ch & 1];
+                                tc_ld_wait(x);
+                                if (ch < 3) tc_ld32_issue(taddr + (uint32_t)(32 * ch + 32), d[1 - (ch & 1)]);
+                                else release();
+                                auto v = [&](int j) { return __uint_as_float(x[j]); };
+                                const int tc0 = t0 + ch * 32;
                                 if (tc0 <= lv) {
                                     if (tc0 + 31 > lv) {
 #pragma unroll
-                                        for (int j = 0; j < 32; ++j) if (tc0 + j > lv) v[j] = -INFINITY;
+                                        for (int j = 0; j < 32; ++j) if (tc0 + j > lv) x[j] = 0xff800000u; // -infinity
                                     }
                                     // tree of three-input maxima
                                     float a[11];
 #pragma unroll
-                                    for (int j = 0; j < 10; ++j) a[j] = max3(v[3 * j], v[3 * j + 1], v[3 * j + 2]);
-                                    a[10] = fmaxf(v[30], v[31]);
+                                    for (int j = 0; j < 10; ++j) a[j] = max3(v(3 * j), v(3 * j + 1), v(3 * j + 2));
+                                    a[10] = fmaxf(v(30), v(31));
                                     const float b0 = max3(a[0], a[1], a[2]), b1 = max3(a[3], a[4], a[5]), b2 = max3(a[6], a[7], a[8]);
                                     const float cm = fmaxf(max3(b0, b1, b2), fmaxf(a[9], a[10]));
                                     const float mn = fmaxf(mr, cm * c);
                                     zr *= ex2(mr - mn);
                                     mr = mn;
-                                    float zs[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                                    u64 zs[2] = {0, 0}; // (0.0f, 0.0f)
+                                    const u64 c2 = pack_f32x2(c, c), n2 = pack_f32x2(-mn, -mn);
 #pragma unroll
-                                    for (int j = 0; j < 32; ++j) zs[j & 3] += ex2(fmaf(v[j], c, -mn));
-                                    zr += (zs[0] + zs[1]) + (zs[2] + zs[3]);
+                                    for (int j = 0; j < 32; j += 2) {
+                                        const float2 e = ex2_pair(fma_f32x2(pack_f32x2(v(j), v(j + 1)), c2, n2));
+                                        zs[(j >> 1) & 1] = add_f32x2(zs[(j >> 1) & 1], pack_f32x2(e.x, e.y));
+                                    }
+                                    zr += sum_f32x2(add_f32x2(zs[0], zs[1]));
                                 }
                             }
                             m[rb] = mr; z[rb] = zr;
                         } else {
                             const int t = t0 + li;
-                            const bool plain = !p.causal || t0 + kTileTokens - 1 <= T - p.W;
-                            const float4 *fr4 = reinterpret_cast<const float4 *>(fs + rb * 128 + half * 64);
-                            float ac[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-                            uint32_t d[32];
-                            tc_ld32_issue(taddr, d);
+                            const bool plain = !p.causal || t0 + kTileTokens - 1 <= T - p.W; // every row sees every token
+                            const float4 *fr4 = reinterpret_cast<const float4 *>(fs + rb * 128);
+                            const u64 c2 = pack_f32x2(c, c);
+                            u64 ac[2] = {0, 0}; // (0.0f, 0.0f)
+                            uint32_t d[2][16];
+                            tc_ld16_issue(taddr, d[0]);
 #pragma unroll
-                            for (int ch = 0; ch < 2; ++ch) { // 32 columns (query rows) at a time
-                                tc_ld_wait(d);
+                            for (int ch = 0; ch < 8; ++ch) { // 16 columns (query rows) at a time, the next 16 on their way meanwhile
+                                uint32_t (&x)[16] = d[ch & 1];
+                                tc_ld16_wait(x);
+                                if (ch < 7) tc_ld16_issue(taddr + (uint32_t)(16 * ch + 16), d[1 - (ch & 1)]);
+                                else release();
                                 if (plain) {
 #pragma unroll
-                                    for (int j4 = 0; j4 < 8; ++j4) {
-                                        const float4 f = fr4[ch * 8 + j4];
-                                        ac[0] += ex2(fmaf(__uint_as_float(d[4 * j4]), c, -f.x));
-                                        ac[1] += ex2(fmaf(__uint_as_float(d[4 * j4 + 1]), c, -f.y));
-                                        ac[2] += ex2(fmaf(__uint_as_float(d[4 * j4 + 2]), c, -f.z));
-                                        ac[3] += ex2(fmaf(__uint_as_float(d[4 * j4 + 3]), c, -f.w));
+                                    for (int j4 = 0; j4 < 4; ++j4) {
+                                        const float4 f = fr4[ch * 4 + j4];
+                                        const float2 e0 = ex2_pair(fma_f32x2(pack_f32x2(__uint_as_float(x[4 * j4]), __uint_as_float(x[4 * j4 + 1])), c2, pack_f32x2(f.x, f.y)));
+                                        const float2 e1 = ex2_pair(fma_f32x2(pack_f32x2(__uint_as_float(x[4 * j4 + 2]), __uint_as_float(x[4 * j4 + 3])), c2, pack_f32x2(f.z, f.w)));
+                                        ac[0] = add_f32x2(ac[0], pack_f32x2(e0.x, e0.y));
+                                        ac[1] = add_f32x2(ac[1], pack_f32x2(e1.x, e1.y));
                                     }
                                 } else {
-                                    const int rbase = rb * 128 + half * 64 + ch * 32;
+                                    const int rbase = rb * 128 + ch * 16;
 #pragma unroll
-                                    for (int j = 0; j < 32; ++j) {
-                                        const int r = rbase + j;
-                                        const bool seen = t <= T - p.W + (r % p.W);
-                                        ac[j & 3] += seen ? ex2(fmaf(__uint_as_float(d[j]), c, -fs[r])) : 0.0f;
+                                    for (int j = 0; j < 16; j += 2) {
+                                        float e[2];
+#pragma unroll
+                                        for (int i2 = 0; i2 < 2; ++i2) {
+                                            const int r = rbase + j + i2;
+                                            const bool seen = t <= T - p.W + (r % p.W);
+                                            e[i2] = seen ? ex2(fmaf(__uint_as_float(x[j + i2]), c, fs[r])) : 0.0f;
+                                        }
+                                        ac[(j >> 1) & 1] = add_f32x2(ac[(j >> 1) & 1], pack_f32x2(e[0], e[1]));
                                     }
                                 }
-                                if (ch == 0) tc_ld32_issue(taddr + 32, d);
                             }
-                            acc += (ac[0] + ac[1]) + (ac[2] + ac[3]);
-                        }
-                        if (PHASE == 2 && rb == n_rb - 1) break; // the slot of a tile's last query block is released below
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&sh.tempty[slot]));
-                    }
-                    if (PHASE == 2 && ok) {
-                        // The two halves of the query rows meet here: the second warpgroup leaves its sum in shared
-                        // memory, the first adds it and writes the token's usage.  The buffer is the one of the slot,
-                        // and the first warpgroup releases the slot only after reading it, so the next tile that
-                        // maps to this slot cannot overwrite it early.
-                        ++wsit; // (the loop above left through its break)
-                        const int bit = last_slot & 1;
-                        float *pa = sh.pacc[pair][bit];
-                        const uint32_t pbar = smem_u32(&sh.pfull[pair][bit]);
-                        if (half == 1) {
-                            pa[li] = acc;
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) { mbar_arrive(pbar); mbar_arrive(smem_u32(&sh.tempty[last_slot])); }
-                        } else {
-                            ok = mbar_wait(pbar, (uint32_t)((bit ? pc1 : pc0) & 1), abort_flag);
-                            if (ok) {
-                                acc += pa[li];
-                                const int t = t0 + li;
-                                // the slot is released before the usage goes to global memory: an arrive (a release) issued
-                                // after the store would wait until the store has been performed
-                                tc_fence_before();
+                            float acc = sum_f32x2(add_f32x2(ac[0], ac[1]));
+                            // a tile's query blocks meet in the warpgroup that has the last one
+                            const int buf = kit & 1;
+                            if (rb < n_rb - 1) {
+                                ok = mbar_wait(smem_u32(&sh.pempty[buf]), (uint32_t)(((kit >> 1) & 1) ^ 1), abort_flag);
+                                ok = __all_sync(0xffffffffu, ok) != 0;
+                                if (!ok) break;
+                                sh.pacc[buf][rb][li] = acc;
                                 __syncwarp();
-                                if (lane == 0) mbar_arrive(smem_u32(&sh.tempty[last_slot]));
+                                if (lane == 0) mbar_arrive(smem_u32(&sh.pfull[buf]));
+                            } else {
+                                if (n_rb > 1) {
+                                    ok = mbar_wait(smem_u32(&sh.pfull[buf]), (uint32_t)((kit >> 1) & 1), abort_flag);
+                                    ok = __all_sync(0xffffffffu, ok) != 0;
+                                    if (!ok) break;
+                                    for (int o = 0; o < n_rb - 1; ++o) acc += sh.pacc[buf][o][li];
+                                    __syncwarp();
+                                    if (lane == 0) mbar_arrive(smem_u32(&sh.pempty[buf]));
+                                }
                                 if (t < T) {
                                     const int ninv = p.causal ? p.G * max(0, t - (T - p.W)) : 0;
                                     p.scores[(size_t)s.uid * p.T_cap + t] = (acc + (float)ninv * pmax) * (1.0f / (float)p.rows);
                                 }
                             }
                         }
-                        if (bit) ++pc1; else ++pc0;
                     }
                 }
                 if (PHASE == 1) {
