@@ -7,8 +7,8 @@
 //               stage (eight 16-token pages, one 4 KB copy each, 128-byte swizzle);
 //   warps 1, 3  MMA issuers (one lane each, one per parity of the products): per product of a tile and a 128-row
 //               query block eight tcgen05.mma m128 n128 k16 into one of four 128-column TMEM slots, used in turn;
-//   warps 4-19  four consumer warpgroups, one per slot: thread i of a warpgroup owns TMEM lane i and takes all 128 columns, the next
-//               16 or 32 of them on their way while it works on the last.  (Two warpgroups to a slot with half of the columns each spent
+//   warps 4-19  four consumer warpgroups, one per slot: thread i of a warpgroup owns TMEM lane i and takes all 128 columns, in the
+//               first phase the next 32 on their way while it works on the last.  (Two warpgroups to a slot with half of the columns each spent
 //               more on waits and hand-over, and had no registers left to fetch ahead: 512 rows, 640 units of 8704 tokens.
 //               statistics 963, now 875 us; usage 887, now 900; the event 2865, now 2782.)
 // Phase 1 puts query rows on the TMEM lanes (A = Q, B = K), so a thread folds its row's
@@ -106,20 +106,25 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
                 const int my_h = my_h0 + (int)(gv / g_span) * my_hs;
                 const long long g = g_begin + gv % g_span;
                 const Segment s = decode_segment(p, prefix, tiles_lh, tpc, g, g_end, my_h);
-                ok = mbar_wait(smem_u32(&sh.qempty), (uint32_t)((seg & 1) ^ 1), abort_flag);
-                if (!ok) break;
-                if (lane == 0) {
-                    mbar_expect_tx(smem_u32(&sh.qfull), (uint32_t)(n_rb * kTileBytes));
-                    const int qrow0 = ((s.l * p.B + s.b) * p.H * p.G + s.h * p.G) * p.W;
-                    for (int rb = 0; rb < n_rb; ++rb)
-                        for (int hf = 0; hf < 2; ++hf)
-                            tma_load_2d(smem_u32(Qs + (size_t)rb * kTileBytes + hf * kHalfBytes), &q_map, smem_u32(&sh.qfull),
-                                        hf * 64, qrow0 + rb * 128);
-                }
-                blocks_issued = seg + 1;
                 const int *table = p.block_table + (size_t)s.b * p.bt_stride;
                 const int last_page = (s.T - 1) >> 4;
                 for (int i = 0; i < s.n && ok; ++i, ++kit) {
+                    // The query block goes behind the unit's first K tiles: it waits for the products of the unit before, they only
+                    // for a stage each, and the K stream runs on.  (A tile whose stage an earlier one of the same unit holds needs
+                    // those products, so no later than before the last of NS.)
+                    if (i == min(NS, s.n) - 1) {
+                        ok = mbar_wait(smem_u32(&sh.qempty), (uint32_t)((seg & 1) ^ 1), abort_flag);
+                        if (!ok) break;
+                        if (lane == 0) {
+                            mbar_expect_tx(smem_u32(&sh.qfull), (uint32_t)(n_rb * kTileBytes));
+                            const int qrow0 = ((s.l * p.B + s.b) * p.H * p.G + s.h * p.G) * p.W;
+                            for (int rb = 0; rb < n_rb; ++rb)
+                                for (int hf = 0; hf < 2; ++hf)
+                                    tma_load_2d(smem_u32(Qs + (size_t)rb * kTileBytes + hf * kHalfBytes), &q_map, smem_u32(&sh.qfull),
+                                                hf * 64, qrow0 + rb * 128);
+                        }
+                        blocks_issued = seg + 1;
+                    }
                     const int st = kit % NS;
                     ok = mbar_wait(smem_u32(&sh.kempty[st]), (uint32_t)(((kit / NS) & 1) ^ (p.expire_polls ? 0 : 1)), abort_flag,
                                    p.expire_polls ? p.expire_polls : kWaitLimit);
@@ -206,14 +211,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
                 const long long g = g_begin + gv % g_span;
                 const Segment s = decode_segment(p, prefix, tiles_lh, tpc, g, g_end, my_h);
                 const int T = s.T;
-                float m[4], z[4];
+                float m[4], z[4], lost[4]; // lost: what rounding has added to z so far (Kahan)
                 int lastv[4];
                 float *fs = fin_s + (seg & 1) * p.rows_pad;
                 float pmax = 0.0f;
                 if (PHASE == 1) {
 #pragma unroll
                     for (int rb = 0; rb < 4; ++rb) {
-                        m[rb] = -INFINITY; z[rb] = 0.0f;
+                        m[rb] = -INFINITY; z[rb] = lost[rb] = 0.0f;
                         const int r = rb * 128 + li;
                         lastv[rb] = r < p.rows ? (p.causal ? T - p.W + (r % p.W) : T - 1) : -1;
                     }
@@ -264,7 +269,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
                             // 32 columns at a time, the next 32 on their way meanwhile: one running-maximum update (one rescaling
                             // exponential) per 32 logits
                             const int lv = min(lastv[rb], T - 1);
-                            float mr = m[rb], zr = z[rb];
+                            float mr = m[rb], zr = z[rb], zl = lost[rb];
                             uint32_t d[2][32];
                             tc_ld32_issue(taddr, d[0]);
 #pragma unroll
@@ -288,7 +293,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
                                     const float b0 = max3(a[0], a[1], a[2]), b1 = max3(a[3], a[4], a[5]), b2 = max3(a[6], a[7], a[8]);
                                     const float cm = fmaxf(max3(b0, b1, b2), fmaxf(a[9], a[10]));
                                     const float mn = fmaxf(mr, cm * c);
-                                    zr *= ex2(mr - mn);
+                                    const float down = ex2(mr - mn);
+                                    zr *= down;
+                                    zl *= down;
                                     mr = mn;
                                     u64 zs[2] = {0, 0}; // (0.0f, 0.0f)
                                     const u64 c2 = pack_f32x2(c, c), n2 = pack_f32x2(-mn, -mn);
@@ -297,47 +304,49 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
                                         const float2 e = ex2_pair(fma_f32x2(pack_f32x2(v(j), v(j + 1)), c2, n2));
                                         zs[(j >> 1) & 1] = add_f32x2(zs[(j >> 1) & 1], pack_f32x2(e.x, e.y));
                                     }
-                                    zr += sum_f32x2(add_f32x2(zs[0], zs[1]));
+                                    // compensated: a thread adds up to 4096 such sums
+                                    const float more = __fsub_rn(sum_f32x2(add_f32x2(zs[0], zs[1])), zl), sum = __fadd_rn(zr, more);
+                                    zl = __fsub_rn(__fsub_rn(sum, zr), more);
+                                    zr = sum;
                                 }
                             }
-                            m[rb] = mr; z[rb] = zr;
+                            m[rb] = mr; z[rb] = zr; lost[rb] = zl;
                         } else {
                             const int t = t0 + li;
                             const bool plain = !p.causal || t0 + kTileTokens - 1 <= T - p.W; // every row sees every token
                             const float4 *fr4 = reinterpret_cast<const float4 *>(fs + rb * 128);
                             const u64 c2 = pack_f32x2(c, c);
                             u64 ac[2] = {0, 0}; // (0.0f, 0.0f)
-                            uint32_t d[2][16];
-                            tc_ld16_issue(taddr, d[0]);
+                            uint32_t d[32];
+                            tc_ld32_issue(taddr, d);
 #pragma unroll
-                            for (int ch = 0; ch < 8; ++ch) { // 16 columns (query rows) at a time, the next 16 on their way meanwhile
-                                uint32_t (&x)[16] = d[ch & 1];
-                                tc_ld16_wait(x);
-                                if (ch < 7) tc_ld16_issue(taddr + (uint32_t)(16 * ch + 16), d[1 - (ch & 1)]);
-                                else release();
+                            for (int ch = 0; ch < 4; ++ch) { // 32 columns (query rows) at a time
+                                tc_ld_wait(d);
+                                if (ch == 3) release();
                                 if (plain) {
 #pragma unroll
-                                    for (int j4 = 0; j4 < 4; ++j4) {
-                                        const float4 f = fr4[ch * 4 + j4];
-                                        const float2 e0 = ex2_pair(fma_f32x2(pack_f32x2(__uint_as_float(x[4 * j4]), __uint_as_float(x[4 * j4 + 1])), c2, pack_f32x2(f.x, f.y)));
-                                        const float2 e1 = ex2_pair(fma_f32x2(pack_f32x2(__uint_as_float(x[4 * j4 + 2]), __uint_as_float(x[4 * j4 + 3])), c2, pack_f32x2(f.z, f.w)));
+                                    for (int j4 = 0; j4 < 8; ++j4) {
+                                        const float4 f = fr4[ch * 8 + j4];
+                                        const float2 e0 = ex2_pair(fma_f32x2(pack_f32x2(__uint_as_float(d[4 * j4]), __uint_as_float(d[4 * j4 + 1])), c2, pack_f32x2(f.x, f.y)));
+                                        const float2 e1 = ex2_pair(fma_f32x2(pack_f32x2(__uint_as_float(d[4 * j4 + 2]), __uint_as_float(d[4 * j4 + 3])), c2, pack_f32x2(f.z, f.w)));
                                         ac[0] = add_f32x2(ac[0], pack_f32x2(e0.x, e0.y));
                                         ac[1] = add_f32x2(ac[1], pack_f32x2(e1.x, e1.y));
                                     }
                                 } else {
-                                    const int rbase = rb * 128 + ch * 16;
+                                    const int rbase = rb * 128 + ch * 32;
 #pragma unroll
-                                    for (int j = 0; j < 16; j += 2) {
+                                    for (int j = 0; j < 32; j += 2) {
                                         float e[2];
 #pragma unroll
                                         for (int i2 = 0; i2 < 2; ++i2) {
                                             const int r = rbase + j + i2;
                                             const bool seen = t <= T - p.W + (r % p.W);
-                                            e[i2] = seen ? ex2(fmaf(__uint_as_float(x[j + i2]), c, fs[r])) : 0.0f;
+                                            e[i2] = seen ? ex2(fmaf(__uint_as_float(d[j + i2]), c, fs[r])) : 0.0f;
                                         }
                                         ac[(j >> 1) & 1] = add_f32x2(ac[(j >> 1) & 1], pack_f32x2(e[0], e[1]));
                                     }
                                 }
+                                if (ch < 3) tc_ld32_issue(taddr + (uint32_t)(32 * ch + 32), d);
                             }
                             float acc = sum_f32x2(add_f32x2(ac[0], ac[1]));
                             // a tile's query blocks meet in the warpgroup that has the last one
