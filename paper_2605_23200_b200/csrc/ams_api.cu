@@ -8,7 +8,7 @@
 namespace ams {
 
 struct Layout {
-    size_t status, eff_lens, seq_bad, scores, usage, ex_logits, n_seg, seg_bounds, quotas, keep_idx, part, fin, group_count, group_part, total;
+    size_t status, eff_lens, seq_bad, scores, usage, ex_logits, n_seg, seg_bounds, quotas, keep_idx, part, fin, group_count, group_part, move_count, src_pages, total;
     int units, T_cap, seg_cap, n_slices, slice_len, rows_pad_cap;
 };
 
@@ -101,6 +101,8 @@ static Layout make_layout(const ams_config *c)
     y.ex_logits = off;  off = align_up(off + (c->expected_scorer ? U * T * (size_t)(c->n_q_heads / c->n_kv_heads) * 4 : 0), 256);
     y.group_count = off; off = align_up(off + (size_t)2 * kGroupCounters * kGroupCounterPad * 4, 256);
     y.group_part = off;  off = align_up(off + (size_t)kGroupBlocks * 4 * kGroupSlot, 256);
+    y.move_count = off;  off = align_up(off + ((size_t)c->n_layers * c->max_batch + 2) * 4, 256);
+    y.src_pages = off;   off = align_up(off + (size_t)c->max_batch * (y.T_cap / kPage) * 4, 256);
     y.total = off;
     return y;
 }
@@ -266,6 +268,9 @@ int ams_compress(ams_state *st, void *k_pages, void *v_pages, int64_t num_pages,
     p.seg_out = dbg && (dbg->n_segments || dbg->seg_bounds || dbg->quotas || dbg->keep_idx);
     p.part = (float *)(st->ws + y.part); p.fin = (float *)(st->ws + y.fin);
     p.group_count = (int *)(st->ws + y.group_count); p.group_part = st->ws + y.group_part;
+    p.move_count = (int *)(st->ws + y.move_count);
+    p.src_pages = (int *)(st->ws + y.src_pages);
+    p.rewrite = dbg ? 0 : 1;
     p.slice_len = y.slice_len; p.n_slices = y.n_slices;
     p.rows_pad = scorer_id == AMS_SCORER_TOVA ? rows_padded(p.rows) : kHeadDim;
     p.tc_tpc_min = tc_tiles_per_block_min(y.T_cap);
@@ -308,14 +313,15 @@ int ams_compress(ams_state *st, void *k_pages, void *v_pages, int64_t num_pages,
         rc = launch_smooth_usage(p, p.usage, usage_buf, c.pool_kernel, ctx);
         p.usage = usage_buf;
     }
-    if (rc == AMS_OK) rc = segsel_supported(p) ? launch_segsel(p, ctx) : AMS_ERR_UNSUPPORTED;
+    bool moved = false;
+    if (rc == AMS_OK) rc = segsel_supported(p) ? launch_segsel(p, ctx, dbg ? nullptr : &moved) : AMS_ERR_UNSUPPORTED;
     if (rc == AMS_OK && dbg) {
         // inspection copies are taken before the table is rewritten
         if (dbg->scores || dbg->usage) rc = launch_inspect_scores(p, *dbg, ctx);
         if (rc == AMS_OK && p.seg_out) rc = launch_inspect(p, *dbg, ctx);
         if (rc == AMS_OK && dbg->prev_kept && dbg->retained_iou) rc = launch_retained_iou(p, dbg->prev_kept, dbg->retained_iou, ctx);
     }
-    if (rc == AMS_OK) rc = launch_gather(p, ctx);
+    if (rc == AMS_OK && !moved) rc = launch_gather(p, ctx);
     st->last_launches = ctx.launches;
     st->n_ev = ctx.n_ev;
     memcpy(st->ev_ids, ctx.ids, sizeof ctx.ids);

@@ -42,6 +42,8 @@ struct DevParams {
     const __nv_bfloat16 *q;           // [L][B][H*G][W][128]
     float *ema;                       // [L][Bmax][H][T_cap]
     const int *dst_pages;             // [B][n_dst]
+    int *src_pages;                   // [B][T_cap / 16] the pages of what is compressed, as the event found them (workspace)
+    int rewrite;                      // the row moves rewrite the block table as well
     // per-unit working arrays, [L*B*H][...]
     const float *usage;               // u: what the mass is built from
     float *scores;                    // g: what segments rank by (== usage unless external)
@@ -68,6 +70,8 @@ struct DevParams {
     int group_size;                   // blocks that work on a unit together: their number if the launcher sets it (a cluster);
     int *group_count;                 // counters, cleared by the first kernel of an event,
     unsigned char *group_part;        // and the slots of what they exchange
+    int *move_count;                  // ticket counter, parts of the row moves finished, and per (layer, sequence) the units selected;
+                                      // cleared by the first kernel of an event
     int *seq_bad;                     // [B]: set when a unit of the sequence, or for all of them a scorer, reported a device-side
                                       // error: what follows leaves the sequence as it is
     int *status;                      // [4]: code, unit, a, b
@@ -327,7 +331,8 @@ int launch_score_keydiff(const DevParams &p, LaunchCtx &ctx);
 bool expected_supported(const DevParams &p);
 int launch_score_expected(const DevParams &p, LaunchCtx &ctx);
 bool segsel_supported(const DevParams &p);   // shared-memory need of the selection kernels fits (always, within the configuration limits)
-int launch_segsel(const DevParams &p, LaunchCtx &ctx); // Algorithm 1 steps 1-5
+// Algorithm 1 steps 1-5; with `moved` given, row moves and block table too where that is the better way (then true)
+int launch_segsel(const DevParams &p, LaunchCtx &ctx, bool *moved);
 int launch_gather(const DevParams &p, LaunchCtx &ctx);
 int launch_smooth_usage(const DevParams &p, const float *src, float *dst, int k, LaunchCtx &ctx);
 // First kernel of an event: validates lengths and page ids, writes the effective lengths (lens_in: the caller's).

@@ -1,7 +1,7 @@
 // Paged head-wise compaction: K_new[pi_new(b, j), h, :] <- K_old[pi_old(b, I[b,h,j]), h, :]
 // and the same for V (the two display equations of the paper's paged-KV appendix),
 // followed by the block-table row and sequence-length rewrite of its runtime routine.
-#include "ams_common.cuh"
+#include "ams_move.cuh"
 
 namespace ams {
 
@@ -21,10 +21,12 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(DevParams p)
     const int b = lb % p.B, l = lb / p.B;
     const int T = p.seq_lens[b];
     if (T <= p.Tk || T > p.T_cap || p.seq_bad[b]) return;
+    // (nobody reads the block table any more: the rows are found by the event's copy of it)
+    if (p.rewrite && blockIdx.x == 0 && l == 0) update_table(p, b);
     const int n_rows = p.Tk * p.H;
     const int lane = threadIdx.x & 15, rsub = threadIdx.x >> 4;
     const int r0 = blockIdx.x * kRowsPerBlock + rsub;
-    const int *table = p.block_table + (size_t)b * p.bt_stride;
+    const int *table = p.src_pages + (size_t)b * (p.T_cap / kPage);
     const int *dst = p.dst_pages + (size_t)b * p.n_dst;
     const int *keep_base = p.keep_idx + (size_t)(l * p.B + b) * p.H * p.Tk;
 
@@ -53,19 +55,14 @@ __global__ void __launch_bounds__(kGatherThreads) k_gather(DevParams p)
     }
 }
 
-// Block-table row <- replacement pages followed by -1; length <- budget.  Runs after
-// every kernel that reads the old table.
+// The rewrite in a launch of its own, for events with views.
 __global__ void k_table_update(DevParams p)
 {
     wait_for_previous_kernel(); // the gather kernel reads the table this kernel rewrites
     const int b = blockIdx.x;
     const int T = p.seq_lens[b];
     if (T <= p.Tk || T > p.T_cap || p.seq_bad[b]) return;
-    int *row = p.block_table + (size_t)b * p.bt_stride;
-    for (int i = threadIdx.x; i < p.bt_stride; i += blockDim.x)
-        row[i] = i < p.n_dst ? p.dst_pages[(size_t)b * p.n_dst + i] : -1;
-    __syncthreads();
-    if (threadIdx.x == 0) p.seq_lens_out[b] = p.Tk;
+    update_table(p, b);
 }
 
 } // namespace
@@ -76,6 +73,7 @@ int launch_gather(const DevParams &p, LaunchCtx &ctx)
     dim3 grid((n_rows + kRowsPerBlock - 1) / kRowsPerBlock, p.L * p.B);
     if (launch_after(k_gather, grid, dim3(kGatherThreads), 0, ctx.s, p) != cudaSuccess) return AMS_ERR_CUDA;
     ctx.mark(kKernGather);
+    if (p.rewrite) return AMS_OK;
     if (launch_after(k_table_update, dim3((unsigned)p.B), dim3(128), 0, ctx.s, p) != cudaSuccess) return AMS_ERR_CUDA;
     ctx.mark(kKernTable);
     return cudaGetLastError() == cudaSuccess ? AMS_OK : AMS_ERR_CUDA;

@@ -36,6 +36,7 @@
 #include <type_traits>
 
 #include "ams_common.cuh"
+#include "ams_move.cuh"
 #include "ams_select.cuh"
 
 namespace ams {
@@ -51,6 +52,7 @@ constexpr int kWarpBins = 128;      // bins of a warp's own histogram, four per 
 constexpr int kBatch = 64;          // long segments searched together
 constexpr int kMaxBins = 1024;      // histogram bins per long segment
 constexpr unsigned kOctaves = 12;   // octaves below a long segment's largest score that its histogram resolves
+constexpr int kMoveLimit = 1 << 22;  // polls of a move for the units that it needs, 100 ns and more each
 constexpr int kBest = 512;          // entries of the table of the pieces' best rejected keys
 
 // Working arrays of the search of long segments, one entry per segment of the batch.
@@ -1075,15 +1077,13 @@ __device__ void block_select_stream(const float *g, int T, int q, SelShared &sh,
 
 // -------------------------------------------------------------------------------------- k_select_compact
 
+// Steps 1-5 of one unit, by the block.
 template <int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, int longs)
+__device__ __forceinline__ void select_unit(const DevParams &p, int longs, int uid, unsigned char *dyn, SelShared &sh)
 {
-    extern __shared__ __align__(16) unsigned char dyn[];
-    __shared__ SelShared sh;
     constexpr int NW = NT / 32, kList = Tune<NT>::kList;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, uid = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int h = uid % p.H, bq = (uid / p.H) % p.B, l = uid / (p.H * p.B);
-    wait_for_previous_kernel(); // scores, effective lengths
     const int T = seq_len_of(p, bq);
     if (T <= p.Tk || T > p.T_cap) return;
     if (p.seq_lens && p.seq_bad[bq]) return; // no scores to go by (the allocation-free entry point has no scorer and keeps its flags)
@@ -1320,12 +1320,118 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
 }
 
 template <int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, int longs)
+{
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ SelShared sh;
+    wait_for_previous_kernel(); // scores, effective lengths
+    select_unit<NT>(p, longs, blockIdx.x, dyn, sh);
+}
+
+// The rest of an event in one launch: selection, row moves, block table.  Selection is bound by instructions and latency, the moves by
+// HBM, so blocks doing the one run beside blocks doing the other.  A block takes a ticket from a counter when it starts: the first
+// `lag` are units to select, then units and parts of the moves in turn, the moves `lag` units behind, then what is left of
+// the moves.  A move waits for the units of its (layer, sequence), whose tickets all came before its own, to
+// blocks that are running or through: no wait needs a block that has not started.  Whoever finishes the last part rewrites the
+// table.  (Blocks that stay and take one ticket after the other need 200 to 800 bytes of spills, as the compiler keeps
+// what does not depend on the ticket in registers throughout.)
+struct MovePlan { int lag, parts, rows; }; // parts of a (layer, sequence), rows in each
+
+template <int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_select_move(DevParams p, int longs, MovePlan plan)
+{
+    extern __shared__ __align__(16) unsigned char dyn[];
+    __shared__ SelShared sh;
+    const int tid = threadIdx.x, groups = p.L * p.B, n_sel = groups * p.H, n_mov = groups * plan.parts;
+    int *finished = p.move_count + 1, *done = p.move_count + 2;
+    wait_for_previous_kernel(); // scores, effective lengths; the counters
+    if (tid == 0) {
+        const int t = atomicAdd(p.move_count, 1);
+        int what = t; // a unit, or n_sel + a part
+        if (t >= plan.lag) {
+            const long long A = n_sel - plan.lag, mixed = A + A * n_mov / n_sel, m = t - plan.lag;
+            if (m < mixed) {
+                const long long s = m * A / mixed;
+                what = (m + 1) * A / mixed > s ? plan.lag + (int)s : n_sel + (int)(m - s);
+            } else {
+                what = n_sel + (int)(m - A);
+            }
+        }
+        sh.total = what;
+    }
+    __syncthreads();
+    const int what = sh.total;
+    if (what < n_sel) {
+        select_unit<NT>(p, longs, what, dyn, sh);
+        __syncthreads();
+        if (tid == 0) {
+            __threadfence();
+            asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(done + what / p.H) : "memory");
+        }
+        return;
+    }
+    const int part = what - n_sel, group = part / plan.parts, b = group % p.B, T = p.seq_lens[b];
+    if (T > p.Tk && T <= p.T_cap) {
+        if (tid == 0) {
+            int have = 0, bad = 0;
+            for (int i = 0; i < kMoveLimit && !bad; ++i) {
+                asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(have) : "l"(done + group) : "memory");
+                if (have >= p.H) break;
+                __nanosleep(100);
+                if ((i & 255) == 255) bad = __ldcg(p.seq_bad + b);
+            }
+            bad = __ldcg(p.seq_bad + b);
+            if (have < p.H && !bad) { // cannot happen; the wait is bounded all the same
+                set_status(p.status, AMS_ERR_INTERNAL, group * p.H, have, p.H);
+                for (int i = 0; i < p.B; ++i) p.seq_bad[i] = 1;
+            }
+            sh.level = have >= p.H && !bad;
+        }
+        __syncthreads();
+        if (sh.level) {
+            const int r0 = (part - group * plan.parts) * plan.rows;
+            move_rows<NT>(p, group / p.B, b, r0, min(p.Tk * p.H, r0 + plan.rows));
+        }
+        __syncthreads();
+    }
+    if (tid == 0) {
+        __threadfence();
+        sh.level = atomicAdd(finished, 1) == n_mov - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (sh.level)
+        for (int i = 0; i < p.B; ++i) {
+            const int Ti = p.seq_lens[i];
+            if (Ti > p.Tk && Ti <= p.T_cap && !__ldcg(p.seq_bad + i)) update_table(p, i);
+        }
+}
+
+template <int NT>
 cudaError_t launch_nt(const DevParams &p, int units, bool longs, LaunchCtx &ctx)
 {
     static SmemGrant grant;
     const size_t smem = sel_smem<NT>(p.T_cap, p.seg_cap, p.S, longs).total;
     if (!grant_dynamic_smem(k_select_compact<NT>, smem, grant)) return cudaErrorInvalidValue;
     return launch_after(k_select_compact<NT>, dim3((unsigned)units), dim3(NT), smem, ctx.s, p, longs ? 1 : 0);
+}
+
+template <int NT>
+cudaError_t launch_move_nt(const DevParams &p, int units, bool longs, int fit, int n_sm, LaunchCtx &ctx)
+{
+    static SmemGrant grant;
+    const size_t smem = sel_smem<NT>(p.T_cap, p.seg_cap, p.S, longs).total;
+    if (!grant_dynamic_smem(k_select_move<NT>, smem, grant)) return cudaErrorInvalidValue;
+    const int blocks = fit * n_sm, n_rows = p.Tk * p.H;
+    constexpr int kRound = NT / 4; // rows of one round of a block
+    MovePlan plan;
+    const long long per = (long long)p.L * p.B * n_rows / (2LL * blocks); // two parts for each block where there is little to move
+    plan.rows = (int)std::min(1024LL, std::max((long long)kRound, per / kRound * kRound));
+    plan.parts = (n_rows + plan.rows - 1) / plan.rows;
+    plan.lag = std::min(units, std::max(blocks, 2 * p.H + 2));
+    const long long tickets = units + (long long)p.L * p.B * plan.parts;
+    if (tickets > 0x7fffffffLL) return cudaErrorInvalidValue;
+    return launch_after(k_select_move<NT>, dim3((unsigned)tickets), dim3(NT), smem, ctx.s, p, longs ? 1 : 0, plan);
 }
 
 constexpr size_t kSmShared = 228 * 1024, kBlockReserve = 1024; // shared memory of an SM; what each block takes besides its own
@@ -1336,8 +1442,9 @@ bool long_segments(const DevParams &p) { return p.l_max == 0 || p.l_max > kPiece
 
 bool segsel_supported(const DevParams &p) { return sel_smem<1024>(p.T_cap, p.seg_cap, p.S, long_segments(p)).total <= (size_t)224 * 1024; }
 
-int launch_segsel(const DevParams &p, LaunchCtx &ctx)
+int launch_segsel(const DevParams &p, LaunchCtx &ctx, bool *moved)
 {
+    bool move = moved != nullptr;
     const int units = p.L * p.B * p.H, n_sm = sm_count();
     if (n_sm <= 0) return AMS_ERR_CUDA;
     const bool longs = long_segments(p);
@@ -1346,14 +1453,23 @@ int launch_segsel(const DevParams &p, LaunchCtx &ctx)
     // ceil(units / resident blocks) rounds of it.  160 units of 125840 tokens, l_max 4096: 512 threads by the registers alone 500 us,
     // 1024 by both 384; 640 of 131072 take 1024 either way, since one block of 512 fits as well.  The host knows the
     // capacity, not the lengths: rows far below it take the capacity's size (640 of 8704 tokens under 131072: 230 us).
-    auto cost = [&](int nt, size_t smem) {
-        const long long fit = std::max(1LL, std::min(1024LL / nt, (long long)(kSmShared / (smem + sizeof(SelShared) + kBlockReserve))));
-        return (units + fit * n_sm - 1) / (fit * n_sm) * (p.T_cap / nt + 24);
-    };
-    const long long c256 = cost(256, sel_smem<256>(p.T_cap, p.seg_cap, p.S, longs).total), c512 = cost(512, sel_smem<512>(p.T_cap, p.seg_cap, p.S, longs).total),
-                    c1024 = cost(1024, sel_smem<1024>(p.T_cap, p.seg_cap, p.S, longs).total);
-    const cudaError_t e = c256 <= c512 && c256 <= c1024 ? launch_nt<256>(p, units, longs, ctx)
-                        : c512 <= c1024 ? launch_nt<512>(p, units, longs, ctx) : launch_nt<1024>(p, units, longs, ctx);
+    auto fits = [&](int nt, size_t smem) { return (int)std::max(1LL, std::min(1024LL / nt, (long long)(kSmShared / (smem + sizeof(SelShared) + kBlockReserve)))); };
+    const int f256 = fits(256, sel_smem<256>(p.T_cap, p.seg_cap, p.S, longs).total), f512 = fits(512, sel_smem<512>(p.T_cap, p.seg_cap, p.S, longs).total),
+              f1024 = fits(1024, sel_smem<1024>(p.T_cap, p.seg_cap, p.S, longs).total);
+    auto cost = [&](int nt, int fit) { return ((long long)units + fit * n_sm - 1) / (fit * n_sm) * (p.T_cap / nt + 24); };
+    const long long c256 = cost(256, f256), c512 = cost(512, f512), c1024 = cost(1024, f1024);
+    // The moves go along with the selection where there is something to run beside (three rounds of units at least, chosen in
+    // registers) and enough to move to pay for the tickets (some 5 % of a unit of 1024 tokens).  Events, apart / together: 1792 units of
+    // 8192 to 32768 tokens, budget 4096, 3361 / 3267 us; 2048 of 1900 to 9001, 1000: 1357 / 1324; 3024 of 1169 to 3146, 967: 904 / 863;
+    // 3456 of 4728, 461: 1308 / 1232; 17672 of 1024 tokens, budget 69, 1028 / 1183; 1944 of 694 to 1024, 152: 240 / 267.
+    // 2048 units in long segments 1176 / 1224 (selection and moves).
+    const int fit = c256 <= c512 && c256 <= c1024 ? f256 : c512 <= c1024 ? f512 : f1024;
+    move = move && !longs && p.Tk >= 320 && units >= 3LL * fit * n_sm;
+    if (moved) *moved = move;
+    cudaError_t e;
+    if (c256 <= c512 && c256 <= c1024) e = move ? launch_move_nt<256>(p, units, longs, f256, n_sm, ctx) : launch_nt<256>(p, units, longs, ctx);
+    else if (c512 <= c1024) e = move ? launch_move_nt<512>(p, units, longs, f512, n_sm, ctx) : launch_nt<512>(p, units, longs, ctx);
+    else e = move ? launch_move_nt<1024>(p, units, longs, f1024, n_sm, ctx) : launch_nt<1024>(p, units, longs, ctx);
     if (e != cudaSuccess) return AMS_ERR_CUDA;
     ctx.mark(kKernSelect);
     return AMS_OK;

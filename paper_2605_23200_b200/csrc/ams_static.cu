@@ -88,7 +88,7 @@ extern "C" int ams_select_static(const ams_config *cfg, const float *scores, int
     ctx.ev = nullptr;
     ctx.max_ev = 0;
     ctx.begin();
-    return launch_segsel(p, ctx);
+    return launch_segsel(p, ctx, nullptr);
 }
 
 // Device-side conditions of the calls above (a segment table that overflowed, a count that did not add up)

@@ -96,6 +96,7 @@ __global__ void __launch_bounds__(256) k_prepare(DevParams p, const int *lens_in
     wait_for_previous_kernel(); // the caller's table and lengths
     const int b = blockIdx.x;
     for (int i = b * blockDim.x + threadIdx.x; i < 2 * kGroupCounters; i += gridDim.x * blockDim.x) p.group_count[i * kGroupCounterPad] = 0;
+    for (int i = b * blockDim.x + threadIdx.x; i < p.L * p.B + 2; i += gridDim.x * blockDim.x) p.move_count[i] = 0;
     const int T = lens_in[b];
     int eff = 0;
     if (T > p.Tk) {
@@ -110,6 +111,7 @@ __global__ void __launch_bounds__(256) k_prepare(DevParams p, const int *lens_in
             for (int i = threadIdx.x; i < n_src && !bad; i += blockDim.x) {
                 const int pg = row[i];
                 if (pg < 0 || (long long)pg >= p.num_pages) { bad = 1; set_status(p.status, AMS_ERR_INVALID_ARG, b, i, pg); }
+                p.src_pages[(size_t)b * (p.T_cap / kPage) + i] = pg;
             }
             for (int i = threadIdx.x; i < p.n_dst; i += blockDim.x) {
                 const int pg = p.dst_pages[(size_t)b * p.n_dst + i];

@@ -1,0 +1,70 @@
+"""Row moves: the kernel that selects and moves in one launch (many units of short segments, no views) and the one that only moves and
+rewrites the table leave the same bytes, table, lengths and credit as an event with views, whose launches are separate and are
+checked against the oracle elsewhere.  External scores, so that every value is determined."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2605_23200_b200 import binding, inputs
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _event(wl, views, seed=5):
+    cache = inputs.make_cache(wl, DEV)
+    comp = binding.AmsCompressor(binding.config_for(wl), DEV)
+    g = torch.Generator(device=DEV)
+    g.manual_seed(seed)
+    ext = torch.randn((wl.n_layers, wl.batch, wl.n_kv_heads, wl.max_seq_len), generator=g, device=DEV).exp_()
+    comp.ema_state.copy_(torch.rand(comp.ema_state.shape, generator=g, device=DEV))
+    dst = torch.from_numpy(inputs.alloc_dst_pages(cache)).to(DEV)
+    dbg = comp.make_debug_views(wl.batch, wl.budget) if views else None
+    for _ in range(1 if views else 2):  # (the second finds every sequence within the budget and changes nothing)
+        comp.compress(cache.k_pages, cache.v_pages, cache.block_table, cache.seq_lens, None, wl.budget, wl.n_segments,
+                      binding.AMS_SCORER_EXTERNAL, dst, ext_scores=ext, dbg=dbg)
+        n = comp.last_launch_count
+        comp.status()
+    return cache, comp, n
+
+
+@pytest.mark.parametrize("kw,launches", [
+    # at least three rounds of units: one launch after the validation
+    (dict(n_layers=37, batch=9, n_kv_heads=8, n_q_heads=8, seq_len_min=300, seq_len_max=900, budget=327), 2),   # part of a page left over
+    (dict(n_layers=80, batch=23, n_kv_heads=1, n_q_heads=1, seq_len_min=330, seq_len_max=700, budget=320), 2),  # one head
+    (dict(n_layers=65, batch=11, n_kv_heads=3, n_q_heads=3, seq_len_min=200, seq_len_max=1000, budget=650), 2), # some within the budget
+    (dict(n_layers=30, batch=2, n_kv_heads=40, n_q_heads=40, seq_len_min=500, seq_len_max=600, budget=337), 2), # more heads than a part's rows divide into
+    # few units, little to move, or segments above a piece: moves of their own, with the table
+    (dict(n_layers=37, batch=9, n_kv_heads=8, n_q_heads=8, seq_len_min=300, seq_len_max=900, budget=319), 3),
+    (dict(n_layers=2, batch=3, n_kv_heads=8, n_q_heads=8, seq_len_min=300, seq_len_max=900, budget=257), 3),
+    (dict(n_layers=37, batch=9, n_kv_heads=8, n_q_heads=8, seq_len_min=300, seq_len_max=900, budget=327, l_max=600), 3),
+])
+def test_event_without_views_equals_event_with_views(kw, launches):
+    wl = inputs.CONFIGS[2].scaled(resident_layers=0, **kw)
+    a, ca, _ = _event(wl, True)
+    b, cb, n = _event(wl, False)
+    assert n == launches
+    assert torch.equal(a.k_pages.view(torch.int16), b.k_pages.view(torch.int16))
+    assert torch.equal(a.v_pages.view(torch.int16), b.v_pages.view(torch.int16))
+    assert torch.equal(a.block_table, b.block_table) and torch.equal(a.seq_lens, b.seq_lens)
+    assert torch.equal(ca.ema_state, cb.ema_state)
+    assert int((b.seq_lens == wl.budget).sum()) > 0
+
+
+def test_bad_page_is_skipped_in_the_joint_launch():
+    """A sequence with a page outside the pool keeps its row and length; the others are compressed."""
+    wl = inputs.CONFIGS[2].scaled(resident_layers=0, n_layers=37, batch=9, n_kv_heads=8, n_q_heads=8, seq_len_min=400, seq_len_max=900, budget=327)
+    cache = inputs.make_cache(wl, DEV)
+    comp = binding.AmsCompressor(binding.config_for(wl), DEV)
+    ext = torch.rand((wl.n_layers, wl.batch, wl.n_kv_heads, wl.max_seq_len), device=DEV)
+    cache.block_table[4, 3] = cache.k_pages.shape[1]
+    table, lens = cache.block_table.clone(), cache.seq_lens.clone()
+    dst = torch.from_numpy(inputs.alloc_dst_pages(cache)).to(DEV)
+    comp.compress(cache.k_pages, cache.v_pages, cache.block_table, cache.seq_lens, None, wl.budget, wl.n_segments,
+                  binding.AMS_SCORER_EXTERNAL, dst, ext_scores=ext)
+    assert comp.last_launch_count == 2
+    rc, detail = comp.status(check=False)
+    assert rc == binding.AMS_ERR_INVALID_ARG and detail[1:4] == [4, 3, cache.k_pages.shape[1]]
+    assert torch.equal(cache.block_table[4], table[4]) and cache.seq_lens[4] == lens[4]
+    others = [b for b in range(wl.batch) if b != 4]
+    assert (cache.seq_lens[others] == wl.budget).all() and torch.equal(cache.block_table[others][:, :dst.shape[1]], dst[others])
