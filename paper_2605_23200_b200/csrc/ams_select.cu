@@ -151,14 +151,27 @@ __device__ __forceinline__ void walk_pieces(int T, F f)
     }
 }
 
-// Block-wide sum of doubles that are multiples of one unit and whose sum has fewer than 53 bits of it (exact, hence
-// independent of the order).
-__device__ __forceinline__ double block_sum_exact_f64(double v, u64 *scratch)
+// Sum over a warp of integers below 2^51 whose total is below 2^53: two reductions of 32 bits, where five steps of two shuffles
+// and an addition take five times as long.
+__device__ __forceinline__ u64 warp_sum_wide(u64 v)
+{
+    const unsigned lo = __reduce_add_sync(kFull, (unsigned)v & 0x3ffffffu), hi = __reduce_add_sync(kFull, (unsigned)(v >> 26));
+    return ((u64)hi << 26) + lo;
+}
+// Block-wide sum of doubles v that are multiples of 1 / scale (a power of two) and whose sum has fewer than 53 bits of it, times
+// scale: exact, hence independent of the order.  They are added as integers (the images of 131072 tokens below 2^53 in all, a
+// quarter of that to a warp) unless a credit that the caller restored is negative or not a number.
+__device__ __forceinline__ double block_sum_images(double v, double scale, u64 *scratch)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    v = __dmul_rn(v, scale);
+    const bool fits = v >= 0.0 && v < 1125899906842624.0; // 2^50
+    const u64 w = warp_sum_wide(fits ? (u64)v : 0ull);
+    __syncthreads();
+    if (lane == 0) scratch[warp] = w;
+    if (!__syncthreads_or(!fits)) return (double)warp_sum_wide(lane < nw ? scratch[lane] : 0ull);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    __syncthreads();
     if (lane == 0) scratch[warp] = (u64)__double_as_longlong(v);
     __syncthreads();
     double x = lane < nw ? __longlong_as_double((long long)scratch[lane]) : 0.0;
@@ -187,7 +200,8 @@ __device__ __forceinline__ u64 warp_sum_mass(u64 h)
 struct Mass {
     const float *u, *credit;
     float eps, cut_w, cut_c;
-    double inv_sa_w, inv_sc_c, beta, omb; // 2^(36 - e_w) / SA, 2^(36 - e_c) / SC
+    double inv_sa_w, inv_sc_c; // 2^(36 - e_w) / SA, 2^(36 - e_c) / SC
+    double beta, omb;          // weights of the current and the past mass, times 2^36 (exactly)
     bool ema, have_credit;
 
     __device__ __forceinline__ double share(float x) const // Eq. 1 mass of a token with usage x
@@ -197,13 +211,9 @@ struct Mass {
     // history-aware integer mass floor((beta m + (1 - beta) normalize(c)) 2^36)
     __device__ __forceinline__ u64 of(float x, float c) const
     {
-        double r = share(x);
-        if (ema) {
-            double hist = 0.0;
-            if (have_credit) hist = __dmul_rn(omb, __dmul_rn((double)fixed_trunc_by_add(c, cut_c), inv_sc_c));
-            r = __dadd_rn(__dmul_rn(beta, r), hist);
-        }
-        return floor_to_u64(__dmul_rn(r, (double)(1ull << kFixBits)));
+        double r = __dmul_rn(beta, share(x)); // (beta is 2^36 where there is no credit)
+        if (have_credit) r = __dadd_rn(r, __dmul_rn(omb, __dmul_rn((double)fixed_trunc_by_add(c, cut_c), inv_sc_c)));
+        return floor_to_u64(r);
     }
     __device__ __forceinline__ u64 at(int t) const { return of(u[t], have_credit ? credit[t] : 0.0f); }
 };
@@ -221,7 +231,8 @@ __device__ u64 mass_of_unit(const DevParams &p, int uid, int T, float *credit, u
     ms.ema = p.beta != 1.0f;
     ms.have_credit = false;
     ms.cut_c = 0.0f; ms.inv_sc_c = 0.0;
-    ms.beta = (double)p.beta; ms.omb = __dsub_rn(1.0, ms.beta);
+    ms.beta = __dmul_rn((double)p.beta, (double)(1ull << kFixBits)); // (1 where there is no credit)
+    ms.omb = __dmul_rn(__dsub_rn(1.0, (double)p.beta), (double)(1ull << kFixBits));
     // ---- largest Eq. 1 weight (that of the largest usage) -> exponent of the fixed-point images
     float umax = 0.0f;
     walk_pieces<NT>(T, [&](int a, int room, auto full) {
@@ -245,7 +256,7 @@ __device__ u64 mass_of_unit(const DevParams &p, int uid, int T, float *credit, u
         for (int j = 0; j < kPer; ++j)
             if (decltype(full)::value || j * 32 < room) sa += (double)fixed_trunc_by_add(weight_of(x[j], p.eps), ms.cut_w);
     });
-    const double SA = __dmul_rn(block_sum_exact_f64(sa, sh.scratch), scale_w);
+    const double SA = block_sum_images(sa, scale_w, sh.scratch);
     ms.inv_sa_w = __dmul_rn(__ddiv_rn(1.0, SA), scale_w); // normalisations multiply by the rounded reciprocal; the scaling is exact
 
     // ---- EMA credit: c <- lambda c + (1 - lambda) m, updated in place (the block-wide reductions that follow
@@ -284,7 +295,7 @@ __device__ u64 mass_of_unit(const DevParams &p, int uid, int T, float *credit, u
 #pragma unroll
                 for (int j = 0; j < kPer; ++j) sc += (double)fixed_trunc_by_add(c[j], ms.cut_c);
             });
-            const double SC = __dmul_rn(block_sum_exact_f64(sc, sh.scratch), scale_c);
+            const double SC = block_sum_images(sc, scale_c, sh.scratch);
             ms.have_credit = SC > 0.0;
             if (ms.have_credit) ms.inv_sc_c = __dmul_rn(__ddiv_rn(1.0, SC), scale_c);
         }
@@ -316,13 +327,11 @@ __device__ u64 mass_of_unit(const DevParams &p, int uid, int T, float *credit, u
     const int n_win = (T + 31) >> 5, per = (n_win + NW - 1) / NW, w0 = min(n_win, warp * per), w1 = min(n_win, w0 + per);
     u64 mine = 0;
     for (int w = w0 + lane; w < w1; w += 32) mine += wsum[w];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(kFull, mine, o);
+    mine = warp_sum_wide(mine);
     if (lane == 0) sh.scratch[warp] = mine; // (the reductions above ended with reads of this table two barriers ago)
     __syncthreads();
-    u64 run = lane < warp ? sh.scratch[lane] : 0ull, tot = lane < NW ? sh.scratch[lane] : 0ull;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) { run += __shfl_xor_sync(kFull, run, o); tot += __shfl_xor_sync(kFull, tot, o); }
+    const u64 tot = warp_sum_wide(lane < NW ? sh.scratch[lane] : 0ull);
+    u64 run = warp_sum_wide(lane < warp ? sh.scratch[lane] : 0ull);
     for (int g = w0; g < w1; g += 32) {
         const u64 v = g + lane < w1 ? wsum[g + lane] : 0ull;
         u64 inc = v;
@@ -349,10 +358,13 @@ __device__ __forceinline__ u64 mass_before(const Mass &ms, const u64 *wsum, int 
 __device__ __forceinline__ int mass_cut(const Mass &ms, const u64 *wsum, int T, u64 thr)
 {
     const int lane = threadIdx.x & 31;
-    int w = 0; // the last window that starts below thr
-    for (int hi = (T + 31) >> 5; hi - w > 1;) {
-        const int mid = (w + hi) >> 1;
-        if (wsum[mid] < thr) w = mid; else hi = mid;
+    int w = 0; // the last window that starts below thr: a lane to each of 32 places at a time (the windows' sums ascend from 0)
+    for (int n = (T + 31) >> 5; n > 1;) {
+        const int step = (n + 31) >> 5, at = lane * step;
+        const unsigned below = __ballot_sync(kFull, at < n && wsum[w + at] < thr); // (lane 0's always)
+        const int i = 31 - __clz(below);
+        w += i * step;
+        n = min(step, n - i * step);
     }
     const int t = w * 32 + lane;
     u64 inc = t < T ? ms.at(t) : 0ull;
@@ -465,7 +477,17 @@ __device__ int segments_and_quotas(const DevParams &p, int T, int Bq, const Mass
         // short raw segments merge forward: the next boundary is the first cut at least l_min past the last one
         int nm = 0, start = 0;
         if (lane == 0) merged[0] = 0;
+        bool plain = true; // no raw segment is short: every cut is a boundary
         for (int k0 = 1; k0 < p.S; k0 += 32) {
+            const int k = k0 + lane, e = k < p.S ? raw[k] : 0, before = k > 1 && k < p.S ? raw[k - 1] : 0;
+            plain = plain && (k >= p.S || (e < T && e - before >= p.l_min));
+        }
+        if (__all_sync(kFull, plain)) {
+            for (int k = lane + 1; k < p.S; k += 32) merged[k] = raw[k];
+            nm = p.S - 1;
+            start = p.S > 1 ? raw[p.S - 1] : 0;
+            __syncwarp();
+        } else for (int k0 = 1; k0 < p.S; k0 += 32) {
             const int k = k0 + lane;
             const int e = k < p.S ? raw[k] : T;
             for (;;) {
@@ -1084,9 +1106,8 @@ __device__ __forceinline__ void select_unit(const DevParams &p, int longs, int u
     constexpr int NW = NT / 32, kList = Tune<NT>::kList;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int h = uid % p.H, bq = (uid / p.H) % p.B, l = uid / (p.H * p.B);
-    const int T = seq_len_of(p, bq);
-    if (T <= p.Tk || T > p.T_cap) return;
-    if (p.seq_lens && p.seq_bad[bq]) return; // no scores to go by (the allocation-free entry point has no scorer and keeps its flags)
+    const int T = seq_len_of(p, bq), bad = p.seq_lens ? p.seq_bad[bq] : 0; // (the allocation-free entry point has no scorer and keeps its flags)
+    if (T <= p.Tk || T > p.T_cap || bad) return; // (bad: no scores to go by)
     const int sc = p.seg_cap;
     const SelSmem mp = sel_smem<NT>(p.T_cap, sc, p.S, longs != 0);
     unsigned *mask = reinterpret_cast<unsigned *>(dyn + mp.mask);
@@ -1109,6 +1130,8 @@ __device__ __forceinline__ void select_unit(const DevParams &p, int longs, int u
     for (int i = tid; i < kBest; i += NT) best[i] = 0u;
     if (tid == 0) { sh.n_list = 0; sh.n_look = 0; sh.bound = 0u; }
     float *credit = p.ema ? p.ema + (((size_t)l * p.Bmax + bq) * p.H + h) * (size_t)p.T_cap : nullptr;
+    if (p.beta != 1.0f) // on its way from HBM while the weights are summed
+        for (int t = tid * 32; t < T; t += NT * 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(credit + t));
     Mass ms;
     u64 *wsum = reinterpret_cast<u64 *>(dyn + mp.list);
     const u64 SH = mass_of_unit<NT>(p, uid, T, credit, wsum, ms, sh);
