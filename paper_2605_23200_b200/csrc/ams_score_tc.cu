@@ -7,10 +7,13 @@
 //               stage (eight 16-token pages, one 4 KB copy each, 128-byte swizzle);
 //   warps 1, 3  MMA issuers (one lane each, one per parity of the products): per product of a tile and a 128-row
 //               query block eight tcgen05.mma m128 n128 k16 into one of four 128-column TMEM slots, used in turn;
-//   warps 4-19  four consumer warpgroups, one per slot: thread i of a warpgroup owns TMEM lane i and takes all 128 columns, in the
-//               first phase the next 32 on their way while it works on the last.  (Two warpgroups to a slot with half of the columns each spent
-//               more on waits and hand-over, and had no registers left to fetch ahead: 512 rows, 640 units of 8704 tokens.
-//               statistics 963, now 875 us; usage 887, now 900; the event 2865, now 2782.)
+//   warps 4-19  four consumer warpgroups: thread i of one owns TMEM lane i of a slot; from two query blocks on a warpgroup has a
+//               slot to itself and takes all 128 columns, with one block two share a slot (see there).  In the first phase the
+//               next 32 columns are on their way while it works on the last; the slot is free again as soon as its last columns
+//               are in registers.  At 512 rows the special-function unit is 80 % busy at the clock that the power limit leaves
+//               (1.69 GHz; two warpgroups to a slot, half of the columns each: 71 %): 640 units of 8704 tokens, statistics 963,
+//               now 873 us, usage 887, now 866; of 131072 tokens 15.4 and 13.8, now 13.6 and 13.5 ms.  Three warpgroups of 128
+//               registers, exponentials shared with the FMA pipe and tiles fetched ahead into L2 were no faster.
 // Phase 1 puts query rows on the TMEM lanes (A = Q, B = K), so a thread folds its row's
 // logits into a running (max, sum of 2^x) without leaving registers; phase 2 puts tokens
 // on the lanes (A = K, B = Q), so a thread sums 2^(x - b_r) over the query rows of its
@@ -32,8 +35,10 @@ namespace {
 struct TcShared {
     unsigned long long kfull[kMaxStages], kempty[kMaxStages], tfull[kSlots], tempty[kSlots];
     unsigned long long qfull, qempty, done[2];
-    unsigned long long pfull[2], pempty[2];          // usage pass: the sums of a tile's earlier query blocks are in pacc; are used
-    float pacc[2][3][128];
+    unsigned long long pfull[kSlots];                // usage pass, one query block: the second half's sums of a slot's tile are in pacc
+    int psum[2][4], pused[2][4];                     // more: how many sums of a tile's earlier query blocks a quarter of the lanes has
+                                                     // received in pacc so far, and how many tiles' it has used
+    float2 pacc[2][3][128];
     uint32_t tmem_base;
     int abort_flag;
     float wmax[2][16];
@@ -42,7 +47,26 @@ struct TcShared {
 };
 
 constexpr int kConsumerWarp = 4; // first warp of the consumers
-template <int PHASE>
+
+// Counters in shared memory that only grow, for a hand-over between warps that do not see every turn of its buffer (a wait by
+// parity must not skip one).  By whole warps; the wait is bounded.
+__device__ __forceinline__ void count_up(int *counter)
+{
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) asm volatile("red.release.cta.shared::cta.add.s32 [%0], 1;" ::"r"(smem_u32(counter)) : "memory");
+}
+__device__ __forceinline__ bool count_wait(const int *counter, int want, volatile int *abort_flag)
+{
+    for (uint32_t i = 0;; ++i) {
+        int have;
+        asm volatile("ld.acquire.cta.shared::cta.s32 %0, [%1];" : "=r"(have) : "r"(smem_u32(counter)) : "memory");
+        if (__all_sync(0xffffffffu, have >= want)) return true;
+        if (i == kWaitLimit) *abort_flag = 1;
+        if ((i & 1023u) == 1023u && __any_sync(0xffffffffu, *abort_flag)) return false;
+    }
+}
+// FORM: 1: one query block, 4: four, 2: two or three (see the consumers)
+template <int PHASE, int FORM>
 __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __grid_constant__ CUtensorMap k_map,
                                                            const __grid_constant__ CUtensorMap q_map)
 {
@@ -60,8 +84,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
 
     if (tid == 0) {
         for (int i = 0; i < kMaxStages; ++i) { mbar_init(smem_u32(&sh.kfull[i]), 1); mbar_init(smem_u32(&sh.kempty[i]), n_rb > 1 ? 2 : 1); }
-        for (int i = 0; i < kSlots; ++i) { mbar_init(smem_u32(&sh.tfull[i]), 1); mbar_init(smem_u32(&sh.tempty[i]), 4); }
-        for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&sh.pfull[i]), (uint32_t)(n_rb > 1 ? 4 * (n_rb - 1) : 1)); mbar_init(smem_u32(&sh.pempty[i]), 4); }
+        for (int i = 0; i < kSlots; ++i) { mbar_init(smem_u32(&sh.tfull[i]), 1); mbar_init(smem_u32(&sh.tempty[i]), FORM == 1 ? 8 : 4); }
+        for (int i = 0; i < kSlots; ++i) mbar_init(smem_u32(&sh.pfull[i]), 4);
+        for (int i = 0; i < 8; ++i) sh.psum[i >> 2][i & 3] = sh.pused[i >> 2][i & 3] = 0;
         mbar_init(smem_u32(&sh.qfull), 1);
         mbar_init(smem_u32(&sh.qempty), 2); // both MMA issuers release the query block
         mbar_init(smem_u32(&sh.done[0]), 1);
@@ -106,25 +131,20 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
                 const int my_h = my_h0 + (int)(gv / g_span) * my_hs;
                 const long long g = g_begin + gv % g_span;
                 const Segment s = decode_segment(p, prefix, tiles_lh, tpc, g, g_end, my_h);
+                ok = mbar_wait(smem_u32(&sh.qempty), (uint32_t)((seg & 1) ^ 1), abort_flag);
+                if (!ok) break;
+                if (lane == 0) {
+                    mbar_expect_tx(smem_u32(&sh.qfull), (uint32_t)(n_rb * kTileBytes));
+                    const int qrow0 = ((s.l * p.B + s.b) * p.H * p.G + s.h * p.G) * p.W;
+                    for (int rb = 0; rb < n_rb; ++rb)
+                        for (int hf = 0; hf < 2; ++hf)
+                            tma_load_2d(smem_u32(Qs + (size_t)rb * kTileBytes + hf * kHalfBytes), &q_map, smem_u32(&sh.qfull),
+                                        hf * 64, qrow0 + rb * 128);
+                }
+                blocks_issued = seg + 1;
                 const int *table = p.block_table + (size_t)s.b * p.bt_stride;
                 const int last_page = (s.T - 1) >> 4;
                 for (int i = 0; i < s.n && ok; ++i, ++kit) {
-                    // The query block goes behind the unit's first K tiles: it waits for the products of the unit before, they only
-                    // for a stage each, and the K stream runs on.  (A tile whose stage an earlier one of the same unit holds needs
-                    // those products, so no later than before the last of NS.)
-                    if (i == min(NS, s.n) - 1) {
-                        ok = mbar_wait(smem_u32(&sh.qempty), (uint32_t)((seg & 1) ^ 1), abort_flag);
-                        if (!ok) break;
-                        if (lane == 0) {
-                            mbar_expect_tx(smem_u32(&sh.qfull), (uint32_t)(n_rb * kTileBytes));
-                            const int qrow0 = ((s.l * p.B + s.b) * p.H * p.G + s.h * p.G) * p.W;
-                            for (int rb = 0; rb < n_rb; ++rb)
-                                for (int hf = 0; hf < 2; ++hf)
-                                    tma_load_2d(smem_u32(Qs + (size_t)rb * kTileBytes + hf * kHalfBytes), &q_map, smem_u32(&sh.qfull),
-                                                hf * 64, qrow0 + rb * 128);
-                        }
-                        blocks_issued = seg + 1;
-                    }
                     const int st = kit % NS;
                     ok = mbar_wait(smem_u32(&sh.kempty[st]), (uint32_t)(((kit / NS) & 1) ^ (p.expire_polls ? 0 : 1)), abort_flag,
                                    p.expire_polls ? p.expire_polls : kWaitLimit);
@@ -199,9 +219,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
             __syncwarp();
         } else if (warp >= kConsumerWarp) {
             // ------------------------------------------------------------ consumers
-            // Product number q = tile * n_rb + query block goes to warpgroup and slot q % 4: thread li of it owns TMEM lane li and
-            // all 128 columns.
+            // Product number q = tile * n_rb + query block goes to slot q % 4, thread li of a warpgroup owning TMEM lane li.  From two
+            // query blocks on a slot belongs to one warpgroup, which takes all 128 columns.  With one block two warpgroups take half
+            // of the columns each and the tiles of one parity, in two slots in turn: a tile is through sooner, which a block with
+            // few tiles of a unit feels (92 units of 322 to 1024 tokens at 119 rows: event 114 us, with a slot each 122).
+            constexpr bool kShare = FORM == 1;
+            constexpr int kChunks = kShare ? 2 : 4; // of 32 columns
             const int wgq = (warp - kConsumerWarp) >> 2, quad = warp & 3, li = quad * 32 + lane;
+            const int col0 = kShare ? (wgq >> 1) * 64 : 0; // first column
             int kit = 0, seg = 0;
             bool ok = true;
             // a thread whose wait ran out keeps walking the segments without touching the pipeline, so that
@@ -211,7 +236,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
                 const long long g = g_begin + gv % g_span;
                 const Segment s = decode_segment(p, prefix, tiles_lh, tpc, g, g_end, my_h);
                 const int T = s.T;
-                float m[4], z[4], lost[4]; // lost: what rounding has added to z so far (Kahan)
+                // (max, sum) of each query block.  Two and three blocks: what rounding has added to the sum (Kahan), as a thread adds up
+                // to 2048 chunks.  Four blocks, where a thread has one of them and all its tiles: instead four parts of that one's
+                // sum, by parity of the tile and half of its columns, which is how one block's are spread over the warpgroups.
+                float m[4], z[4], lost[4];
                 int lastv[4];
                 float *fs = fin_s + (seg & 1) * p.rows_pad;
                 float pmax = 0.0f;
@@ -252,9 +280,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
                 }
                 for (int i = 0; i < s.n && ok; ++i, ++kit) {
                     const int t0 = (s.tile0 + i) * kTileTokens;
-                    for (int rb = (wgq - kit * n_rb) & 3; rb < n_rb && ok; rb += 4) {
-                        const int slot = wgq;
-                        const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(slot * 128);
+                    for (int rb = kShare ? (kit ^ wgq) & 1 : (wgq - kit * n_rb) & 3; rb < n_rb && ok; rb += 4) {
+                        const int slot = kShare ? kit & 3 : wgq;
+                        const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(slot * 128 + col0);
                         ok = mbar_wait(smem_u32(&sh.tfull[slot]), (uint32_t)(((kit * n_rb + rb) >> 2) & 1), abort_flag);
                         ok = __all_sync(0xffffffffu, ok) != 0; // one answer per warp: what follows is warp-wide
                         if (!ok) break;
@@ -269,17 +297,23 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
                             // 32 columns at a time, the next 32 on their way meanwhile: one running-maximum update (one rescaling
                             // exponential) per 32 logits
                             const int lv = min(lastv[rb], T - 1);
-                            float mr = m[rb], zr = z[rb], zl = lost[rb];
+                            int at = FORM == 4 ? kit & 1 : rb;
+                            float mr = m[at], zr = z[at], zl = lost[at];
                             uint32_t d[2][32];
                             tc_ld32_issue(taddr, d[0]);
 #pragma unroll
-                            for (int ch = 0; ch < 4; ++ch) {
+                            for (int ch = 0; ch < kChunks; ++ch) {
                                 uint32_t (&x)[32] = d[ch & 1];
                                 tc_ld_wait(x);
-                                if (ch < 3) tc_ld32_issue(taddr + (uint32_t)(32 * ch + 32), d[1 - (ch & 1)]);
+                                if (ch < kChunks - 1) tc_ld32_issue(taddr + (uint32_t)(32 * ch + 32), d[1 - (ch & 1)]);
                                 else release();
                                 auto v = [&](int j) { return __uint_as_float(x[j]); };
-                                const int tc0 = t0 + ch * 32;
+                                if (FORM == 4 && ch == 2) { // the second half
+                                    m[at] = mr; z[at] = zr;
+                                    at += 2;
+                                    mr = m[at]; zr = z[at];
+                                }
+                                const int tc0 = t0 + col0 + ch * 32;
                                 if (tc0 <= lv) {
                                     if (tc0 + 31 > lv) {
 #pragma unroll
@@ -295,7 +329,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
                                     const float mn = fmaxf(mr, cm * c);
                                     const float down = ex2(mr - mn);
                                     zr *= down;
-                                    zl *= down;
+                                    if (FORM == 2) zl *= down;
                                     mr = mn;
                                     u64 zs[2] = {0, 0}; // (0.0f, 0.0f)
                                     const u64 c2 = pack_f32x2(c, c), n2 = pack_f32x2(-mn, -mn);
@@ -304,25 +338,33 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
                                         const float2 e = ex2_pair(fma_f32x2(pack_f32x2(v(j), v(j + 1)), c2, n2));
                                         zs[(j >> 1) & 1] = add_f32x2(zs[(j >> 1) & 1], pack_f32x2(e.x, e.y));
                                     }
-                                    // compensated: a thread adds up to 4096 such sums
-                                    const float more = __fsub_rn(sum_f32x2(add_f32x2(zs[0], zs[1])), zl), sum = __fadd_rn(zr, more);
-                                    zl = __fsub_rn(__fsub_rn(sum, zr), more);
-                                    zr = sum;
+                                    float s0, s1, s2, s3;
+                                    unpack_f32x2(zs[0], s0, s1);
+                                    unpack_f32x2(zs[1], s2, s3);
+                                    if (FORM != 2) {
+                                        zr += (s0 + s1) + (s2 + s3);
+                                    } else {
+                                        const float more = __fsub_rn((s0 + s1) + (s2 + s3), zl), sum = __fadd_rn(zr, more);
+                                        zl = __fsub_rn(__fsub_rn(sum, zr), more);
+                                        zr = sum;
+                                    }
                                 }
                             }
-                            m[rb] = mr; z[rb] = zr; lost[rb] = zl;
+                            m[at] = mr; z[at] = zr;
+                            if (FORM == 2) lost[at] = zl;
                         } else {
                             const int t = t0 + li;
                             const bool plain = !p.causal || t0 + kTileTokens - 1 <= T - p.W; // every row sees every token
-                            const float4 *fr4 = reinterpret_cast<const float4 *>(fs + rb * 128);
+                            const float4 *fr4 = reinterpret_cast<const float4 *>(fs + rb * 128 + col0);
                             const u64 c2 = pack_f32x2(c, c);
-                            u64 ac[2] = {0, 0}; // (0.0f, 0.0f)
+                            u64 acs[2][2] = {{0, 0}, {0, 0}}; // (0.0f, 0.0f), of either half of the columns
                             uint32_t d[32];
                             tc_ld32_issue(taddr, d);
 #pragma unroll
-                            for (int ch = 0; ch < 4; ++ch) { // 32 columns (query rows) at a time
+                            for (int ch = 0; ch < kChunks; ++ch) { // 32 columns (query rows) at a time
+                                u64 (&ac)[2] = acs[ch >> 1];
                                 tc_ld_wait(d);
-                                if (ch == 3) release();
+                                if (!kShare && ch == kChunks - 1) release();
                                 if (plain) {
 #pragma unroll
                                     for (int j4 = 0; j4 < 8; ++j4) {
@@ -333,7 +375,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
                                         ac[1] = add_f32x2(ac[1], pack_f32x2(e1.x, e1.y));
                                     }
                                 } else {
-                                    const int rbase = rb * 128 + ch * 32;
+                                    const int rbase = rb * 128 + col0 + ch * 32;
 #pragma unroll
                                     for (int j = 0; j < 32; j += 2) {
                                         float e[2];
@@ -346,26 +388,50 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
                                         ac[(j >> 1) & 1] = add_f32x2(ac[(j >> 1) & 1], pack_f32x2(e[0], e[1]));
                                     }
                                 }
-                                if (ch < 3) tc_ld32_issue(taddr + (uint32_t)(32 * ch + 32), d);
+                                if (ch < kChunks - 1) tc_ld32_issue(taddr + (uint32_t)(32 * ch + 32), d);
                             }
-                            float acc = sum_f32x2(add_f32x2(ac[0], ac[1]));
-                            // a tile's query blocks meet in the warpgroup that has the last one
-                            const int buf = kit & 1;
-                            if (rb < n_rb - 1) {
-                                ok = mbar_wait(smem_u32(&sh.pempty[buf]), (uint32_t)(((kit >> 1) & 1) ^ 1), abort_flag);
-                                ok = __all_sync(0xffffffffu, ok) != 0;
-                                if (!ok) break;
-                                sh.pacc[buf][rb][li] = acc;
+                            float half[2]; // of the query block: the sum over either half of its rows
+#pragma unroll
+                            for (int i2 = 0; i2 < 2; ++i2) {
+                                float s0, s1, s2, s3;
+                                unpack_f32x2(acs[i2][0], s0, s1);
+                                unpack_f32x2(acs[i2][1], s2, s3);
+                                half[i2] = (s0 + s1) + (s2 + s3);
+                            }
+                            // the halves of a tile's columns meet in the first half's warpgroup, the sums of its query blocks in the one
+                            // that has the last; a quarter of the lanes at a time
+                            const int buf = kit & 1, turn = kit >> 1;
+                            if (kShare && col0 > 0) {
+                                sh.pacc[slot & 1][slot >> 1][li].x = half[0];
+                                tc_fence_before();
                                 __syncwarp();
-                                if (lane == 0) mbar_arrive(smem_u32(&sh.pfull[buf]));
+                                if (lane == 0) { mbar_arrive(smem_u32(&sh.pfull[slot])); mbar_arrive(smem_u32(&sh.tempty[slot])); }
+                            } else if (!kShare && rb < n_rb - 1) {
+                                ok = count_wait(&sh.pused[buf][quad], turn, abort_flag);
+                                if (!ok) break;
+                                sh.pacc[buf][rb][li] = make_float2(half[0], half[1]);
+                                count_up(&sh.psum[buf][quad]);
                             } else {
-                                if (n_rb > 1) {
-                                    ok = mbar_wait(smem_u32(&sh.pfull[buf]), (uint32_t)((kit >> 1) & 1), abort_flag);
+                                float acc;
+                                if (kShare) {
+                                    // the slot is released only after its sums are read, so the next tile in it cannot overwrite them, and
+                                    // before the usage goes to global memory: an arrive after the store would wait until that is performed
+                                    ok = mbar_wait(smem_u32(&sh.pfull[slot]), (uint32_t)((kit >> 2) & 1), abort_flag);
                                     ok = __all_sync(0xffffffffu, ok) != 0;
                                     if (!ok) break;
-                                    for (int o = 0; o < n_rb - 1; ++o) acc += sh.pacc[buf][o][li];
-                                    __syncwarp();
-                                    if (lane == 0) mbar_arrive(smem_u32(&sh.pempty[buf]));
+                                    acc = half[0] + sh.pacc[slot & 1][slot >> 1][li].x;
+                                    release();
+                                } else {
+                                    ok = count_wait(&sh.psum[buf][quad], (turn + 1) * (n_rb - 1), abort_flag);
+                                    if (!ok) break;
+                                    float2 sum = sh.pacc[buf][0][li];
+                                    for (int o = 1; o < n_rb - 1; ++o) {
+                                        const float2 v = sh.pacc[buf][o][li];
+                                        sum.x += v.x;
+                                        sum.y += v.y;
+                                    }
+                                    acc = (sum.x + half[0]) + (sum.y + half[1]);
+                                    count_up(&sh.pused[buf][quad]);
                                 }
                                 if (t < T) {
                                     const int ninv = p.causal ? p.G * max(0, t - (T - p.W)) : 0;
@@ -378,6 +444,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tova_tc(DevParams p, const __
                 if (PHASE == 1) {
                     // fold the four warpgroups' statistics (fixed order) and store this block's part of the unit
                     float2 *rd = red;
+                    if (FORM == 4) {
+#pragma unroll
+                        for (int i = 1; i < 4; ++i) lse_merge(m[0], z[0], m[i], z[i]);
+                        const float mm = m[0], zz = z[0];
+#pragma unroll
+                        for (int rb = 0; rb < 4; ++rb) { m[rb] = rb == wgq ? mm : -INFINITY; z[rb] = rb == wgq ? zz : 0.0f; }
+                    }
                     if (wgq > 0)
                         for (int rb = 0; rb < n_rb; ++rb) rd[((wgq - 1) * n_rb + rb) * 128 + li] = make_float2(m[rb], z[rb]);
                     asm volatile("bar.sync 1, %0;" ::"n"(kConsumerThreads) : "memory");
@@ -432,14 +505,17 @@ int launch_score_tova_tc(const DevParams &p_in, LaunchCtx &ctx)
     const int n_sm = sm_count();
     if (n_sm <= 0) return AMS_ERR_CUDA;
     const size_t smem = tova_tc_smem_bytes(p);
-    static SmemGrant grant1, grant2;
-    if (!grant_dynamic_smem(k_tova_tc<1>, smem, grant1) || !grant_dynamic_smem(k_tova_tc<2>, smem, grant2)) return AMS_ERR_CUDA;
+    const int form = p.rows_pad == 128 ? 0 : p.rows_pad == 512 ? 2 : 1;
+    auto kernel1 = form == 0 ? k_tova_tc<1, 1> : form == 1 ? k_tova_tc<1, 2> : k_tova_tc<1, 4>;
+    auto kernel2 = form == 0 ? k_tova_tc<2, 1> : k_tova_tc<2, 2>; // (two blocks or more)
+    static SmemGrant grant1[3], grant2[2];
+    if (!grant_dynamic_smem(kernel1, smem, grant1[form]) || !grant_dynamic_smem(kernel2, smem, grant2[form > 0])) return AMS_ERR_CUDA;
     const TcGrid tg = tc_grid(p, n_sm);
     const int hpb = tg.hpb, grid = tg.grid;
     p.tc_hpb = hpb;
-    if (launch_after(k_tova_tc<1>, dim3((unsigned)grid), dim3(kTcThreads), smem, ctx.s, p, k_map, q_map) != cudaSuccess) return AMS_ERR_CUDA;
+    if (launch_after(kernel1, dim3((unsigned)grid), dim3(kTcThreads), smem, ctx.s, p, k_map, q_map) != cudaSuccess) return AMS_ERR_CUDA;
     ctx.mark(kKernScore1);
-    if (launch_after(k_tova_tc<2>, dim3((unsigned)grid), dim3(kTcThreads), smem, ctx.s, p, k_map, q_map) != cudaSuccess) return AMS_ERR_CUDA;
+    if (launch_after(kernel2, dim3((unsigned)grid), dim3(kTcThreads), smem, ctx.s, p, k_map, q_map) != cudaSuccess) return AMS_ERR_CUDA;
     ctx.mark(kKernScore2);
     return cudaGetLastError() == cudaSuccess ? AMS_OK : AMS_ERR_CUDA;
 }
