@@ -255,8 +255,9 @@ def roofline_of(wl, kern_ms, k_read, moved, lens, peaks, traffic=None):
     rows = wl.group * max(wl.window, 1)
     note = []
     if overall != dom:
-        note.append(f"longest kernel of the step is {overall} ({kern_ms[overall]:.4f} ms), which moves no K/V byte; the roofline is "
-                    f"quoted for the longest kernel that does")
+        what = "which selects and moves the kept rows in one launch" if overall == "select_compact" and not kern_ms.get("gather") else "which moves no K/V byte"
+        note.append(f"longest kernel of the step is {overall} ({kern_ms[overall]:.4f} ms), {what}; the roofline is "
+                    f"quoted for the longest kernel that only streams")
     if dom == "gather":
         bytes_launch, bound = moved, "hbm"
     elif wl.scorer_id == 3 and dom == "score_phase1":

@@ -231,7 +231,8 @@ int32_t ams_last_launch_count(const ams_state *st);
  * event on its stream after every kernel it launches (events are host objects; no
  * device memory is allocated).  ams_get_kernel_times waits for the last call's final
  * event and writes AMS_KERNEL_SLOTS durations in milliseconds, one per kernel slot
- * named by ams_kernel_name (a slot launched more than once holds the sum). */
+ * named by ams_kernel_name (a slot launched more than once holds the sum; row moves that go along with the
+ * selection of many units, in one launch, count as "select_compact"). */
 #define AMS_KERNEL_SLOTS 10
 int ams_set_profiling(ams_state *st, int enable);
 int ams_get_kernel_times(ams_state *st, float *ms);
