@@ -437,7 +437,8 @@ void orc_must_keep(int32_t T, int32_t Tk, int32_t n_sink, int32_t n_last, int32_
  * token per visit, visiting segments heaviest first (ties: lower index) and
  * cycling while any has room; a surplus is taken back one token per visit,
  * lightest first (ties: higher index), never below q_i^min unless the budget
- * cannot even cover the minima (then a second round goes down to zero). */
+ * cannot even cover the minima (then a second round goes down to zero).  A unit whose mass is 0
+ * throughout (beta = 0 and a credit that says nothing) has no shares: the deficit is the whole of T_rem. */
 void orc_quotas(const uint64_t *C, const int32_t *bounds, int32_t n_seg, int32_t q_min, int32_t Bq,
                 int32_t *q)
 {
@@ -460,7 +461,7 @@ void orc_quotas(const uint64_t *C, const int32_t *bounds, int32_t n_seg, int32_t
     for (int i = 0; i < n_seg; ++i) {
         const int32_t L = bounds[i + 1] - bounds[i];
         int64_t qi = qmin[i];
-        if (Trem >= 0) qi += (int64_t)((2 * (uint64_t)Trem * M[i] + SH) / (2 * SH));
+        if (Trem >= 0 && SH > 0) qi += (int64_t)((2 * (uint64_t)Trem * M[i] + SH) / (2 * SH));
         if (qi > L) qi = L;
         q[i] = (int32_t)qi;
         sum_q += qi;

@@ -151,16 +151,17 @@ __device__ __forceinline__ void walk_pieces(int T, F f)
     }
 }
 
-// Sum over a warp of integers below 2^51 whose total is below 2^53: two reductions of 32 bits, where five steps of two shuffles
-// and an addition take five times as long.
+// Sum over a warp of any 64-bit integers, modulo 2^64: three reductions of 32 bits (22 + 22 + 20 bits of each), where five steps of
+// two shuffles and an addition take several times as long.
 __device__ __forceinline__ u64 warp_sum_wide(u64 v)
 {
-    const unsigned lo = __reduce_add_sync(kFull, (unsigned)v & 0x3ffffffu), hi = __reduce_add_sync(kFull, (unsigned)(v >> 26));
-    return ((u64)hi << 26) + lo;
+    const unsigned lo = __reduce_add_sync(kFull, (unsigned)v & 0x3fffffu), mid = __reduce_add_sync(kFull, (unsigned)(v >> 22) & 0x3fffffu),
+                   hi = __reduce_add_sync(kFull, (unsigned)(v >> 44));
+    return ((u64)hi << 44) + ((u64)mid << 22) + lo;
 }
 // Block-wide sum of doubles v that are multiples of 1 / scale (a power of two) and whose sum has fewer than 53 bits of it, times
-// scale: exact, hence independent of the order.  They are added as integers (the images of 131072 tokens below 2^53 in all, a
-// quarter of that to a warp) unless a credit that the caller restored is negative or not a number.
+// scale: exact, hence independent of the order.  They are added as integers (the images of 131072 tokens below 2^53 in all)
+// unless a credit that the caller restored is negative or not a number.
 __device__ __forceinline__ double block_sum_images(double v, double scale, u64 *scratch)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -354,15 +355,16 @@ __device__ __forceinline__ u64 mass_before(const Mass &ms, const u64 *wsum, int 
     return wsum[b >> 5] + warp_sum_mass(lane < (b & 31) ? ms.at((b & ~31) + lane) : 0ull);
 }
 
-// Boundary after the token that reaches `thr` (0 < thr <= total), by one warp.
+// Boundary after the token that reaches `thr` (at most the total), by one warp.  Always from 0 to the last window's end, whatever
+// the sums are: a total of 0 (no credit and ema_beta = 0) has thresholds of 0, below which no window starts.
 __device__ __forceinline__ int mass_cut(const Mass &ms, const u64 *wsum, int T, u64 thr)
 {
     const int lane = threadIdx.x & 31;
     int w = 0; // the last window that starts below thr: a lane to each of 32 places at a time (the windows' sums ascend from 0)
     for (int n = (T + 31) >> 5; n > 1;) {
         const int step = (n + 31) >> 5, at = lane * step;
-        const unsigned below = __ballot_sync(kFull, at < n && wsum[w + at] < thr); // (lane 0's always)
-        const int i = 31 - __clz(below);
+        const unsigned below = __ballot_sync(kFull, at < n && wsum[w + at] < thr);
+        const int i = below ? 31 - __clz(below) : 0;
         w += i * step;
         n = min(step, n - i * step);
     }
@@ -553,7 +555,7 @@ __device__ int segments_and_quotas(const DevParams &p, int T, int Bq, const Mass
         if (i >= n_seg) break;
         const int L = bounds[i + 1] - bounds[i];
         long long qi = max(0, min(p.q_min, L));
-        if (Trem >= 0) qi += (long long)quotient(2ull * (u64)Trem * M[j] + SHq, 2ull * SHq, inv);
+        if (Trem >= 0 && SHq > 0) qi += (long long)quotient(2ull * (u64)Trem * M[j] + SHq, 2ull * SHq, inv); // (no mass: equal shares)
         if (qi > L) qi = L;
         Ms[i] = M[j];
         quota[i] = (int)qi;
