@@ -151,13 +151,13 @@ __device__ __forceinline__ void walk_pieces(int T, F f)
     }
 }
 
-// Sum over a warp of any 64-bit integers, modulo 2^64: three reductions of 32 bits (22 + 22 + 20 bits of each), where five steps of
-// two shuffles and an addition take several times as long.
+// Sum over a warp of integers below 2^51 whose total is below 2^53: two reductions of 32 bits, where five steps of two shuffles
+// and an addition take five times as long.  (A credit that the caller restored with negative entries makes larger masses: their
+// sum is some number then, and so are the cuts and shares, within the bounds that these keep for any.)
 __device__ __forceinline__ u64 warp_sum_wide(u64 v)
 {
-    const unsigned lo = __reduce_add_sync(kFull, (unsigned)v & 0x3fffffu), mid = __reduce_add_sync(kFull, (unsigned)(v >> 22) & 0x3fffffu),
-                   hi = __reduce_add_sync(kFull, (unsigned)(v >> 44));
-    return ((u64)hi << 44) + ((u64)mid << 22) + lo;
+    const unsigned lo = __reduce_add_sync(kFull, (unsigned)v & 0x3ffffffu), hi = __reduce_add_sync(kFull, (unsigned)(v >> 26));
+    return ((u64)hi << 26) + lo;
 }
 // Block-wide sum of doubles v that are multiples of 1 / scale (a power of two) and whose sum has fewer than 53 bits of it, times
 // scale: exact, hence independent of the order.  They are added as integers (the images of 131072 tokens below 2^53 in all)
@@ -297,7 +297,7 @@ __device__ u64 mass_of_unit(const DevParams &p, int uid, int T, float *credit, u
                 for (int j = 0; j < kPer; ++j) sc += (double)fixed_trunc_by_add(c[j], ms.cut_c);
             });
             const double SC = block_sum_images(sc, scale_c, sh.scratch);
-            ms.have_credit = SC > 0.0;
+            ms.have_credit = SC > 0.0 && SC < (double)INFINITY; // (a restored credit may be infinite: it has no shares)
             if (ms.have_credit) ms.inv_sc_c = __dmul_rn(__ddiv_rn(1.0, SC), scale_c);
         }
     } else if (mass_dbg) {
@@ -554,12 +554,12 @@ __device__ int segments_and_quotas(const DevParams &p, int T, int Bq, const Mass
         const int i = j * NT + tid;
         if (i >= n_seg) break;
         const int L = bounds[i + 1] - bounds[i];
-        long long qi = max(0, min(p.q_min, L));
-        if (Trem >= 0 && SHq > 0) qi += (long long)quotient(2ull * (u64)Trem * M[j] + SHq, 2ull * SHq, inv); // (no mass: equal shares)
-        if (qi > L) qi = L;
+        int qi = max(0, min(p.q_min, L));
+        if (Trem >= 0 && SHq > 0) // (no mass: equal shares)
+            qi += (int)min((u64)(L - qi), quotient(2ull * (u64)Trem * M[j] + SHq, 2ull * SHq, inv)); // at most L, whatever the masses are
         Ms[i] = M[j];
-        quota[i] = (int)qi;
-        sq += (int)qi;
+        quota[i] = qi;
+        sq += qi;
     }
     const int Dq = Bq - block_count<NT>(sq, round, sh);
     if (Dq != 0) {

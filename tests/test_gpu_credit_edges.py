@@ -1,4 +1,4 @@
-"""Credit rows that say nothing: a restored credit that is negative or not a number throughout is left out of the mass, and with
+"""Credit rows that say nothing: a restored credit that is negative or not a number throughout, or infinite anywhere, is left out of the mass, and with
 ema_beta = 0 the unit then has no mass at all (every threshold of the cut search is 0, every share of the budget too)."""
 import numpy as np
 import pytest
@@ -24,7 +24,11 @@ def _event(kw, beta, fill):
     comp = binding.AmsCompressor(binding.config_for(wl), "cuda:0")
     rng = np.random.default_rng(17)
     ext = np.exp(2.0 * rng.standard_normal((wl.n_layers, wl.batch, wl.n_kv_heads, wl.max_seq_len))).astype(np.float32)
-    comp.ema_state.fill_(fill)
+    if fill == "one":
+        comp.ema_state.uniform_(0.0, 1e-3)
+        comp.ema_state[..., 300] = float("inf")
+    else:
+        comp.ema_state.fill_(fill)
     snap, credit0 = HostSnapshot(cache), comp.ema_state.cpu().numpy()
     dst = inputs.alloc_dst_pages(cache)
     dbg = gpu_event(comp, cache, dst, inputs.SCORER_EXTERNAL, torch.from_numpy(ext).to("cuda:0"))
@@ -42,11 +46,12 @@ def test_negative_credit(kw, beta):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("fill", [float("nan"), float("inf"), "one"])
 @pytest.mark.parametrize("beta", [0.0, 0.9])
 @pytest.mark.parametrize("kw", SHAPES)
-def test_credit_that_is_not_a_number(kw, beta):
-    """Kept rows as with a negative credit; the credit itself stays what it is."""
-    wl, cache, comp, snap, credit0, dst, dbg, ext = _event(kw, beta, float("nan"))
+def test_credit_that_is_not_finite(kw, beta, fill):
+    """Kept rows as with a negative credit; the credit itself stays what it is.  "one": one infinite token in each unit."""
+    wl, cache, comp, snap, credit0, dst, dbg, ext = _event(kw, beta, fill)
     prm = oracle.Params(wl.n_segments, wl.l_min, wl.l_max, wl.q_min, wl.n_sink, wl.n_last, wl.ema_lambda, beta, wl.eps)
     res = oracle.compress(snap.k, snap.v, snap.table, snap.lens, None, np.full_like(credit0, -1.0), wl.budget, prm,
                           oracle.SCORER_EXTERNAL, dst, ext_scores=ext, threads=8)
@@ -54,7 +59,8 @@ def test_credit_that_is_not_a_number(kw, beta):
     for u, r in res.items():
         assert (keep[u] == r.keep_idx).all(), u
     assert (inputs.as_u16(cache.k_pages) == snap.k).all() and (inputs.as_u16(cache.v_pages) == snap.v).all()
-    assert bool(torch.isnan(comp.ema_state[..., :wl.budget]).all())
+    if fill != "one":
+        assert not bool(torch.isfinite(comp.ema_state[..., :wl.budget]).any())
 
 
 def test_oracle_shares_equally_where_there_is_no_mass():
