@@ -72,12 +72,15 @@ struct DevParams {
     unsigned char *group_part;        // and the slots of what they exchange
     int *move_count;                  // ticket counter, parts of the row moves finished, and per (layer, sequence) the units selected;
                                       // cleared by the first kernel of an event
-    int *seq_bad;                     // [B]: set when a unit of the sequence, or for all of them a scorer, reported a device-side
-                                      // error: what follows leaves the sequence as it is
+    int *seq_bad;                     // [B]: kBad* flags of a reported device-side error: what follows leaves the sequence as it is
     int *status;                      // [4]: code, unit, a, b
     uint32_t expire_polls;            // test hook: a wait of this event's scorer is for something that never comes, and gives up
                                       // after so many polls (0: off)
 };
+
+// kBadScores is set by scorers alone, for all sequences, so it cannot change while units are selected: the threads of a block that
+// read it there agree.  kBadUnit may be set by other blocks of the same launch at any time.
+enum { kBadScores = 1, kBadUnit = 2 };
 
 __device__ __forceinline__ void set_status(int *status, int code, int unit, int a, int b)
 {
@@ -92,7 +95,7 @@ __device__ __forceinline__ void set_status(int *status, int code, int unit, int 
 __device__ __forceinline__ void report_timeout(const DevParams &p, int a, int b)
 {
     set_status(p.status, AMS_ERR_TIMEOUT, blockIdx.x, a, b);
-    for (int i = 0; i < p.B; ++i) p.seq_bad[i] = 1;
+    for (int i = 0; i < p.B; ++i) p.seq_bad[i] = kBadScores;
 }
 
 __device__ __forceinline__ int seq_len_of(const DevParams &p, int b) { return p.seq_lens ? p.seq_lens[b] : p.fixed_len; }

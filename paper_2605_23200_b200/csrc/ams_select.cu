@@ -1108,7 +1108,7 @@ __device__ __forceinline__ void select_unit(const DevParams &p, int longs, int u
     constexpr int NW = NT / 32, kList = Tune<NT>::kList;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int h = uid % p.H, bq = (uid / p.H) % p.B, l = uid / (p.H * p.B);
-    const int T = seq_len_of(p, bq), bad = p.seq_lens ? p.seq_bad[bq] : 0; // (the allocation-free entry point has no scorer and keeps its flags)
+    const int T = seq_len_of(p, bq), bad = p.seq_lens ? p.seq_bad[bq] & kBadScores : 0; // (the allocation-free entry point has no scorer)
     if (T <= p.Tk || T > p.T_cap || bad) return; // (bad: no scores to go by)
     const int sc = p.seg_cap;
     const SelSmem mp = sel_smem<NT>(p.T_cap, sc, p.S, longs != 0);
@@ -1140,7 +1140,7 @@ __device__ __forceinline__ void select_unit(const DevParams &p, int longs, int u
     const int n_seg = segments_and_quotas<NT>(p, T, p.Tk - ns - nl, ms, wsum, SH, reinterpret_cast<u64 *>(dyn + mp.ms), bounds, quota,
                                               reinterpret_cast<int *>(dyn + mp.hist), sh, round);
     if (n_seg < 0) { // cannot happen with the capacity formula of the header; reported all the same
-        if (tid == 0) { set_status(p.status, AMS_ERR_CAPACITY, uid, sh.n_seg, sc); p.n_seg[uid] = -1; p.seq_bad[bq] = 1; }
+        if (tid == 0) { set_status(p.status, AMS_ERR_CAPACITY, uid, sh.n_seg, sc); p.n_seg[uid] = -1; atomicOr(&p.seq_bad[bq], kBadUnit); }
         return;
     }
     __syncthreads();
@@ -1295,7 +1295,7 @@ __device__ __forceinline__ void select_unit(const DevParams &p, int longs, int u
     int pos = warp_sum(lane < warp ? sh.wc[0][lane] : 0);
     const int total = warp_sum(lane < NW ? sh.wc[0][lane] : 0);
     if (total != p.Tk) {
-        if (tid == 0) { set_status(p.status, AMS_ERR_INTERNAL, uid, total, p.Tk); p.seq_bad[bq] = 1; }
+        if (tid == 0) { set_status(p.status, AMS_ERR_INTERNAL, uid, total, p.Tk); atomicOr(&p.seq_bad[bq], kBadUnit); }
         return;
     }
     for (int g0 = w0; g0 < w1; g0 += 32) {
@@ -1408,7 +1408,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_move(DevParams p, int 
             bad = __ldcg(p.seq_bad + b);
             if (have < p.H && !bad) { // cannot happen; the wait is bounded all the same
                 set_status(p.status, AMS_ERR_INTERNAL, group * p.H, have, p.H);
-                for (int i = 0; i < p.B; ++i) p.seq_bad[i] = 1;
+                for (int i = 0; i < p.B; ++i) atomicOr(&p.seq_bad[i], kBadUnit);
             }
             sh.level = have >= p.H && !bad;
         }

@@ -3,7 +3,8 @@ and leaves pages, table, lengths and credit alone, and the next event on the han
 import pytest
 import torch
 
-from helpers import HostSnapshot, compare_event, gpu_event
+import oracle
+from helpers import HostSnapshot, compare_event, gpu_event, params_of
 from paper_2605_23200_b200 import binding, inputs
 
 pytestmark = pytest.mark.gpu
@@ -53,3 +54,43 @@ def test_a_wait_that_runs_out_inside_a_scorer(kw, polls):
     compare_event(snap, cache, comp, dbg, dst, credit0, dbg.scores.cpu().numpy(), units=units)
     with pytest.raises(binding.AmsError):
         comp.expire_event(0)
+
+
+JOINT = dict(n_layers=37, batch=12, seq_len_min=520, seq_len_max=900, budget=460)  # 1776 units: selection and moves in one launch
+
+
+@pytest.mark.parametrize("kw,launches", [
+    (dict(cfg=3, n_q_heads=32, n_kv_heads=4, l_max=256, **JOINT), 3),                                            # key-only scores
+    (dict(cfg=2, n_q_heads=28, n_kv_heads=4, window=1, **JOINT), 3),                                             # 7 rows
+    (dict(cfg=2, n_q_heads=32, n_kv_heads=4, window=16, **JOINT), 4),                                            # 128 rows
+    (dict(cfg=2, n_q_heads=28, n_kv_heads=4, window=1, n_layers=2, batch=5, seq_len_min=700, seq_len_max=3000, budget=512), 4),  # moves of their own
+])
+def test_a_scorer_that_gave_up_without_views(kw, launches):
+    """Nothing changes, and the next event on the handle, without views too, is the oracle's."""
+    kw = dict(kw)
+    wl = inputs.CONFIGS[kw.pop("cfg")].scaled(resident_layers=0, **kw)
+    cache = inputs.make_cache(wl, DEV)
+    comp = binding.AmsCompressor(binding.config_for(wl), DEV)
+    comp.ema_state.uniform_(0.0, 1e-3)
+    dst_np = inputs.alloc_dst_pages(cache)
+    dst = torch.from_numpy(dst_np).to(DEV)
+    own = [cache.k_pages, cache.v_pages, cache.block_table, cache.seq_lens, comp.ema_state]
+    before = [t.clone() for t in own]
+    comp.expire_event(3)
+    comp.compress(cache.k_pages, cache.v_pages, cache.block_table, cache.seq_lens, cache.obs_queries if wl.window else None, wl.budget,
+                  wl.n_segments, wl.scorer_id, dst)
+    assert comp.last_launch_count == launches
+    assert comp.status(check=False)[0] == binding.AMS_ERR_TIMEOUT
+    for t, b in zip(own, before):
+        raw = torch.int16 if t.element_size() == 2 else torch.int32
+        assert torch.equal(t.view(raw), b.view(raw))
+    ext = torch.rand((wl.n_layers, wl.batch, wl.n_kv_heads, wl.max_seq_len), device=DEV)
+    snap, credit = HostSnapshot(cache), comp.ema_state.cpu().numpy()
+    comp.compress(cache.k_pages, cache.v_pages, cache.block_table, cache.seq_lens, None, wl.budget, wl.n_segments,
+                  binding.AMS_SCORER_EXTERNAL, dst, ext_scores=ext)
+    comp.status()
+    oracle.compress(snap.k, snap.v, snap.table, snap.lens, None, credit, wl.budget, params_of(wl), oracle.SCORER_EXTERNAL, dst_np,
+                    ext_scores=ext.cpu().numpy(), threads=8)
+    assert (inputs.as_u16(cache.k_pages) == snap.k).all() and (inputs.as_u16(cache.v_pages) == snap.v).all()
+    assert (cache.block_table.cpu().numpy() == snap.table).all() and (cache.seq_lens.cpu().numpy() == snap.lens).all()
+    assert wl.ema_beta == 1.0 or (comp.ema_state.cpu().numpy() == credit).all()
