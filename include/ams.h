@@ -48,8 +48,11 @@
  * one whose block-table row or replacement pages name a page outside [0, num_pages)
  * (AMS_ERR_INVALID_ARG, detail = sequence, index in the row, page id) is skipped
  * entirely: its pages, table row, length and credit stay as they were.  A bounded
- * wait that ran out is AMS_ERR_TIMEOUT; the scores are then incomplete, and no sequence
- * of the event is compressed: all pages, table rows, lengths and credit stay as they were.  The library serves any number of devices
+ * wait that ran out is AMS_ERR_TIMEOUT.  In a scorer: the scores are then incomplete, and no sequence
+ * of the event is compressed: all pages, table rows, lengths and credit stay as they were.  In the row moves
+ * (detail = unit, units of its layer and sequence that are selected, units waited for), as with AMS_ERR_INTERNAL
+ * of a unit: the sequence keeps its live pages, table row and length, but credit rows of units that were
+ * selected have moved and its replacement pages may hold rows.  The library serves any number of devices
  * per process (launch state is kept per device); a handle belongs to the device that
  * was current when it was created.
  */
@@ -220,8 +223,8 @@ int ams_get_status(ams_state *st, void *stream, int32_t *detail);
 int ams_debug_expire_wait(ams_state *st, uint32_t polls, void *stream);
 
 /* The same inside an event: in the next ams_compress on this handle the scorer waits for something that never comes (an arrival
- * from one block more than share the work, or a free place that nobody frees) and gives up after `polls` polls (1 .. 2^20).  A
- * scorer without such waits runs as usual. */
+ * from one block more than share the work, or a free place that nobody frees) and gives up after `polls` polls (1 .. 2^20), and so
+ * do row moves that go along with the selection (for one unit more than there are).  What has no such waits runs as usual. */
 int ams_debug_expire_event(ams_state *st, uint32_t polls);
 
 /* Number of kernels the last ams_compress on this handle launched. */

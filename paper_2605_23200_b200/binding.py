@@ -234,7 +234,8 @@ class AmsCompressor:
             raise AmsError(rc, "ams_debug_expire_wait")
 
     def expire_event(self, polls: int = 1000) -> None:
-        """Failure-handling check: a wait inside the next event's scorer runs out after `polls` polls."""
+        """Failure-handling check: the waits of the next event's scorer, and of moves that go along with the selection, run out
+        after `polls` polls."""
         rc = lib().ams_debug_expire_event(self._h, polls)
         if rc != AMS_OK:
             raise AmsError(rc, "ams_debug_expire_event")

@@ -74,8 +74,8 @@ struct DevParams {
                                       // cleared by the first kernel of an event
     int *seq_bad;                     // [B]: kBad* flags of a reported device-side error: what follows leaves the sequence as it is
     int *status;                      // [4]: code, unit, a, b
-    uint32_t expire_polls;            // test hook: a wait of this event's scorer is for something that never comes, and gives up
-                                      // after so many polls (0: off)
+    uint32_t expire_polls;            // test hook: the waits of this event's scorer, and of moves that go along with the selection, are
+                                      // for something that never comes, and give up after so many polls (0: off)
 };
 
 // kBadScores is set by scorers alone, for all sequences, so it cannot change while units are selected: the threads of a block that

@@ -52,7 +52,7 @@ constexpr int kWarpBins = 128;      // bins of a warp's own histogram, four per 
 constexpr int kBatch = 64;          // long segments searched together
 constexpr int kMaxBins = 1024;      // histogram bins per long segment
 constexpr unsigned kOctaves = 12;   // octaves below a long segment's largest score that its histogram resolves
-constexpr int kMoveLimit = 1 << 22;  // polls of a move for the units that it needs, 100 ns and more each
+constexpr int kMoveLimit = 1 << 22; // polls of a move for the units that it needs: a second and more, as each goes to L2
 constexpr int kBest = 512;          // entries of the table of the pieces' best rejected keys
 
 // Working arrays of the search of long segments, one entry per segment of the batch.
@@ -1398,19 +1398,20 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_move(DevParams p, int 
     const int part = what - n_sel, group = part / plan.parts, b = group % p.B, T = p.seq_lens[b];
     if (T > p.Tk && T <= p.T_cap) {
         if (tid == 0) {
+            const int want = p.H + (p.expire_polls ? 1 : 0), limit = p.expire_polls ? (int)p.expire_polls : kMoveLimit;
             int have = 0, bad = 0;
-            for (int i = 0; i < kMoveLimit && !bad; ++i) {
+            for (int i = 0; i < limit && !bad; ++i) {
                 asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(have) : "l"(done + group) : "memory");
-                if (have >= p.H) break;
+                if (have >= want) break;
                 __nanosleep(100);
                 if ((i & 255) == 255) bad = __ldcg(p.seq_bad + b);
             }
             bad = __ldcg(p.seq_bad + b);
-            if (have < p.H && !bad) { // cannot happen; the wait is bounded all the same
-                set_status(p.status, AMS_ERR_INTERNAL, group * p.H, have, p.H);
-                for (int i = 0; i < p.B; ++i) atomicOr(&p.seq_bad[i], kBadUnit);
+            if (have < want && !bad) { // (only where the device stood still, or as a test)
+                set_status(p.status, AMS_ERR_TIMEOUT, group * p.H, have, want);
+                atomicOr(&p.seq_bad[b], kBadUnit);
             }
-            sh.level = have >= p.H && !bad;
+            sh.level = have >= want && !bad;
         }
         __syncthreads();
         if (sh.level) {

@@ -1,5 +1,6 @@
-"""A wait inside a scorer that runs out: every role of every block returns with its copies landed, the event reports AMS_ERR_TIMEOUT
-and leaves pages, table, lengths and credit alone, and the next event on the handle is exact.  The wait is made to run out by construction (for an arrival that nobody makes)."""
+"""A wait inside a scorer, or of the row moves, that runs out: every role of every block returns with its copies landed, the event
+reports AMS_ERR_TIMEOUT and leaves pages, table and lengths alone (a scorer also the credit), and the next event on the handle is exact.
+The wait is made to run out by construction (for an arrival that nobody makes)."""
 import pytest
 import torch
 
@@ -94,3 +95,34 @@ def test_a_scorer_that_gave_up_without_views(kw, launches):
     assert (inputs.as_u16(cache.k_pages) == snap.k).all() and (inputs.as_u16(cache.v_pages) == snap.v).all()
     assert (cache.block_table.cpu().numpy() == snap.table).all() and (cache.seq_lens.cpu().numpy() == snap.lens).all()
     assert wl.ema_beta == 1.0 or (comp.ema_state.cpu().numpy() == credit).all()
+
+
+@pytest.mark.parametrize("polls", [1, 300])
+def test_a_wait_of_the_moves_that_runs_out(polls):
+    """External scores, so that only the moves of the joint launch wait: table, lengths and live pages stay, and the next event is exact."""
+    wl = inputs.CONFIGS[2].scaled(resident_layers=0, n_q_heads=28, n_kv_heads=4, **JOINT)
+    cache = inputs.make_cache(wl, DEV)
+    short = 3
+    cache.seq_lens[short] = wl.budget - 5  # within the budget: its moves have nothing to wait for
+    comp = binding.AmsCompressor(binding.config_for(wl), DEV)
+    dst_np = inputs.alloc_dst_pages(cache)
+    dst = torch.from_numpy(dst_np).to(DEV)
+    ext = torch.rand((wl.n_layers, wl.batch, wl.n_kv_heads, wl.max_seq_len), device=DEV)
+    args = (cache.k_pages, cache.v_pages, cache.block_table, cache.seq_lens, None, wl.budget, wl.n_segments, binding.AMS_SCORER_EXTERNAL, dst)
+    before = [t.clone() for t in (cache.block_table, cache.seq_lens, cache.k_pages, cache.v_pages)]
+    comp.expire_event(polls)
+    comp.compress(*args, ext_scores=ext)
+    assert comp.last_launch_count == 2
+    rc, detail = comp.status(check=False)
+    assert rc == binding.AMS_ERR_TIMEOUT and detail[1] % wl.n_kv_heads == 0 and detail[3] == wl.n_kv_heads + 1
+    assert torch.equal(cache.block_table, before[0]) and torch.equal(cache.seq_lens, before[1])
+    assert torch.equal(cache.k_pages.view(torch.int16), before[2].view(torch.int16))  # (no part moved a row)
+    assert torch.equal(cache.v_pages.view(torch.int16), before[3].view(torch.int16))
+    snap, credit = HostSnapshot(cache), comp.ema_state.cpu().numpy()
+    comp.compress(*args, ext_scores=ext)
+    comp.status()
+    oracle.compress(snap.k, snap.v, snap.table, snap.lens, None, credit, wl.budget, params_of(wl), oracle.SCORER_EXTERNAL, dst_np,
+                    ext_scores=ext.cpu().numpy(), threads=8)
+    assert (inputs.as_u16(cache.k_pages) == snap.k).all() and (inputs.as_u16(cache.v_pages) == snap.v).all()
+    assert (cache.block_table.cpu().numpy() == snap.table).all() and (cache.seq_lens.cpu().numpy() == snap.lens).all()
+    assert (comp.ema_state.cpu().numpy() == credit).all()
