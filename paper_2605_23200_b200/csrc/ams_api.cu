@@ -101,7 +101,7 @@ static Layout make_layout(const ams_config *c)
     y.ex_logits = off;  off = align_up(off + (c->expected_scorer ? U * T * (size_t)(c->n_q_heads / c->n_kv_heads) * 4 : 0), 256);
     y.group_count = off; off = align_up(off + (size_t)2 * kGroupCounters * kGroupCounterPad * 4, 256);
     y.group_part = off;  off = align_up(off + (size_t)kGroupBlocks * 4 * kGroupSlot, 256);
-    y.move_count = off;  off = align_up(off + ((size_t)c->n_layers * c->max_batch + 2) * 4, 256);
+    y.move_count = off;  off = align_up(off + ((size_t)c->n_layers * c->max_batch + c->max_batch + 1) * 4, 256);
     y.src_pages = off;   off = align_up(off + (size_t)c->max_batch * (y.T_cap / kPage) * 4, 256);
     y.total = off;
     return y;

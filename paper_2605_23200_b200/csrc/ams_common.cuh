@@ -70,8 +70,8 @@ struct DevParams {
     int group_size;                   // blocks that work on a unit together: their number if the launcher sets it (a cluster);
     int *group_count;                 // counters, cleared by the first kernel of an event,
     unsigned char *group_part;        // and the slots of what they exchange
-    int *move_count;                  // ticket counter, parts of the row moves finished, and per (layer, sequence) the units selected;
-                                      // cleared by the first kernel of an event
+    int *move_count;                  // ticket counter, per sequence the parts of its row moves finished, per (layer, sequence) the units
+                                      // selected; cleared by the first kernel of an event
     int *seq_bad;                     // [B]: kBad* flags of a reported device-side error: what follows leaves the sequence as it is
     int *status;                      // [4]: code, unit, a, b
     uint32_t expire_polls;            // test hook: the waits of this event's scorer, and of moves that go along with the selection, are

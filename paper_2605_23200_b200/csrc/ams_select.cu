@@ -1357,8 +1357,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
 // HBM, so blocks doing the one run beside blocks doing the other.  A block takes a ticket from a counter when it starts: the first
 // `lag` are units to select, then units and parts of the moves in turn, the moves `lag` units behind, then what is left of
 // the moves.  A move waits for the units of its (layer, sequence), whose tickets all came before its own, to
-// blocks that are running or through: no wait needs a block that has not started.  Whoever finishes the last part rewrites the
-// table.  (Blocks that stay and take one ticket after the other need 200 to 800 bytes of spills, as the compiler keeps
+// blocks that are running or through: no wait needs a block that has not started.  Whoever finishes a sequence's last part rewrites
+// its row of the table, beside the others' moves (one block that rewrites 128 rows of 8192 entries at the end: event of 2048 units of 600 to 900 tokens 472 us, so 310, apart 341).  (Blocks that stay and take one ticket after the other need 200 to 800 bytes of spills, as the compiler keeps
 // what does not depend on the ticket in registers throughout.)
 struct MovePlan { int lag, parts, rows; }; // parts of a (layer, sequence), rows in each
 
@@ -1368,7 +1368,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_move(DevParams p, int 
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ SelShared sh;
     const int tid = threadIdx.x, groups = p.L * p.B, n_sel = groups * p.H, n_mov = groups * plan.parts;
-    int *finished = p.move_count + 1, *done = p.move_count + 2;
+    int *finished = p.move_count + 1, *done = finished + p.B;
     wait_for_previous_kernel(); // scores, effective lengths; the counters
     if (tid == 0) {
         const int t = atomicAdd(p.move_count, 1);
@@ -1419,18 +1419,15 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_move(DevParams p, int 
             move_rows<NT>(p, group / p.B, b, r0, min(p.Tk * p.H, r0 + plan.rows));
         }
         __syncthreads();
-    }
-    if (tid == 0) {
-        __threadfence();
-        sh.level = atomicAdd(finished, 1) == n_mov - 1;
-        __threadfence();
-    }
-    __syncthreads();
-    if (sh.level)
-        for (int i = 0; i < p.B; ++i) {
-            const int Ti = p.seq_lens[i];
-            if (Ti > p.Tk && Ti <= p.T_cap && !__ldcg(p.seq_bad + i)) update_table(p, i);
+        if (tid == 0) {
+            __threadfence();
+            sh.level = atomicAdd(finished + b, 1) == p.L * plan.parts - 1;
+            __threadfence();
+            if (sh.level && __ldcg(p.seq_bad + b)) sh.level = 0; // (no unit of the sequence is under way any more, or a move has flagged it)
         }
+        __syncthreads();
+        if (sh.level) update_table(p, b);
+    }
 }
 
 template <int NT>

@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(256) k_prepare(DevParams p, const int *lens_in
     wait_for_previous_kernel(); // the caller's table and lengths
     const int b = blockIdx.x;
     for (int i = b * blockDim.x + threadIdx.x; i < 2 * kGroupCounters; i += gridDim.x * blockDim.x) p.group_count[i * kGroupCounterPad] = 0;
-    for (int i = b * blockDim.x + threadIdx.x; i < p.L * p.B + 2; i += gridDim.x * blockDim.x) p.move_count[i] = 0;
+    for (int i = b * blockDim.x + threadIdx.x; i < p.L * p.B + p.B + 1; i += gridDim.x * blockDim.x) p.move_count[i] = 0;
     const int T = lens_in[b];
     int eff = 0;
     if (T > p.Tk) {
