@@ -1359,7 +1359,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_select_compact(DevParams p, i
 // the moves.  A move waits for the units of its (layer, sequence), whose tickets all came before its own, to
 // blocks that are running or through: no wait needs a block that has not started.  Whoever finishes a sequence's last part rewrites
 // its row of the table, beside the others' moves (one block that rewrites 128 rows of 8192 entries at the end: event of 2048 units of 600 to 900 tokens 472 us, so 310, apart 341).  (Blocks that stay and take one ticket after the other need 200 to 800 bytes of spills, as the compiler keeps
-// what does not depend on the ticket in registers throughout.)
+// what does not depend on the ticket in registers throughout; this form spills 64 to 68.  `longs` is 0 in every launch, but not for
+// the compiler: with that known it spills 28 to 36 bytes and orders the moves' loads so that 1792 units of 4224 tokens, budget 4096,
+// take 1789 instead of 1335 us.)
 struct MovePlan { int lag, parts, rows; }; // parts of a (layer, sequence), rows in each
 
 template <int NT>
@@ -1440,21 +1442,22 @@ cudaError_t launch_nt(const DevParams &p, int units, bool longs, LaunchCtx &ctx)
 }
 
 template <int NT>
-cudaError_t launch_move_nt(const DevParams &p, int units, bool longs, int fit, int n_sm, LaunchCtx &ctx)
+cudaError_t launch_move_nt(const DevParams &p, int units, int fit, int n_sm, LaunchCtx &ctx)
 {
     static SmemGrant grant;
-    const size_t smem = sel_smem<NT>(p.T_cap, p.seg_cap, p.S, longs).total;
+    const size_t smem = sel_smem<NT>(p.T_cap, p.seg_cap, p.S, false).total;
     if (!grant_dynamic_smem(k_select_move<NT>, smem, grant)) return cudaErrorInvalidValue;
     const int blocks = fit * n_sm, n_rows = p.Tk * p.H;
     constexpr int kRound = NT / 4; // rows of one round of a block
-    MovePlan plan;
     const long long per = (long long)p.L * p.B * n_rows / (2LL * blocks); // two parts for each block where there is little to move
-    plan.rows = (int)std::min(1024LL, std::max((long long)kRound, per / kRound * kRound));
-    plan.parts = (n_rows + plan.rows - 1) / plan.rows;
+    const int most = (int)std::min(1024LL, std::max((long long)kRound, per / kRound * kRound));
+    MovePlan plan; // equal parts: with a remainder of its own (720 rows as 704 and 16), 2442 units of 400 tokens took 282 instead of 242 us
+    plan.parts = (n_rows + most - 1) / most;
+    plan.rows = (n_rows + plan.parts - 1) / plan.parts;
     plan.lag = std::min(units, std::max(blocks, 2 * p.H + 2));
     const long long tickets = units + (long long)p.L * p.B * plan.parts;
     if (tickets > 0x7fffffffLL) return cudaErrorInvalidValue;
-    return launch_after(k_select_move<NT>, dim3((unsigned)tickets), dim3(NT), smem, ctx.s, p, longs ? 1 : 0, plan);
+    return launch_after(k_select_move<NT>, dim3((unsigned)tickets), dim3(NT), smem, ctx.s, p, 0, plan);
 }
 
 constexpr size_t kSmShared = 228 * 1024, kBlockReserve = 1024; // shared memory of an SM; what each block takes besides its own
@@ -1481,18 +1484,24 @@ int launch_segsel(const DevParams &p, LaunchCtx &ctx, bool *moved)
               f1024 = fits(1024, sel_smem<1024>(p.T_cap, p.seg_cap, p.S, longs).total);
     auto cost = [&](int nt, int fit) { return ((long long)units + fit * n_sm - 1) / (fit * n_sm) * (p.T_cap / nt + 24); };
     const long long c256 = cost(256, f256), c512 = cost(512, f512), c1024 = cost(1024, f1024);
-    // The moves go along with the selection where there is something to run beside (three rounds of units at least, chosen in
-    // registers) and enough to move to pay for the tickets (some 5 % of a unit of 1024 tokens).  Events, apart / together: 1792 units of
-    // 8192 to 32768 tokens, budget 4096, 3361 / 3267 us; 2048 of 1900 to 9001, 1000: 1357 / 1324; 3024 of 1169 to 3146, 967: 904 / 863;
-    // 3456 of 4728, 461: 1308 / 1232; 17672 of 1024 tokens, budget 69, 1028 / 1183; 1944 of 694 to 1024, 152: 240 / 267.
-    // 2048 units in long segments 1176 / 1224 (selection and moves).
-    const int fit = c256 <= c512 && c256 <= c1024 ? f256 : c512 <= c1024 ? f512 : f1024;
-    move = move && !longs && p.Tk >= 320 && units >= 3LL * fit * n_sm;
+    const int nt = c256 <= c512 && c256 <= c1024 ? 256 : c512 <= c1024 ? 512 : 1024, fit = nt == 256 ? f256 : nt == 512 ? f512 : f1024;
+    // Selection and moves in one launch, by figures of events apart / together / (apart, before there was a joint launch), us.  The host
+    // knows the capacity, not the lengths, so the line lies where lengths just above the budget, which leave least to run beside, do not lose:
+    // - 12 units per SM: 1184 units of 4224 tokens, budget 4096, 874 / 904 / (876); 1776 of 4096, 2048: 716 / 701 / (719); 1792 of
+    //   8192 to 32768, 4096: 1611 / 1485 / (1619); 2048 of 1900 to 9001, 1000: 497 / 456 / (506).
+    // - Two blocks to an SM, so that both kinds are on it: 640 units under 131072 tokens take blocks of 1024, 8704 tokens, 8192: 970 / 1005 /
+    //   (983); 444 of 65536, 512: 339 / 396 / (340); 640 of 131072, 8192, that gain (1848 / 1691) are given up for those.
+    //   Long segments (2048 units, 1176 / 1224) leave room for one block as well.
+    // - A budget that pays for the tickets: 600 tokens, 1792 units, four heads, 320: 184 / 171 / (190), one head: 192 / 174 / (195); 3584
+    //   units, one head, 320: 353 / 380 / (360); 2664, four heads, 360: 273 / 281 / (280); 400: 292 / 286 / (299).
+    // - The separate moves read a token's rows of all heads together, which from 8 heads on is 2 KB in a piece and as fast as copying;
+    //   selection of few units then hides less than the joint moves lose: 2560 units of 4136 tokens, 8 heads, 4096: 1853 / 1875 /
+    //   (1864); 2088, 2048: 972 / 969 / (979); 8704, 8192, 8 heads: 3651 / 3700 / (3666), 4 heads: 3778 / 3702 / (3784).
+    move = move && !longs && fit >= 2 && units >= 12LL * n_sm && p.Tk >= (units < 16LL * n_sm ? 320 : 400) && (p.H <= 4 || p.Tk <= 128LL * units / n_sm);
     if (moved) *moved = move;
-    cudaError_t e;
-    if (c256 <= c512 && c256 <= c1024) e = move ? launch_move_nt<256>(p, units, longs, f256, n_sm, ctx) : launch_nt<256>(p, units, longs, ctx);
-    else if (c512 <= c1024) e = move ? launch_move_nt<512>(p, units, longs, f512, n_sm, ctx) : launch_nt<512>(p, units, longs, ctx);
-    else e = move ? launch_move_nt<1024>(p, units, longs, f1024, n_sm, ctx) : launch_nt<1024>(p, units, longs, ctx);
+    const cudaError_t e = nt == 256 ? (move ? launch_move_nt<256>(p, units, fit, n_sm, ctx) : launch_nt<256>(p, units, longs, ctx))
+                        : nt == 512 ? (move ? launch_move_nt<512>(p, units, fit, n_sm, ctx) : launch_nt<512>(p, units, longs, ctx))
+                                    : launch_nt<1024>(p, units, longs, ctx);
     if (e != cudaSuccess) return AMS_ERR_CUDA;
     ctx.mark(kKernSelect);
     return AMS_OK;
