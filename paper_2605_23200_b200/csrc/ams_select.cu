@@ -1132,8 +1132,6 @@ __device__ __forceinline__ void select_unit(const DevParams &p, int longs, int u
     for (int i = tid; i < kBest; i += NT) best[i] = 0u;
     if (tid == 0) { sh.n_list = 0; sh.n_look = 0; sh.bound = 0u; }
     float *credit = p.ema ? p.ema + (((size_t)l * p.Bmax + bq) * p.H + h) * (size_t)p.T_cap : nullptr;
-    if (p.beta != 1.0f) // on its way from HBM while the weights are summed
-        for (int t = tid * 32; t < T; t += NT * 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(credit + t));
     Mass ms;
     u64 *wsum = reinterpret_cast<u64 *>(dyn + mp.list);
     const u64 SH = mass_of_unit<NT>(p, uid, T, credit, wsum, ms, sh);
