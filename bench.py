@@ -60,21 +60,20 @@ def _peaks():
     return {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "sm_max_mhz": 1965.0, "kind": "fallback"}
 
 
-# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per launch from ncu captures summarised under
-# profiles/ (workload -> kernel slot -> bytes per launch).  A kernel or workload without a capture of the
-# current code reports null.
+# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) per launch from ncu captures (workload -> kernel slot ->
+# bytes per launch).  A kernel or workload without a capture of the current code reports null.
 NCU_TRAFFIC_BYTES: dict = {
-    # two-layer capture (profiles/tc_scorer_cfg4_2layers_ncu_full.md) x 40: the 80-layer launch holds 50 GB, too much to
-    # capture under full counters; units are independent and each is read once per pass, so traffic grows with the layers
-    "cfg4_llama70b_L80_T131072_k8192_w64": {"score_phase1": 40 * (540_616_448 + 6_414_080),
-                                            "score_phase2": 40 * (542_741_760 + 11_199_488)},
-    # captured at the timed size (profiles/tc_scorer_cfg1_32layers_ncu_full.md, profiles/gather_cfg1_cfg2_ncu_full.md)
-    "cfg1_llama8b_L32_T16384_k2048_w32": {"score_phase1": 1_089_513_472 + 14_958_336,
-                                          "score_phase2": 1_090_619_136 + 20_133_632,
-                                          "gather": 270_614_528 + 219_303_168},
-    # capture of one layer and half of the sequences x 8 (profiles/group_scorers_ncu.md)
+    # two-layer capture x 40: the 80-layer launch holds 50 GB, too much to capture under full counters; units are
+    # independent and each is read once per pass, so traffic grows with the layers
+    "cfg4_llama70b_L80_T131072_k8192_w64": {"score_phase1": 40 * (540_276_224 + 7_217_152),
+                                            "score_phase2": 40 * (542_973_952 + 14_032_384)},
+    # captured at the timed size
+    "cfg1_llama8b_L32_T16384_k2048_w32": {"score_phase1": 1_089_468_928 + 14_519_552,
+                                          "score_phase2": 1_090_427_392 + 18_597_376,
+                                          "gather": 270_609_408 + 222_114_816},
+    # capture of one layer and half of the sequences x 8
     "cfg3_qwen3_8b_L36_B64_T32768_k2048_keydiff": {"score_phase1": 8 * (2_159_701_504 + 37_753_856)},
-    # four-layer capture x 8 (profiles/expected_attention_cfg5_4layers_ncu_full.md)
+    # four-layer capture x 8
     "cfg5_llama8b_L32_T16384_k2048_expected": {"score_phase1": 8 * (138_547_456 + 6_842_624),
                                                "score_phase2": 8 * (142_662_656 + 4_295_936)},
 }
@@ -245,20 +244,21 @@ SELECT_SLOTS = ("select_compact",)
 def roofline_of(wl, kern_ms, k_read, moved, lens, peaks, traffic=None):
     """Roofline object of the dominant kernel that has an algorithmic byte (or operation) count: the scorer
     passes (K bytes; exponentials and tensor flops when the query block is wide) and the gather (kept rows).
-    The selection kernels read no K/V byte; if one of them is the longest kernel the note says so."""
+    The selection kernel reads no K/V byte; if it is the longest kernel the note says so, unless it moves the kept rows as well
+    (many units: no launch of the gather's own), when it counts with those bytes."""
     if not kern_ms:
         return None
     overall = max(kern_ms, key=kern_ms.get)
-    cands = {k: v for k, v in kern_ms.items() if k in ("score_phase1", "score_phase2", "gather")}
+    joint = "gather" not in kern_ms and "select_compact" in kern_ms and moved > 0
+    cands = {k: v for k, v in kern_ms.items() if k in ("score_phase1", "score_phase2", "gather") or (joint and k == "select_compact")}
     dom = max(cands, key=cands.get)
     ms = cands[dom]
     rows = wl.group * max(wl.window, 1)
     note = []
     if overall != dom:
-        what = "which selects and moves the kept rows in one launch" if overall == "select_compact" and not kern_ms.get("gather") else "which moves no K/V byte"
-        note.append(f"longest kernel of the step is {overall} ({kern_ms[overall]:.4f} ms), {what}; the roofline is "
-                    f"quoted for the longest kernel that only streams")
-    if dom == "gather":
+        note.append(f"longest kernel of the step is {overall} ({kern_ms[overall]:.4f} ms), which moves no K/V byte; the roofline is "
+                    f"quoted for the longest kernel that does")
+    if dom in ("gather", "select_compact"):
         bytes_launch, bound = moved, "hbm"
     elif wl.scorer_id == 3 and dom == "score_phase1":
         # K once (the V pass is the other scorer kernel); 2 * 128 * 128 flops per (query head, token) on the tensor pipe
@@ -299,6 +299,10 @@ def roofline_of(wl, kern_ms, k_read, moved, lens, peaks, traffic=None):
         note.append("512 query rows per KV head: the pass takes one exp2 per (row, token) on the special-function unit "
                     "(16 results per clock and SM x 148 SMs x the maximum SM clock = peak) and is bound by it before HBM; "
                     "hbm and tensor fractions of the same launch are under 'also'")
+    if joint:
+        gbs = moved / (kern_ms["select_compact"] * 1e-3) / 1e9
+        out["select_and_move"] = {"algorithmic_bytes_per_launch": moved, "achieved": gbs, "unit": "GB/s", "frac": gbs / peaks["hbm_gbs"]}
+        note.append("select_and_move: kept rows read and written by the launch that also selects them, over its whole duration")
     out["note"] = "; ".join(note)
     return out
 

@@ -208,7 +208,7 @@ int ams_set_query_stats(ams_state *st, const float *q_mean, const void *q_cov, f
  * are such (key-only scores, windows below 64 query rows per KV head): they run on whatever SMs are free, beside kernels that
  * never leave theirs, and a sequence's scores do not depend on the other sequences of the call.  They read K twice and
  * take up to 1.7 times as long.  Default: off.  Wider windows and the expected-attention scorer need no two blocks
- * at the same time either way. */
+ * at the same time either way; row moves that go along with the selection wait for units, but only for such whose block has started. */
 int ams_set_independent_blocks(ams_state *st, int enable);
 
 /* Synchronises `stream`, then returns and clears the device status: AMS_OK or the

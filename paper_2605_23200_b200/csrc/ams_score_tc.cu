@@ -10,10 +10,11 @@
 //   warps 4-19  four consumer warpgroups: thread i of one owns TMEM lane i of a slot; from two query blocks on a warpgroup has a
 //               slot to itself and takes all 128 columns, with one block two share a slot (see there).  In the first phase the
 //               next 32 columns are on their way while it works on the last; the slot is free again as soon as its last columns
-//               are in registers.  At 512 rows the special-function unit is 80 % busy at the clock that the power limit leaves
-//               (1.69 GHz; two warpgroups to a slot, half of the columns each: 71 %): 640 units of 8704 tokens, statistics 963,
-//               now 873 us, usage 887, now 866; of 131072 tokens 15.4 and 13.8, now 13.6 and 13.5 ms.  Three warpgroups of 128
-//               registers, exponentials shared with the FMA pipe and tiles fetched ahead into L2 were no faster.
+//               are in registers.  At 512 rows the special-function pipe binds: 84 % (statistics) and 81 % (usage) of its peak
+//               while active, 16 layers of 16384 tokens in 669 us for both passes; with two warpgroups to a slot, half of the
+//               columns each, 76 and 79 %, 716 us.  In a loop of 640 units of 131072 tokens the power limit takes part of that
+//               back (1.72 GHz instead of 1.75): 13.97 + 13.75 ms against 15.27 + 13.68.  Three warpgroups of 128 registers,
+//               exponentials shared with the FMA pipe and tiles fetched ahead into L2 were no faster.
 // Phase 1 puts query rows on the TMEM lanes (A = Q, B = K), so a thread folds its row's
 // logits into a running (max, sum of 2^x) without leaving registers; phase 2 puts tokens
 // on the lanes (A = K, B = Q), so a thread sums 2^(x - b_r) over the query rows of its
