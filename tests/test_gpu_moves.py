@@ -62,6 +62,7 @@ def _event(wl, views, cap=0, seed=5):
     (dict(n_layers=37, batch=9, n_kv_heads=8, n_q_heads=8, seq_len_min=300, seq_len_max=900, budget=319), 3),
     (dict(n_layers=2, batch=3, n_kv_heads=8, n_q_heads=8, seq_len_min=300, seq_len_max=900, budget=257), 3),
     (dict(n_layers=37, batch=9, n_kv_heads=8, n_q_heads=8, seq_len_min=300, seq_len_max=900, budget=407, l_max=600), 3),
+    (dict(n_layers=37, batch=9, n_kv_heads=8, n_q_heads=8, seq_len_min=300, seq_len_max=900, budget=327, l_max=600), 3),
 ])
 def test_event_without_views_equals_event_with_views(kw, launches):
     kw = dict(kw)
@@ -77,9 +78,12 @@ def test_event_without_views_equals_event_with_views(kw, launches):
     assert int((b.seq_lens == wl.budget).sum()) > 0
 
 
-def test_bad_page_is_skipped_in_the_joint_launch():
-    """A sequence with a page outside the pool keeps its row and length; the others are compressed."""
-    wl = inputs.CONFIGS[2].scaled(resident_layers=0, n_layers=37, batch=9, n_kv_heads=8, n_q_heads=8, seq_len_min=420, seq_len_max=900, budget=407)
+@pytest.mark.parametrize("shortest,budget,launches", [(420, 407, 2), (400, 327, 3)])
+def test_bad_page_is_skipped_in_the_joint_launch(shortest, budget, launches):
+    """A sequence with a page outside the pool keeps its row and length; the others are compressed (with the smaller budget in separate
+    launches)."""
+    wl = inputs.CONFIGS[2].scaled(resident_layers=0, n_layers=37, batch=9, n_kv_heads=8, n_q_heads=8, seq_len_min=shortest, seq_len_max=900,
+                                  budget=budget)
     cache = inputs.make_cache(wl, DEV)
     comp = binding.AmsCompressor(binding.config_for(wl), DEV)
     ext = torch.rand((wl.n_layers, wl.batch, wl.n_kv_heads, wl.max_seq_len), device=DEV)
@@ -88,7 +92,7 @@ def test_bad_page_is_skipped_in_the_joint_launch():
     dst = torch.from_numpy(inputs.alloc_dst_pages(cache)).to(DEV)
     comp.compress(cache.k_pages, cache.v_pages, cache.block_table, cache.seq_lens, None, wl.budget, wl.n_segments,
                   binding.AMS_SCORER_EXTERNAL, dst, ext_scores=ext)
-    assert comp.last_launch_count == 2
+    assert comp.last_launch_count == launches
     rc, detail = comp.status(check=False)
     assert rc == binding.AMS_ERR_INVALID_ARG and detail[1:4] == [4, 3, cache.k_pages.shape[1]]
     assert torch.equal(cache.block_table[4], table[4]) and cache.seq_lens[4] == lens[4]
