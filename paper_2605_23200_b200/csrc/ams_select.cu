@@ -465,7 +465,7 @@ __device__ int segments_and_quotas(const DevParams &p, int T, int Bq, const Mass
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int *merged = tmp, *poff = merged + p.S + 1, *raw = poff + p.S + 1, *cap = raw + p.S + 1;
-    const u64 SHq = p.uniform_q ? (u64)T : SH; // total of what the quotas are proportional to
+    const u64 SHq = p.uniform_q ? (u64)T : max(SH, 1ull); // total of what the quotas are proportional to (no mass: nobody has a share)
     const double inv = 1.0 / (double)(2ull * SHq);
     const double inv_s = 1.0 / (double)p.S;
     // raw cuts, ascending: the token that reaches quantile k closes its segment, c(t) >= k / S <=> C(t) >= ceil(k SH / S)
@@ -554,12 +554,12 @@ __device__ int segments_and_quotas(const DevParams &p, int T, int Bq, const Mass
         const int i = j * NT + tid;
         if (i >= n_seg) break;
         const int L = bounds[i + 1] - bounds[i];
-        int qi = max(0, min(p.q_min, L));
-        if (Trem >= 0 && SHq > 0) // (no mass: equal shares)
-            qi += (int)min((u64)(L - qi), quotient(2ull * (u64)Trem * M[j] + SHq, 2ull * SHq, inv)); // at most L, whatever the masses are
+        u64 qi = (u64)max(0, min(p.q_min, L));
+        if (Trem >= 0) qi += quotient(2ull * (u64)Trem * M[j] + SHq, 2ull * SHq, inv);
+        if (qi > (u64)L) qi = (u64)L; // (whatever the masses are)
         Ms[i] = M[j];
-        quota[i] = qi;
-        sq += qi;
+        quota[i] = (int)qi;
+        sq += (int)qi;
     }
     const int Dq = Bq - block_count<NT>(sq, round, sh);
     if (Dq != 0) {
